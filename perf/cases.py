@@ -6,9 +6,9 @@ V^T with sigma geometric from 1 to 1/kappa and V Haar; U is a Gaussian m x n mat
 orthonormal columns for m >> n and is quick to draw.  Entries of A have full FP64 significands.  b = A x_true + noise
 of relative size rho.
 
-The calls write FP64 vectors whatever the working precision.  Where the caller asked for single working precision the
-program keeps the result in single, as the method delivers it (forward errors of a few units in the last place of
-single); sketches, FP64 factors and solves in double stay FP64.
+The calls write FP64 buffers whatever the precision they were computed in.  Where that was single (u_w or u_p single; a
+tensor-core sketch, which accumulates in FP32) the program keeps the result in single, as the method delivers it
+(forward errors of a few units in the last place of single); FP64 factors and solves in double stay FP64.
 """
 import math
 import random
@@ -189,7 +189,7 @@ def run(st):
     m, n, s = c["m"], c["n"], c["s"]
     if c["kind"] == "sketch":
         lsq.lsq_sketch(h, st["A"], st["b"], m, n, s, c["u_s"], "f32", "f32", "f64", 1.0, st["seed"], None, st["Y"])
-        return st["Y"]
+        return st["Y"].float()
     args = (h, st["A"], st["b"], m, n, s, c["u_s"], c["u_p"], c["u_w"], c["u_r"], c["tol"], st["seed"], None)
     out = F32 if c["u_w"] == "f32" else F64
     if c["kind"] == "lsqr":
