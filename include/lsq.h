@@ -114,10 +114,9 @@ typedef struct lsq_opts {
                              on the handle's stream (info->kern_ms / kern_launches) */
   int32_t no_graph;       /* 1: launch LSQR / FGMRES iteration batches directly instead of
                              replaying cached CUDA graphs (same arithmetic) */
-  int32_t sketch_exact;   /* 1: tensor-core sketch resolves the entries of fl_s(G) whose FP32
-                             estimate lies near a rounding midpoint inside the GEMM pipeline;
-                             0 (default): the GEMM uses the estimates and a correction kernel
-                             adds the exact differences afterwards (same product, faster) */
+  int32_t sketch_exact;   /* accepted, without effect: the tensor-core sketch multiplies fl_s(G)
+                             itself (entries whose FP32 estimate lies near a rounding midpoint
+                             are resolved inside the GEMM pipeline) */
   double gmres_tol;       /* FGMRES relative-residual tolerance; 0 -> tol */
   double kappa_hint;      /* kappa(A) for the escalation rule; 0 -> estimate from R */
   const double* Y_in;     /* optional device sketch, s x (n+1) column-major (ld = s):
@@ -371,8 +370,8 @@ lsq_status lsq_lsir_batched(lsq_handle* h, int32_t nprob, const lsq_problem* pro
 /*
  * lsq_omega -- the sketch operand fl_s(G)[i, j] for i in [0, s) and
  * j in [j0, j0 + cols), written as FP64 to `out` (device, row-major s x cols),
- * computed by the same device code the sketch kernels use (fast FP32
- * evaluation with the FP64 definition as fallback near rounding boundaries).
+ * computed by the same device code the sketch kernels use (FP32 estimate,
+ * double-float and the FP64 definition near rounding boundaries).
  * For testing that the in-kernel Gaussian is the defined one, bit for bit.
  */
 lsq_status lsq_omega(lsq_handle* h, int64_t s, int64_t j0, int64_t cols, lsq_prec u_s,

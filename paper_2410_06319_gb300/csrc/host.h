@@ -39,7 +39,6 @@ struct StatusFail {
   } while (0)
 
 constexpr int kBatch = 8;        // iterations enqueued between host checks
-constexpr size_t kRecMaxBytes = (size_t)4 << 30;   // deferred sketch-correction lists, at most
 constexpr int kMaxGmres = 127;   // cap of the FGMRES basis size
 
 struct Buf {

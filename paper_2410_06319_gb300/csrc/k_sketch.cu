@@ -368,14 +368,11 @@ cudaError_t launch_cast_transpose(int fmt, const double* A, int64_t lda, const d
 // ============================================================ tcgen05 sketch
 constexpr int kSkGenWarps = 16;
 constexpr int kSkGenThreads = kSkGenWarps * 32;
-constexpr int kSkFixWarps = 2;                // resolve the FP64 fallbacks of a stage
+constexpr int kSkFixWarps = 2;                // resolve the undecided pairs of a stage
 constexpr int kSkFixThreads = kSkFixWarps * 32;
 constexpr int kSkFixFirst = 2 + kSkGenWarps;
-constexpr int kSkQMax = 256;                 // FP64 fallbacks queued per stage
-// threads of the kernel: TMA + MMA warps, generators, and (exact mode) fixers
-__host__ __device__ constexpr int sk_threads(bool defer) {
-  return (2 + kSkGenWarps + (defer ? 0 : kSkFixWarps)) * 32;
-}
+constexpr int kSkQMax = 256;                 // undecided pairs queued per stage
+constexpr int kSkThreads = (2 + kSkGenWarps + kSkFixWarps) * 32;   // TMA, MMA, generators, fixers
 
 __device__ __forceinline__ void fix_barrier() {
   asm volatile("bar.sync 1, %0;" ::"n"(kSkFixThreads) : "memory");
@@ -402,30 +399,38 @@ __device__ __forceinline__ uint32_t swz_chunk(int row, int kc) {
 }
 
 // Y partial = fl_s(G)[128 rows] x (sum over NT planes of Bt)[bn columns] over one split of m.
-// Exact mode (DEFER = false): pairs whose FP32 estimate is too close to a rounding
-// midpoint of u_s are queued per stage and replaced by the FP64 definition by the
-// fixer warps before the stage is multiplied.  Deferred mode: the stage is
-// multiplied with the FP32 estimates at once and those pairs are recorded;
-// sketch_fix_kernel then evaluates them in FP64 and adds (fl_s(G) - estimate) times
-// the matching rows of A_s to the partials, which gives the same product.
+//
+// A stage passes through three groups of warps: the generators write the tile from FP32
+// estimates and queue the pairs that the estimate leaves undecided (gauss.cuh: about 1 %
+// for BF16, 3 % for F16); the fixers evaluate those in double-float and patch the tile while
+// the generators are on the next stage; the MMA warp multiplies it.  So the GEMM always
+// multiplies fl_s(G) itself.
+//
+// What bounds it: the generators' instruction issue (BF16, m = 1e5, n = 500, s = 2000:
+// 176 instructions a pair, 66 % of the issue slots, 706 us, with the earlier FP32 estimate;
+// see gauss.cuh).  Before, the GEMM multiplied the estimates, kept lists of the undecided
+// pairs and a second kernel evaluated them in FP64 and corrected the partials: 17 ms beside
+// the GEMM's 17 ms for F16 at m = 1e6, n = 1000, s = 3000, a host round trip to see whether
+// a list had overflowed, and in E4M3, whose subnormal range no estimate decided, always a
+// second GEMM with every such pair in FP64 (131 ms at m = 6e5, n = 601, s = 1803).
 //
 // GROUPED: one launch for a batch of problems.  CTA b belongs to the problem p with
 // grp.start[p] <= b < grp.start[p + 1]; its local index gives (tile, column group, split)
 // in that problem's grid; the problem's arguments come from grp.tab[p] and its tensor map
 // from grp.maps[p] (global memory, written by the host before the launch).
 //
-// SHARE (deferred mode, two column groups): the CTAs of the two column groups of a
-// (tile, split) form a cluster and share the sketch operand: each generates half of the
-// 128-row tile (rows 64 r .. 64 r + 63 for cluster rank r) into its own shared memory and
-// copies it into its partner's stage with one bulk copy per generator warp, completing the
-// partner's full barrier; each MMA commit releases the stage in both CTAs (the empty
-// barriers count two arrivals), so neither CTA overwrites a stage its partner still reads.
-// Before exiting, the producer waits for the last release of every stage, so no arrival
-// from the partner can land in a CTA that has exited.
-template <int FMT, int STAGES, int ROWB, int NT, bool DEFER, bool GROUPED, bool SHARE = false>
-__global__ void __launch_bounds__(sk_threads(DEFER), 1)
+// SHARE (two column groups): the CTAs of the two column groups of a (tile, split) form a
+// cluster and share the sketch operand: each generates and fixes half of the 128-row tile
+// (rows 64 r .. 64 r + 63 for cluster rank r) in its own shared memory and copies it into its
+// partner's stage with one bulk copy, completing the partner's full barrier; each MMA commit
+// releases the stage in both CTAs (the empty barriers count two arrivals), so neither CTA
+// overwrites a stage its partner still reads.  Before exiting, the producer waits for the
+// last release of every stage, so no arrival from the partner can land in a CTA that has
+// exited.
+template <int FMT, int STAGES, int ROWB, int NT, bool GROUPED, bool SHARE = false>
+__global__ void __launch_bounds__(kSkThreads, 1)
     sketch_tc_kernel(const __grid_constant__ CUtensorMap tmB, const SketchTcArgs a_in, const SketchGroup grp) {
-  static_assert(!SHARE || (DEFER && !GROUPED), "operand sharing runs in deferred mode, one problem");
+  static_assert(!SHARE || !GROUPED, "operand sharing runs for one problem");
   constexpr int GF = (FMT == FMT_BF16X3) ? FMT_BF16 : FMT;   // format of the sketch operand
   constexpr int EB = (GF == FMT_E4M3) ? 1 : 2;                // bytes per element
   constexpr int BK = ROWB / EB;                               // K elements per stage
@@ -458,8 +463,8 @@ __global__ void __launch_bounds__(sk_threads(DEFER), 1)
   uint32_t* tslot = reinterpret_cast<uint32_t*>(bars + 4 * STAGES + 1);
   uint32_t* qcnt = tslot + 4;                                 // [STAGES]
   uint32_t* qbuf = qcnt + 4;                                  // [STAGES][kSkQMax][3]
-  // full: TMA bytes + fixer warps; empty: MMA commit; genned: generator warps done
-  // with the FP32 pass; fixed: fallbacks written and the queue reset.
+  // full: TMA bytes + fixer warps (+ the partner's half); empty: MMA commit; genned: generator
+  // warps done with the estimates; fixed: undecided pairs written and the queue reset.
   const uint32_t full0 = smem_u32(bars), empty0 = smem_u32(bars + STAGES);
   const uint32_t genned0 = smem_u32(bars + 2 * STAGES), fixed0 = smem_u32(bars + 3 * STAGES);
   const uint32_t done_bar = smem_u32(bars + 4 * STAGES);
@@ -474,7 +479,7 @@ __global__ void __launch_bounds__(sk_threads(DEFER), 1)
 
   if (threadIdx.x == 0) {
     for (int st = 0; st < STAGES; ++st) {
-      mbar_init(full0 + 8 * st, DEFER ? 1 + kSkGenWarps : kSkFixWarps + 1);
+      mbar_init(full0 + 8 * st, kSkFixWarps + 1);
       mbar_init(empty0 + 8 * st, SHARE ? 2 : 1);
       mbar_init(genned0 + 8 * st, kSkGenWarps);
       mbar_init(fixed0 + 8 * st, kSkFixWarps);
@@ -558,14 +563,11 @@ __global__ void __launch_bounds__(sk_threads(DEFER), 1)
   } else if (warp < kSkFixFirst) {
     // ---------------- generator warps: fl_s(G) tile, 128 rows x BK columns
     const int g = threadIdx.x - 64;
-    uint32_t wcnt = 0;   // deferred mode: pairs recorded by this warp
-    const int64_t cta = blockIdx.x + (int64_t)gridDim.x * (blockIdx.y + (int64_t)gridDim.y * blockIdx.z);
-    uint64_t* rec_w = DEFER ? a.rec + (cta * kSkGenWarps + (warp - 2)) * (int64_t)a.rec_cap : nullptr;
     for (int ks = 0; ks < nk; ++ks) {
       const int st = ks % STAGES;
       const uint32_t ph = (uint32_t)(ks / STAGES) & 1u;
       if (!mbar_wait(empty0 + 8 * st, ph ^ 1u, a.err, DEV_TIMEOUT_EMPTY)) break;
-      if (!DEFER && !mbar_wait(fixed0 + 8 * st, ph ^ 1u, a.err, DEV_TIMEOUT_EMPTY)) break;
+      if (!mbar_wait(fixed0 + 8 * st, ph ^ 1u, a.err, DEV_TIMEOUT_EMPTY)) break;
       uint8_t* S = smem + st * stage_bytes;
       uint32_t* qb = qbuf + st * (kSkQMax * 3);
       const int64_t kbase = k_begin + (int64_t)ks * BK;
@@ -583,27 +585,10 @@ __global__ void __launch_bounds__(sk_threads(DEFER), 1)
         for (int hh = 0; hh < HPI; ++hh) {
           const int h = hp * HPI + hh;
           const uint4 x = philox4x32_10(gauss_counter(q0 + h, i), a.k0, a.k1);
-          uint32_t e0, o0, e1, o1;
-          const bool ok0 = gauss_pair_fast<GF>(x.x, x.y, e0, o0);
-          const bool ok1 = gauss_pair_fast<GF>(x.z, x.w, e1, o1);
-          if constexpr (DEFER) {
-            // record the uncertain pairs, in lane order (deterministic lists)
-            const unsigned act = __activemask();
-            const unsigned m0 = __ballot_sync(act, !ok0), m1 = __ballot_sync(act, !ok1);
-            if ((m0 | m1) != 0u) {
-              const unsigned lt = (1u << lane) - 1u;
-              const uint64_t j0 = (q0 + (uint64_t)h) * 4u;
-              if (!ok0) {
-                const uint32_t x0 = wcnt + __popc(m0 & lt);
-                if (x0 < a.rec_cap) rec_w[x0] = (j0 << 16) | i;
-              }
-              if (!ok1) {
-                const uint32_t x1 = wcnt + __popc(m0) + __popc(m1 & lt);
-                if (x1 < a.rec_cap) rec_w[x1] = ((j0 + 2u) << 16) | i;
-              }
-              wcnt += __popc(m0) + __popc(m1);
-            }
-          } else if (!ok0 || !ok1) {
+          uint32_t p0, p1;   // the two pairs of the call, packed
+          const bool ok0 = gauss_pair_est<GF>(x.x, x.y, p0);
+          const bool ok1 = gauss_pair_est<GF>(x.z, x.w, p1);
+          if (!ok0 || !ok1) {
 #pragma unroll
             for (int p2 = 0; p2 < 2; ++p2) {
               if (p2 == 0 ? ok0 : ok1) continue;
@@ -613,18 +598,20 @@ __global__ void __launch_bounds__(sk_threads(DEFER), 1)
                 qb[slot * 3 + 0] = ((uint32_t)row << 8) | ((uint32_t)kc << 4) | (uint32_t)(2 * h + p2);
                 qb[slot * 3 + 1] = pa;
                 qb[slot * 3 + 2] = pb;
-              } else if (p2 == 0) {
-                gauss_pair_slow<GF>(pa, pb, e0, o0);   // queue full: resolve in place
-              } else {
-                gauss_pair_slow<GF>(pa, pb, e1, o1);
+              } else {   // queue full: resolve in place
+                uint32_t be, bo;
+                gauss_pair_slow<GF>(pa, pb, be, bo);
+                const uint32_t v = be | (bo << (8 * EB));
+                if (p2 == 0) p0 = v;
+                else p1 = v;
               }
             }
           }
           if constexpr (EB == 2) {
-            w[2 * hh] = e0 | (o0 << 16);
-            w[2 * hh + 1] = e1 | (o1 << 16);
+            w[2 * hh] = p0;
+            w[2 * hh + 1] = p1;
           } else {
-            w[hh] = e0 | (o0 << 8) | (e1 << 16) | (o1 << 24);
+            w[hh] = p0 | (p1 << 16);
           }
         }
         if constexpr (SPL == 1)
@@ -634,24 +621,11 @@ __global__ void __launch_bounds__(sk_threads(DEFER), 1)
       }
       fence_proxy_async_smem();
       __syncwarp();
-      if constexpr (SHARE) {
-        // this warp's 32 items cover 32 / SPL chunks, whole rows of the tile: one contiguous run
-        constexpr int SPLc = (EB == 2 && GCH * 2 <= kSkGenThreads) ? 2 : 1;
-        static_assert(GCH * SPLc <= kSkGenThreads && (GCH * SPLc) % 32 == 0 && (32 / SPLc) % CPR == 0,
-                      "one item per generator thread, whole rows per warp");
-        const int i0 = (warp - 2) * 32;
-        if (lane == 0 && i0 < GCH * SPLc) {
-          const uint32_t off = (uint32_t)((i0 / SPLc / CPR + (int)rank * 64) * ROWB);
-          const uint32_t src = smem_u32(S) + off;
-          bulk_s2s(cl_map(src, rank ^ 1u), src, (uint32_t)(32 / SPLc) * 16u, cl_map(full0 + 8 * st, rank ^ 1u));
-        }
-      }
-      if (lane == 0) mbar_arrive(DEFER ? full0 + 8 * st : genned0 + 8 * st);
+      if (lane == 0) mbar_arrive(genned0 + 8 * st);
     }
-    if (DEFER && lane == 0) a.rec_cnt[cta * kSkGenWarps + (warp - 2)] = wcnt;
-  } else if constexpr (!DEFER) {
-    // ---------------- fixer warps: FP64 definition for the queued pairs of a stage,
-    // overlapping the generation of the next stage
+  } else {
+    // ---------------- fixer warps: the queued pairs of a stage, overlapping the generation
+    // of the next one
     const int fx = threadIdx.x - kSkFixFirst * 32;
     for (int ks = 0; ks < nk; ++ks) {
       const int st = ks % STAGES;
@@ -663,7 +637,7 @@ __global__ void __launch_bounds__(sk_threads(DEFER), 1)
       for (uint32_t qi = fx; qi < nq; qi += kSkFixThreads) {
         const uint32_t pos = qb[qi * 3];
         uint32_t be, bo;
-        gauss_pair_slow<GF>(qb[qi * 3 + 1], qb[qi * 3 + 2], be, bo);
+        gauss_pair_resolve<GF>(qb[qi * 3 + 1], qb[qi * 3 + 2], be, bo);
         const int row = (int)(pos >> 8), kc = (int)((pos >> 4) & 15), pi = (int)(pos & 15);
         uint8_t* cp = S + swz_chunk<ROWB>(row, kc);
         if constexpr (EB == 2)
@@ -673,7 +647,13 @@ __global__ void __launch_bounds__(sk_threads(DEFER), 1)
       }
       fence_proxy_async_smem();
       fix_barrier();            // every fixer has read qcnt and written its pairs
-      if (fx == 0) qcnt[st] = 0;
+      if (fx == 0) {
+        qcnt[st] = 0;
+        if constexpr (SHARE) {   // the finished half tile: whole rows, one contiguous run
+          const uint32_t src = smem_u32(S) + rank * HALF;
+          bulk_s2s(cl_map(src, rank ^ 1u), src, HALF, cl_map(full0 + 8 * st, rank ^ 1u));
+        }
+      }
       __syncwarp();
       if (lane == 0) {
         mbar_arrive(full0 + 8 * st);
@@ -817,14 +797,14 @@ static cudaError_t launch_tc_inst(const SketchPlan& p, const CUtensorMap& tm, co
                                   cudaStream_t st) {
   dim3 grid((unsigned)p.mtiles, (unsigned)p.ngroups, (unsigned)p.splits);
   const SketchGroup none{};
-  if (a.rec && p.ngroups == 2) {
+  if (p.ngroups == 2) {
     // the two column groups of a (tile, split) share the generated operand (a cluster of two)
-    auto kern = sketch_tc_kernel<FMT, STAGES, ROWB, NT, true, false, true>;
+    auto kern = sketch_tc_kernel<FMT, STAGES, ROWB, NT, false, true>;
     cudaError_t e = allow_dyn_smem(kern, (size_t)p.smem);
     if (e != cudaSuccess) return e;
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = grid;
-    cfg.blockDim = dim3(sk_threads(true));
+    cfg.blockDim = dim3(kSkThreads);
     cfg.dynamicSmemBytes = p.smem;
     cfg.stream = st;
     cudaLaunchAttribute attr[1];
@@ -836,55 +816,27 @@ static cudaError_t launch_tc_inst(const SketchPlan& p, const CUtensorMap& tm, co
     cfg.numAttrs = 1;
     return cudaLaunchKernelEx(&cfg, kern, tm, a, none);
   }
-  if (a.rec) {
-    auto kern = sketch_tc_kernel<FMT, STAGES, ROWB, NT, true, false>;
-    cudaError_t e = allow_dyn_smem(kern, (size_t)p.smem);
-    if (e != cudaSuccess) return e;
-    kern<<<grid, sk_threads(true), p.smem, st>>>(tm, a, none);
-  } else {
-    auto kern = sketch_tc_kernel<FMT, STAGES, ROWB, NT, false, false>;
-    cudaError_t e = allow_dyn_smem(kern, (size_t)p.smem);
-    if (e != cudaSuccess) return e;
-    kern<<<grid, sk_threads(false), p.smem, st>>>(tm, a, none);
-  }
+  auto kern = sketch_tc_kernel<FMT, STAGES, ROWB, NT, false>;
+  cudaError_t e = allow_dyn_smem(kern, (size_t)p.smem);
+  if (e != cudaSuccess) return e;
+  kern<<<grid, kSkThreads, p.smem, st>>>(tm, a, none);
   return cudaGetLastError();
 }
 
 template <int FMT, int STAGES, int ROWB, int NT>
 static cudaError_t launch_tc_grouped_inst(const SketchGroup& g, int64_t ctas, size_t smem, cudaStream_t st) {
-  auto kern = sketch_tc_kernel<FMT, STAGES, ROWB, NT, false, true>;
+  auto kern = sketch_tc_kernel<FMT, STAGES, ROWB, NT, true>;
   cudaError_t e = allow_dyn_smem(kern, smem);
   if (e != cudaSuccess) return e;
   CUtensorMap unused;
   std::memset(&unused, 0, sizeof(unused));
-  kern<<<(unsigned)ctas, sk_threads(false), smem, st>>>(unused, SketchTcArgs{}, g);
+  kern<<<(unsigned)ctas, kSkThreads, smem, st>>>(unused, SketchTcArgs{}, g);
   return cudaGetLastError();
 }
 
 cudaError_t launch_sketch_tc(const SketchPlan& p, const CUtensorMap& tm, uint64_t seed,
-                             float* partial, int* err, cudaStream_t st, uint64_t* rec,
-                             uint32_t* rec_cnt, uint32_t rec_cap) {
-  SketchTcArgs a;
-  a.s = p.s;
-  a.m = p.m;
-  a.ncols = p.ncols;
-  a.kchunk = p.kchunk;
-  a.s_pad = p.s_pad;
-  a.bn = p.bn;
-  a.nsub = p.nsub;
-  a.rows_per_plane = p.ngroups * p.bn;
-  a.mtiles = p.mtiles;
-  a.ngroups = p.ngroups;
-  int tc = 32;
-  while (tc < p.bn) tc <<= 1;
-  a.tmem_cols = tc;
-  a.k0 = (uint32_t)seed;
-  a.k1 = (uint32_t)(seed >> 32);
-  a.partial = partial;
-  a.err = err;
-  a.rec = rec;
-  a.rec_cnt = rec_cnt;
-  a.rec_cap = rec_cap;
+                             float* partial, int* err, cudaStream_t st) {
+  const SketchTcArgs a = sketch_tc_args(p, seed, partial, err);
   const bool four = p.stages == 4;
   switch (p.fmt) {
     case FMT_F16: return four ? launch_tc_inst<FMT_F16, 4, 128, 1>(p, tm, a, st)
@@ -939,172 +891,8 @@ cudaError_t launch_sketch_tc_grouped(int fmt, int stages, const SketchGroup& g, 
   return cudaErrorInvalidValue;
 }
 
-// ============================================================ deferred correction
-// One block per sketch CTA (same grid): the pairs recorded by its generator warps,
-// in list order, 512 at a time.  Phase 1 (one pair per thread, full warps on the
-// FP64 pipe): d = fl_s(G) - fl_s(g32) for both entries of the pair; pairs with
-// d != 0 are compacted in order.  Phase 2 (one column per thread): for each kept
-// pair, partial[i][c] += d * A_s[j][c], with A_s[j][c] recomputed from A by the
-// cast's own rounding.  Every partial entry is updated by one thread in a fixed
-// order, so the result is deterministic.
-constexpr int kFixThreads = 512;
-
-struct SketchFixArgs {
-  int64_t s, m, n, ncols, s_pad, lda;
-  int bn;
-  int share;   // the two column groups shared the operand: read both CTAs' lists
-  uint32_t k0, k1, cap;
-  const uint64_t* rec;
-  const uint32_t* rec_cnt;
-  const double* A;
-  const double* b;
-  const int* kexp;
-  float* partial;
-  int* overflow;
-};
-
-struct FixRec {
-  uint32_t i, pad;
-  uint64_t j0;
-  float de, dodd;   // exact minus estimate: differences of nearby values of the format, exact in FP32
-};
-
-template <int FMT>
-__global__ void __launch_bounds__(kFixThreads)
-    sketch_fix_kernel(const SketchFixArgs f) {
-  constexpr int GF = (FMT == FMT_BF16X3) ? FMT_BF16 : FMT;
-  __shared__ uint32_t off[2 * kSkGenWarps + 1];
-  __shared__ int ovf;
-  __shared__ int wsum[kFixThreads / 32];
-  __shared__ FixRec kept[kFixThreads];
-  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  const int64_t cta = blockIdx.x + (int64_t)gridDim.x * (blockIdx.y + (int64_t)gridDim.y * blockIdx.z);
-  // with a shared operand, the partner CTA (other column group) generated half of the rows
-  const int64_t peer = blockIdx.x + (int64_t)gridDim.x * ((blockIdx.y ^ 1u) + (int64_t)gridDim.y * blockIdx.z);
-  const int nl = f.share ? 2 * kSkGenWarps : kSkGenWarps;
-  auto list_of = [&](int w) { return (w < kSkGenWarps ? cta : peer) * kSkGenWarps + (w % kSkGenWarps); };
-  if (tid == 0) {
-    uint32_t o = 0;
-    int bad = 0;
-    for (int w = 0; w < nl; ++w) {
-      const uint32_t c = f.rec_cnt[list_of(w)];
-      if (c > f.cap) bad = 1;
-      off[w] = o;
-      o += min(c, f.cap);
-    }
-    off[nl] = o;
-    ovf = bad;
-  }
-  __syncthreads();
-  if (ovf) {   // lists incomplete: the caller reruns the exact kernel
-    if (tid == 0) atomicExch(f.overflow, 1);
-    return;
-  }
-  const uint32_t total = off[nl];
-  const int64_t split = blockIdx.z;
-  const int64_t col = (int64_t)blockIdx.y * f.bn + tid;
-  const bool has_col = tid < f.bn && col < f.ncols;
-  const int kc = has_col ? f.kexp[col] : 0;
-  const uint64_t* Au = reinterpret_cast<const uint64_t*>(f.A);
-  const uint64_t* bu = reinterpret_cast<const uint64_t*>(f.b);
-  for (uint32_t base = 0; base < total; base += kFixThreads) {
-    // ---- phase 1: exact minus estimate for one recorded pair
-    FixRec r{};
-    bool keep = false;
-    const uint32_t idx = base + tid;
-    if (idx < total) {
-      int w = 0;
-      while (idx >= off[w + 1]) ++w;
-      const uint64_t pk = f.rec[list_of(w) * (int64_t)f.cap + (idx - off[w])];
-      r.i = (uint32_t)(pk & 0xFFFFu);
-      r.j0 = pk >> 16;
-      const uint4 x = philox4x32_10(gauss_counter(r.j0 >> 2, r.i), f.k0, f.k1);
-      const uint32_t pa = (r.j0 & 2u) ? x.z : x.x, pb = (r.j0 & 2u) ? x.w : x.y;
-      uint32_t fe, fo, xe, xo;
-      gauss_pair_fast<GF>(pa, pb, fe, fo);
-      gauss_pair_slow<GF>(pa, pb, xe, xo);
-      r.de = __fsub_rn(bits_to_float<GF>(xe), bits_to_float<GF>(fe));
-      r.dodd = __fsub_rn(bits_to_float<GF>(xo), bits_to_float<GF>(fo));
-      keep = (r.de != 0.0f || r.dodd != 0.0f) && (int64_t)r.i < f.s;
-    }
-    // ---- ordered compaction of the kept pairs
-    const unsigned bal = __ballot_sync(0xffffffffu, keep);
-    if (lane == 0) wsum[warp] = __popc(bal);
-    __syncthreads();
-    int before = 0, nkept = 0;
-    for (int q = 0; q < kFixThreads / 32; ++q) {
-      if (q < warp) before += wsum[q];
-      nkept += wsum[q];
-    }
-    if (keep) kept[before + __popc(bal & ((1u << lane) - 1u))] = r;
-    __syncthreads();
-    // ---- phase 2: partial[i][col] += d * A_s[j][col], in FP32 like the GEMM.  d is one
-    // step of the format (a power of two) or the difference of two nearby values of it,
-    // and A_s[j][col] has at most 24 significant bits (BF16X3: hi + lo + lo2, exact in
-    // FP32), so each product is exact; the two of a pair are summed in FP32.
-    if (has_col) {
-      float* pc = f.partial + (split * f.ncols + col) * f.s_pad;
-      for (int q = 0; q < nkept; ++q) {
-        const FixRec& k = kept[q];
-        float add = 0.0f;
-#pragma unroll
-        for (int e = 0; e < 2; ++e) {
-          const float d = e ? k.dodd : k.de;
-          const int64_t j = (int64_t)k.j0 + e;
-          if (d == 0.0f || j >= f.m) continue;
-          const uint64_t u = (col < f.n) ? Au[j * f.lda + col] : bu[j];
-          uint32_t t[3];
-          cast_bits<FMT>(u, kc, t);
-          float v = bits_to_float<GF>(t[0]);
-          if constexpr (FMT == FMT_BF16X3)
-            v = __fadd_rn(__fadd_rn(v, bits_to_float<GF>(t[1])), bits_to_float<GF>(t[2]));
-          add = __fmaf_rn(d, v, add);
-        }
-        pc[k.i] += add;
-      }
-    }
-    __syncthreads();
-  }
-}
-
-cudaError_t launch_sketch_fix(const SketchPlan& p, uint64_t seed, const uint64_t* rec,
-                              const uint32_t* rec_cnt, uint32_t cap, const double* A, int64_t lda,
-                              const double* b, const int* kexp, float* partial, int* overflow,
-                              cudaStream_t st) {
-  if (p.bn > kFixThreads) return cudaErrorInvalidValue;
-  SketchFixArgs f;
-  f.s = p.s;
-  f.m = p.m;
-  f.n = p.ncols - 1;
-  f.ncols = p.ncols;
-  f.s_pad = p.s_pad;
-  f.lda = lda;
-  f.bn = p.bn;
-  f.share = p.ngroups == 2 ? 1 : 0;   // launch_sketch_tc shares the operand exactly then (deferred mode)
-  f.k0 = (uint32_t)seed;
-  f.k1 = (uint32_t)(seed >> 32);
-  f.cap = cap;
-  f.rec = rec;
-  f.rec_cnt = rec_cnt;
-  f.A = A;
-  f.b = b;
-  f.kexp = kexp;
-  f.partial = partial;
-  f.overflow = overflow;
-  dim3 grid((unsigned)p.mtiles, (unsigned)p.ngroups, (unsigned)p.splits);
-  switch (p.fmt) {
-    case FMT_F16: sketch_fix_kernel<FMT_F16><<<grid, kFixThreads, 0, st>>>(f); break;
-    case FMT_BF16: sketch_fix_kernel<FMT_BF16><<<grid, kFixThreads, 0, st>>>(f); break;
-    case FMT_E4M3: sketch_fix_kernel<FMT_E4M3><<<grid, kFixThreads, 0, st>>>(f); break;
-    case FMT_BF16X3: sketch_fix_kernel<FMT_BF16X3><<<grid, kFixThreads, 0, st>>>(f); break;
-    default: return cudaErrorInvalidValue;
-  }
-  return cudaGetLastError();
-}
-
-// Records per generator warp for deferred correction: the warp sees 4 * kchunk
-// (a, b) pairs; expected fractions near a midpoint are ~0.2% (BF16), ~1.6%
-// (FP16), ~0.01% (E4M3), so the capacity leaves a 4x or larger margin.
+// The pairs of one split a generator warp can leave undecided (4 * kchunk pairs a warp, with a
+// margin over the fractions in gauss.cuh), and the number of generator warps of the grid.
 uint32_t sketch_rec_cap(const SketchPlan& p) {
   const int64_t pairs = 4 * p.kchunk;
   const int64_t div = (p.fmt == FMT_F16) ? 16 : (p.fmt == FMT_E4M3) ? 1024 : 128;

@@ -44,11 +44,6 @@ struct SketchTcArgs {
   uint32_t k0, k1;
   float* partial;
   int* err;
-  // deferred mode: per generator warp a list of the (a, b) pairs whose FP32
-  // estimate was too close to a rounding midpoint, packed (data row << 16 | sketch row)
-  uint64_t* rec;
-  uint32_t* rec_cnt;
-  uint32_t rec_cap;
 };
 
 // A grouped sketch launch: problem p owns CTAs [start[p], start[p + 1]); tab[p] and
@@ -109,11 +104,7 @@ bool plan_sketch_tc(int fmt, int64_t s, int64_t m, int64_t ncols, int num_sms, S
 // (`rows` = planes x plane_rows).
 bool encode_bt_tmap(CUtensorMap* tm, const void* Bt, int fmt, int64_t rows, int64_t m, int box_rows,
                     int rowb);
-// rec == nullptr: exact mode (FP64 fallbacks resolved inside the kernel).  Otherwise
-// deferred mode: the uncertain pairs go to sketch_rec_lists(p) lists of
-// sketch_rec_cap(p) entries (counts in rec_cnt) and launch_sketch_fix corrects the
-// partials; if it reports *overflow != 0 the exact mode must be rerun.
-// The arguments launch_sketch_tc builds for plan p (exact mode), for a grouped table.
+// The arguments launch_sketch_tc builds for plan p, for a grouped table.
 SketchTcArgs sketch_tc_args(const SketchPlan& p, uint64_t seed, float* partial, int* err);
 // One launch for a batch: ctas = start[nprob]; smem = the largest plan's; every plan must
 // have the same format and stage count.
@@ -128,14 +119,9 @@ cudaError_t launch_grouped_cast(int fmt, const GCast* tab, const int* colmax_sta
 cudaError_t launch_grouped_sketch_reduce(const GReduce* tab, const int* start, int64_t ctas, int nprob,
                                          cudaStream_t st);
 cudaError_t launch_sketch_tc(const SketchPlan& p, const CUtensorMap& tm, uint64_t seed,
-                             float* partial, int* err, cudaStream_t st, uint64_t* rec = nullptr,
-                             uint32_t* rec_cnt = nullptr, uint32_t rec_cap = 0);
+                             float* partial, int* err, cudaStream_t st);
 uint32_t sketch_rec_cap(const SketchPlan& p);
 int64_t sketch_rec_lists(const SketchPlan& p);
-cudaError_t launch_sketch_fix(const SketchPlan& p, uint64_t seed, const uint64_t* rec,
-                              const uint32_t* rec_cnt, uint32_t cap, const double* A, int64_t lda,
-                              const double* b, const int* kexp, float* partial, int* overflow,
-                              cudaStream_t st);
 // CUDA-core sketch in FP64 (fmt F64) or FP32 (fmt F32) from the FP64 data.
 cudaError_t launch_sketch_cc(int fmt, const double* A, int64_t lda, const double* b, int64_t m,
                              int64_t n, int64_t s, uint64_t seed, int splits, int64_t kchunk,
