@@ -52,7 +52,7 @@ void stage_sketch(Ctx& c, double* Y, const float* a32) {
     }
     StageTimer tt(c.h, ST_SKETCH);
     CUtensorMap tm;
-    if (!encode_bt_tmap(&tm, Bt, fmt, (int64_t)p.nt * rows, c.m, p.bn / p.nsub, p.rowb))
+    if (!encode_bt_tmap(&tm, Bt, fmt, (int64_t)p.nt * rows, c.m, p.bn / p.nsub))
       throw StatusFail{LSQ_E_UNSUPPORTED};
     float* partial = static_cast<float*>(ws(c.h, "partial", (size_t)p.splits * ncols * p.s_pad * 4));
     {

@@ -385,10 +385,6 @@ lsq_status lsq_batch_grouped(lsq_handle* h, int32_t nprob, const lsq_problem* pr
     b.lda32[p] = (b.n[p] + 3) / 4 * 4;
     if (b.n[p] > 256 || b.s[p] > 1024 || !probs[p].x) return LSQ_E_UNSUPPORTED;
   }
-  // one kernel instantiation for the batch: the smallest stage count of the plans and the
-  // largest shared-memory size (a plan's layout needs at most its own stage count)
-  int stages = 4;
-  size_t sk_smem = 0;
   for (int p = 0; p < np; ++p) {
     // the plan depends on the problem alone (about one CTA-wave share per 8192 rows), so
     // that its result does not depend on the rest of the batch
@@ -396,8 +392,6 @@ lsq_status lsq_batch_grouped(lsq_handle* h, int32_t nprob, const lsq_problem* pr
     if (!plan_sketch_tc(fmt, b.s[p], b.m[p], b.n[p] + 1, share, &plans[p], b.o.sketch_kchunk))
       return LSQ_E_UNSUPPORTED;
     if (plans[p].splits > 65535) return LSQ_E_UNSUPPORTED;
-    stages = std::min(stages, plans[p].stages);
-    sk_smem = std::max(sk_smem, plans[p].smem);
   }
   std::vector<lsq_info> local((size_t)np);
   lsq_info* inf = infos ? infos : local.data();
@@ -464,7 +458,7 @@ lsq_status lsq_batch_grouped(lsq_handle* h, int32_t nprob, const lsq_problem* pr
       for (int p = 0; p < np; ++p) {
         const SketchPlan& pl = plans[p];
         const int64_t rows = (int64_t)pl.ngroups * pl.bn;
-        if (!encode_bt_tmap(&maps[p], aBt.at<void>(p), fmt, (int64_t)pl.nt * rows, b.m[p], pl.bn / pl.nsub, pl.rowb))
+        if (!encode_bt_tmap(&maps[p], aBt.at<void>(p), fmt, (int64_t)pl.nt * rows, b.m[p], pl.bn / pl.nsub))
           throw StatusFail{LSQ_E_UNSUPPORTED};
         targs[p] = sketch_tc_args(pl, probs[p].seed, aPart.at<float>(p), h->d_err);
         tred[p] = GReduce{aPart.at<float>(p), pl.splits, pl.ncols, b.s[p], pl.s_pad, aK.at<int>(p), aY.at<double>(p)};
@@ -476,7 +470,7 @@ lsq_status lsq_batch_grouped(lsq_handle* h, int32_t nprob, const lsq_problem* pr
       sg.start = gs.dev;
       sg.nprob = np;
       CK(cudaStreamSynchronize(b.st));
-      LB(launch_sketch_tc_grouped(fmt, stages, sg, gs.total, sk_smem, b.st));
+      LB(launch_sketch_tc_grouped(fmt, sg, gs.total, b.st));
       Groups gr = make_groups(h, "b_gred", redc);
       GReduce* dred = upload(h, "b_tred", tred);
       LB(launch_grouped_sketch_reduce(dred, gr.dev, gr.total, np, b.st));

@@ -147,12 +147,12 @@ __device__ __forceinline__ void spec_gauss_pair(uint32_t a, uint32_t b, double& 
 // d > rad and no sign of g passes the test.
 //  * BF16, E4M3 (coarse): sin.approx and cos.approx, 2^-20.5 absolute, on an angle from the
 //    23 leading bits of U2 (centred: 2^-21.3, plus 2^-22.2 of roundings):
-//    d = 2.7e-6 rad + 6e-7 / rad, against a first-order sum of 1.8e-6 rad + 4.5e-7 / rad.
-//    About 1 % of the BF16 pairs and 0.1 % of the E4M3 pairs are left undecided.
+//    d = 2e-6 rad + 5e-7 / rad, against a first-order sum of 1.8e-6 rad + 4.5e-7 / rad.
+//    About 1.4 % of the BF16 pairs and 0.06 % of the E4M3 pairs are left undecided.
 //  * F16 (three more bits): sin and cos by quadrant reduction on the exact integer and a short
 //    series, 4e-7 relative, so that small entries keep their relative accuracy:
-//    d = |g| (1.5e-6 + 6e-7 / rad2); about 3 % of the pairs are left undecided (8 % with
-//    the approximate functions).
+//    d = |g| (1.2e-6 + 5e-7 / rad2), against 1.1e-6 + 4.5e-7 / rad2; about 1.7 % of the pairs
+//    are left undecided (8 % with the approximate functions).
 __device__ __forceinline__ float mufu_lg2(float x) {
   float r;
   asm("lg2.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
@@ -226,7 +226,7 @@ __device__ __forceinline__ bool gauss_pair_est(uint32_t a, uint32_t b, uint32_t&
     const uint32_t cb = __float_as_uint(swap ? sp : cp) ^ (((q + 1u) & 2u) << 30);
     const uint32_t sb = __float_as_uint(swap ? cp : sp) ^ ((q & 2u) << 30);
     const float ge = rad * __uint_as_float(cb), go = rad * __uint_as_float(sb);
-    const float t = fmaf(irad * irad, 6e-7f, 1.5e-6f);
+    const float t = fmaf(irad * irad, 5e-7f, 1.2e-6f);
     packed = pack2<FMT>(fmaf(ge, -t, ge), fmaf(go, -t, go));
     return packed == pack2<FMT>(fmaf(ge, t, ge), fmaf(go, t, go));
   } else {
@@ -236,7 +236,7 @@ __device__ __forceinline__ bool gauss_pair_est(uint32_t a, uint32_t b, uint32_t&
     const float th = fmaf(u, 6.28318530717958648f, (float)(6.28318530717958648 * 0x1p-24));
     const float nrad = -rad2 * irad;
     const float ge = nrad * mufu_cos(th), go = nrad * mufu_sin(th);
-    const float d = fmaf(nrad, -2.7e-6f, irad * 6e-7f);
+    const float d = fmaf(nrad, -2e-6f, irad * 5e-7f);
     packed = pack2<FMT>(ge - d, go - d);
     return packed == pack2<FMT>(ge + d, go + d);
   }

@@ -14,6 +14,7 @@
 //  * reduce: FP64 sum of the split partials, times s^-1/2 and 2^-k_j.
 #include <cudaTypedefs.h>
 
+#include <algorithm>
 #include <cstring>
 
 #include "cast.cuh"
@@ -368,34 +369,41 @@ cudaError_t launch_cast_transpose(int fmt, const double* A, int64_t lda, const d
 // ============================================================ tcgen05 sketch
 constexpr int kSkGenWarps = 16;
 constexpr int kSkGenThreads = kSkGenWarps * 32;
-constexpr int kSkFixWarps = 2;                // resolve the undecided pairs of a stage
+// Fixers: two groups of warps take the stages in turn.  A double-float evaluation is a chain
+// of about 1.4 us, so one group of two warps held every stage for that long (F16, m = 2e5,
+// n = 1000, s = 3000: 1.73 ms, 1.75 us a stage).
+constexpr int kSkFixGroups = 2;
+constexpr int kSkFixWarps = 2;                // of a group
 constexpr int kSkFixThreads = kSkFixWarps * 32;
 constexpr int kSkFixFirst = 2 + kSkGenWarps;
 constexpr int kSkQMax = 256;                 // undecided pairs queued per stage
-constexpr int kSkThreads = (2 + kSkGenWarps + kSkFixWarps) * 32;   // TMA, MMA, generators, fixers
+constexpr size_t kSkSmem = 232448;           // the SM's shared memory: one CTA per SM
+// Rings: three or four sketch tiles of 128 rows, and as many Bt slots as fit (at most
+// kSkBRing).  A slot is one box of one plane (chunk rows), so a slot is refilled as soon as its
+// own products are done, and the generators run up to four stages ahead.  Whole stages as
+// slots (sketch tile and all boxes of Bt: 80 KB at 512 columns, so two of them) left both
+// waiting for the refill's latency.  Rings, 128-byte rows and fixer groups together: BF16, m =
+// 1e5, n = 500, s = 2000 459 -> 355 us (instruction issue of the generators), F16, m = 2e5, n =
+// 1000, s = 3000 2.50 -> 1.65 ms, BF16X3, m = 2e5, n = 1000, s = 4000 4.99 -> 3.5 ms (tensor
+// pipe 42 -> 60 %).
+constexpr int sk_a_ring(int nt) { return nt == 1 ? 4 : 3; }
+constexpr int kSkBRing = 16;
+constexpr size_t kSkCtrl = 5120;             // barriers and queue counters (512 bytes), queues
+static_assert(512 + sk_a_ring(1) * kSkQMax * 4 <= kSkCtrl, "a queue per sketch tile");
+constexpr int kSkThreads = (2 + kSkGenWarps + kSkFixGroups * kSkFixWarps) * 32;   // TMA, MMA, generators, fixers
 
-__device__ __forceinline__ void fix_barrier() {
-  asm volatile("bar.sync 1, %0;" ::"n"(kSkFixThreads) : "memory");
+__device__ __forceinline__ void fix_barrier(int group) {
+  asm volatile("bar.sync %0, %1;" ::"r"(1 + group), "n"(kSkFixThreads) : "memory");
 }
 
-// Smem descriptor for a K-major operand whose rows are ROWB bytes (128: 128-byte
-// swizzle; 64: 64-byte swizzle), 8-row core groups 8 * ROWB bytes apart.
-template <int ROWB>
-__device__ __forceinline__ uint64_t kmajor_desc(uint32_t saddr) {
-  uint64_t d = 0;
-  d |= (uint64_t)((saddr & 0x3FFFFu) >> 4);
-  d |= (uint64_t)(16u >> 4) << 16;
-  d |= (uint64_t)((8u * ROWB) >> 4) << 32;
-  d |= (uint64_t)1 << 46;
-  d |= (uint64_t)(ROWB == 128 ? 2 : 4) << 61;
-  return d;
-}
+// A stage is 128 bytes of K (64 elements of the 16-bit formats, 128 of E4M3): K-major
+// operands in 128-byte rows, 128-byte swizzle.  (Stages of 64-byte rows for the three planes
+// of BF16X3 issued twice the TMA rows and gave every generator thread a single Philox call.)
+constexpr int kSkRowB = 128;
 
 // Byte offset of 16-byte chunk kc of row `row` in a swizzled K-major tile.
-template <int ROWB>
 __device__ __forceinline__ uint32_t swz_chunk(int row, int kc) {
-  const int sw = (ROWB == 128) ? (row & 7) : ((row >> 1) & 3);
-  return (uint32_t)(row * ROWB + ((kc ^ sw) << 4));
+  return (uint32_t)(row * kSkRowB + ((kc ^ (row & 7)) << 4));
 }
 
 // Y partial = fl_s(G)[128 rows] x (sum over NT planes of Bt)[bn columns] over one split of m.
@@ -406,9 +414,9 @@ __device__ __forceinline__ uint32_t swz_chunk(int row, int kc) {
 // the generators are on the next stage; the MMA warp multiplies it.  So the GEMM always
 // multiplies fl_s(G) itself.
 //
-// What bounds it: the generators' instruction issue (BF16, m = 1e5, n = 500, s = 2000:
-// 176 instructions a pair, 66 % of the issue slots, 706 us, with the earlier FP32 estimate;
-// see gauss.cuh).  Before, the GEMM multiplied the estimates, kept lists of the undecided
+// What bounds it: the generators' instruction issue where n is below about 500 a format
+// term, the tensor pipe and the refill of Bt beyond.  (With the earlier FP32 estimate, 176
+// instructions a pair against 72 now, BF16, m = 1e5, n = 500, s = 2000 took 706 us.)  Before, the GEMM multiplied the estimates, kept lists of the undecided
 // pairs and a second kernel evaluated them in FP64 and corrected the partials: 17 ms beside
 // the GEMM's 17 ms for F16 at m = 1e6, n = 1000, s = 3000, a host round trip to see whether
 // a list had overflowed, and in E4M3, whose subnormal range no estimate decided, always a
@@ -427,19 +435,19 @@ __device__ __forceinline__ uint32_t swz_chunk(int row, int kc) {
 // overwrites a stage its partner still reads.  Before exiting, the producer waits for the
 // last release of every stage, so no arrival from the partner can land in a CTA that has
 // exited.
-template <int FMT, int STAGES, int ROWB, int NT, bool GROUPED, bool SHARE = false>
+template <int FMT, int NT, bool GROUPED, bool SHARE = false>
 __global__ void __launch_bounds__(kSkThreads, 1)
     sketch_tc_kernel(const __grid_constant__ CUtensorMap tmB, const SketchTcArgs a_in, const SketchGroup grp) {
   static_assert(!SHARE || !GROUPED, "operand sharing runs for one problem");
   constexpr int GF = (FMT == FMT_BF16X3) ? FMT_BF16 : FMT;   // format of the sketch operand
   constexpr int EB = (GF == FMT_E4M3) ? 1 : 2;                // bytes per element
-  constexpr int BK = ROWB / EB;                               // K elements per stage
+  constexpr int BK = kSkRowB / EB;                            // K elements per stage
   constexpr int EPC = 16 / EB;                                // elements per 16-byte chunk
-  constexpr int CPR = ROWB / 16;                              // chunks per row
+  constexpr int CPR = kSkRowB / 16;                           // chunks per row
   constexpr int NCHUNK = 128 * CPR;                           // chunks per sketch tile
   constexpr int PPC = EPC / 2;                                // (a, b) pairs per chunk
-  constexpr uint32_t S_BYTES = 128u * ROWB;
-  constexpr int KSLICES = ROWB / 32;                          // MMA K slices (32 bytes) per stage
+  constexpr uint32_t S_BYTES = 128u * kSkRowB;
+  constexpr int KSLICES = kSkRowB / 32;                         // MMA K slices (32 bytes) per stage
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) &
                                              ~static_cast<uintptr_t>(1023));
@@ -457,33 +465,42 @@ __global__ void __launch_bounds__(kSkThreads, 1)
     tmp = grp.maps + gp;
   }
   const SketchTcArgs a = GROUPED ? grp.tab[gp] : a_in;
-  const uint32_t b_bytes = (uint32_t)a.bn * ROWB;              // one plane of Bt per stage
-  const uint32_t stage_bytes = S_BYTES + NT * b_bytes;
-  uint64_t* bars = reinterpret_cast<uint64_t*>(smem + STAGES * stage_bytes);
-  uint32_t* tslot = reinterpret_cast<uint32_t*>(bars + 4 * STAGES + 1);
-  uint32_t* qcnt = tslot + 4;                                 // [STAGES]
-  uint32_t* qbuf = qcnt + 4;                                  // [STAGES][kSkQMax][3]
-  // full: TMA bytes + fixer warps (+ the partner's half); empty: MMA commit; genned: generator
-  // warps done with the estimates; fixed: undecided pairs written and the queue reset.
-  const uint32_t full0 = smem_u32(bars), empty0 = smem_u32(bars + STAGES);
-  const uint32_t genned0 = smem_u32(bars + 2 * STAGES), fixed0 = smem_u32(bars + 3 * STAGES);
-  const uint32_t done_bar = smem_u32(bars + 4 * STAGES);
+  constexpr int NA = sk_a_ring(NT), ROWB = kSkRowB;
+  const int chunk = a.bn / a.nsub;
+  const uint32_t slot_bytes = (uint32_t)chunk * ROWB;         // one box of one plane of Bt
+  const int NB = min(kSkBRing, (int)((kSkSmem - 1024 - kSkCtrl - NA * S_BYTES) / slot_bytes));
+  uint64_t* bars = reinterpret_cast<uint64_t*>(smem);
+  uint32_t* tslot = reinterpret_cast<uint32_t*>(bars + 4 * NA + 2 * kSkBRing + 1);
+  uint32_t* qcnt = tslot + 1;                                 // [NA]
+  uint32_t* qbuf = reinterpret_cast<uint32_t*>(smem + 512);   // [NA][kSkQMax]
+  uint8_t* ringA = smem + kSkCtrl;
+  uint8_t* ringB = ringA + NA * S_BYTES;
+  // sketch tiles -- afull: fixer warps (+ the partner's half); aempty: MMA commit (of both
+  // CTAs, SHARE); genned: generator warps done with the estimates; fixed: undecided pairs
+  // written and the queue reset.  Bt slots -- bfull: TMA bytes; bempty: MMA commit.
+  const uint32_t afull0 = smem_u32(bars), aempty0 = smem_u32(bars + NA);
+  const uint32_t genned0 = smem_u32(bars + 2 * NA), fixed0 = smem_u32(bars + 3 * NA);
+  const uint32_t bfull0 = smem_u32(bars + 4 * NA), bempty0 = smem_u32(bars + 4 * NA + kSkBRing);
+  const uint32_t done_bar = smem_u32(bars + 4 * NA + 2 * kSkBRing);
 
   const int64_t k_begin = split * a.kchunk;
   const int64_t k_end = min(a.m, k_begin + a.kchunk);
   const int nk = (int)((k_end - k_begin + BK - 1) / BK);
-  const int chunk = a.bn / a.nsub;
   constexpr uint32_t HALF = S_BYTES / 2;                      // the half tile a CTA generates (SHARE)
   constexpr int GCH = SHARE ? NCHUNK / 2 : NCHUNK;            // chunks this CTA generates per stage
   const uint32_t rank = SHARE ? cl_rank() : 0u;
 
   if (threadIdx.x == 0) {
-    for (int st = 0; st < STAGES; ++st) {
-      mbar_init(full0 + 8 * st, kSkFixWarps + 1);
-      mbar_init(empty0 + 8 * st, SHARE ? 2 : 1);
+    for (int st = 0; st < NA; ++st) {
+      mbar_init(afull0 + 8 * st, kSkFixWarps);
+      mbar_init(aempty0 + 8 * st, SHARE ? 2 : 1);
       mbar_init(genned0 + 8 * st, kSkGenWarps);
       mbar_init(fixed0 + 8 * st, kSkFixWarps);
       qcnt[st] = 0;
+    }
+    for (int sl = 0; sl < NB; ++sl) {
+      mbar_init(bfull0 + 8 * sl, 1);
+      mbar_init(bempty0 + 8 * sl, 1);
     }
     mbar_init(done_bar, 1);
     fence_barrier_init();
@@ -498,8 +515,21 @@ __global__ void __launch_bounds__(kSkThreads, 1)
   const uint32_t tmem_base = *tslot;
   if constexpr (SHARE) cl_sync();   // the partner's barriers are initialised before any copy or commit
 
+  // Pair pi of chunk kc, row `row` of a sketch tile: its words drawn again, fl_s(G) stored.
+  auto resolve_pair = [&](uint8_t* S, int row, int kc, int pi, int64_t kbase) {
+    const uint64_t q = ((uint64_t)(kbase + kc * EPC) >> 2) + (uint64_t)(pi >> 1);
+    const uint4 x = philox4x32_10(gauss_counter(q, (uint32_t)(mt * 128 + row)), a.k0, a.k1);
+    uint32_t be, bo;
+    gauss_pair_resolve<GF>((pi & 1) ? x.z : x.x, (pi & 1) ? x.w : x.y, be, bo);
+    uint8_t* cp = S + swz_chunk(row, kc);
+    if constexpr (EB == 2)
+      *reinterpret_cast<uint32_t*>(cp + 4 * pi) = be | (bo << 16);
+    else
+      *reinterpret_cast<uint16_t*>(cp + 2 * pi) = (uint16_t)(be | (bo << 8));
+  };
+
   if (warp == 0) {
-    // ---------------- TMA producer: NT planes x nsub boxes of [chunk rows x ROWB bytes]
+    // ---------------- TMA producer: NT planes x nsub boxes of [chunk rows x 128 bytes]
     if (lane == 0) {
       if constexpr (GROUPED) {   // the map was written through the generic proxy
         asm volatile("fence.proxy.tensormap::generic.acquire.gpu [%0], 128;" ::"l"(
@@ -507,24 +537,30 @@ __global__ void __launch_bounds__(kSkThreads, 1)
                      : "memory");
       }
       prefetch_tmap(tmp);
-      for (int ks = 0; ks < nk; ++ks) {
-        const int st = ks % STAGES;
-        const uint32_t ph = (uint32_t)(ks / STAGES) & 1u;
-        if (!mbar_wait(empty0 + 8 * st, ph ^ 1u, a.err, DEV_TIMEOUT_EMPTY)) break;
-        mbar_arrive_expect_tx(full0 + 8 * st, (uint32_t)NT * b_bytes + (SHARE ? HALF : 0u));
-        const uint32_t sb = smem_u32(smem + st * stage_bytes + S_BYTES);
+      int sl = 0;
+      uint32_t ph = 0;
+      bool ok = true;
+      for (int ks = 0; ks < nk && ok; ++ks) {
         const int64_t kx = k_begin + (int64_t)ks * BK;
         const int32_t kin = (int32_t)(kx % kBtBlock), kblk = (int32_t)(kx / kBtBlock);
-        for (int t = 0; t < NT; ++t)
-          for (int c = 0; c < a.nsub; ++c)
-            tma_load_3d(sb + t * b_bytes + (uint32_t)(c * chunk * ROWB), tmp, kin,
-                        (int32_t)(t * a.rows_per_plane + ng * a.bn + c * chunk), kblk, full0 + 8 * st);
+        for (int c = 0; c < a.nsub && ok; ++c)
+          for (int t = 0; t < NT; ++t) {
+            ok = mbar_wait(bempty0 + 8 * sl, ph ^ 1u, a.err, DEV_TIMEOUT_EMPTY);
+            if (!ok) break;
+            mbar_arrive_expect_tx(bfull0 + 8 * sl, slot_bytes);
+            tma_load_3d(smem_u32(ringB) + (uint32_t)sl * slot_bytes, tmp, kin,
+                        (int32_t)(t * a.rows_per_plane + ng * a.bn + c * chunk), kblk, bfull0 + 8 * sl);
+            if (++sl == NB) {
+              sl = 0;
+              ph ^= 1u;
+            }
+          }
       }
       if constexpr (SHARE) {
-        // tail: the last release of every stage (both MMAs) has arrived here
-        for (int st = 0; st < STAGES && st < nk; ++st) {
-          const int last = st + ((nk - 1 - st) / STAGES) * STAGES;
-          if (!mbar_wait(empty0 + 8 * st, (uint32_t)(last / STAGES) & 1u, a.err, DEV_TIMEOUT_EMPTY)) break;
+        // tail: the last release of every sketch tile (both MMAs) has arrived here
+        for (int st = 0; st < NA && st < nk; ++st) {
+          const int last = st + ((nk - 1 - st) / NA) * NA;
+          if (!mbar_wait(aempty0 + 8 * st, (uint32_t)(last / NA) & 1u, a.err, DEV_TIMEOUT_EMPTY)) break;
         }
       }
     }
@@ -532,31 +568,39 @@ __global__ void __launch_bounds__(kSkThreads, 1)
     // ---------------- MMA issuer
     if (lane == 0) {
       const uint32_t idesc = make_idesc(GF == FMT_BF16 ? 1u : 0u, 128u, (uint32_t)chunk);
-      for (int ks = 0; ks < nk; ++ks) {
-        const int st = ks % STAGES;
-        const uint32_t ph = (uint32_t)(ks / STAGES) & 1u;
-        if (!mbar_wait(full0 + 8 * st, ph, a.err, DEV_TIMEOUT_FULL)) break;
-        tc_fence_after();
-        const uint32_t sa = smem_u32(smem + st * stage_bytes);
-        const uint32_t sb = sa + S_BYTES;
+      int sl = 0;
+      uint32_t ph = 0;
+      bool ok = true;
+      for (int ks = 0; ks < nk && ok; ++ks) {
+        const int st = ks % NA;
+        ok = mbar_wait(afull0 + 8 * st, (uint32_t)(ks / NA) & 1u, a.err, DEV_TIMEOUT_FULL);
+        if (!ok) break;
+        const uint32_t sa = smem_u32(ringA) + (uint32_t)st * S_BYTES;
+        for (int c = 0; c < a.nsub && ok; ++c) {
 #pragma unroll
-        for (int kk = 0; kk < KSLICES; ++kk) {
-          const uint64_t ad = kmajor_desc<ROWB>(sa + kk * 32);
-          for (int c = 0; c < a.nsub; ++c) {
+          for (int t = 0; t < NT; ++t) {
+            ok = mbar_wait(bfull0 + 8 * sl, ph, a.err, DEV_TIMEOUT_FULL);
+            if (!ok) break;
+            tc_fence_after();
+            const uint32_t sb = smem_u32(ringB) + (uint32_t)sl * slot_bytes;
 #pragma unroll
-            for (int t = 0; t < NT; ++t) {
-              const uint64_t bd =
-                  kmajor_desc<ROWB>(sb + t * b_bytes + (uint32_t)(c * chunk * ROWB) + kk * 32);
+            for (int kk = 0; kk < KSLICES; ++kk) {
+              const uint64_t ad = sw128_desc(sa + kk * 32), bd = sw128_desc(sb + kk * 32);
               const uint32_t acc = (ks | kk | t) != 0 ? 1u : 0u;
               if constexpr (GF == FMT_E4M3)
                 mma_f8(tmem_base + (uint32_t)(c * chunk), ad, bd, idesc, acc);
               else
                 mma_f16(tmem_base + (uint32_t)(c * chunk), ad, bd, idesc, acc);
             }
+            tc_commit(bempty0 + 8 * sl);
+            if (++sl == NB) {
+              sl = 0;
+              ph ^= 1u;
+            }
           }
         }
-        if constexpr (SHARE) tc_commit_mc(empty0 + 8 * st, (uint16_t)0x3);
-        else tc_commit(empty0 + 8 * st);
+        if constexpr (SHARE) tc_commit_mc(aempty0 + 8 * st, (uint16_t)0x3);
+        else tc_commit(aempty0 + 8 * st);
       }
       tc_commit(done_bar);
     }
@@ -564,60 +608,51 @@ __global__ void __launch_bounds__(kSkThreads, 1)
     // ---------------- generator warps: fl_s(G) tile, 128 rows x BK columns
     const int g = threadIdx.x - 64;
     for (int ks = 0; ks < nk; ++ks) {
-      const int st = ks % STAGES;
-      const uint32_t ph = (uint32_t)(ks / STAGES) & 1u;
-      if (!mbar_wait(empty0 + 8 * st, ph ^ 1u, a.err, DEV_TIMEOUT_EMPTY)) break;
+      const int st = ks % NA;
+      const uint32_t ph = (uint32_t)(ks / NA) & 1u;
+      if (!mbar_wait(aempty0 + 8 * st, ph ^ 1u, a.err, DEV_TIMEOUT_EMPTY)) break;
       if (!mbar_wait(fixed0 + 8 * st, ph ^ 1u, a.err, DEV_TIMEOUT_EMPTY)) break;
-      uint8_t* S = smem + st * stage_bytes;
-      uint32_t* qb = qbuf + st * (kSkQMax * 3);
+      uint8_t* S = ringA + st * S_BYTES;
       const int64_t kbase = k_begin + (int64_t)ks * BK;
-      // SPL threads per 16-byte chunk (two when a half tile has fewer chunks than there are
-      // generator threads: each then takes one Philox call and writes 8 bytes)
-      constexpr int SPL = (SHARE && EB == 2 && GCH * 2 <= kSkGenThreads) ? 2 : 1;
-      constexpr int HPI = (EPC / 4) / SPL;   // Philox calls per thread and chunk
-      for (int itm = g; itm < GCH * SPL; itm += kSkGenThreads) {
-        const int c = itm / SPL, hp = itm % SPL;
+      // One 16-byte chunk (HPI Philox calls, PPC pairs) per item.  No branch until every pair of
+      // the thread is estimated: the calls interleave, and und collects the undecided pairs.
+      constexpr int HPI = EPC / 4;
+      constexpr int IPT = (GCH + kSkGenThreads - 1) / kSkGenThreads;   // items per thread
+      static_assert(GCH % kSkGenThreads == 0 && IPT * PPC <= 32, "whole items, one bit per pair");
+      uint32_t und = 0;
+#pragma unroll
+      for (int it = 0; it < IPT; ++it) {
+        const int c = g + it * kSkGenThreads;
         const int row = c / CPR + (int)rank * 64, kc = c % CPR;
         const uint32_t i = (uint32_t)(mt * 128 + row);
         const uint64_t q0 = (uint64_t)(kbase + kc * EPC) >> 2;
-        uint32_t w[4] = {0u, 0u, 0u, 0u};
+        uint32_t w[4];
 #pragma unroll
-        for (int hh = 0; hh < HPI; ++hh) {
-          const int h = hp * HPI + hh;
+        for (int h = 0; h < HPI; ++h) {
           const uint4 x = philox4x32_10(gauss_counter(q0 + h, i), a.k0, a.k1);
           uint32_t p0, p1;   // the two pairs of the call, packed
           const bool ok0 = gauss_pair_est<GF>(x.x, x.y, p0);
           const bool ok1 = gauss_pair_est<GF>(x.z, x.w, p1);
-          if (!ok0 || !ok1) {
-#pragma unroll
-            for (int p2 = 0; p2 < 2; ++p2) {
-              if (p2 == 0 ? ok0 : ok1) continue;
-              const uint32_t pa = p2 == 0 ? x.x : x.z, pb = p2 == 0 ? x.y : x.w;
-              const uint32_t slot = atomicAdd(qcnt + st, 1u);
-              if (slot < (uint32_t)kSkQMax) {
-                qb[slot * 3 + 0] = ((uint32_t)row << 8) | ((uint32_t)kc << 4) | (uint32_t)(2 * h + p2);
-                qb[slot * 3 + 1] = pa;
-                qb[slot * 3 + 2] = pb;
-              } else {   // queue full: resolve in place
-                uint32_t be, bo;
-                gauss_pair_slow<GF>(pa, pb, be, bo);
-                const uint32_t v = be | (bo << (8 * EB));
-                if (p2 == 0) p0 = v;
-                else p1 = v;
-              }
-            }
-          }
+          und |= (ok0 ? 0u : 1u << (it * PPC + 2 * h)) | (ok1 ? 0u : 2u << (it * PPC + 2 * h));
           if constexpr (EB == 2) {
-            w[2 * hh] = p0;
-            w[2 * hh + 1] = p1;
+            w[2 * h] = p0;
+            w[2 * h + 1] = p1;
           } else {
-            w[hh] = p0 | (p1 << 16);
+            w[h] = p0 | (p1 << 16);
           }
         }
-        if constexpr (SPL == 1)
-          *reinterpret_cast<uint4*>(S + swz_chunk<ROWB>(row, kc)) = make_uint4(w[0], w[1], w[2], w[3]);
-        else
-          *reinterpret_cast<uint2*>(S + swz_chunk<ROWB>(row, kc) + 8 * hp) = make_uint2(w[0], w[1]);
+        *reinterpret_cast<uint4*>(S + swz_chunk(row, kc)) = make_uint4(w[0], w[1], w[2], w[3]);
+      }
+      while (und != 0u) {
+        const int bit = __ffs((int)und) - 1;
+        und &= und - 1u;
+        const int c = g + (bit / PPC) * kSkGenThreads;
+        const int row = c / CPR + (int)rank * 64, kc = c % CPR, pi = bit % PPC;
+        const uint32_t slot = atomicAdd(qcnt + st, 1u);
+        if (slot < (uint32_t)kSkQMax)
+          qbuf[st * kSkQMax + slot] = ((uint32_t)row << 8) | ((uint32_t)kc << 4) | (uint32_t)pi;
+        else   // queue full: resolve in place
+          resolve_pair(S, row, kc, pi, kbase);
       }
       fence_proxy_async_smem();
       __syncwarp();
@@ -626,49 +661,45 @@ __global__ void __launch_bounds__(kSkThreads, 1)
   } else {
     // ---------------- fixer warps: the queued pairs of a stage, overlapping the generation
     // of the next one
-    const int fx = threadIdx.x - kSkFixFirst * 32;
-    for (int ks = 0; ks < nk; ++ks) {
-      const int st = ks % STAGES;
-      const uint32_t ph = (uint32_t)(ks / STAGES) & 1u;
+    const int group = (warp - kSkFixFirst) / kSkFixWarps;
+    const int fx = threadIdx.x - (kSkFixFirst + group * kSkFixWarps) * 32;
+    for (int ks = group; ks < nk; ks += kSkFixGroups) {
+      const int st = ks % NA;
+      const uint32_t ph = (uint32_t)(ks / NA) & 1u;
       if (!mbar_wait(genned0 + 8 * st, ph, a.err, DEV_TIMEOUT_FULL)) break;
-      uint8_t* S = smem + st * stage_bytes;
-      const uint32_t* qb = qbuf + st * (kSkQMax * 3);
+      uint8_t* S = ringA + st * S_BYTES;
+      const int64_t kbase = k_begin + (int64_t)ks * BK;
       const uint32_t nq = min(qcnt[st], (uint32_t)kSkQMax);
       for (uint32_t qi = fx; qi < nq; qi += kSkFixThreads) {
-        const uint32_t pos = qb[qi * 3];
-        uint32_t be, bo;
-        gauss_pair_resolve<GF>(qb[qi * 3 + 1], qb[qi * 3 + 2], be, bo);
-        const int row = (int)(pos >> 8), kc = (int)((pos >> 4) & 15), pi = (int)(pos & 15);
-        uint8_t* cp = S + swz_chunk<ROWB>(row, kc);
-        if constexpr (EB == 2)
-          *reinterpret_cast<uint32_t*>(cp + 4 * pi) = be | (bo << 16);
-        else
-          *reinterpret_cast<uint16_t*>(cp + 2 * pi) = (uint16_t)(be | (bo << 8));
+        const uint32_t pos = qbuf[st * kSkQMax + qi];
+        resolve_pair(S, (int)(pos >> 8), (int)((pos >> 4) & 15), (int)(pos & 15), kbase);
       }
       fence_proxy_async_smem();
-      fix_barrier();            // every fixer has read qcnt and written its pairs
+      fix_barrier(group);       // the group has read qcnt and written its pairs
       if (fx == 0) {
         qcnt[st] = 0;
         if constexpr (SHARE) {   // the finished half tile: whole rows, one contiguous run
           const uint32_t src = smem_u32(S) + rank * HALF;
-          bulk_s2s(cl_map(src, rank ^ 1u), src, HALF, cl_map(full0 + 8 * st, rank ^ 1u));
+          bulk_s2s(cl_map(src, rank ^ 1u), src, HALF, cl_map(afull0 + 8 * st, rank ^ 1u));
         }
       }
       __syncwarp();
       if (lane == 0) {
-        mbar_arrive(full0 + 8 * st);
+        if (SHARE && fx == 0) mbar_arrive_expect_tx(afull0 + 8 * st, HALF);   // the partner's half
+        else mbar_arrive(afull0 + 8 * st);
         mbar_arrive(fixed0 + 8 * st);
       }
     }
   }
 
-  // ---------------- epilogue: warps 4..7 drain TMEM lanes 32q .. 32q+31
-  if (warp >= 4 && warp < 8) {
+  // ---------------- epilogue: the generator warps drain TMEM, four warps to each quarter of
+  // its lanes (a warp reaches lanes 32 (warp % 4) ..), 32 columns at a time
+  if (warp >= 2 && warp < kSkFixFirst) {
     mbar_wait(done_bar, 0, a.err, DEV_TIMEOUT_DONE);
     tc_fence_after();
     const int q = warp & 3;
     const int64_t i = mt * 128 + q * 32 + lane;
-    for (int c0 = 0; c0 < a.bn; c0 += 32) {
+    for (int c0 = 32 * ((warp - 2) >> 2); c0 < a.bn; c0 += 32 * (kSkGenWarps / 4)) {
       uint32_t r[32];
       tmem_ld_32x32b_x32(tmem_base + ((uint32_t)(q * 32) << 16) + (uint32_t)c0, r);
       tmem_ld_wait();
@@ -699,7 +730,7 @@ bool plan_sketch_tc(int fmt, int64_t s, int64_t m, int64_t ncols, int num_sms, S
   const int EB = (fmt == FMT_E4M3) ? 1 : 2;
   p->nt = (fmt == FMT_BF16X3) ? 3 : 1;
   p->rowb = (p->nt == 3) ? 64 : 128;
-  const int BK = p->rowb / EB;
+  const int BK = kSkRowB / EB;   // the kernel's K step
   p->fmt = fmt;
   p->s = s;
   p->m = m;
@@ -715,6 +746,8 @@ bool plan_sketch_tc(int fmt, int64_t s, int64_t m, int64_t ncols, int num_sms, S
   p->bn = bn;
   p->mtiles = (int)((s + 127) / 128);
   const size_t stage = (size_t)128 * p->rowb + (size_t)p->nt * bn * p->rowb;
+  // the ring the plan guarantees room for: whole stages of rowb-byte rows, at least two (the
+  // kernel lays out its rings in the SM's whole shared memory)
   p->stages = (4 * stage + 1024 + 512 + 4 * kSkQMax * 12 <= 232448) ? 4 : 2;
   p->smem = 1024 + (size_t)p->stages * stage + 512 + (size_t)p->stages * kSkQMax * 12;
   if (p->smem > 232448) return false;
@@ -763,8 +796,7 @@ bool plan_sketch_tc(int fmt, int64_t s, int64_t m, int64_t ncols, int num_sms, S
   return true;
 }
 
-bool encode_bt_tmap(CUtensorMap* tm, const void* Bt, int fmt, int64_t rows, int64_t m, int box_rows,
-                    int rowb) {
+bool encode_bt_tmap(CUtensorMap* tm, const void* Bt, int fmt, int64_t rows, int64_t m, int box_rows) {
   // looked up once (thread-safe static initialisation; batched solves call this
   // from several host threads)
   static const PFN_cuTensorMapEncodeTiled_v12000 fn = []() -> PFN_cuTensorMapEncodeTiled_v12000 {
@@ -778,34 +810,34 @@ bool encode_bt_tmap(CUtensorMap* tm, const void* Bt, int fmt, int64_t rows, int6
   }();
   if (!fn) return false;
   const int EB = (fmt == FMT_E4M3) ? 1 : 2;
-  if (kBtBlock % (rowb / EB) != 0) return false;   // a stage never straddles two blocks
+  static_assert(kBtBlock % kSkRowB == 0, "a stage never straddles two blocks");
   // (k within the block, row over all planes, block)
   cuuint64_t dims[3] = {(cuuint64_t)kBtBlock, (cuuint64_t)rows, (cuuint64_t)bt_blocks(m)};
   cuuint64_t strides[2] = {(cuuint64_t)(kBtBlock * EB), (cuuint64_t)(rows * kBtBlock * EB)};
-  cuuint32_t box[3] = {(cuuint32_t)(rowb / EB), (cuuint32_t)box_rows, 1};
+  cuuint32_t box[3] = {(cuuint32_t)(kSkRowB / EB), (cuuint32_t)box_rows, 1};
   cuuint32_t es[3] = {1, 1, 1};
   CUresult r = fn(tm, EB == 2 ? CU_TENSOR_MAP_DATA_TYPE_UINT16 : CU_TENSOR_MAP_DATA_TYPE_UINT8, 3,
                   const_cast<void*>(Bt), dims, strides, box, es, CU_TENSOR_MAP_INTERLEAVE_NONE,
-                  rowb == 128 ? CU_TENSOR_MAP_SWIZZLE_128B : CU_TENSOR_MAP_SWIZZLE_64B,
+                  CU_TENSOR_MAP_SWIZZLE_128B,
                   CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
                   CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
   return r == CUDA_SUCCESS;
 }
 
-template <int FMT, int STAGES, int ROWB, int NT>
+template <int FMT, int NT>
 static cudaError_t launch_tc_inst(const SketchPlan& p, const CUtensorMap& tm, const SketchTcArgs& a,
                                   cudaStream_t st) {
   dim3 grid((unsigned)p.mtiles, (unsigned)p.ngroups, (unsigned)p.splits);
   const SketchGroup none{};
   if (p.ngroups == 2) {
     // the two column groups of a (tile, split) share the generated operand (a cluster of two)
-    auto kern = sketch_tc_kernel<FMT, STAGES, ROWB, NT, false, true>;
-    cudaError_t e = allow_dyn_smem(kern, (size_t)p.smem);
+    auto kern = sketch_tc_kernel<FMT, NT, false, true>;
+    cudaError_t e = allow_dyn_smem(kern, kSkSmem);
     if (e != cudaSuccess) return e;
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = grid;
     cfg.blockDim = dim3(kSkThreads);
-    cfg.dynamicSmemBytes = p.smem;
+    cfg.dynamicSmemBytes = kSkSmem;
     cfg.stream = st;
     cudaLaunchAttribute attr[1];
     attr[0].id = cudaLaunchAttributeClusterDimension;
@@ -816,37 +848,32 @@ static cudaError_t launch_tc_inst(const SketchPlan& p, const CUtensorMap& tm, co
     cfg.numAttrs = 1;
     return cudaLaunchKernelEx(&cfg, kern, tm, a, none);
   }
-  auto kern = sketch_tc_kernel<FMT, STAGES, ROWB, NT, false>;
-  cudaError_t e = allow_dyn_smem(kern, (size_t)p.smem);
+  auto kern = sketch_tc_kernel<FMT, NT, false>;
+  cudaError_t e = allow_dyn_smem(kern, kSkSmem);
   if (e != cudaSuccess) return e;
-  kern<<<grid, kSkThreads, p.smem, st>>>(tm, a, none);
+  kern<<<grid, kSkThreads, kSkSmem, st>>>(tm, a, none);
   return cudaGetLastError();
 }
 
-template <int FMT, int STAGES, int ROWB, int NT>
-static cudaError_t launch_tc_grouped_inst(const SketchGroup& g, int64_t ctas, size_t smem, cudaStream_t st) {
-  auto kern = sketch_tc_kernel<FMT, STAGES, ROWB, NT, true>;
-  cudaError_t e = allow_dyn_smem(kern, smem);
+template <int FMT, int NT>
+static cudaError_t launch_tc_grouped_inst(const SketchGroup& g, int64_t ctas, cudaStream_t st) {
+  auto kern = sketch_tc_kernel<FMT, NT, true>;
+  cudaError_t e = allow_dyn_smem(kern, kSkSmem);
   if (e != cudaSuccess) return e;
   CUtensorMap unused;
   std::memset(&unused, 0, sizeof(unused));
-  kern<<<(unsigned)ctas, kSkThreads, smem, st>>>(unused, SketchTcArgs{}, g);
+  kern<<<(unsigned)ctas, kSkThreads, kSkSmem, st>>>(unused, SketchTcArgs{}, g);
   return cudaGetLastError();
 }
 
 cudaError_t launch_sketch_tc(const SketchPlan& p, const CUtensorMap& tm, uint64_t seed,
                              float* partial, int* err, cudaStream_t st) {
   const SketchTcArgs a = sketch_tc_args(p, seed, partial, err);
-  const bool four = p.stages == 4;
   switch (p.fmt) {
-    case FMT_F16: return four ? launch_tc_inst<FMT_F16, 4, 128, 1>(p, tm, a, st)
-                              : launch_tc_inst<FMT_F16, 2, 128, 1>(p, tm, a, st);
-    case FMT_BF16: return four ? launch_tc_inst<FMT_BF16, 4, 128, 1>(p, tm, a, st)
-                               : launch_tc_inst<FMT_BF16, 2, 128, 1>(p, tm, a, st);
-    case FMT_E4M3: return four ? launch_tc_inst<FMT_E4M3, 4, 128, 1>(p, tm, a, st)
-                               : launch_tc_inst<FMT_E4M3, 2, 128, 1>(p, tm, a, st);
-    case FMT_BF16X3: return four ? launch_tc_inst<FMT_BF16X3, 4, 64, 3>(p, tm, a, st)
-                                 : launch_tc_inst<FMT_BF16X3, 2, 64, 3>(p, tm, a, st);
+    case FMT_F16: return launch_tc_inst<FMT_F16, 1>(p, tm, a, st);
+    case FMT_BF16: return launch_tc_inst<FMT_BF16, 1>(p, tm, a, st);
+    case FMT_E4M3: return launch_tc_inst<FMT_E4M3, 1>(p, tm, a, st);
+    case FMT_BF16X3: return launch_tc_inst<FMT_BF16X3, 3>(p, tm, a, st);
   }
   return cudaErrorInvalidValue;
 }
@@ -873,20 +900,14 @@ SketchTcArgs sketch_tc_args(const SketchPlan& p, uint64_t seed, float* partial, 
   return a;
 }
 
-cudaError_t launch_sketch_tc_grouped(int fmt, int stages, const SketchGroup& g, int64_t ctas, size_t smem,
-                                     cudaStream_t st) {
+cudaError_t launch_sketch_tc_grouped(int fmt, const SketchGroup& g, int64_t ctas, cudaStream_t st) {
   if (ctas <= 0) return cudaSuccess;
   if (ctas > 2147483647LL) return cudaErrorInvalidValue;
-  const bool four = stages == 4;
   switch (fmt) {
-    case FMT_F16: return four ? launch_tc_grouped_inst<FMT_F16, 4, 128, 1>(g, ctas, smem, st)
-                              : launch_tc_grouped_inst<FMT_F16, 2, 128, 1>(g, ctas, smem, st);
-    case FMT_BF16: return four ? launch_tc_grouped_inst<FMT_BF16, 4, 128, 1>(g, ctas, smem, st)
-                               : launch_tc_grouped_inst<FMT_BF16, 2, 128, 1>(g, ctas, smem, st);
-    case FMT_E4M3: return four ? launch_tc_grouped_inst<FMT_E4M3, 4, 128, 1>(g, ctas, smem, st)
-                               : launch_tc_grouped_inst<FMT_E4M3, 2, 128, 1>(g, ctas, smem, st);
-    case FMT_BF16X3: return four ? launch_tc_grouped_inst<FMT_BF16X3, 4, 64, 3>(g, ctas, smem, st)
-                                 : launch_tc_grouped_inst<FMT_BF16X3, 2, 64, 3>(g, ctas, smem, st);
+    case FMT_F16: return launch_tc_grouped_inst<FMT_F16, 1>(g, ctas, st);
+    case FMT_BF16: return launch_tc_grouped_inst<FMT_BF16, 1>(g, ctas, st);
+    case FMT_E4M3: return launch_tc_grouped_inst<FMT_E4M3, 1>(g, ctas, st);
+    case FMT_BF16X3: return launch_tc_grouped_inst<FMT_BF16X3, 3>(g, ctas, st);
   }
   return cudaErrorInvalidValue;
 }

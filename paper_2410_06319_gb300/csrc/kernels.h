@@ -92,7 +92,7 @@ struct SketchPlan {
   int64_t s_pad;       // rows of the partial buffers
   int stages;
   int nt;              // B planes (1, or 3 for the split-term BF16 sketch)
-  int rowb;            // bytes per K-major row of a stage (128 or 64)
+  int rowb;            // bytes per K-major row of the ring that smem counts (128 or 64)
   size_t smem;
 };
 
@@ -102,14 +102,11 @@ bool plan_sketch_tc(int fmt, int64_t s, int64_t m, int64_t ncols, int num_sms, S
                     int64_t max_kchunk = 0);
 // Encodes the 3-D TMA descriptor (k within a block, row over all planes, block) of Bt
 // (`rows` = planes x plane_rows).
-bool encode_bt_tmap(CUtensorMap* tm, const void* Bt, int fmt, int64_t rows, int64_t m, int box_rows,
-                    int rowb);
+bool encode_bt_tmap(CUtensorMap* tm, const void* Bt, int fmt, int64_t rows, int64_t m, int box_rows);
 // The arguments launch_sketch_tc builds for plan p, for a grouped table.
 SketchTcArgs sketch_tc_args(const SketchPlan& p, uint64_t seed, float* partial, int* err);
-// One launch for a batch: ctas = start[nprob]; smem = the largest plan's; every plan must
-// have the same format and stage count.
-cudaError_t launch_sketch_tc_grouped(int fmt, int stages, const SketchGroup& g, int64_t ctas, size_t smem,
-                                     cudaStream_t st);
+// One launch for a batch: ctas = start[nprob]; every plan must have the same format.
+cudaError_t launch_sketch_tc_grouped(int fmt, const SketchGroup& g, int64_t ctas, cudaStream_t st);
 // Grouped cast: colmax CTAs (ceil(m / kGroupedColmaxRows) per problem), exponent CTAs
 // (ceil((n + 1) / 256)), cast CTAs (cast_gx x ceil(plane_rows / 32)); t as in launch_scale_exps.
 cudaError_t launch_grouped_cast(int fmt, const GCast* tab, const int* colmax_start, int64_t colmax_ctas,
