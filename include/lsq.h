@@ -189,7 +189,7 @@ typedef struct lsq_info {
   double gmres_relres[32];  /* FGMRES relative residual reached in each refinement step */
   double kern_ms[8];        /* with opts->timing: summed device time of the sketch GEMM, LSQR
                                pass, FGMRES pass, residual pass, FGMRES Arnoldi step, FGMRES
-                               triangular solves and the sketch's deferred correction; one
+                               triangular products and the sum of the sketch's splits; one
                                entry spare */
   int64_t kern_launches[8]; /* number of launches behind each kern_ms entry */
   int64_t arnoldi_second_passes; /* FGMRES Arnoldi steps that ran the second Gram-Schmidt pass */

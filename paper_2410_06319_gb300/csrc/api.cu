@@ -59,6 +59,7 @@ void stage_sketch(Ctx& c, double* Y, const float* a32) {
       KernTimer kt(c.h, K_SKETCH, c.o.timing);
       L(launch_sketch_tc(p, tm, c.seed, partial, c.h->d_err, c.st));
     }
+    KernTimer kt(c.h, K_SKETCH_SUM, c.o.timing);
     L(launch_sketch_reduce(partial, false, p.splits, ncols, c.s, p.s_pad, kexp, Y, c.st));
   } else {
     StageTimer tt(c.h, ST_SKETCH);

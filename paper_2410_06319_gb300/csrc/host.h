@@ -136,7 +136,7 @@ struct StageTimer {
 };
 
 enum Stage { ST_CAST = 0, ST_SKETCH, ST_QR, ST_LSQR, ST_RES, ST_FGMRES, ST_UPDATE, ST_TOTAL };
-enum Kern { K_SKETCH = 0, K_LSQR_PASS, K_FGM_PASS, K_RES_PASS, K_ARNOLDI, K_TRSV, K_SKETCH_FIX,
+enum Kern { K_SKETCH = 0, K_LSQR_PASS, K_FGM_PASS, K_RES_PASS, K_ARNOLDI, K_TRSV, K_SKETCH_SUM,
             K_NKERN = 8 };
 constexpr int kKernMark = 100;   // marks with stage >= kKernMark time single kernels
 
