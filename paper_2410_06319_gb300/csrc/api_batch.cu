@@ -435,7 +435,6 @@ lsq_status lsq_batch_grouped(lsq_handle* h, int32_t nprob, const lsq_problem* pr
       g.kexp = aK.at<int>(p);
       g.Bt = aBt.at<void>(p);
       g.plane_rows = (int64_t)pl.ngroups * pl.bn;
-      g.cast_gx = cast_row_tiles(fmt, b.m[p]);
       tcast[p] = g;
     }
     {

@@ -100,6 +100,36 @@ LSQ_HD bool cast_terms_int(uint64_t u, int k, uint32_t (&t)[3]) {
   return enc_term<F>(sg, a, E - 1075 + k, t[0], rd);
 }
 
+// fl(2^k x) for a 16- or 8-bit format from the two words of x alone, for results in the
+// format's normal range: the low word only breaks ties, so it is folded into the last bit of
+// the high word as a sticky bit, and one add rounds the high word at the format's last bit
+// (nearest, ties to even); a carry moves into the exponent.  Per column (k) the exponent
+// range and rebias are fixed: about 15 instructions an element against 90 for the general
+// rounding on the 53-bit significand.
+struct CastRange {
+  uint32_t lo, hi;   // |x|'s high word before rounding >= lo, after rounding < hi
+  uint32_t base;     // subtracted from the rounded pattern: the exponent's rebias
+};
+template <class F>
+LSQ_HD CastRange cast_range(int k) {
+  // normal FP64 exponents E (1 .. 2046) with EMIN <= E - 1023 + k <= EMAX
+  int e0 = F::EMIN + 1023 - k, e1 = F::EMAX + 1023 - k + 1;
+  if (e0 < 1) e0 = 1;
+  if (e0 > 2047) e0 = 2047;
+  if (e1 > 2047) e1 = 2047;
+  if (e1 < 0) e1 = 0;
+  return CastRange{(uint32_t)e0 << 20, (uint32_t)e1 << 20, (uint32_t)(1023 - k - F::BIAS) << F::MB};
+}
+template <class F>
+LSQ_HD bool cast_hi(uint64_t u, const CastRange& c, uint32_t& bits) {
+  constexpr int SH = 20 - F::MB;
+  const uint32_t w = (uint32_t)(u >> 32) | ((uint32_t)u != 0u ? 1u : 0u);
+  const uint32_t mag = w & 0x7FFFFFFFu;
+  const uint32_t r = mag + ((1u << (SH - 1)) - 1u) + ((mag >> SH) & 1u);
+  bits = ((r >> SH) - c.base) | ((w >> 31) << (F::W - 1));
+  return mag >= c.lo && r < c.hi;
+}
+
 // fl32(x) for x given by its FP64 bits, when the result is a normal FP32 number or an
 // infinity reached by rounding (biased FP64 exponent 897 .. 1150): round the 53-bit
 // significand at bit 29 to nearest even by one 64-bit add (a carry out of the fraction

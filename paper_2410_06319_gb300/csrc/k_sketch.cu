@@ -14,8 +14,8 @@
 //  * reduce: FP64 sum of the split partials, times s^-1/2 and 2^-k_j.
 #include <cudaTypedefs.h>
 
-#include <algorithm>
 #include <cstring>
+#include <type_traits>
 
 #include "cast.cuh"
 #include "common.cuh"
@@ -215,47 +215,55 @@ __device__ __forceinline__ void cast_bits(uint64_t u, int k, uint32_t (&t)[3]) {
 // sketch CTA's K chunk of its column group lies in one contiguous stretch of a
 // few MB (a K-major layout with m-long rows puts every row of a stage on its
 // own page once m is in the millions).
+//
+// Single-term formats: tiles of 32 columns by as many rows as make 128 bytes of a column of
+// Bt (64 rows; 128 for E4M3).  Each thread issues its loads of a column eight at a time and
+// rounds on the high word (cast_hi; the general rounding of the few other values follows),
+// the tile is transposed in its final format, and a warp stores 128 contiguous bytes.  Column
+// tile fastest, as in the BF16X3 cast.  Bound by HBM (8 bytes read, 2 or 1 written a value):
+// at 116 instructions an element and 32 x 32 tiles of 8-byte words it was bound by
+// instruction issue (BF16, m = 1e5, n = 500: 201 us; now 87 us).
+template <int FMT>
+constexpr int kCastRows = FMT == FMT_E4M3 ? 128 : 64;
 template <int FMT>
 __device__ __forceinline__ void cast_transpose_body(const double* __restrict__ A, int64_t lda,
                                                     const double* __restrict__ b, int64_t m, int64_t n,
                                                     const int* __restrict__ kexp, void* __restrict__ Bt,
-                                                    int64_t plane_rows, int planes, int64_t bx, int64_t by) {
-  __shared__ uint64_t tile[32][33];
-  const int64_t j0 = bx * 32, c0 = by * 32;
-  const uint64_t* Au = reinterpret_cast<const uint64_t*>(A);
-  const uint64_t* bu = reinterpret_cast<const uint64_t*>(b);
-  for (int r = threadIdx.y; r < 32; r += 8) {
-    const int64_t j = j0 + r, c = c0 + threadIdx.x;
-    uint64_t v = 0;
-    if (j < m) {
-      if (c < n) v = __ldcs(Au + j * lda + c);
-      else if (c == n) v = bu[j];
+                                                    int64_t plane_rows, int64_t bx, int64_t by) {
+  using F = typename FmtEnc<FMT>::T;
+  using E = typename std::conditional<FMT == FMT_E4M3, uint8_t, uint16_t>::type;
+  constexpr int ROWS = kCastRows<FMT>, VPW = 4 / (int)sizeof(E);
+  __shared__ uint32_t tile[32][33];   // [column][row], VPW values a word, one word of padding
+  const int64_t j0 = bx * ROWS, c0 = by * 32, c = c0 + threadIdx.x;
+  const uint64_t* src = reinterpret_cast<const uint64_t*>(c < n ? A + c : b);
+  const int64_t stride = c < n ? lda : 1;
+  const int k = c <= n ? kexp[c] : 0;
+  const CastRange cr = cast_range<F>(k);
+  E* col = reinterpret_cast<E*>(tile[threadIdx.x]);
+#pragma unroll
+  for (int h = 0; h < ROWS / 64; ++h) {
+    uint64_t u[8];
+#pragma unroll
+    for (int q = 0; q < 8; ++q) {
+      const int64_t j = j0 + h * 64 + threadIdx.y + 8 * q;
+      u[q] = (c <= n && j < m) ? __ldcs(src + j * stride) : 0ull;
     }
-    tile[r][threadIdx.x] = v;
+#pragma unroll
+    for (int q = 0; q < 8; ++q) {
+      uint32_t v;
+      if (!cast_hi<F>(u[q], cr, v)) {
+        uint32_t t[3];
+        cast_bits<FMT>(u[q], k, t);
+        v = t[0];
+      }
+      col[h * 64 + threadIdx.y + 8 * q] = (E)v;
+    }
   }
   __syncthreads();
-  for (int r = threadIdx.y; r < 32; r += 8) {
-    const int64_t c = c0 + r, j = j0 + threadIdx.x;
-    if (c >= plane_rows) continue;
-    // every (row, k) of the padded blocks is written: zeros past column n and row m
-    const int64_t blk = j / kBtBlock, kk = j % kBtBlock;
-    const int64_t base = (blk * planes * plane_rows + c) * kBtBlock + kk;
-    const bool live = c <= n && j < m;
-    const uint64_t u = tile[threadIdx.x][r];
-    const int k = live ? kexp[c] : 0;
-    if constexpr (FMT == FMT_F32) {
-      const double v = ldexp(__longlong_as_double((long long)u), k);
-      reinterpret_cast<float*>(Bt)[base] = live ? __double2float_rn(v) : 0.0f;
-    } else {
-      uint32_t tt[3] = {0u, 0u, 0u};
-      if (live) cast_bits<FMT>(u, k, tt);
-      if constexpr (FMT == FMT_E4M3) {
-        reinterpret_cast<uint8_t*>(Bt)[base] = (uint8_t)tt[0];
-      } else {
-        reinterpret_cast<uint16_t*>(Bt)[base] = (uint16_t)tt[0];
-      }
-    }
-  }
+  const int64_t j = j0 + VPW * threadIdx.x, blk = j / kBtBlock, kk = j % kBtBlock;
+  uint32_t* P = reinterpret_cast<uint32_t*>(Bt);
+  for (int r = threadIdx.y; r < 32; r += 8)   // rows past column n and data rows past m: zeros
+    if (c0 + r < plane_rows) P[((blk * plane_rows + c0 + r) * kBtBlock + kk) / VPW] = tile[r][threadIdx.x];
 }
 
 // BF16X3: y = fl32(2^k x) in three BF16 planes hi, lo, lo2 (same Bt layout).  Tiles of
@@ -302,12 +310,15 @@ __device__ __forceinline__ void cast_bf16x3_body(const double* __restrict__ A, i
     const int64_t cc = c0 + r;
     if (cc >= plane_rows) continue;
     const int64_t base = ((blk * 3 * plane_rows + cc) * kBtBlock + kk) / 2;
-    uint32_t t0[3], t1[3];
-    split3_f32(tile[r][2 * threadIdx.x], t0);
-    split3_f32(tile[r][2 * threadIdx.x + 1], t1);
-    P[base] = t0[0] | (t1[0] << 16);
-    P[base + pstride] = t0[1] | (t1[1] << 16);
-    P[base + 2 * pstride] = t0[2] | (t1[2] << 16);
+    // the split of two values (cast.cuh: split3_f32) with the packed FP32 -> BF16 rounding
+    float y0 = __uint_as_float(tile[r][2 * threadIdx.x]), y1 = __uint_as_float(tile[r][2 * threadIdx.x + 1]);
+#pragma unroll
+    for (int t = 0; t < 3; ++t) {
+      const uint32_t w = pack2<FMT_BF16>(y0, y1);
+      P[base + t * pstride] = w;
+      y0 = __fsub_rn(y0, __uint_as_float(w << 16));
+      y1 = __fsub_rn(y1, __uint_as_float(w & 0xFFFF0000u));
+    }
   }
 }
 
@@ -325,42 +336,36 @@ template <int FMT>
 __global__ void cast_transpose_kernel(const double* __restrict__ A, int64_t lda,
                                       const double* __restrict__ b, int64_t m, int64_t n,
                                       const int* __restrict__ kexp, void* __restrict__ Bt,
-                                      int64_t plane_rows, int planes) {
-  cast_transpose_body<FMT>(A, lda, b, m, n, kexp, Bt, plane_rows, planes, blockIdx.x, blockIdx.y);
+                                      int64_t plane_rows) {
+  const int64_t ct = (plane_rows + 31) / 32, id = blockIdx.x;
+  cast_transpose_body<FMT>(A, lda, b, m, n, kexp, Bt, plane_rows, id / ct, id % ct);
 }
 
 int64_t bt_blocks(int64_t m) { return (m + kBtBlock - 1) / kBtBlock; }
 
 size_t bt_bytes(int fmt, int64_t m, int64_t plane_rows) {
-  const int esz = (fmt == FMT_E4M3) ? 1 : (fmt == FMT_F32 ? 4 : 2);
+  const int esz = (fmt == FMT_E4M3) ? 1 : 2;
   const int planes = (fmt == FMT_BF16X3) ? 3 : 1;
   return (size_t)bt_blocks(m) * planes * plane_rows * kBtBlock * esz;
 }
 
 int64_t cast_row_tiles(int fmt, int64_t m) {
-  return bt_blocks(m) * kBtBlock / (fmt == FMT_BF16X3 ? kCast3Rows : 32);
+  return bt_blocks(m) * kBtBlock / (fmt == FMT_BF16X3 ? kCast3Rows : fmt == FMT_E4M3 ? kCastRows<FMT_E4M3> : kCastRows<FMT_BF16>);
 }
 
 cudaError_t launch_cast_transpose(int fmt, const double* A, int64_t lda, const double* b, const float* a32,
                                   int64_t lda32, int64_t m, int64_t n, const int* kexp, void* Bt,
                                   int64_t plane_rows, cudaStream_t st) {
   if (plane_rows < n + 1) return cudaErrorInvalidValue;
-  const int planes = (fmt == FMT_BF16X3) ? 3 : 1;
-  const int64_t gx = cast_row_tiles(fmt, m);
-  if (gx > 2147483647LL) return cudaErrorInvalidValue;
-  dim3 grid((unsigned)gx, (unsigned)((plane_rows + 31) / 32));
-  dim3 block(32, 8);
+  const int64_t tiles = cast_row_tiles(fmt, m) * ((plane_rows + 31) / 32);
+  if (tiles > 2147483647LL) return cudaErrorInvalidValue;
+  const unsigned grid = (unsigned)tiles;
+  const dim3 block(32, 8);
   switch (fmt) {
-    case FMT_F16: cast_transpose_kernel<FMT_F16><<<grid, block, 0, st>>>(A, lda, b, m, n, kexp, Bt, plane_rows, planes); break;
-    case FMT_BF16: cast_transpose_kernel<FMT_BF16><<<grid, block, 0, st>>>(A, lda, b, m, n, kexp, Bt, plane_rows, planes); break;
-    case FMT_E4M3: cast_transpose_kernel<FMT_E4M3><<<grid, block, 0, st>>>(A, lda, b, m, n, kexp, Bt, plane_rows, planes); break;
-    case FMT_F32: cast_transpose_kernel<FMT_F32><<<grid, block, 0, st>>>(A, lda, b, m, n, kexp, Bt, plane_rows, planes); break;
-    case FMT_BF16X3: {
-      const int64_t tiles = gx * ((plane_rows + 31) / 32);
-      if (tiles > 2147483647LL) return cudaErrorInvalidValue;
-      cast_bf16x3_kernel<<<(unsigned)tiles, block, 0, st>>>(A, lda, b, a32, lda32, m, n, kexp, Bt, plane_rows);
-      break;
-    }
+    case FMT_F16: cast_transpose_kernel<FMT_F16><<<grid, block, 0, st>>>(A, lda, b, m, n, kexp, Bt, plane_rows); break;
+    case FMT_BF16: cast_transpose_kernel<FMT_BF16><<<grid, block, 0, st>>>(A, lda, b, m, n, kexp, Bt, plane_rows); break;
+    case FMT_E4M3: cast_transpose_kernel<FMT_E4M3><<<grid, block, 0, st>>>(A, lda, b, m, n, kexp, Bt, plane_rows); break;
+    case FMT_BF16X3: cast_bf16x3_kernel<<<grid, block, 0, st>>>(A, lda, b, a32, lda32, m, n, kexp, Bt, plane_rows); break;
     default: return cudaErrorInvalidValue;
   }
   return cudaGetLastError();
@@ -1081,18 +1086,14 @@ __global__ void grouped_scale_exps_kernel(const GCast* __restrict__ tab, const i
 }
 
 template <int FMT>
-__global__ void grouped_cast_kernel(const GCast* __restrict__ tab, const int* __restrict__ start, int nprob,
-                                    int planes) {
+__global__ void grouped_cast_kernel(const GCast* __restrict__ tab, const int* __restrict__ start, int nprob) {
   const int p = group_of(start, nprob, blockIdx.x);
   const GCast& g = tab[p];
-  const int64_t local = (int64_t)blockIdx.x - start[p];
-  if constexpr (FMT == FMT_BF16X3) {   // column tile fastest, as cast_bf16x3_kernel
-    const int64_t ct = (g.plane_rows + 31) / 32;
+  const int64_t local = (int64_t)blockIdx.x - start[p], ct = (g.plane_rows + 31) / 32;   // column tile fastest
+  if constexpr (FMT == FMT_BF16X3)
     cast_bf16x3_body(g.A, g.lda, g.b, g.a32, g.lda32, g.m, g.n, g.kexp, g.Bt, g.plane_rows, local / ct, local % ct);
-  } else {
-    cast_transpose_body<FMT>(g.A, g.lda, g.b, g.m, g.n, g.kexp, g.Bt, g.plane_rows, planes, local % g.cast_gx,
-                             local / g.cast_gx);
-  }
+  else
+    cast_transpose_body<FMT>(g.A, g.lda, g.b, g.m, g.n, g.kexp, g.Bt, g.plane_rows, local / ct, local % ct);
 }
 
 __global__ void grouped_sketch_reduce_kernel(const GReduce* __restrict__ tab, const int* __restrict__ start,
@@ -1114,10 +1115,10 @@ cudaError_t launch_grouped_cast(int fmt, const GCast* tab, const int* colmax_sta
   const int planes = (fmt == FMT_BF16X3) ? 3 : 1;
   const dim3 block(32, 8);
   switch (fmt) {
-    case FMT_F16: grouped_cast_kernel<FMT_F16><<<(unsigned)cast_ctas, block, 0, st>>>(tab, cast_start, nprob, planes); break;
-    case FMT_BF16: grouped_cast_kernel<FMT_BF16><<<(unsigned)cast_ctas, block, 0, st>>>(tab, cast_start, nprob, planes); break;
-    case FMT_E4M3: grouped_cast_kernel<FMT_E4M3><<<(unsigned)cast_ctas, block, 0, st>>>(tab, cast_start, nprob, planes); break;
-    case FMT_BF16X3: grouped_cast_kernel<FMT_BF16X3><<<(unsigned)cast_ctas, block, 0, st>>>(tab, cast_start, nprob, planes); break;
+    case FMT_F16: grouped_cast_kernel<FMT_F16><<<(unsigned)cast_ctas, block, 0, st>>>(tab, cast_start, nprob); break;
+    case FMT_BF16: grouped_cast_kernel<FMT_BF16><<<(unsigned)cast_ctas, block, 0, st>>>(tab, cast_start, nprob); break;
+    case FMT_E4M3: grouped_cast_kernel<FMT_E4M3><<<(unsigned)cast_ctas, block, 0, st>>>(tab, cast_start, nprob); break;
+    case FMT_BF16X3: grouped_cast_kernel<FMT_BF16X3><<<(unsigned)cast_ctas, block, 0, st>>>(tab, cast_start, nprob); break;
     default: return cudaErrorInvalidValue;
   }
   return cudaGetLastError();

@@ -23,15 +23,15 @@ cudaError_t launch_scale_exps(const unsigned long long* cmax_bits, int64_t ncols
 // Pass 2 over A: the K-major tensor-core operand Bt: fl_s(2^k_c [A | b][j][c]) for
 // column c and data row j, stored in blocks of kBtBlock data rows, each block
 // [plane][row c < plane_rows][j % kBtBlock]; rows past n and data rows past m are
-// zero.  fmt in {F16, BF16, E4M3, F32, BF16X3}; element size 2, 2, 1, 4, 2;
+// zero.  fmt in {F16, BF16, E4M3, BF16X3}; element size 2, 2, 1, 2;
 // BF16X3 has three planes (hi, lo, lo2) of y = fl32(2^k_c x), read from the FP32
 // copy a32 (row-major, lda32; may be null) where its power-of-two scaling is exact
 // and from A elsewhere.  plane_rows >= n + 1.
 constexpr int64_t kBtBlock = 2048;
-constexpr int kCast3Rows = 64;   // data rows of a BF16X3 cast tile (32 for the other formats)
+constexpr int kCast3Rows = 64;   // data rows of a BF16X3 cast tile
 int64_t bt_blocks(int64_t m);
 size_t bt_bytes(int fmt, int64_t m, int64_t plane_rows);
-int64_t cast_row_tiles(int fmt, int64_t m);   // x extent of the cast grid
+int64_t cast_row_tiles(int fmt, int64_t m);   // row tiles of the cast
 cudaError_t launch_cast_transpose(int fmt, const double* A, int64_t lda, const double* b, const float* a32,
                                   int64_t lda32, int64_t m, int64_t n, const int* kexp, void* Bt,
                                   int64_t plane_rows, cudaStream_t st);
@@ -69,7 +69,6 @@ struct GCast {
   int* kexp;
   void* Bt;
   int64_t plane_rows;
-  int64_t cast_gx;            // row tiles of this problem's cast grid (cast_row_tiles)
 };
 // Per-problem arguments of the grouped split reduction of the FP32 sketch partials.
 struct GReduce {
@@ -108,7 +107,7 @@ SketchTcArgs sketch_tc_args(const SketchPlan& p, uint64_t seed, float* partial, 
 // One launch for a batch: ctas = start[nprob]; every plan must have the same format.
 cudaError_t launch_sketch_tc_grouped(int fmt, const SketchGroup& g, int64_t ctas, cudaStream_t st);
 // Grouped cast: colmax CTAs (ceil(m / kGroupedColmaxRows) per problem), exponent CTAs
-// (ceil((n + 1) / 256)), cast CTAs (cast_gx x ceil(plane_rows / 32)); t as in launch_scale_exps.
+// (ceil((n + 1) / 256)), cast CTAs (cast_row_tiles x ceil(plane_rows / 32)); t as in launch_scale_exps.
 cudaError_t launch_grouped_cast(int fmt, const GCast* tab, const int* colmax_start, int64_t colmax_ctas,
                                 const int* exps_start, int64_t exps_ctas, const int* cast_start,
                                 int64_t cast_ctas, int nprob, int t, int* err, cudaStream_t st);
