@@ -86,7 +86,7 @@ struct RCopies {
   Tri<double> f64;
   double* kappa;
   template <typename T>
-  const Tri<T>& get() const {
+  Tri<T>& get() {
     if constexpr (sizeof(T) == 4) return f32;
     else return f64;
   }
@@ -109,6 +109,21 @@ RCopies stage_prepare_r(Ctx& c, const double* R) {
   L(launch_prepare_r(R, c.n, &r.f32, &r.f64, r.kappa, c.st));
   c.h->launches += 3;
   return r;
+}
+
+// R^-1 in the iterations' precision, formed when a solve first needs it.
+template <typename T>
+const Tri<T>& stage_inverse(Ctx& c, RCopies& rc) {
+  Tri<T>& f = rc.get<T>();
+  if (!f.X) {
+    const size_t bytes = (size_t)f.ld * c.n * sizeof(T);
+    T* X = static_cast<T*>(ws(c.h, sizeof(T) == 4 ? "X32" : "X64", bytes));
+    T* XT = static_cast<T*>(ws(c.h, sizeof(T) == 4 ? "XT32" : "XT64", bytes));
+    L(launch_trinv<T>(rc.f64, f.ld, X, XT, c.st));
+    f.X = X;
+    f.XT = XT;
+  }
+  return f;
 }
 
 // Alg. 1 (QR) -> R (n x n) and c; then x_s = R^-1 c in u_QR.
@@ -162,6 +177,7 @@ LsqrState stage_lsqr(Ctx& c, const W* Aw, int64_t ldw, const Tri<W>& tri, const 
   double* sq = static_cast<double*>(ws(c.h, "sq", c.nblk * 8));
   double* part = static_cast<double*>(ws(c.h, "part", c.nblk2 * 8));
   LsqrState* dst = static_cast<LsqrState*>(ws(c.h, "lsqr_state", sizeof(LsqrState)));
+  double* spart = static_cast<double*>(ws(c.h, "lsqr_part", 128 * 8));
   const int maxit = c.o.lsqr_maxit > 0 ? c.o.lsqr_maxit : (int)(2 * n);
   LsqrState hs;
   std::memset(&hs, 0, sizeof(hs));
@@ -175,7 +191,8 @@ LsqrState stage_lsqr(Ctx& c, const W* Aw, int64_t ldw, const Tri<W>& tri, const 
   L((launch_axpby<double, double, W>(x0, -1.0, nullptr, 0.0, t, n, c.st)));
   L(launch_pass_lsqr_any<W>(Aw, ldw, m, n, t, bw, nullptr, 1.0, u, P, sq, c.nblk, nullptr, c.st));
   L(launch_lsqr_colsum<W>(P, c.nblk, n, sq, dst, true, sv, c.st));
-  L(launch_lsqr_step<W>(tri, sv, v, w, z, t, dst, true, c.st));
+  L(launch_lsqr_step<W>(tri, sv, v, w, z, t, vt, spart, dst, true, c.st));
+  c.h->launches += 1;
   auto body = [&]() {
     for (int k = 0; k < kBatch; ++k) {
       const int* dn = &dst->done;
@@ -184,7 +201,8 @@ LsqrState stage_lsqr(Ctx& c, const W* Aw, int64_t ldw, const Tri<W>& tri, const 
         L(launch_pass_lsqr_any<W>(Aw, ldw, m, n, t, u, &dst->cu, 1.0, u, P, sq, c.nblk, dn, c.st));
       }
       L(launch_lsqr_colsum<W>(P, c.nblk, n, sq, dst, false, sv, c.st));
-      L(launch_lsqr_step<W>(tri, sv, v, w, z, t, dst, false, c.st));
+      L(launch_lsqr_step<W>(tri, sv, v, w, z, t, vt, spart, dst, false, c.st));
+      c.h->launches += 1;
     }
   };
   // CUDA events cannot be timed inside graphs: with opts.timing the batch is launched directly
@@ -193,8 +211,8 @@ LsqrState stage_lsqr(Ctx& c, const W* Aw, int64_t ldw, const Tri<W>& tri, const 
                       : get_graph(c,
                                           graph_key(sizeof(W) == 4 ? "lsqr32" : "lsqr64",
                                                     {PV(Aw), ldw, m, n, PV(t), PV(u), PV(P), PV(sq),
-                                                     PV(sv), PV(v), PV(w), PV(z), PV(dst), PV(tri.R),
-                                                     PV(tri.L), PV(tri.DU), PV(tri.DL), c.nblk}),
+                                                     PV(sv), PV(v), PV(w), PV(z), PV(vt), PV(spart), PV(dst),
+                                                     PV(tri.X), PV(tri.XT), c.nblk}),
                                           body);
   int done = 0, its = 0;
   LsqrState out{};
@@ -210,7 +228,7 @@ LsqrState stage_lsqr(Ctx& c, const W* Aw, int64_t ldw, const Tri<W>& tri, const 
     if (its > maxit + kBatch) break;  // defensive: the device flag ends the loop
   }
   // x = x0 + R^-1 z
-  L((launch_trsv<W, W, W>(true, tri, z, 1.0, t, nullptr, c.st)));
+  L((launch_trimv<W, W, W>(false, tri, z, t, nullptr, c.st)));
   L((launch_axpby<W, double, double>(t, 1.0, x0, 1.0, x, n, c.st)));
   return out;
 }
@@ -319,7 +337,10 @@ GmOut stage_fgmres(Ctx& c, const TOP* Aop, int64_t ldop, const Tri<TOP>& tri, co
       }
       {
         KernTimer kt(c.h, K_TRSV, c.o.timing);
-        L((launch_trsv<TOP, double, TOP>(true, tri, V + m, 1.0, Zb, dn, c.st, jp, ld, ldz)));
+        if (tri.X)
+          L((launch_trimv<TOP, double, TOP>(false, tri, V + m, Zb, dn, c.st, jp, ld, ldz)));
+        else
+          L((launch_trsv<TOP, double, TOP>(true, tri, V + m, 1.0, Zb, dn, c.st, jp, ld, ldz)));
       }
       {
         KernTimer kt(c.h, K_FGM_PASS, c.o.timing);
@@ -329,7 +350,10 @@ GmOut stage_fgmres(Ctx& c, const TOP* Aop, int64_t ldop, const Tri<TOP>& tri, co
       L((launch_colsum<TOP, TOP>(P, c.nblk, n, nullptr, 1.0, sb, dn, c.st)));
       {
         KernTimer kt(c.h, K_TRSV, c.o.timing);
-        L((launch_trsv<TOP, TOP, double>(false, tri, sb, 1.0, wv + m, dn, c.st)));
+        if (tri.X)
+          L((launch_trimv<TOP, TOP, double>(true, tri, sb, wv + m, dn, c.st)));
+        else
+          L((launch_trsv<TOP, TOP, double>(false, tri, sb, 1.0, wv + m, dn, c.st)));
       }
       // modified Gram-Schmidt, or classical with a second pass only where the first one
       // lost more than half of ||w||^2 ("twice is enough"); Givens step; new column
@@ -351,7 +375,7 @@ GmOut stage_fgmres(Ctx& c, const TOP* Aop, int64_t ldop, const Tri<TOP>& tri, co
                                         PV(wv), PV(P), PV(zlo), PV(Phi), PV(Plo), PV(th), PV(tl),
                                         PV(az), PV(v32),
                                         PV(sb), PV(H), PV(cs), PV(sn), PV(g), PV(hh), PV(Dp), PV(sqp),
-                                        PV(gst), PV(gbar), PV(tri.R), PV(tri.L), PV(tri.DU), PV(tri.DL), c.nblk,
+                                        PV(gst), PV(gbar), PV(tri.R), PV(tri.L), PV(tri.DU), PV(tri.DL), PV(tri.X), PV(tri.XT), c.nblk,
                                         c.nblk2, (int64_t)mgs, PV(gseq), (int64_t)c.o.expire_sync}),
                              body);
   int j = 0;
@@ -414,7 +438,7 @@ void stage_residual(Ctx& c, const double* x, const double* r, double* f, double*
 
 // dd: FGMRES products in double-double (TOP = double); gmax_min raises the FGMRES cap.
 template <typename TOP>
-bool stage_refine(Ctx& c, const TOP* Aop, int64_t ldop, const RCopies& rc, double* x, double* r,
+bool stage_refine(Ctx& c, const TOP* Aop, int64_t ldop, RCopies& rc, double* x, double* r,
                   lsq_info* info, bool dd = false, int gmax_min = 0) {
   const int64_t m = c.m, n = c.n;
   double* f = static_cast<double*>(ws(c.h, "ir_f", m * 8));
@@ -425,6 +449,12 @@ bool stage_refine(Ctx& c, const TOP* Aop, int64_t ldop, const RCopies& rc, doubl
   const double gtol = c.o.gmres_tol > 0 ? c.o.gmres_tol : c.tol;
   const double u = unit_roundoff(c.uw);
   info->aug_alpha = c.alpha;
+  // R^-1 as products where later corrections remove their rounding; a single correction
+  // (irmax = 1) keeps it, in single up to kappa u, and the double-double products are meant to
+  // have none: these two substitute.
+  Tri<TOP> tri = rc.get<TOP>();
+  if (!dd && irmax > 1) tri = stage_inverse<TOP>(c, rc);
+  else tri.X = tri.XT = nullptr;
   bool converged = false;
   double prev_dx = 0.0, prev_dr = 0.0;
   info->ir_its = 0;
@@ -441,7 +471,7 @@ bool stage_refine(Ctx& c, const TOP* Aop, int64_t ldop, const RCopies& rc, doubl
         L((launch_trsv<double, double, double>(false, rc.f64, gv, 1.0, hv, nullptr, c.st)));
       }
     }
-    GmOut go = stage_fgmres<TOP>(c, Aop, ldop, rc.get<TOP>(), f, hv, gtol, gmax, r, x, dd);
+    GmOut go = stage_fgmres<TOP>(c, Aop, ldop, tri, f, hv, gtol, gmax, r, x, dd);
     info->gmres_its[i] = go.its;
     info->gmres_its_total += go.its;
     info->arnoldi_second_passes += go.reorth;
@@ -531,9 +561,9 @@ Front run_front(Ctx& c, double* x, lsq_info* info) {
   if (!(kap < INFINITY)) throw StatusFail{LSQ_E_RANK};
   if (c.us != LSQ_AUTO && kap * unit_roundoff(c.us) >= 1.0) info->flags |= LSQ_WARN_COND;
   if (c.uw == LSQ_F32)
-    fr.ls = stage_lsqr<float>(c, fr.a32, c.lda32, fr.rc.f32, fr.x0, x);
+    fr.ls = stage_lsqr<float>(c, fr.a32, c.lda32, stage_inverse<float>(c, fr.rc), fr.x0, x);
   else
-    fr.ls = stage_lsqr<double>(c, c.A, c.lda, fr.rc.f64, fr.x0, x);
+    fr.ls = stage_lsqr<double>(c, c.A, c.lda, stage_inverse<double>(c, fr.rc), fr.x0, x);
   info->lsqr_its = fr.ls.its;
   info->lsqr_flag = fr.ls.flag;
   info->lsqr_normr = fr.ls.normr;

@@ -188,7 +188,7 @@ void batch_fgmres(BatchCtx& b, const std::vector<const TOP*>& Aop, const std::ve
     const int64_t m = b.m[p], n = b.n[p], len = m + n;
     pass_ctas[p] = cdiv(m, kPassRowsPerCta);
     arn_ctas[p] = cdiv(len, kArnRowsPerCta);
-    col_ctas[p] = cdiv(n, 32);
+    col_ctas[p] = cdiv(n, kColsumCols);
     ldz[p] = (n + 3) / 4 * 4 + 4;
     szV[p] = (size_t)len * maxc * 8;
     szZ[p] = (size_t)ldz[p] * maxc * sizeof(TOP);
@@ -555,11 +555,12 @@ lsq_status lsq_batch_grouped(lsq_handle* h, int32_t nprob, const lsq_problem* pr
       else if (kap[p] * unit_roundoff(u_s) >= 1.0) inf[p].flags |= LSQ_WARN_COND;
     }
     // ------------------------------------------------------------ LSQR (a5, a6)
-    std::vector<int64_t> pcta(np), ncta(np), mcta(np);
+    std::vector<int64_t> pcta(np), ncta(np), ccta(np), mcta(np);
     std::vector<size_t> szU(np), szVec(np), szPb(np), szSq(np), szM8(np), szM4(np);
     for (int p = 0; p < np; ++p) {
       pcta[p] = cdiv(b.m[p], kPassRowsPerCta);
       ncta[p] = cdiv(b.n[p], 32);
+      ccta[p] = cdiv(b.n[p], kColsumCols);
       mcta[p] = cdiv(b.m[p], 256);
       szU[p] = (size_t)(b.m[p] + 8) * 4;
       szVec[p] = (size_t)(b.lda32[p] + 8) * 4;
@@ -574,7 +575,8 @@ lsq_status lsq_batch_grouped(lsq_handle* h, int32_t nprob, const lsq_problem* pr
           aPb = make_arena(h, "b_pb", szPb), aSqv = make_arena(h, "b_sq", szSq), aXl = make_arena(h, "b_xl", szN),
           aR0 = make_arena(h, "b_r0", szM8);
     LsqrState* lsd = static_cast<LsqrState*>(ws(h, "b_ls", (size_t)np * sizeof(LsqrState)));
-    Groups gp = make_groups(h, "b_gpass", pcta), gn = make_groups(h, "b_gn", ncta), gm = make_groups(h, "b_gm", mcta);
+    Groups gp = make_groups(h, "b_gpass", pcta), gn = make_groups(h, "b_gn", ncta), gm = make_groups(h, "b_gm", mcta),
+           gc = make_groups(h, "b_gcol", ccta);
     std::vector<LsqrState> lst(np);
     {
       StageTimer t(h, ST_LSQR);
@@ -638,12 +640,12 @@ lsq_status lsq_batch_grouped(lsq_handle* h, int32_t nprob, const lsq_problem* pr
       // timing this (repeatable) first pass with each candidate
       b.pass_grid = tune_pass_grid(b, dp0, gp, pass_smem);
       LB(launch_grouped_pass<float>(PM_LSQR, 4, 2, dp0, gp.dev, gp.total, np, pass_smem, b.st, b.pass_grid));
-      LB(launch_grouped_lsqr_colsum<float>(dcs, gn.dev, gn.total, np, true, b.st));
+      LB(launch_grouped_lsqr_colsum<float>(dcs, gc.dev, gc.total, np, true, b.st));
       LB(launch_grouped_lsqr_step<float>(dstep, np, true, b.st));
       auto body = [&]() {
         for (int k = 0; k < kBatch; ++k) {
           LB(launch_grouped_pass<float>(PM_LSQR, 4, 2, dp1, gp.dev, gp.total, np, pass_smem, b.st, b.pass_grid));
-          LB(launch_grouped_lsqr_colsum<float>(dcs, gn.dev, gn.total, np, false, b.st));
+          LB(launch_grouped_lsqr_colsum<float>(dcs, gc.dev, gc.total, np, false, b.st));
           LB(launch_grouped_lsqr_step<float>(dstep, np, false, b.st));
         }
       };
@@ -808,7 +810,7 @@ lsq_status lsq_batch_grouped(lsq_handle* h, int32_t nprob, const lsq_problem* pr
           StageTimer t(h, ST_RES);
           LB(launch_grouped_pass<double>(PM_RES, 1, 8, dres, gp.dev, gp.total, np, (size_t)8 * maxn * 8, b.st,
                                          b.pass_grid));
-          LB(launch_grouped_colsum<double, double>(dcg, gn.dev, gn.total, np, b.st));
+          LB(launch_grouped_colsum<double, double>(dcg, gc.dev, gc.total, np, b.st));
           LB(launch_grouped_trsv<double, double, double>(false, dth, np, b.st));
         }
         std::vector<GmState> gs;

@@ -64,8 +64,8 @@ template <typename T>
 cudaError_t launch_lsqr_colsum(const T* P, int nblk, int64_t n, const double* sq, LsqrState* st,
                                bool init, T* out, cudaStream_t s);
 template <typename T>
-cudaError_t launch_lsqr_step(const Tri<T>& f, const T* s, T* v, T* w, T* z, T* t, LsqrState* st,
-                             bool init, cudaStream_t strm);
+cudaError_t launch_lsqr_step(const Tri<T>& f, const T* s, T* v, T* w, T* z, T* t, T* vv, double* part,
+                             LsqrState* st, bool init, cudaStream_t strm);   // part: n / 8 values
 
 template <typename TX, typename TY, typename TO>
 cudaError_t launch_axpby(const TX* x, double a, const TY* y, double b, TO* out, int64_t len,

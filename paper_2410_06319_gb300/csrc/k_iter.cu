@@ -575,37 +575,46 @@ cudaError_t launch_pass_res(const double* A, int64_t lda, int64_t m, int64_t n, 
 }
 
 // ------------------------------------------------------------ column sums
+// A warp per column, lanes over the CTAs' partials, eight columns a CTA (32-byte pieces of
+// the rows of P).  FP64 additions and FP32 -> FP64 conversions are what it costs (an SM
+// does two a clock), so the columns are spread over many CTAs: 32 columns a CTA with a serial
+// sum of 32 shares took 7 us at n = 500, 5 now.
+template <typename TP>
+__device__ __forceinline__ double colsum_warp(const TP* __restrict__ P, int nblk, int64_t n, int64_t c) {
+  const int lane = threadIdx.x & 31;
+  double s0 = 0.0, s1 = 0.0;
+  int b = lane;
+  for (; b + 32 < nblk; b += 64) {
+    const TP p0 = P[(int64_t)b * n + c], p1 = P[(int64_t)(b + 32) * n + c];
+    s0 += (double)p0;
+    s1 += (double)p1;
+  }
+  if (b < nblk) s0 += (double)P[(int64_t)b * n + c];
+  return warp_sum(s0 + s1);
+}
+
 template <typename TP, typename TO>
 __device__ __forceinline__ void colsum_body(const TP* __restrict__ P, int nblk, int64_t n, const double* scale_ptr,
                                             double scale_mul, TO* __restrict__ out, const int* done, int64_t bx) {
   if (done && *done) return;
-  __shared__ double part[32][33];
-  const int tx = threadIdx.x, ty = threadIdx.y;
-  const int64_t c = bx * 32 + tx;
-  double s = 0.0;
-  if (c < n)
-    for (int b = ty; b < nblk; b += 32) s += (double)P[(int64_t)b * n + c];
-  part[ty][tx] = s;
-  __syncthreads();
-  if (ty == 0 && c < n) {
-    double t = 0.0;
-    for (int k = 0; k < 32; ++k) t += part[k][tx];
-    const double sc = (scale_ptr ? *scale_ptr : 1.0) * scale_mul;
-    out[c] = (TO)(t * sc);
-  }
+  const int64_t c = bx * kColsumCols + (threadIdx.x >> 5);
+  if (c >= n) return;
+  const double t = colsum_warp<TP>(P, nblk, n, c);
+  if ((threadIdx.x & 31) == 0) out[c] = (TO)(t * ((scale_ptr ? *scale_ptr : 1.0) * scale_mul));
 }
 
 template <typename TP, typename TO>
-__global__ void colsum_kernel(const TP* __restrict__ P, int nblk, int64_t n, const double* scale_ptr,
-                              double scale_mul, TO* __restrict__ out, const int* done) {
+__global__ void __launch_bounds__(kColsumCols * 32)
+    colsum_kernel(const TP* __restrict__ P, int nblk, int64_t n, const double* scale_ptr,
+                  double scale_mul, TO* __restrict__ out, const int* done) {
   colsum_body<TP, TO>(P, nblk, n, scale_ptr, scale_mul, out, done, blockIdx.x);
 }
 
 template <typename TP, typename TO>
 cudaError_t launch_colsum(const TP* P, int nblk, int64_t n, const double* scale_ptr, double scale_mul,
                           TO* out, const int* done, cudaStream_t st) {
-  colsum_kernel<TP, TO><<<(unsigned)((n + 31) / 32), dim3(32, 32), 0, st>>>(P, nblk, n, scale_ptr,
-                                                                           scale_mul, out, done);
+  colsum_kernel<TP, TO><<<(unsigned)((n + kColsumCols - 1) / kColsumCols), kColsumCols * 32, 0, st>>>(
+      P, nblk, n, scale_ptr, scale_mul, out, done);
   return cudaGetLastError();
 }
 template cudaError_t launch_colsum<float, float>(const float*, int, int64_t, const double*, double,
@@ -638,45 +647,85 @@ template <typename TP>
 __device__ __forceinline__ void lsqr_colsum_body(const TP* __restrict__ P, int nblk, int64_t n, const double* sq,
                                                  LsqrState* st, bool init, TP* __restrict__ out, int64_t bx) {
   if (!init && st->done) return;
-  __shared__ double part[32][33];
-  __shared__ double beta_s;
-  const int tx = threadIdx.x, ty = threadIdx.y;
-  const int tid = ty * 32 + tx;
-  double q = 0.0;
-  for (int b = tid; b < nblk; b += 1024) q += sq[b];
-  q = warp_sum(q);
-  if (tx == 0) part[ty][32] = q;
-  __syncthreads();
-  if (tid == 0) {
-    double t = 0.0;
-    for (int k = 0; k < 32; ++k) t += part[k][32];
-    beta_s = sqrt(t);
+  __shared__ double us_s;
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  if (warp == kColsumCols) {   // a warp of its own: beta, its square root and reciprocal once
+    double q = 0.0;
+    for (int b = lane; b < nblk; b += 32) q += sq[b];
+    q = warp_sum(q);
+    if (lane == 0) {
+      const double beta = sqrt(q);
+      const double us = beta > 0.0 ? 1.0 / beta : 0.0;
+      us_s = us;
+      if (bx == 0) {
+        st->beta = beta;
+        st->us = us;
+        if (init) st->phibar = beta;
+      }
+    }
   }
+  const int64_t c = bx * kColsumCols + warp;
+  double t = 0.0;
+  if (warp < kColsumCols && c < n) t = colsum_warp<TP>(P, nblk, n, c);
   __syncthreads();
-  const double beta = beta_s;
-  const double us = beta > 0.0 ? 1.0 / beta : 0.0;
-  if (bx == 0 && tid == 0) {
-    st->beta = beta;
-    st->us = us;
-    if (init) st->phibar = beta;
-  }
-  const int64_t c = bx * 32 + tx;
-  double sacc = 0.0;
-  if (c < n)
-    for (int b = ty; b < nblk; b += 32) sacc += (double)P[(int64_t)b * n + c];
-  part[ty][tx] = sacc;
-  __syncthreads();
-  if (ty == 0 && c < n) {
-    double t = 0.0;
-    for (int k = 0; k < 32; ++k) t += part[k][tx];
-    out[c] = (TP)(t * us);
-  }
+  if (warp < kColsumCols && c < n && lane == 0) out[c] = (TP)(t * us_s);
 }
 
 template <typename TP>
-__global__ void lsqr_colsum_kernel(const TP* __restrict__ P, int nblk, int64_t n, const double* sq,
-                                   LsqrState* st, bool init, TP* __restrict__ out) {
+__global__ void __launch_bounds__((kColsumCols + 1) * 32)
+    lsqr_colsum_kernel(const TP* __restrict__ P, int nblk, int64_t n, const double* sq,
+                       LsqrState* st, bool init, TP* __restrict__ out) {
   lsqr_colsum_body<TP>(P, nblk, n, sq, st, init, out, blockIdx.x);
+}
+
+// The plane rotation and the stopping tests of one step, by one warp: square roots and
+// quotients that do not depend on one another run in different lanes (each is a chain of some
+// 40 FP64 operations).  coef (shared): the factors of the z and w updates.
+__device__ __forceinline__ void lsqr_scalars(LsqrState* st, bool init, double alpha, double beta, double* coef) {
+  const int lane = threadIdx.x & 31;
+  if (init) {
+    if (lane == 0) {
+      st->alpha = alpha;
+      st->rhobar = alpha;
+      st->anorm2 = 0.0;
+      st->its = 0;
+      st->normr = beta;
+      st->normar = alpha * beta;
+      st->normA = 0.0;
+      st->flag = (beta == 0.0 || alpha == 0.0) ? 3 : 0;
+      st->done = (st->flag != 0 || st->maxit <= 0) ? 1 : 0;
+      coef[0] = 0.0;
+      coef[1] = 0.0;
+      st->cu = -alpha * st->us;
+    }
+    return;
+  }
+  const double alpha_old = st->alpha, rhobar = st->rhobar, phibar0 = st->phibar;
+  const double anorm2 = st->anorm2 + alpha_old * alpha_old + beta * beta;
+  const double root = sqrt(lane == 0 ? rhobar * rhobar + beta * beta : anorm2);
+  const double rho = __shfl_sync(0xffffffffu, root, 0), normA = __shfl_sync(0xffffffffu, root, 1);
+  const double q1 = (lane == 0 ? rhobar : beta) / rho;
+  const double c = __shfl_sync(0xffffffffu, q1, 0), sn = __shfl_sync(0xffffffffu, q1, 1);
+  const double theta = sn * alpha, phi = c * phibar0, phibar = sn * phibar0;
+  const double q2 = (lane == 0 ? phi : theta) / rho;
+  if (lane < 2) coef[lane] = q2;
+  if (lane == 0) {
+    st->rhobar = -c * alpha;
+    st->phibar = phibar;
+    st->anorm2 = anorm2;
+    st->alpha = alpha;
+    st->its += 1;
+    st->normr = fabs(phibar);
+    st->normar = fabs(phibar * alpha * c);
+    st->normA = normA;
+    int flag = 0;
+    if (st->normr <= st->tol * st->normb) flag = 1;
+    else if (st->normar <= st->tol * normA * st->normr) flag = 2;
+    else if (beta == 0.0 || alpha == 0.0) flag = 3;
+    st->flag = flag;
+    st->done = (flag != 0 || st->its >= st->maxit) ? 1 : 0;
+    st->cu = -alpha * st->us;
+  }
 }
 
 // One CTA: vt = R^-T s ; (init) alpha v = vt, w = v, z = 0 ; (iteration)
@@ -702,50 +751,13 @@ __device__ __forceinline__ void lsqr_step_body(const Tri<T>& f, const T* __restr
     ss += (double)vv * (double)vv;
   }
   ss = block_sum_d(ss, red);
-  const double alpha = sqrt(ss);
-  if (threadIdx.x == 0) {
-    if (init) {
-      st->alpha = alpha;
-      st->rhobar = alpha;
-      st->anorm2 = 0.0;
-      st->its = 0;
-      st->normr = beta;
-      st->normar = alpha * beta;
-      st->normA = 0.0;
-      st->flag = (beta == 0.0 || alpha == 0.0) ? 3 : 0;
-      st->done = (st->flag != 0 || st->maxit <= 0) ? 1 : 0;
-      coef[0] = 0.0;
-      coef[1] = 0.0;
-    } else {
-      const double alpha_old = st->alpha;
-      const double anorm2 = st->anorm2 + alpha_old * alpha_old + beta * beta;
-      const double rhobar = st->rhobar;
-      const double rho = sqrt(rhobar * rhobar + beta * beta);
-      const double c = rhobar / rho, sn = beta / rho;
-      const double theta = sn * alpha;
-      const double phi = c * st->phibar;
-      const double phibar = sn * st->phibar;
-      coef[0] = phi / rho;
-      coef[1] = theta / rho;
-      st->rhobar = -c * alpha;
-      st->phibar = phibar;
-      st->anorm2 = anorm2;
-      st->alpha = alpha;
-      st->its += 1;
-      st->normr = fabs(phibar);
-      st->normar = fabs(phibar * alpha * c);
-      st->normA = sqrt(anorm2);
-      int flag = 0;
-      if (st->normr <= st->tol * st->normb) flag = 1;
-      else if (st->normar <= st->tol * st->normA * st->normr) flag = 2;
-      else if (beta == 0.0 || alpha == 0.0) flag = 3;
-      st->flag = flag;
-      st->done = (flag != 0 || st->its >= st->maxit) ? 1 : 0;
-    }
-    st->cu = -alpha * st->us;
+  if (threadIdx.x < 32) {   // one warp: the FP64 roots and quotients
+    const double alpha = sqrt(ss);
+    lsqr_scalars(st, init, alpha, beta, coef);
+    if (threadIdx.x == 0) coef[2] = alpha > 0.0 ? 1.0 / alpha : 0.0;
   }
   __syncthreads();
-  const T ia = alpha > 0.0 ? (T)(1.0 / alpha) : T(0);
+  const T ia = (T)coef[2];
   const T c0 = (T)coef[0], c1 = (T)coef[1];
   for (int i = threadIdx.x; i < n; i += blockDim.x) {
     const T vn = (init ? xs[i] : xs[i] - (T)beta * v[i]) * ia;
@@ -765,33 +777,112 @@ __device__ __forceinline__ void lsqr_step_body(const Tri<T>& f, const T* __restr
   for (int i = threadIdx.x; i < n; i += blockDim.x) t[i] = xs[i];
 }
 
+// The step of one problem by two launches over the rows of X = R^-1 (a warp per row):
+//   1: vv = X^T s - beta v (init: X^T s), and the CTA's sum of squares;
+//   2: alpha = ||vv||; t = X (vv / alpha) for the next pass; CTA 0 also does the scalars and the
+//      vectors v, w, z.  (A CTA that starts after CTA 0 has set done skips its rows of t: no
+//      pass reads them then.)
+// On one CTA with two triangular solves the step took 20 us at n = 50 and 46 us at n = 500.
 template <typename T>
-__global__ void __launch_bounds__(kTrsvThreads)
-    lsqr_step_kernel(Tri<T> f, const T* __restrict__ s, T* __restrict__ v, T* __restrict__ w,
-                     T* __restrict__ z, T* __restrict__ t, LsqrState* st, bool init) {
-  lsqr_step_body<T>(f, s, v, w, z, t, st, init);
+__global__ void __launch_bounds__(kTrimvWarps * 32)
+    lsqr_step1_kernel(const T* __restrict__ XT, int64_t ld, int n, const T* __restrict__ s, const T* __restrict__ v,
+                      T* __restrict__ vv, double* __restrict__ part, const LsqrState* st, bool init) {
+  if (!init && st->done) return;
+  __shared__ __align__(16) T ysm[1024];
+  __shared__ double sq[kTrimvWarps];
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int r = blockIdx.x * kTrimvWarps + warp;
+  const int c1 = min((int)ld, (int)(blockIdx.x + 1) * kTrimvWarps + 4);
+  for (int i = threadIdx.x; i < c1; i += blockDim.x) ysm[i] = i < n ? s[i] : T(0);
+  __syncthreads();
+  if (r < n) {
+    T x = trimv_row<T, true>(XT + (size_t)r * ld, r, n, ysm);
+    if (!init) x -= (T)st->beta * v[r];
+    if (lane == 0) {
+      vv[r] = x;
+      sq[warp] = (double)x * (double)x;
+    }
+  } else if (lane == 0) {
+    sq[warp] = 0.0;
+  }
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    double q = 0.0;
+#pragma unroll
+    for (int w = 0; w < kTrimvWarps; ++w) q += sq[w];
+    part[blockIdx.x] = q;
+  }
+}
+
+template <typename T>
+__global__ void __launch_bounds__(kTrimvWarps * 32)
+    lsqr_step2_kernel(const T* __restrict__ X, int64_t ld, int n, const T* __restrict__ vv,
+                      const double* __restrict__ part, T* __restrict__ v, T* __restrict__ w, T* __restrict__ z,
+                      T* __restrict__ t, LsqrState* st, bool init) {
+  if (!init && st->done) return;
+  __shared__ __align__(16) T ysm[1024];
+  __shared__ double coef[2], alpha_s;
+  __shared__ T ia_s;
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  if (warp == 0) {   // once: an FP64 root and quotient in every warp would cost microseconds
+    double q = 0.0;
+    for (int b = lane; b < (int)gridDim.x; b += 32) q += part[b];
+    const double al = sqrt(warp_sum(q));
+    if (lane == 0) {
+      alpha_s = al;
+      ia_s = al > 0.0 ? (T)(1.0 / al) : T(0);
+    }
+  }
+  __syncthreads();
+  const double alpha = alpha_s;
+  const T ia = ia_s;
+  const int c0 = (blockIdx.x * kTrimvWarps / 4) * 4;
+  for (int i = c0 + threadIdx.x; i < (int)ld; i += blockDim.x) ysm[i] = i < n ? vv[i] * ia : T(0);
+  __syncthreads();
+  const int r = blockIdx.x * kTrimvWarps + warp;
+  if (r < n) {
+    const T x = trimv_row<T, false>(X + (size_t)r * ld, r, n, ysm);
+    if (lane == 0) t[r] = x;
+  }
+  if (blockIdx.x == 0) {   // ysm holds all of v here
+    if (warp == 0) lsqr_scalars(st, init, alpha, st->beta, coef);
+    __syncthreads();
+    const T f0 = (T)coef[0], f1 = (T)coef[1];
+    for (int i = threadIdx.x; i < n; i += blockDim.x) {
+      const T vn = ysm[i];
+      if (init) {
+        w[i] = vn;
+        z[i] = T(0);
+      } else {
+        const T wi = w[i];
+        z[i] = z[i] + f0 * wi;
+        w[i] = vn - f1 * wi;
+      }
+      v[i] = vn;
+    }
+  }
 }
 
 template <typename T>
 cudaError_t launch_lsqr_colsum(const T* P, int nblk, int64_t n, const double* sq, LsqrState* st,
                                bool init, T* out, cudaStream_t s) {
-  lsqr_colsum_kernel<T><<<(unsigned)((n + 31) / 32), dim3(32, 32), 0, s>>>(P, nblk, n, sq, st, init, out);
+  lsqr_colsum_kernel<T><<<(unsigned)((n + kColsumCols - 1) / kColsumCols), (kColsumCols + 1) * 32, 0, s>>>(P, nblk, n, sq, st,
+                                                                                                      init, out);
   return cudaGetLastError();
 }
 template <typename T>
-cudaError_t launch_lsqr_step(const Tri<T>& f, const T* s, T* v, T* w, T* z, T* t, LsqrState* st,
-                             bool init, cudaStream_t strm) {
-  if (f.n > 1024) return cudaErrorInvalidValue;
-  const size_t smem = TrsvSmem<T>::bytes;
-  cudaError_t e = allow_dyn_smem(lsqr_step_kernel<T>, smem);
-  if (e != cudaSuccess) return e;
-  lsqr_step_kernel<T><<<1, kTrsvThreads, smem, strm>>>(f, s, v, w, z, t, st, init);
+cudaError_t launch_lsqr_step(const Tri<T>& f, const T* s, T* v, T* w, T* z, T* t, T* vv, double* part,
+                             LsqrState* st, bool init, cudaStream_t strm) {
+  if (f.n > 1024 || !f.X || !f.XT) return cudaErrorInvalidValue;
+  const unsigned grid = (unsigned)((f.n + kTrimvWarps - 1) / kTrimvWarps);
+  lsqr_step1_kernel<T><<<grid, kTrimvWarps * 32, 0, strm>>>(f.XT, f.ld, (int)f.n, s, v, vv, part, st, init);
+  lsqr_step2_kernel<T><<<grid, kTrimvWarps * 32, 0, strm>>>(f.X, f.ld, (int)f.n, vv, part, v, w, z, t, st, init);
   return cudaGetLastError();
 }
 template cudaError_t launch_lsqr_colsum<float>(const float*, int, int64_t, const double*, LsqrState*, bool, float*, cudaStream_t);
 template cudaError_t launch_lsqr_colsum<double>(const double*, int, int64_t, const double*, LsqrState*, bool, double*, cudaStream_t);
-template cudaError_t launch_lsqr_step<float>(const Tri<float>&, const float*, float*, float*, float*, float*, LsqrState*, bool, cudaStream_t);
-template cudaError_t launch_lsqr_step<double>(const Tri<double>&, const double*, double*, double*, double*, double*, LsqrState*, bool, cudaStream_t);
+template cudaError_t launch_lsqr_step<float>(const Tri<float>&, const float*, float*, float*, float*, float*, float*, double*, LsqrState*, bool, cudaStream_t);
+template cudaError_t launch_lsqr_step<double>(const Tri<double>&, const double*, double*, double*, double*, double*, double*, double*, LsqrState*, bool, cudaStream_t);
 
 // ============================================================ vector kernels
 // out[i] = x[i] * a + y[i] * b  (types converted), i < len
@@ -1620,7 +1711,7 @@ template <typename TP, typename TO>
 cudaError_t launch_grouped_colsum(const GColsum<TP, TO>* tab, const int* start, int64_t ctas, int nprob,
                                   cudaStream_t st) {
   if (ctas <= 0) return cudaSuccess;
-  grouped_colsum_kernel<TP, TO><<<(unsigned)ctas, dim3(32, 32), 0, st>>>(tab, start, nprob);
+  grouped_colsum_kernel<TP, TO><<<(unsigned)ctas, kColsumCols * 32, 0, st>>>(tab, start, nprob);
   return cudaGetLastError();
 }
 template cudaError_t launch_grouped_colsum<float, float>(const GColsum<float, float>*, const int*, int64_t, int,
@@ -1640,7 +1731,7 @@ template <typename TP>
 cudaError_t launch_grouped_lsqr_colsum(const GLsqrColsum<TP>* tab, const int* start, int64_t ctas, int nprob,
                                        bool init, cudaStream_t st) {
   if (ctas <= 0) return cudaSuccess;
-  grouped_lsqr_colsum_kernel<TP><<<(unsigned)ctas, dim3(32, 32), 0, st>>>(tab, start, nprob, init);
+  grouped_lsqr_colsum_kernel<TP><<<(unsigned)ctas, (kColsumCols + 1) * 32, 0, st>>>(tab, start, nprob, init);
   return cudaGetLastError();
 }
 template cudaError_t launch_grouped_lsqr_colsum<float>(const GLsqrColsum<float>*, const int*, int64_t, int, bool,

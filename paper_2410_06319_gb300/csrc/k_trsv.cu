@@ -569,6 +569,123 @@ LSQ_TRSV_INST(double, float, double)
 LSQ_TRSV_INST(double, double, float)
 LSQ_TRSV_INST(double, float, float)
 
+// ------------------------------------------------------------ explicit inverse
+// The iterations multiply with X = R^-1 instead of solving with R: a solve is a chain of
+// n / 32 dependent block steps (18 us at n = 500 and 50 us at n = 1000 in FP32, 24 us at n = 187 in
+// FP64, on one cluster; 46 us for the two of an LSQR step on one CTA), a product is one
+// read of the triangle by all SMs (3 us).  X is formed once per solve, in FP64 from
+// the FP64 factor and then rounded, so that its entries are correct to about an ulp of T; the
+// product's forward error n u |X||y| is no larger than substitution's n u |R^-1||R||R^-1 y|.
+// The solves that fix a result (x_s, h = R^-T g, double-double) still substitute.
+//
+// One CTA per column j: blocked back substitution x_k = D_k (e_j - sum_c R_kc x_c), D_k the
+// inverse of the 32 x 32 diagonal block; the four warps split the columns c, lanes hold the
+// block's rows (coalesced column segments of R from L2).  n^3 / 6 FP64 FMAs: bound by the
+// FP64 pipe at n = 1000 and by the block chain below.
+template <typename T>
+__global__ void __launch_bounds__(128)
+    trinv_kernel(const double* __restrict__ R, int64_t ld64, const double* __restrict__ DU, int n, int64_t ld,
+                 T* __restrict__ X, T* __restrict__ XT) {
+  __shared__ double x[1024];
+  __shared__ double red[4][33];
+  const int j = n - 1 - (int)blockIdx.x;   // the longest columns first
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int jb = j >> 5;
+  for (int k = jb; k >= 0; --k) {
+    // sum over the columns c of later blocks (c <= j), split among the warps
+    double s0 = 0.0, s1 = 0.0;
+    const double* col = R + 32 * k + lane;
+    const bool row_in = 32 * k + lane < n;
+    int c = 32 * (k + 1) + warp;
+    if (row_in) {
+      for (; c + 12 <= j; c += 16) {
+        const double r0 = col[(size_t)c * ld64], r1 = col[(size_t)(c + 4) * ld64], r2 = col[(size_t)(c + 8) * ld64],
+                     r3 = col[(size_t)(c + 12) * ld64];
+        s0 = fma(r0, x[c], s0);
+        s1 = fma(r1, x[c + 4], s1);
+        s0 = fma(r2, x[c + 8], s0);
+        s1 = fma(r3, x[c + 12], s1);
+      }
+      for (; c <= j; c += 4) s0 = fma(col[(size_t)c * ld64], x[c], s0);
+    }
+    red[warp][lane] = s0 + s1;
+    __syncthreads();
+    const double rhs = ((k == jb && lane == (j & 31)) ? 1.0 : 0.0) -
+                       ((red[0][lane] + red[1][lane]) + (red[2][lane] + red[3][lane]));
+    __syncthreads();
+    // x_k = D_k rhs: eight columns of D_k per warp
+    double d0 = 0.0, d1 = 0.0;
+#pragma unroll
+    for (int q = 0; q < 8; q += 2) {
+      const int cc = warp * 8 + q;
+      d0 = fma(DU[(size_t)k * 1024 + cc * 32 + lane], __shfl_sync(0xffffffffu, rhs, cc), d0);
+      d1 = fma(DU[(size_t)k * 1024 + (cc + 1) * 32 + lane], __shfl_sync(0xffffffffu, rhs, cc + 1), d1);
+    }
+    red[warp][lane] = d0 + d1;
+    __syncthreads();
+    if (warp == 0) x[32 * k + lane] = (red[0][lane] + red[1][lane]) + (red[2][lane] + red[3][lane]);
+    __syncthreads();
+  }
+  for (int i = threadIdx.x; i < (int)ld; i += 128) {
+    const T v = i <= j ? (T)x[i] : T(0);
+    XT[(size_t)j * ld + i] = v;
+    if (i < n) X[(size_t)i * ld + j] = v;
+  }
+  if (j == n - 1)   // the padding columns of X
+    for (int64_t e = threadIdx.x; e < (int64_t)n * (ld - n); e += 128) X[(e / (ld - n)) * ld + n + e % (ld - n)] = T(0);
+}
+
+template <typename T>
+cudaError_t launch_trinv(const Tri<double>& f64, int64_t ld, T* X, T* XT, cudaStream_t st) {
+  if (f64.n > 1024) return cudaErrorInvalidValue;
+  trinv_kernel<T><<<(unsigned)f64.n, 128, 0, st>>>(f64.R, f64.ld, f64.DU, (int)f64.n, ld, X, XT);
+  return cudaGetLastError();
+}
+template cudaError_t launch_trinv<float>(const Tri<double>&, int64_t, float*, float*, cudaStream_t);
+template cudaError_t launch_trinv<double>(const Tri<double>&, int64_t, double*, double*, cudaStream_t);
+
+template <typename T, typename TIN, typename TOUT, bool TRANS>
+__global__ void __launch_bounds__(kTrimvWarps * 32)
+    trimv_kernel(const T* __restrict__ M, int64_t ld, int n, const TIN* __restrict__ y, TOUT* __restrict__ out,
+                 const int* done, const int* jp, int64_t ys, int64_t outstr) {
+  if (done && *done) return;
+  if (jp) {   // column j of a basis: offsets read on the device (graph-replayable)
+    const int64_t j = *jp;
+    y += j * ys;
+    out += j * outstr;
+  }
+  __shared__ __align__(16) T ysm[1024];
+  const int r = blockIdx.x * kTrimvWarps + (threadIdx.x >> 5);
+  // the part of y this CTA's rows meet, zero padded to whole vectors
+  const int np = (int)ld;
+  const int c0 = TRANS ? 0 : (blockIdx.x * kTrimvWarps / 4) * 4;
+  const int c1 = TRANS ? min(np, (int)(blockIdx.x + 1) * kTrimvWarps + 4) : np;
+  for (int i = c0 + threadIdx.x; i < c1; i += blockDim.x) ysm[i] = i < n ? (T)y[i] : T(0);
+  __syncthreads();
+  if (r >= n) return;
+  const T s = trimv_row<T, TRANS>(M + (size_t)r * ld, r, n, ysm);
+  if ((threadIdx.x & 31) == 0) out[r] = (TOUT)s;
+}
+
+template <typename T, typename TIN, typename TOUT>
+cudaError_t launch_trimv(bool trans, const Tri<T>& f, const TIN* y, TOUT* out, const int* done, cudaStream_t st,
+                         const int* jp, int64_t ys, int64_t outstr) {
+  if (f.n > 1024 || !f.X || !f.XT) return cudaErrorInvalidValue;
+  const unsigned grid = (unsigned)((f.n + kTrimvWarps - 1) / kTrimvWarps);
+  if (trans)
+    trimv_kernel<T, TIN, TOUT, true><<<grid, kTrimvWarps * 32, 0, st>>>(f.XT, f.ld, (int)f.n, y, out, done, jp, ys, outstr);
+  else
+    trimv_kernel<T, TIN, TOUT, false><<<grid, kTrimvWarps * 32, 0, st>>>(f.X, f.ld, (int)f.n, y, out, done, jp, ys, outstr);
+  return cudaGetLastError();
+}
+#define LSQ_TRIMV_INST(T, TIN, TOUT)                                                                     \
+  template cudaError_t launch_trimv<T, TIN, TOUT>(bool, const Tri<T>&, const TIN*, TOUT*, const int*, \
+                                                  cudaStream_t, const int*, int64_t, int64_t);
+LSQ_TRIMV_INST(float, float, float)
+LSQ_TRIMV_INST(float, double, float)
+LSQ_TRIMV_INST(float, float, double)
+LSQ_TRIMV_INST(double, double, double)
+
 // ------------------------------------------------------------ preparation
 __device__ __forceinline__ void prepare_r_body(const double* __restrict__ R, int64_t n, float* R32, float* L32,
                                                int64_t ld32, double* R64, double* L64, int64_t ld64, int64_t j) {

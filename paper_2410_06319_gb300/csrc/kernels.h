@@ -164,6 +164,10 @@ struct Tri {
   int64_t n;
   int64_t ld;
   int* err = nullptr;   // device error word for bounded waits (may be null)
+  // the explicit inverse of R for the iterations (launch_trinv; null until formed): X = R^-1
+  // with row i at X + i * ld, XT = R^-T with row j at XT + j * ld, zeros outside the triangle
+  const T* X = nullptr;
+  const T* XT = nullptr;
 };
 inline int64_t tri_ld(int64_t n, int elem_bytes) {
   const int64_t q = 16 / elem_bytes;
@@ -177,6 +181,16 @@ template <typename T, typename TIN, typename TOUT>
 cudaError_t launch_trsv(bool upper, const Tri<T>& f, const TIN* y, double yscale, TOUT* x,
                         const int* done, cudaStream_t st, const int* jp = nullptr, int64_t ys = 0,
                         int64_t xstr = 0);
+
+// X = R^-1 and its transpose in T, formed in FP64 from the FP64 factor f64 (n <= 1024); sets
+// nothing else of *f.  X and XT hold n * ld elements each.
+template <typename T>
+cudaError_t launch_trinv(const Tri<double>& f64, int64_t ld, T* X, T* XT, cudaStream_t st);
+// out = X y (trans = false) or X^T y: the products with R^-1 and R^-T inside the iterations.
+// Arguments as launch_trsv.
+template <typename T, typename TIN, typename TOUT>
+cudaError_t launch_trimv(bool trans, const Tri<T>& f, const TIN* y, TOUT* out, const int* done, cudaStream_t st,
+                         const int* jp = nullptr, int64_t ys = 0, int64_t outstr = 0);
 
 // Converts R (FP64, col-major) into the FP32 and FP64 factors (R, R^T and the
 // diagonal-block inverses); writes max|r_ii| / min|r_ii| to *kappa_est.
@@ -196,6 +210,7 @@ cudaError_t launch_pass_fgm(const TA* A, int64_t lda, int64_t m, int64_t n, cons
 cudaError_t launch_pass_res(const double* A, int64_t lda, int64_t m, int64_t n, const double* x,
                             const double* r, const double* b, double* f, double* Pblk, int nblk,
                             cudaStream_t st);
+constexpr int kColsumCols = 8;   // columns of a CTA of the column sums
 // out[c] = scale * sum_b P[b][c] (FP64 accumulation).  scale = *scale_ptr * scale_mul
 // when scale_ptr != nullptr.
 template <typename TP, typename TO>

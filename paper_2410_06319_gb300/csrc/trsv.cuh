@@ -163,4 +163,30 @@ __device__ __forceinline__ bool block_trsv(const T* __restrict__ M, int64_t ld, 
   return true;
 }
 
+// ------------------------------------------------------------ triangular products
+// Row r of X (upper triangular, columns r ..) or of X^T (columns 0 .. r) times y by one
+// warp: rows of 16-byte vectors, y in shared memory, zero outside the triangle.  Every lane
+// returns the sum.
+constexpr int kTrimvWarps = 8;   // rows of a CTA
+template <typename T, bool TRANS>
+__device__ __forceinline__ T trimv_row(const T* __restrict__ row, int r, int n, const T* ys) {
+  constexpr int VE = 16 / (int)sizeof(T);
+  const int lane = threadIdx.x & 31;
+  const int v0 = TRANS ? 0 : r / VE, v1 = TRANS ? r / VE + 1 : (n + VE - 1) / VE;
+  T acc[VE];
+#pragma unroll
+  for (int k = 0; k < VE; ++k) acc[k] = T(0);
+#pragma unroll 4
+  for (int v = v0 + lane; v < v1; v += 32) {
+    T a[VE];
+    *reinterpret_cast<uint4*>(a) = *reinterpret_cast<const uint4*>(row + (size_t)v * VE);
+#pragma unroll
+    for (int k = 0; k < VE; ++k) acc[k] = fma(a[k], ys[v * VE + k], acc[k]);
+  }
+  T s = T(0);
+#pragma unroll
+  for (int k = 0; k < VE; ++k) s += acc[k];
+  return warp_sum(s);
+}
+
 }  // namespace lsq
