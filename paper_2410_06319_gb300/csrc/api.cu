@@ -276,23 +276,14 @@ GmOut stage_fgmres(Ctx& c, const TOP* Aop, int64_t ldop, const Tri<TOP>& tri, co
   double* sn = static_cast<double*>(ws(c.h, "gmsn", (maxit + 1) * 8));
   double* g = static_cast<double*>(ws(c.h, "gmg", (maxit + 2) * 8, true));
   double* y = static_cast<double*>(ws(c.h, "gmy", (maxit + 1) * 8));
-  double* hh = static_cast<double*>(ws(c.h, "gmhh", (maxit + 2) * 8));
-  double* Dp = static_cast<double*>(ws(c.h, "gmDp", (size_t)c.nblk2 * (maxit + 2) * 8));
+  double* hh = static_cast<double*>(ws(c.h, "gmhh", 2 * (maxit + 2) * 8));
+  double* Dp = static_cast<double*>(ws(c.h, "gmDp", (size_t)2 * c.nblk2 * (maxit + 18) * 8));
   double* sqp = static_cast<double*>(ws(c.h, "gmsq", c.nblk2 * 8));
   double* p4 = static_cast<double*>(ws(c.h, "gmp4", 4 * c.nblk2 * 8));
   double* nrm = static_cast<double*>(ws(c.h, "gmnrm", 4 * 8));
   GmState* gst = static_cast<GmState*>(ws(c.h, "gm_state", sizeof(GmState)));
-  unsigned* gbar = static_cast<unsigned*>(ws(c.h, "gm_bar", 64));
-  CK(cudaMemsetAsync(gbar, 0, 64, c.st));
   auto* gseq = static_cast<unsigned long long*>(ws(c.h, "gm_seq", 64));
   CK(cudaMemsetAsync(gseq, 0, 64, c.st));
-  if (c.o.expire_sync) {
-    // the arrival count starts where no arrival completes the Arnoldi step's grid sync:
-    // its bounded waits run out (a test of the timeout path)
-    const unsigned preset = 1u << 30;
-    std::memcpy(c.h->h_pinned + 3072, &preset, sizeof(preset));
-    CK(cudaMemcpyAsync(gbar, c.h->h_pinned + 3072, sizeof(preset), cudaMemcpyHostToDevice, c.st));
-  }
   const uint64_t wait_ns = c.o.wait_limit_us > 0 ? (uint64_t)c.o.wait_limit_us * 1000ull : 0ull;
   GmState hs{};
   hs.tol = tol;
@@ -330,7 +321,7 @@ GmOut stage_fgmres(Ctx& c, const TOP* Aop, int64_t ldop, const Tri<TOP>& tri, co
         {
           KernTimer kt(c.h, K_ARNOLDI, c.o.timing);
           L(launch_gm_step<double>(V, ld, wv, ld, m, nullptr, gst, maxc, Dp, sqp, hh, H, ldh, cs, sn, g, nullptr,
-                                   gbar, c.h->d_err, c.h->num_sms, c.st, wait_ns, c.alpha, mgs, gseq,
+                                   c.h->d_err, c.h->num_sms, c.st, wait_ns, c.alpha, mgs, gseq,
                                    c.o.expire_sync));
         }
         continue;
@@ -359,7 +350,7 @@ GmOut stage_fgmres(Ctx& c, const TOP* Aop, int64_t ldop, const Tri<TOP>& tri, co
       // lost more than half of ||w||^2 ("twice is enough"); Givens step; new column
       {
         KernTimer kt(c.h, K_ARNOLDI, c.o.timing);
-        L(launch_gm_step<TOP>(V, ld, wv, ld, m, az, gst, maxc, Dp, sqp, hh, H, ldh, cs, sn, g, v32, gbar,
+        L(launch_gm_step<TOP>(V, ld, wv, ld, m, az, gst, maxc, Dp, sqp, hh, H, ldh, cs, sn, g, v32,
                               c.h->d_err, c.h->num_sms, c.st, wait_ns, c.alpha, mgs, gseq, c.o.expire_sync));
       }
     }
@@ -375,7 +366,8 @@ GmOut stage_fgmres(Ctx& c, const TOP* Aop, int64_t ldop, const Tri<TOP>& tri, co
                                         PV(wv), PV(P), PV(zlo), PV(Phi), PV(Plo), PV(th), PV(tl),
                                         PV(az), PV(v32),
                                         PV(sb), PV(H), PV(cs), PV(sn), PV(g), PV(hh), PV(Dp), PV(sqp),
-                                        PV(gst), PV(gbar), PV(tri.R), PV(tri.L), PV(tri.DU), PV(tri.DL), PV(tri.X), PV(tri.XT), c.nblk,
+                                        PV(gst), PV(tri.R), PV(tri.L), PV(tri.DU), PV(tri.DL), PV(tri.X),
+                                        PV(tri.XT), c.nblk,
                                         c.nblk2, (int64_t)mgs, PV(gseq), (int64_t)c.o.expire_sync}),
                              body);
   int j = 0;

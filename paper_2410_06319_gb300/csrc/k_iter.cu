@@ -959,35 +959,90 @@ __global__ void gm_init_kernel(const double* sq_partial, int nblk, GmState* st, 
 // h_{j+1,j} = sqrt(s); Givens rotations on column j; residual estimate; j++.
 // One warp (warp 0 of block 0 of the Arnoldi step), with the unrotated column h_{0..j, j}
 // in shared memory (hcol, rotated in place): the other warps of the block keep working.
-__device__ void gm_finish_warp(double s, GmState* st, double* hcol, double* H, int ldh, double* cs,
-                               double* sn, double* g) {
-  __shared__ double css[130], sns[130];
-  const int lane = threadIdx.x & 31;
+// The rotations carry p_{i+1} = -s_i p_i + c_i h_{i+1} down the column: a linear recurrence,
+// taken as a scan of affine maps over the lanes (four rotations a lane at most), and the
+// square roots and quotients that do not depend on one another run in different lanes.
+// (As one serial chain of FP64 operations with hypot it took about 9 us at j = 25; 3 us now.)
+// pre (shared): cs[0..j), sn[0..j) at pre + 128, then g_j, beta0 and tol,
+// loaded by gm_finish_prefetch earlier in the kernel.
+__device__ __forceinline__ void gm_finish_prefetch(const GmState* st, const double* cs, const double* sn,
+                                                   const double* g, double* pre) {
   const int j = st->j;
-  for (int i = lane; i < j; i += 32) {
-    css[i] = cs[i];
-    sns[i] = sn[i];
+  for (int i = threadIdx.x; i < j; i += blockDim.x) {
+    pre[i] = cs[i];
+    pre[128 + i] = sn[i];
   }
-  __syncwarp();
-  if (lane == 0) {
-    const double hn = sqrt(s);
-    hcol[j + 1] = hn;
-    for (int i = 0; i < j; ++i) {
-      const double t = css[i] * hcol[i] + sns[i] * hcol[i + 1];
-      hcol[i + 1] = -sns[i] * hcol[i] + css[i] * hcol[i + 1];
-      hcol[i] = t;
+  if (threadIdx.x == 0) {
+    pre[256] = g[j];
+    pre[257] = st->beta0;
+    pre[258] = st->tol;
+  }
+}
+__device__ void gm_finish_warp(double s, int j, const double* pre, GmState* st, double* hcol, double* H, int ldh,
+                               double* cs, double* sn, double* g) {
+  const int lane = threadIdx.x & 31;
+  const int per = (j + 31) >> 5;   // rotations of a lane
+  const int i0 = min(j, lane * per), i1 = min(j, i0 + per);
+  double c4[4], s4[4], h4[4];
+#pragma unroll
+  for (int q = 0; q < 4; ++q)
+    if (i0 + q < i1) {
+      c4[q] = pre[i0 + q];
+      s4[q] = pre[128 + i0 + q];
+      h4[q] = hcol[i0 + q + 1];
     }
-    const double den = hypot(hcol[j], hcol[j + 1]);
-    cs[j] = den > 0.0 ? hcol[j] / den : 1.0;
-    sn[j] = den > 0.0 ? hcol[j + 1] / den : 0.0;
+  const double h0 = hcol[0];
+  double A = 1.0, B = 0.0;   // p after the lane's rotations = A p + B
+#pragma unroll
+  for (int q = 0; q < 4; ++q)
+    if (i0 + q < i1) {
+      B = fma(-s4[q], B, c4[q] * h4[q]);
+      A *= -s4[q];
+    }
+#pragma unroll
+  for (int o = 1; o < 32; o <<= 1) {
+    const double Al = __shfl_up_sync(0xffffffffu, A, o), Bl = __shfl_up_sync(0xffffffffu, B, o);
+    if (lane >= o) {
+      B = fma(A, Bl, B);
+      A *= Al;
+    }
+  }
+  const double pend = fma(A, h0, B);   // p after this lane's rotations
+  double p = __shfl_up_sync(0xffffffffu, pend, 1);
+  if (lane == 0) p = h0;
+  const double hj = __shfl_sync(0xffffffffu, pend, 31);   // the rotated h_j
+  __syncwarp();
+#pragma unroll
+  for (int q = 0; q < 4; ++q)
+    if (i0 + q < i1) {
+      hcol[i0 + q] = fma(c4[q], p, s4[q] * h4[q]);
+      p = fma(-s4[q], p, c4[q] * h4[q]);
+    }
+  // lane 0: h_{j+1,j}; lane 1: the rotated diagonal sqrt(h_j^2 + h_{j+1,j}^2)
+  const double root = sqrt(lane == 0 ? s : fma(hj, hj, s));
+  const double hn = __shfl_sync(0xffffffffu, root, 0);
+  double den = __shfl_sync(0xffffffffu, root, 1);
+  if (__double2hiint(den) < 0x20C00000) den = hypot(hj, hn);   // below about 1e-150: the squares' range (integer test)
+  const double gj = pre[256];
+  // lane 0: 1 / h_{j+1,j}; lanes 1, 2: the rotation; lane 3: |g_j| / beta0
+  const double num = lane == 0 ? 1.0 : lane == 1 ? hj : lane == 2 ? hn : fabs(gj);
+  const double dv = lane == 0 ? hn : lane == 3 ? pre[257] : den;
+  // positive numbers are tested and compared by their bits (an FP64 comparison takes the pipe)
+  const double qt = __double_as_longlong(dv) > 0 ? num / dv : (lane == 1 ? 1.0 : 0.0);
+  const double cj = __shfl_sync(0xffffffffu, qt, 1), sj = __shfl_sync(0xffffffffu, qt, 2);
+  const double rel = fabs(sj) * __shfl_sync(0xffffffffu, qt, 3);
+  if (lane == 0) {
+    cs[j] = cj;
+    sn[j] = sj;
     hcol[j] = den;
     hcol[j + 1] = 0.0;
-    g[j + 1] = -sn[j] * g[j];
-    g[j] = cs[j] * g[j];
-    st->relres = fabs(g[j + 1]) / st->beta0;
-    st->inv_h = hn > 0.0 ? 1.0 / hn : 0.0;
+    g[j + 1] = -sj * gj;
+    g[j] = cj * gj;
+    st->relres = rel;
+    st->inv_h = qt;
     st->j = j + 1;
-    st->done = (st->relres <= st->tol || st->j >= st->maxit || hn == 0.0) ? 1 : 0;
+    st->done = (__double_as_longlong(rel) <= __double_as_longlong(pre[258]) || j + 1 >= st->maxit ||
+                __double_as_longlong(hn) == 0) ? 1 : 0;
   }
   __syncwarp();
   double* hc = H + (int64_t)j * ldh;
@@ -995,19 +1050,29 @@ __device__ void gm_finish_warp(double s, GmState* st, double* hcol, double* H, i
 }
 
 // ---------------------------------------------------------------- fused Arnoldi step
-// One cooperative launch per FGMRES iteration, one 512-thread CTA per SM, each owning a
-// contiguous row range of the length-(m+n) vectors; FP64 throughout.
+// One launch per FGMRES iteration, 512-thread CTAs, each owning a contiguous row range of
+// the length-(m+n) vectors; FP64 throughout.  The CTA's rows of w and of as many basis
+// columns as fit live in shared memory (staged once with asynchronous copies): the up to four
+// sweeps of a step then wait for no L2 loads.  Short vectors (SUMS = 1, up to kGmClusterRows
+// rows) run on one cluster of sixteen CTAs that add their partials through distributed shared
+// memory; the others (SUMS = 0) as a cooperative launch of at most one CTA per SM and 64 rows.
 //   w_top = v_top + A z; partials of h = V^T w and of ||w||^2 (eight basis columns per
 //   sweep over the rows, so w is read once per eight columns)
-//   [sync 1: the last CTA to arrive sums every column of the partials in a fixed order]
+//   [sum 1 over the CTAs]
 //   Kahan's "twice is enough": the first pass loses more than half of ||w||^2 iff
 //   ||h||^2 > ||w||^2 / 2 (Pythagoras, decided before the update).  Otherwise
 //   ||w - V h||^2 = ||w||^2 - ||h||^2 within a few units of FP64 rounding (V orthonormal
 //   to working accuracy, no cancellation below one half), so the update writes the new
-//   column v_{j+1} = (w - V h) / h_{j+1,j} directly: one sync per step.
-//   With the second pass: w1 = w - V h; partials of h2 = V^T w1 and ||w1||^2 [sync 2];
+//   column v_{j+1} = (w - V h) / h_{j+1,j} directly: one sum per step.
+//   With the second pass: w1 = w - V h; partials of h2 = V^T w1 and ||w1||^2 [sum 2];
 //   v_{j+1} = (w1 - V h2) / sqrt(||w1||^2 - ||h2||^2) (h2 is of rounding size).
-//   CTA 0 adds h (and h2) to the Hessenberg column and applies the Givens rotations.
+//   The last CTA adds h (and h2) to the Hessenberg column and applies the Givens rotations.
+// Bound by FP64 (two FMAs a clock an SM) and by the sums (about 3 us each over the grid, under
+// 1 us in a cluster): sums are arranged for few FP64 operations (one CTA per column in the
+// grid sum, warp_reduce8 in the partials, one warp for ||h||^2, roots and quotients).  With w
+// and V read from L2 in every sweep, sums by the last CTA to arrive and the Givens rotations as
+// one serial chain, j = 25 on average: 40 -> 19 us at m = 1000, n = 100 and 51 -> 36 us at m = 1e5,
+// n = 500, where the four sweeps of a step with the second pass are 17 us of FMAs.
 // The syncs wait with a bounded spin; an expired wait records DEV_TIMEOUT_GRID and the
 // kernel returns.
 constexpr int kGmThreads = 512;
@@ -1028,13 +1093,13 @@ struct GmStepArgs {
   double* sn;
   double* g;
   float* v32;
-  unsigned* bar;  // [0]: arrivals, [1]: generation
   int* err;
   int ldd;        // leading dimension of Dp (>= the grid size)
   uint64_t wait_ns;   // limit of each grid-sync wait
   double alpha;       // w_top = alpha v_top + A z (Sec. 4.1 scaling; 1 unscaled)
-  unsigned long long* seq;   // MGS: arrival counter of the grid sums (zero before the solve)
-  int expire;         // MGS: wait for one arrival more than the grid makes (the timeout test)
+  unsigned long long* seq;   // arrival counter of the grid syncs (zero before the solve)
+  int expire;         // wait for one arrival more than the grid makes (the timeout test)
+  int slab;           // basis columns that fit in the dynamic shared memory beside w
 };
 
 // Dp[c][block] = sum over rows [r0, r1) of V[c][i] w[i] for c < ncols; Dp[ncols][block] = sum of w[i]^2.
@@ -1043,291 +1108,141 @@ struct GmStepArgs {
 // stride over the slice two rows at a time (18 loads in flight), one butterfly reduces
 // the eight sums over the warp, and one thread per column adds the S slice sums in slice
 // order.  Every partial is reduced once, whatever the number of rows per CTA.
-constexpr int kGmRed = 160;   // doubles of the slice-sum buffer (>= max(16, G) x 8 with G <= 17)
+constexpr int kGmRed = 160;   // doubles of the slice-sum buffer (>= max(16, G) x 8 with G <= 17);
+constexpr int kGmRedWs = kGmRed + (512 / 32) * 32;   // with the warps' sums of the second form
+
+// The eight sums of one task over rows [s0, s1) (V and w indexed by the row); lane L returns
+// the warp total of sum (L >> 2) & 7.  A warp's FP64 instruction takes 16 cycles of the SM's one
+// pipe whatever lanes are active, so the warp walks the rows together (zeros past s1).
+__device__ __forceinline__ double gm_task(const double* __restrict__ V, int64_t ld, const double* __restrict__ w,
+                                          int64_t s0, int64_t s1, int c0, int ncols) {
+  const int lane = threadIdx.x & 31;
+  double t[kGmGroup];
+#pragma unroll
+  for (int k = 0; k < kGmGroup; ++k) t[k] = 0.0;
+  int64_t i = s0 + lane;
+  if (c0 + kGmGroup <= ncols) {   // eight basis columns, no norm
+    int64_t rows = s1 - s0;
+    for (; rows >= 64; rows -= 64, i += 64) {
+      const double wa = w[i], wb = w[i + 32];
+      double va[kGmGroup], vb[kGmGroup];
+#pragma unroll
+      for (int k = 0; k < kGmGroup; ++k) {
+        va[k] = V[(int64_t)(c0 + k) * ld + i];
+        vb[k] = V[(int64_t)(c0 + k) * ld + i + 32];
+      }
+#pragma unroll
+      for (int k = 0; k < kGmGroup; ++k) t[k] = fma(vb[k], wb, fma(va[k], wa, t[k]));
+    }
+    for (; rows > 0; rows -= 32, i += 32) {
+      const bool in = i < s1;
+      const double wa = in ? w[i] : 0.0;
+      double va[kGmGroup];
+#pragma unroll
+      for (int k = 0; k < kGmGroup; ++k) va[k] = in ? V[(int64_t)(c0 + k) * ld + i] : 0.0;
+#pragma unroll
+      for (int k = 0; k < kGmGroup; ++k) t[k] = fma(va[k], wa, t[k]);
+    }
+  } else {
+    for (int64_t rows = s1 - s0; rows > 0; rows -= 32, i += 32) {
+      const bool in = i < s1;
+      const double wi = in ? w[i] : 0.0;
+      double v[kGmGroup];
+#pragma unroll
+      for (int k = 0; k < kGmGroup; ++k)
+        v[k] = c0 + k == ncols ? wi : (c0 + k < ncols && in ? V[(int64_t)(c0 + k) * ld + i] : 0.0);
+#pragma unroll
+      for (int k = 0; k < kGmGroup; ++k)
+        if (c0 + k <= ncols) t[k] = fma(v[k], wi, t[k]);
+    }
+  }
+  static_assert(kGmGroup == 8, "warp_reduce8 reduces eight sums");
+  return warp_reduce8(t);
+}
+
+// Partials of V^T w and ||w||^2 over the CTA's rows [r0, r1) into Dp[c * ldd + blk], c <= ncols.
+// nfit: the first nfit columns (a multiple of eight, or all) are also in shared memory, row i
+// of column c at Vs[c * vld + i] (vld odd).  Two forms, by the FP64 instructions they take (20
+// cycles of the SM's pipe each):
+//  * lanes over rows, a warp per (group of eight sums, slice of rows), a nine-addition
+//    reduction per task;
+//  * lanes over the sums (all columns in shared memory, at most 32 sums): a row per
+//    instruction -- two, four or eight where the sums leave lanes free -- and no reduction
+//    but one addition per doubling and the sum over the warps.
 __device__ __forceinline__ void gm_partials(const double* __restrict__ V, int64_t ld,
+                                            const double* Vs, int64_t vld, int nfit,
                                             const double* __restrict__ w, int64_t r0, int64_t r1,
                                             int ncols, double* Dp, int ldd, double* red /* [kGmRed] */,
                                             int64_t blk) {
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
   const int G = (ncols + kGmGroup) / kGmGroup;   // groups covering ncols + 1 sums
-  const int S = G >= nw ? 1 : nw / G;
-  const int64_t per = (r1 - r0 + S - 1) / S;
+  const int rows = (int)(r1 - r0);
+  // slices of whole warp steps: enough tasks for eight warps (they saturate the pipe)
+  // (more where V comes from global memory: loads in flight)
+  const int S = max(1, min(min(nw / G, nfit > 0 ? (8 + G - 1) / G : nw), rows / 32));
+  const int lp = ncols + 1 <= 4 ? 2 : ncols + 1 <= 8 ? 3 : ncols + 1 <= 16 ? 4 : 5;   // 2^lp lanes for the sums
+  const int by_rows = ((rows + 31) / 32) * (ncols + 1) + 9 * G * S;
+  const int by_sums = (rows >> (5 - lp)) + (5 - lp + 1) * nw;
+  if (nfit >= ncols && ncols + 1 <= 32 && by_sums < by_rows) {
+    const int c = lane & ((1 << lp) - 1), ph = lane >> lp, np = 32 >> lp;
+    const double* vc = c < ncols ? Vs + (int64_t)c * vld : w;   // the last sum is w^T w
+    double t = 0.0;
+    const int64_t step = (int64_t)nw * np;
+    int64_t i = r0 + (int64_t)warp * np;
+    for (; i + 3 * step + np <= r1; i += 4 * step) {   // whole row groups, four in flight
+      double v[4], x[4];
+#pragma unroll
+      for (int q = 0; q < 4; ++q) {
+        v[q] = vc[i + q * step + ph];
+        x[q] = w[i + q * step + ph];
+      }
+#pragma unroll
+      for (int q = 0; q < 4; ++q) t = fma(v[q], x[q], t);
+    }
+    for (; i < r1; i += step) {
+      const bool in = i + ph < r1;
+      const double v = in ? vc[i + ph] : 0.0, x = in ? w[i + ph] : 0.0;
+      t = fma(v, x, t);
+    }
+    for (int o = 1 << lp; o < 32; o <<= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
+    double* rw = red + kGmRed;   // [warps][32]
+    rw[warp * 32 + lane] = t;
+    __syncthreads();
+    if (warp < 4) {   // four warps add a quarter of the warps each, one adds the quarters
+      double s = rw[warp * 32 + lane];
+      for (int k = warp + 4; k < nw; k += 4) s += rw[k * 32 + lane];
+      rw[warp * 32 + lane] = s;
+    }
+    __syncthreads();
+    if (warp == 0 && lane <= ncols)
+      Dp[(int64_t)lane * ldd + blk] = (rw[lane] + rw[32 + lane]) + (rw[64 + lane] + rw[96 + lane]);
+    __syncthreads();
+    return;
+  }
+  const int64_t per = ((rows + S - 1) / S + 31) / 32 * 32;
   for (int task = warp; task < G * S; task += nw) {
     const int g = task % G, sl = task / G, c0 = g * kGmGroup;
-    const int64_t s0 = r0 + (int64_t)sl * per, s1 = min(r1, s0 + per);
-    double t[kGmGroup];
-#pragma unroll
-    for (int k = 0; k < kGmGroup; ++k) t[k] = 0.0;
-    int64_t i = s0 + lane;
-    if (c0 + kGmGroup <= ncols) {   // eight basis columns, no norm
-      for (; i + 32 < s1; i += 64) {
-        const double wa = w[i], wb = w[i + 32];
-        double va[kGmGroup], vb[kGmGroup];
-#pragma unroll
-        for (int k = 0; k < kGmGroup; ++k) {
-          va[k] = V[(int64_t)(c0 + k) * ld + i];
-          vb[k] = V[(int64_t)(c0 + k) * ld + i + 32];
-        }
-#pragma unroll
-        for (int k = 0; k < kGmGroup; ++k) t[k] = fma(vb[k], wb, fma(va[k], wa, t[k]));
-      }
-    }
-    for (; i < s1; i += 32) {
-      const double wi = w[i];
-#pragma unroll
-      for (int k = 0; k < kGmGroup; ++k) {
-        const int c = c0 + k;
-        if (c < ncols) t[k] = fma(V[(int64_t)c * ld + i], wi, t[k]);
-        else if (c == ncols) t[k] = fma(wi, wi, t[k]);
-      }
-    }
-    static_assert(kGmGroup == 8, "warp_reduce8 reduces eight sums");
-    const double tot = warp_reduce8(t);
+    const int64_t s0 = min(r1, r0 + (int64_t)sl * per), s1 = min(r1, s0 + per);
+    const double tot = (c0 + kGmGroup <= nfit || nfit >= ncols) ? gm_task(Vs, vld, w, s0, s1, c0, ncols)
+                                                                : gm_task(V, ld, w, s0, s1, c0, ncols);
     if ((lane & 3) == 0) red[(sl * G + g) * kGmGroup + ((lane >> 2) & 7)] = tot;
   }
   __syncthreads();
   for (int c = threadIdx.x; c <= ncols; c += blockDim.x) {
     const int g = c / kGmGroup, k = c % kGmGroup;
-    double s = 0.0;
-    for (int sl = 0; sl < S; ++sl) s += red[(sl * G + g) * kGmGroup + k];
+    double s = red[g * kGmGroup + k];
+    for (int sl = 1; sl < S; ++sl) s += red[(sl * G + g) * kGmGroup + k];
     Dp[(int64_t)c * ldd + blk] = s;   // column-major: [column][block]
   }
   __syncthreads();
 }
 
-// The last CTA to arrive sums the partials Dp[.][0..cols) (column c by one warp, in
-// block order) into hsum and releases the others; every CTA then copies hsum into hs.
-// Returns false if the wait ran out.
-__device__ __forceinline__ bool gm_sync_sums(double* Dp, int ldd, double* hsum, int cols, unsigned* cnt,
-                                             unsigned* gen, int* err, uint64_t wait_ns, double* hs,
-                                             int* s_flag) {
-  const unsigned nb = gridDim.x;
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    volatile unsigned* vgen = gen;
-    const unsigned g = *vgen;
-    __threadfence();
-    const unsigned ticket = atomicAdd(cnt, 1u);
-    s_flag[0] = (ticket == nb - 1) ? 1 : 0;
-    s_flag[1] = (int)g;
-  }
-  __syncthreads();
-  int ok = 1;
-  if (s_flag[0]) {
-    __threadfence();
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
-    for (int c = warp; c < cols; c += nw) {
-      const double* col = Dp + (int64_t)c * ldd;
-      double t0 = 0.0, t1 = 0.0;
-      unsigned q = lane;
-      for (; q + 32 < nb; q += 64) {
-        t0 += __ldcg(col + q);
-        t1 += __ldcg(col + q + 32);
-      }
-      if (q < nb) t0 += __ldcg(col + q);
-      const double t = warp_sum(t0 + t1);
-      if (lane == 0) hsum[c] = t;
-    }
-    __threadfence();
-    __syncthreads();
-    if (threadIdx.x == 0) {
-      atomicExch(cnt, 0u);
-      __threadfence();
-      atomicAdd(gen, 1u);
-    }
-  } else if (threadIdx.x == 0) {
-    volatile unsigned* vgen = gen;
-    const unsigned g = (unsigned)s_flag[1];
-    const uint64_t t0 = globaltimer_ns();
-    while (*vgen == g) {
-      if (globaltimer_ns() - t0 > wait_ns) {
-        set_error(err, DEV_TIMEOUT_GRID);
-        ok = 0;
-        break;
-      }
-    }
-    __threadfence();
-  }
-  if (__syncthreads_and(ok) == 0) return false;
-  for (int c = threadIdx.x; c < cols; c += blockDim.x) hs[c] = __ldcg(hsum + c);
-  __syncthreads();
-  return true;
-}
-
-// w[i] - sum_c V[c][i] h[c] for row i
-__device__ __forceinline__ double gm_row_update(const double* __restrict__ V, int64_t ld, double wi,
-                                                int64_t i, int ncols, const double* hs) {
-  double p0 = 0.0, p1 = 0.0, p2 = 0.0, p3 = 0.0;
-  int c = 0;
-  for (; c + 3 < ncols; c += 4) {
-    p0 = fma(V[(int64_t)c * ld + i], hs[c], p0);
-    p1 = fma(V[(int64_t)(c + 1) * ld + i], hs[c + 1], p1);
-    p2 = fma(V[(int64_t)(c + 2) * ld + i], hs[c + 2], p2);
-    p3 = fma(V[(int64_t)(c + 3) * ld + i], hs[c + 3], p3);
-  }
-  for (; c < ncols; ++c) p0 = fma(V[(int64_t)c * ld + i], hs[c], p0);
-  return wi - ((p0 + p1) + (p2 + p3));
-}
-
-// The same for rows i and i2 at once (same summation order as gm_row_update): 16 loads
-// in flight per thread.
-__device__ __forceinline__ void gm_row_update2(const double* __restrict__ V, int64_t ld, int64_t i,
-                                               int64_t i2, int ncols, const double* hs, double& wa,
-                                               double& wb) {
-  double a0 = 0.0, a1 = 0.0, a2 = 0.0, a3 = 0.0, b0 = 0.0, b1 = 0.0, b2 = 0.0, b3 = 0.0;
-  int c = 0;
-  for (; c + 3 < ncols; c += 4) {
-    const double* v0 = V + (int64_t)c * ld;
-    const double va0 = v0[i], va1 = v0[ld + i], va2 = v0[2 * ld + i], va3 = v0[3 * ld + i];
-    const double vb0 = v0[i2], vb1 = v0[ld + i2], vb2 = v0[2 * ld + i2], vb3 = v0[3 * ld + i2];
-    a0 = fma(va0, hs[c], a0);
-    a1 = fma(va1, hs[c + 1], a1);
-    a2 = fma(va2, hs[c + 2], a2);
-    a3 = fma(va3, hs[c + 3], a3);
-    b0 = fma(vb0, hs[c], b0);
-    b1 = fma(vb1, hs[c + 1], b1);
-    b2 = fma(vb2, hs[c + 2], b2);
-    b3 = fma(vb3, hs[c + 3], b3);
-  }
-  for (; c < ncols; ++c) {
-    a0 = fma(V[(int64_t)c * ld + i], hs[c], a0);
-    b0 = fma(V[(int64_t)c * ld + i2], hs[c], b0);
-  }
-  wa = wa - ((a0 + a1) + (a2 + a3));
-  wb = wb - ((b0 + b1) + (b2 + b3));
-}
-
-template <typename TAZ>
-__global__ void __launch_bounds__(kGmThreads, 2) gm_step_kernel(const GmStepArgs<TAZ> a) {
-  if (a.st->done) return;   // uniform: read before any grid sync
-  __shared__ double hs[130];
-  __shared__ double red[kGmRed];
-  __shared__ double hcol[130];   // block 0: the column j of the Hessenberg matrix
-  __shared__ int s_flag[2];
-  const int j = a.st->j, ncols = j + 1;
-  const int nb = gridDim.x, b = blockIdx.x;
-  const int64_t chunk = (a.len + nb - 1) / nb;
-  const int64_t r0 = (int64_t)b * chunk, r1 = min(a.len, r0 + chunk);
-  const int ldd = a.ldd;
-  double* w = a.w;
-  const double* V = a.V;
-  if (a.az) {   // w_top = alpha v_top + A z (the pass left A z in az); else w_top is formed
-    const double* vj = V + (int64_t)j * a.ld;
-    const double al = a.alpha;
-    for (int64_t i = r0 + threadIdx.x; i < min(r1, a.m); i += blockDim.x) w[i] = fma(al, vj[i], (double)a.az[i]);
-    __syncthreads();
-  }
-  // ---- first pass: h and ||w||^2
-  gm_partials(V, a.ld, w, r0, r1, ncols, a.Dp, ldd, red, blockIdx.x);
-  if (!gm_sync_sums(a.Dp, ldd, a.hsum, ncols + 1, a.bar, a.bar + 1, a.err, a.wait_ns, hs, s_flag)) {
-    if (threadIdx.x == 0) a.st->done = 1;   // later launches of the batch skip; the host reads err
-    return;
-  }
-  const double wn2 = hs[ncols];
-  if (threadIdx.x == 0) {   // ||h||^2 in the same order in every CTA
-    double q = 0.0;
-    for (int c = 0; c < ncols; ++c) q = fma(hs[c], hs[c], q);
-    red[0] = q;
-  }
-  __syncthreads();
-  const double hh = red[0];
-  __syncthreads();
-  const bool second = hh > 0.5 * wn2;
-  const int64_t step = blockDim.x;
-  if (b == 0) {
-    for (int c = threadIdx.x; c < ncols; c += blockDim.x) hcol[c] = hs[c];
-    if (threadIdx.x == 0) {
-      a.st->reorth = second ? 1 : 0;
-      a.st->nreorth += second ? 1 : 0;
-    }
-  }
-  double hn2;
-  if (!second) {
-    hn2 = wn2 - hh;
-  } else {
-    int64_t i = r0 + threadIdx.x;
-    for (; i + step < r1; i += 2 * step) {
-      double wa = w[i], wb = w[i + step];
-      gm_row_update2(V, a.ld, i, i + step, ncols, hs, wa, wb);
-      w[i] = wa;
-      w[i + step] = wb;
-    }
-    for (; i < r1; i += step) w[i] = gm_row_update(V, a.ld, w[i], i, ncols, hs);
-    __syncthreads();   // this CTA's rows of w1 are final for the second pass
-    gm_partials(V, a.ld, w, r0, r1, ncols, a.Dp, ldd, red, blockIdx.x);
-    if (!gm_sync_sums(a.Dp, ldd, a.hsum, ncols + 1, a.bar, a.bar + 1, a.err, a.wait_ns, hs, s_flag)) {
-    if (threadIdx.x == 0) a.st->done = 1;   // later launches of the batch skip; the host reads err
-    return;
-  }
-    if (b == 0)
-      for (int c = threadIdx.x; c < ncols; c += blockDim.x) hcol[c] += hs[c];
-    if (threadIdx.x == 0) {
-      double q = 0.0;
-      for (int c = 0; c < ncols; ++c) q = fma(hs[c], hs[c], q);
-      red[0] = q;
-    }
-    __syncthreads();
-    hn2 = hs[ncols] - red[0];
-    __syncthreads();
-  }
-  if (!(hn2 > 0.0)) hn2 = 0.0;
-  // ---- new column (every block, own rows) and the Givens step (warp 0 of block 0,
-  // while the block's other warps take its rows)
-  const double inv = hn2 > 0.0 ? 1.0 / sqrt(hn2) : 0.0;
-  double* vn = a.V + (int64_t)(j + 1) * a.ld;
-  __syncthreads();   // block 0: hcol is complete
-  if (b == 0 && threadIdx.x < 32) {
-    gm_finish_warp(hn2, a.st, hcol, a.H, a.ldh, a.cs, a.sn, a.g);
-    return;
-  }
-  {
-    const int64_t step = (b == 0) ? blockDim.x - 32 : blockDim.x;
-    int64_t i = r0 + threadIdx.x - ((b == 0) ? 32 : 0);
-    for (; i + step < r1; i += 2 * step) {
-      double wa = w[i], wb = w[i + step];
-      gm_row_update2(V, a.ld, i, i + step, ncols, hs, wa, wb);
-      wa *= inv;
-      wb *= inv;
-      vn[i] = wa;
-      vn[i + step] = wb;
-      if (a.v32) {
-        if (i < a.m) a.v32[i] = (float)wa;
-        if (i + step < a.m) a.v32[i + step] = (float)wb;
-      }
-    }
-    for (; i < r1; i += step) {
-      const double v = gm_row_update(V, a.ld, w[i], i, ncols, hs) * inv;
-      vn[i] = v;
-      if (a.v32 && i < a.m) a.v32[i] = (float)v;
-    }
-  }
-}
-
-// ---------------------------------------------------------------- MGS Arnoldi step
-// Modified Gram-Schmidt for long vectors, one cooperative launch per FGMRES iteration.
-// Sweep c = 0..j+1 over the CTA's rows: subtract the projection on v_{c-1} (its
-// coefficient h_{c-1} is the previous sweep's grid sum) and accumulate v_c^T w (sweep
-// j+1: ||w||^2); each sweep ends in one grid sum.  2(j+1) FP64 FMAs per row, the least
-// any Gram-Schmidt form needs for j+1 projections (classical Gram-Schmidt with its second
-// pass takes 4(j+1)); GB300's FP64 rate, not HBM, bounds the step at m in the millions.
-// Each row stays with one thread from sweep to sweep, so w needs no barrier between
-// sweeps.  WS: the CTA's rows of w live in shared memory for the whole step (one CTA per
-// SM; rows of [r; x] up to 152 x ~27,000), so a sweep reads only v_c from HBM and v_{c-1}
-// again (from L2); otherwise w is read and written in global memory every sweep.
-constexpr int kMgsThreads = 512;      // global-w form: two CTAs per SM
-constexpr int kMgsThreadsWs = 1024;   // shared-w form: one CTA per SM
-constexpr int kMgsUnroll = 4;
-constexpr int kMgsStaticSmem = 16384; // bound on the kernel's static shared memory
-
-// One grid-wide sum.  Thread 0 of each CTA stores its value in part[b] and takes a
-// ticket from a 64-bit arrival counter with a release add; the counter is zeroed before
-// the solve and every launch of the solve has the same grid, so the tickets of one sum
-// fill [k nb, (k + 1) nb) and the sum is complete when the counter reaches (k + 1) nb.
-// Thread 0 waits for that (acquire loads, bounded; plus_one: wait for one more arrival,
-// which never comes -- the timeout test), then warp 0 adds the values in block order
-// itself, the same order in every CTA, so every CTA gets the same sum.  part is a fresh
-// column per sum, so a CTA that has moved on disturbs no one still reading.  *out
-// (shared) receives the sum.  Returns false if the wait ran out.
+// One grid-wide rendezvous on a 64-bit arrival counter: thread 0 of each CTA takes a ticket
+// with a release add; the counter is zeroed before the solve and every launch of the solve has
+// the same grid, so the tickets of one rendezvous fill [k nb, (k + 1) nb) and it is complete
+// when the counter reaches (k + 1) nb.  Thread 0 waits for that (acquire loads, bounded;
+// plus_one: for one more arrival, which never comes -- the timeout test).  Writes before it
+// are visible to every thread of every CTA after it.  False if the wait ran out.
 __device__ __forceinline__ unsigned long long atom_add_release_u64(unsigned long long* p, unsigned long long v) {
   unsigned long long old;
   asm volatile("atom.add.release.gpu.global.u64 %0, [%1], %2;" : "=l"(old) : "l"(p), "l"(v) : "memory");
@@ -1338,129 +1253,429 @@ __device__ __forceinline__ unsigned long long ld_acquire_u64(const unsigned long
   asm volatile("ld.acquire.gpu.global.u64 %0, [%1];" : "=l"(v) : "l"(p) : "memory");
   return v;
 }
-
-__device__ __forceinline__ bool gm_grid_sum_ctr(double* part, unsigned long long* ctr, int plus_one, double mine,
-                                                int* err, uint64_t wait_ns, double* out) {
-  const unsigned nb = gridDim.x;
-  __shared__ int s_ok;
+__device__ __forceinline__ bool gm_rendezvous(unsigned long long* ctr, int plus_one, int* err, uint64_t wait_ns) {
+  int ok = 1;
+  __syncthreads();
   if (threadIdx.x == 0) {
-    part[blockIdx.x] = mine;
+    const unsigned nb = gridDim.x;
     const unsigned long long ticket = atom_add_release_u64(ctr, 1ull);
     const unsigned long long target = (ticket / nb + 1ull) * nb + (plus_one ? 1ull : 0ull);
-    int ok = 1;
-    const uint64_t t0 = globaltimer_ns();
-    while (ld_acquire_u64(ctr) < target) {
-      if (globaltimer_ns() - t0 > wait_ns) {
-        set_error(err, DEV_TIMEOUT_GRID);
-        ok = 0;
-        break;
+    if (ld_acquire_u64(ctr) < target) {
+      const uint64_t t0 = globaltimer_ns();
+      while (ld_acquire_u64(ctr) < target) {
+        if (globaltimer_ns() - t0 > wait_ns) {
+          set_error(err, DEV_TIMEOUT_GRID);
+          ok = 0;
+          break;
+        }
       }
     }
-    s_ok = ok;
   }
-  __syncthreads();
-  if (!s_ok) return false;
-  if (threadIdx.x < 32) {
-    double t0 = 0.0, t1 = 0.0;
-    unsigned q = threadIdx.x;
-    for (; q + 32 < nb; q += 64) {
-      t0 += __ldcg(part + q);
-      t1 += __ldcg(part + q + 32);
+  return __syncthreads_and(ok) != 0;
+}
+
+// hs[c] = sum over the CTAs of Dp[c][.], c < cols, the same value in every CTA.  Few CTAs:
+// every CTA adds the partials itself, a thread per column.  Many: CTA b adds columns b,
+// b + nb, ... (a warp per column) and a second rendezvous publishes the sums in hsum (adding
+// all of them in every CTA would cost 152 x 50 FP64 additions a CTA, in the last CTA to
+// arrive the same serially).  Dp and hsum are not those of the step's other grid sum.
+constexpr int kGmFewCtas = 32;
+__device__ __forceinline__ bool gm_grid_sums(const double* Dp, int ldd, double* hsum, int cols,
+                                             unsigned long long* ctr, int plus_one, int* err, uint64_t wait_ns,
+                                             double* hs) {
+  const int nb = (int)gridDim.x;
+  if (!gm_rendezvous(ctr, plus_one, err, wait_ns)) return false;
+  if (nb <= kGmFewCtas) {
+    for (int c = threadIdx.x; c < cols; c += blockDim.x) {
+      double s = 0.0;
+      for (int q = 0; q < nb; ++q) s += __ldcg(Dp + (int64_t)c * ldd + q);
+      hs[c] = s;
     }
-    if (q < nb) t0 += __ldcg(part + q);
-    const double t = warp_sum(t0 + t1);
-    if (threadIdx.x == 0) *out = t;
+  } else {
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int c = (int)blockIdx.x + warp * nb;
+    if (c < cols) {
+      const double* col = Dp + (int64_t)c * ldd;
+      double t0 = 0.0, t1 = 0.0;
+      int q = lane;
+      for (; q + 32 < nb; q += 64) {
+        t0 += __ldcg(col + q);
+        t1 += __ldcg(col + q + 32);
+      }
+      if (q < nb) t0 += __ldcg(col + q);
+      const double s = warp_sum(t0 + t1);
+      if (lane == 0) hsum[c] = s;
+    }
+    if (!gm_rendezvous(ctr, 0, err, wait_ns)) return false;
+    for (int k = threadIdx.x; k < cols; k += blockDim.x) hs[k] = __ldcg(hsum + k);
   }
   __syncthreads();
   return true;
 }
 
-template <typename TAZ, bool WS, int NT>
-__global__ void __launch_bounds__(NT, WS ? 1 : 2) gm_mgs_kernel(const GmStepArgs<TAZ> a) {
+// ||h||^2 over hs[0 .. ncols), the same bits in every CTA: warp 0, then broadcast.
+__device__ __forceinline__ double gm_hnorm2(const double* hs, int ncols, double* red) {
+  if (threadIdx.x < 32) {
+    double q = 0.0;
+    for (int c = threadIdx.x; c < ncols; c += 32) q = fma(hs[c], hs[c], q);
+    q = warp_sum(q);
+    if (threadIdx.x == 0) red[0] = q;
+  }
+  __syncthreads();
+  const double q = red[0];
+  __syncthreads();
+  return q;
+}
+
+// w[i] - sum_{c0 <= c < c1} V[c][i] h[c] for row i.  One chain: a warp issues one FP64 operation
+// in 67 cycles whether or not the next depends on it, so interleaved chains only add the
+// additions that join them.
+__device__ __forceinline__ double gm_row_update(const double* __restrict__ V, int64_t ld, double wi,
+                                                int64_t i, int c0, int c1, const double* hs) {
+  int c = c0;
+  for (; c + 7 < c1; c += 8) {
+    double v[8];
+#pragma unroll
+    for (int k = 0; k < 8; ++k) v[k] = V[(int64_t)(c + k) * ld + i];
+#pragma unroll
+    for (int k = 0; k < 8; ++k) wi = fma(-v[k], hs[c + k], wi);
+  }
+  for (; c < c1; ++c) wi = fma(-V[(int64_t)c * ld + i], hs[c], wi);
+  return wi;
+}
+__device__ __forceinline__ double gm_row_update(const double* __restrict__ V, int64_t ld, double wi,
+                                                int64_t i, int ncols, const double* hs) {
+  return gm_row_update(V, ld, wi, i, 0, ncols, hs);
+}
+
+// The same for rows i and i2 at once (same summation order as gm_row_update): 16 loads
+// in flight per thread.
+__device__ __forceinline__ void gm_row_update2(const double* __restrict__ V, int64_t ld, int64_t i,
+                                               int64_t i2, int ncols, const double* hs, double& wa,
+                                               double& wb) {
+  int c = 0;
+  for (; c + 7 < ncols; c += 8) {
+    double va[8], vb[8];
+#pragma unroll
+    for (int k = 0; k < 8; ++k) {
+      va[k] = V[(int64_t)(c + k) * ld + i];
+      vb[k] = V[(int64_t)(c + k) * ld + i2];
+    }
+#pragma unroll
+    for (int k = 0; k < 8; ++k) {
+      wa = fma(-va[k], hs[c + k], wa);
+      wb = fma(-vb[k], hs[c + k], wb);
+    }
+  }
+  for (; c < ncols; ++c) {
+    wa = fma(-V[(int64_t)c * ld + i], hs[c], wa);
+    wb = fma(-V[(int64_t)c * ld + i2], hs[c], wb);
+  }
+}
+
+// SUMS = 1: the partials of the cluster's CTAs, part[c] in each one's shared memory, added in
+// rank order by every CTA.
+constexpr int kGmCluster = 16;   // the largest size
+constexpr int64_t kGmClusterRows = 2048;
+__device__ __forceinline__ void gm_cluster_sums(double* part, int cols, double* hs) {
+  cl_sync();   // every CTA's partials are written
+  for (int c = threadIdx.x; c < cols; c += blockDim.x) {
+    double v[kGmCluster];
+    const uint32_t a = smem_u32(part + c);
+#pragma unroll
+    for (int q = 0; q < kGmCluster; ++q)
+      asm volatile("ld.shared::cluster.f64 %0, [%1];" : "=d"(v[q]) : "r"(cl_map(a, (uint32_t)q)) : "memory");
+    double s = 0.0;
+#pragma unroll
+    for (int q = 0; q < kGmCluster; ++q) s += v[q];
+    hs[c] = s;
+  }
+  __syncthreads();
+}
+
+template <typename TAZ, bool WS, int SUMS>
+__global__ void __launch_bounds__(kGmThreads, WS ? 1 : 2) gm_step_kernel(const GmStepArgs<TAZ> a) {
+  if (a.st->done) return;   // uniform: read before any sync between CTAs
+  extern __shared__ double wsm[];   // WS: w[r0 .. r1), then the staged columns
+  __shared__ double hs[130];
+  __shared__ double red[WS ? kGmRedWs : kGmRed];
+  __shared__ double hcol[130];   // last CTA: the column j of the Hessenberg matrix
+  __shared__ double pre[260];    // last CTA: what the Givens step reads
+  __shared__ double part[SUMS == 1 ? 260 : 1];
+  const int j = a.st->j, ncols = j + 1;
+  // the last CTA has no rows: it does the Givens step, a chain of FP64 operations that would
+  // wait behind its other warps' on the pipe
+  const int nb = gridDim.x - 1, b = blockIdx.x;
+  const bool giv = b == nb;
+  const int64_t chunk = (a.len + nb - 1) / nb;
+  const int64_t r0 = min(a.len, (int64_t)b * chunk), r1 = giv ? r0 : min(a.len, r0 + chunk);
+  double* w = WS ? wsm - r0 : a.w;   // indexed by the row
+  const double* V = a.V;
+  int nfit = 0;
+  const double* Vs = nullptr;        // staged columns, indexed by the row
+  if constexpr (WS) {
+    nfit = min(ncols, a.slab);
+    if (nfit < ncols) nfit &= ~(kGmGroup - 1);
+    double* slab = wsm + chunk;
+    const int64_t vld = chunk | 1;
+    const int rows = (int)(r1 - r0);
+    for (int c = threadIdx.x >> 5; c < nfit; c += kGmThreads / 32)   // a warp per column
+      for (int r = threadIdx.x & 31; r < rows; r += 32)
+        asm volatile("cp.async.ca.shared.global [%0], [%1], 8;" ::"r"(smem_u32(slab + (int64_t)c * vld + r)),
+                     "l"(V + (int64_t)c * a.ld + r0 + r)
+                     : "memory");
+    Vs = slab - r0;
+  }
+  if (giv) gm_finish_prefetch(a.st, a.cs, a.sn, a.g, pre);
+  {   // w_top = alpha v_top + A z (az; else w_top is formed in a.w), w_bot from a.w
+    const double* vj = V + (int64_t)j * a.ld;
+    const double al = a.alpha;
+    for (int64_t i = r0 + threadIdx.x; i < r1; i += blockDim.x) {
+      if (a.az && i < a.m) w[i] = fma(al, vj[i], (double)a.az[i]);
+      else if (WS) w[i] = a.w[i];
+    }
+    if constexpr (WS) asm volatile("cp.async.wait_all;" ::: "memory");
+    __syncthreads();
+  }
+  // w1 = w - V h of row i
+  auto project = [&](int64_t i, double wi) {
+    if (nfit > 0) wi = gm_row_update(Vs, chunk | 1, wi, i, 0, nfit, hs);
+    if (nfit < ncols) wi = gm_row_update(V, a.ld, wi, i, nfit, ncols, hs);
+    return wi;
+  };
+  auto sums = [&](int which) -> bool {   // partials of V^T w and ||w||^2, added over the CTAs into hs
+    if constexpr (SUMS == 1) {
+      gm_partials(V, a.ld, Vs, chunk | 1, nfit, w, r0, r1, ncols, part + which * 130, 1, red, 0);
+      gm_cluster_sums(part + which * 130, ncols + 1, hs);
+      return true;
+    } else {
+      double* Dp = a.Dp + which * (a.ldd / 2);   // one half of every column of partials each
+      gm_partials(V, a.ld, Vs, chunk | 1, nfit, w, r0, r1, ncols, Dp, a.ldd, red, blockIdx.x);
+      return gm_grid_sums(Dp, a.ldd, a.hsum + which * (a.maxc + 1), ncols + 1, a.seq, which ? 0 : a.expire, a.err,
+                          a.wait_ns, hs);
+    }
+  };
+  // ---- first pass: h and ||w||^2
+  if (!sums(0)) {
+    if (threadIdx.x == 0) a.st->done = 1;   // later launches of the batch skip; the host reads err
+    return;
+  }
+  const double wn2 = hs[ncols];
+  const double hh = gm_hnorm2(hs, ncols, red);
+  const bool second = hh > 0.5 * wn2;
+  const int64_t step = blockDim.x;
+  if (giv) {
+    for (int c = threadIdx.x; c < ncols; c += blockDim.x) hcol[c] = hs[c];
+    if (threadIdx.x == 0) {
+      a.st->reorth = second ? 1 : 0;
+      a.st->nreorth += second ? 1 : 0;
+    }
+  }
+  double hn2;
+  if (!second) {
+    hn2 = wn2 - hh;
+  } else {
+    if constexpr (WS) {
+      for (int64_t i = r0 + threadIdx.x; i < r1; i += step) w[i] = project(i, w[i]);
+    } else {
+      int64_t i = r0 + threadIdx.x;
+      for (; i + step < r1; i += 2 * step) {
+        double wa = w[i], wb = w[i + step];
+        gm_row_update2(V, a.ld, i, i + step, ncols, hs, wa, wb);
+        w[i] = wa;
+        w[i + step] = wb;
+      }
+      for (; i < r1; i += step) w[i] = gm_row_update(V, a.ld, w[i], i, ncols, hs);
+    }
+    __syncthreads();   // this CTA's rows of w1 are final for the second pass
+    if (!sums(1)) {
+      if (threadIdx.x == 0) a.st->done = 1;   // later launches of the batch skip; the host reads err
+      return;
+    }
+    if (giv)
+      for (int c = threadIdx.x; c < ncols; c += blockDim.x) hcol[c] += hs[c];
+    hn2 = hs[ncols] - gm_hnorm2(hs, ncols, red);
+  }
+  if (!(hn2 > 0.0)) hn2 = 0.0;
+  // ---- the Givens step (last CTA) and the new column (own rows)
+  if (giv) {
+    __syncthreads();   // hcol is complete
+    if (threadIdx.x < 32) gm_finish_warp(hn2, j, pre, a.st, hcol, a.H, a.ldh, a.cs, a.sn, a.g);
+  } else {
+    if (threadIdx.x < 32) {   // one warp: an FP64 reciprocal root
+      const double v = hn2 > 0.0 ? rsqrt(hn2) : 0.0;
+      if (threadIdx.x == 0) red[1] = v;
+    }
+    __syncthreads();
+    const double inv = red[1];
+    double* vn = a.V + (int64_t)(j + 1) * a.ld;
+    int64_t i = r0 + threadIdx.x;
+    if constexpr (!WS) {
+      for (; i + step < r1; i += 2 * step) {
+        double wa = w[i], wb = w[i + step];
+        gm_row_update2(V, a.ld, i, i + step, ncols, hs, wa, wb);
+        wa *= inv;
+        wb *= inv;
+        vn[i] = wa;
+        vn[i + step] = wb;
+        if (a.v32) {
+          if (i < a.m) a.v32[i] = (float)wa;
+          if (i + step < a.m) a.v32[i + step] = (float)wb;
+        }
+      }
+    }
+    for (; i < r1; i += step) {
+      const double v = (WS ? project(i, w[i]) : gm_row_update(V, a.ld, w[i], i, ncols, hs)) * inv;
+      vn[i] = v;
+      if (a.v32 && i < a.m) a.v32[i] = (float)v;
+    }
+  }
+  if constexpr (SUMS == 1) cl_sync();   // no CTA leaves while another may read its partials
+}
+
+// ---------------------------------------------------------------- MGS Arnoldi step
+// Modified Gram-Schmidt in blocks of eight columns for long vectors, one cooperative launch
+// per FGMRES iteration.  Sweep k = 0 .. K over the CTA's rows (K blocks): subtract the
+// projection on block k-1 (its coefficients are the previous sweep's grid sums) and accumulate
+// the eight products of block k with w (sweep K: ||w||^2); each sweep ends in one grid sum.
+// 2(j+1) FP64 FMAs per row, the least any Gram-Schmidt form needs for j+1 projections
+// (classical Gram-Schmidt with its second pass takes 4(j+1)); GB300's FP64 rate, not HBM,
+// bounds the step at m in the millions.  The columns of a block are orthonormal to working
+// accuracy, so projecting on eight at once loses no more than one after the other does,
+// with an eighth of the grid sums (about 4 us each: column by column, m = 1e6, j = 20 took 222
+// us a step, 152 us now, 67 us of them FMAs).
+// Each row stays with one thread from sweep to sweep, so w needs no barrier between
+// sweeps.  WS: the CTA's rows of w live in shared memory for the whole step (one CTA per
+// SM; rows of [r; x] up to 152 x ~27,000), so a sweep reads only block k from HBM and block k-1
+// again (from L2 while it fits); otherwise w is read and written in global memory every sweep.
+constexpr int kMgsThreads = 512;
+constexpr int kMgsStaticSmem = 16384; // bound on the kernels' static shared memory
+
+// The grid sums of eight values: each CTA's part[c * ldd + block] (one fresh set of columns per
+// sweep, so a CTA that has moved on disturbs no one still reading), added by a warp per column
+// in block order in every CTA.  False if the wait ran out.
+__device__ __forceinline__ bool gm_grid_sum8(const double* part, int ldd, int cols, unsigned long long* ctr,
+                                             int plus_one, int* err, uint64_t wait_ns, double* out) {
+  if (!gm_rendezvous(ctr, plus_one, err, wait_ns)) return false;
+  const int nb = (int)gridDim.x, warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  if (warp < cols) {
+    const double* col = part + (int64_t)warp * ldd;
+    double t0 = 0.0, t1 = 0.0;
+    int q = lane;
+    for (; q + 32 < nb; q += 64) {
+      t0 += __ldcg(col + q);
+      t1 += __ldcg(col + q + 32);
+    }
+    if (q < nb) t0 += __ldcg(col + q);
+    const double t = warp_sum(t0 + t1);
+    if (lane == 0) out[warp] = t;
+  }
+  __syncthreads();
+  return true;
+}
+
+template <typename TAZ, bool WS>
+__global__ void __launch_bounds__(kMgsThreads, WS ? 1 : 2) gm_mgs_kernel(const GmStepArgs<TAZ> a) {
   if (a.st->done) return;   // uniform: read before any grid sync
   extern __shared__ double wsm[];   // WS: w[r0 .. r1)
-  __shared__ double hs[130];
-  __shared__ double red[NT];
+  __shared__ double hs[144];        // the coefficients; zero past ncols up to a whole block
+  __shared__ double red[kMgsThreads / 32][kGmGroup + 1];
   __shared__ double hcol[130];
+  __shared__ double pre[260];
+  __shared__ double wn2_s, inv_s;
   const int j = a.st->j, ncols = j + 1;
-  const int nb = gridDim.x, b = blockIdx.x;
+  const int K = (ncols + kGmGroup - 1) / kGmGroup;
+  const int nb = gridDim.x - 1, b = blockIdx.x;   // the last CTA: the Givens step, no rows
+  const bool giv = b == nb;
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int64_t chunk = (a.len + nb - 1) / nb;
-  const int64_t r0 = (int64_t)b * chunk, r1 = min(a.len, r0 + chunk);
-  constexpr int64_t step = NT;
+  const int64_t r0 = min(a.len, (int64_t)b * chunk), r1 = giv ? r0 : min(a.len, r0 + chunk);
+  constexpr int64_t step = kMgsThreads;
   double* w = WS ? wsm - r0 : a.w;   // indexed by the row
   const double* wg = a.w;
   const double* V = a.V;
   const double* vj = V + (int64_t)j * a.ld;
   const double al = a.alpha;
   const bool form = a.az != nullptr;
-  for (int c = 0; c <= ncols; ++c) {
-    const double* vp = V + (int64_t)(c > 0 ? c - 1 : 0) * a.ld;
-    const double* vc = V + (int64_t)(c < ncols ? c : 0) * a.ld;
-    const double hp = c > 0 ? hs[c - 1] : 0.0;
-    double t = 0.0;
-    int64_t i = r0 + threadIdx.x;
-    for (; i + (kMgsUnroll - 1) * step < r1; i += kMgsUnroll * step) {
-      double wv[kMgsUnroll], pv[kMgsUnroll], cv[kMgsUnroll];
+  if (giv) gm_finish_prefetch(a.st, a.cs, a.sn, a.g, pre);
+  for (int k = 0; k <= K; ++k) {
+    // block k - 1 subtracted, block k accumulated; columns past ncols are read as column 0 with a
+    // zero coefficient, and their sums dropped
+    const double* vp[kGmGroup];
+    const double* vc[kGmGroup];
+    double hp[kGmGroup], t[kGmGroup];
 #pragma unroll
-      for (int u = 0; u < kMgsUnroll; ++u) {
-        const int64_t q = i + u * step;
-        if (c == 0) wv[u] = (form && q < a.m) ? fma(al, vj[q], (double)a.az[q]) : wg[q];
-        else wv[u] = w[q];
-        pv[u] = c > 0 ? vp[q] : 0.0;
-        cv[u] = c < ncols ? vc[q] : 0.0;
+    for (int q = 0; q < kGmGroup; ++q) {
+      const int cp = (k - 1) * kGmGroup + q, cc = k * kGmGroup + q;
+      vp[q] = V + (k > 0 && cp < ncols ? (int64_t)cp * a.ld : 0);
+      vc[q] = V + (cc < ncols ? (int64_t)cc * a.ld : 0);
+      hp[q] = (k > 0 && cp < ncols) ? -hs[cp] : 0.0;
+      t[q] = 0.0;
+    }
+    const int np = k > 0 ? min(kGmGroup, ncols - (k - 1) * kGmGroup) : 0;
+    const int nc = k < K ? min(kGmGroup, ncols - k * kGmGroup) : 0;
+    for (int64_t i = r0 + threadIdx.x; i < r1; i += step) {
+      double pv[kGmGroup], cv[kGmGroup];
+      double wi = k > 0 ? w[i] : ((form && i < a.m) ? fma(al, vj[i], (double)a.az[i]) : wg[i]);
+#pragma unroll
+      for (int q = 0; q < kGmGroup; ++q) pv[q] = q < np ? vp[q][i] : 0.0;
+#pragma unroll
+      for (int q = 0; q < kGmGroup; ++q) cv[q] = q < nc ? vc[q][i] : 0.0;
+      if (k > 0) {
+        double p0 = 0.0, p1 = 0.0;
+#pragma unroll
+        for (int q = 0; q < kGmGroup; q += 2) {
+          if (q < np) p0 = fma(hp[q], pv[q], p0);
+          if (q + 1 < np) p1 = fma(hp[q + 1], pv[q + 1], p1);
+        }
+        wi += p0 + p1;
       }
+      if (WS || k > 0 || (form && i < a.m)) w[i] = wi;
+      if (k < K) {
 #pragma unroll
-      for (int u = 0; u < kMgsUnroll; ++u) {
-        const int64_t q = i + u * step;
-        if (c > 0) wv[u] = fma(-hp, pv[u], wv[u]);
-        if (WS || c > 0 || (form && q < a.m)) w[q] = wv[u];
-        t = fma(c < ncols ? cv[u] : wv[u], wv[u], t);
+        for (int q = 0; q < kGmGroup; ++q)
+          if (q < nc) t[q] = fma(cv[q], wi, t[q]);
+      } else {
+        t[0] = fma(wi, wi, t[0]);
       }
     }
-    for (; i < r1; i += step) {
-      double wi = c > 0 ? w[i] : ((form && i < a.m) ? fma(al, vj[i], (double)a.az[i]) : wg[i]);
-      if (c > 0) wi = fma(-hp, vp[i], wi);
-      if (WS || c > 0 || (form && i < a.m)) w[i] = wi;
-      t = fma(c < ncols ? vc[i] : wi, wi, t);
-    }
-    // block sum in a fixed order: NT / 32 values per lane of warp 0 (four interleaved
-    // chains), then the warp
-    red[threadIdx.x] = t;
+    const double tot = warp_reduce8(t);
+    __syncthreads();   // the previous sweep's red has been read
+    if ((lane & 3) == 0) red[warp][(lane >> 2) & 7] = tot;
     __syncthreads();
-    double mine = 0.0;
-    if (threadIdx.x < 32) {
-      static_assert(NT % 128 == 0, "four chains of NT / 128 values");
-      const double* rl = red + threadIdx.x * (NT / 32);
-      double q0 = 0.0, q1 = 0.0, q2 = 0.0, q3 = 0.0;
+    const int cols = k < K ? nc : 1;
+    double* part = a.Dp + (int64_t)k * kGmGroup * a.ldd;
+    if (threadIdx.x < cols) {
+      double s0 = 0.0, s1 = 0.0;
 #pragma unroll
-      for (int k = 0; k < NT / 32; k += 4) {
-        q0 += rl[k];
-        q1 += rl[k + 1];
-        q2 += rl[k + 2];
-        q3 += rl[k + 3];
+      for (int q = 0; q < kMgsThreads / 32; q += 2) {
+        s0 += red[q][threadIdx.x];
+        s1 += red[q + 1][threadIdx.x];
       }
-      mine = warp_sum((q0 + q1) + (q2 + q3));
+      part[(int64_t)threadIdx.x * a.ldd + b] = s0 + s1;
     }
-    if (!gm_grid_sum_ctr(a.Dp + (int64_t)c * a.ldd, a.seq, a.expire, mine, a.err, a.wait_ns, hs + c)) {
+    if (!gm_grid_sum8(part, a.ldd, cols, a.seq, a.expire, a.err, a.wait_ns, k < K ? hs + k * kGmGroup : &wn2_s)) {
       if (threadIdx.x == 0) a.st->done = 1;   // later launches of the batch skip; the host reads err
       return;
     }
   }
-  double hn2 = hs[ncols];
+  double hn2 = wn2_s;
   if (!(hn2 > 0.0)) hn2 = 0.0;
-  if (b == 0) {
+  if (giv) {
     for (int c = threadIdx.x; c < ncols; c += blockDim.x) hcol[c] = hs[c];
     if (threadIdx.x == 0) a.st->reorth = 0;
-  }
-  const double inv = hn2 > 0.0 ? 1.0 / sqrt(hn2) : 0.0;
-  double* vn = a.V + (int64_t)(j + 1) * a.ld;
-  __syncthreads();   // block 0: hcol is complete; every thread's last w is visible to the CTA
-  if (b == 0 && threadIdx.x < 32) {
-    gm_finish_warp(hn2, a.st, hcol, a.H, a.ldh, a.cs, a.sn, a.g);
+    __syncthreads();
+    if (threadIdx.x < 32) gm_finish_warp(hn2, j, pre, a.st, hcol, a.H, a.ldh, a.cs, a.sn, a.g);
     return;
   }
-  const int64_t nstep = (b == 0) ? NT - 32 : NT;
-  for (int64_t i = r0 + threadIdx.x - ((b == 0) ? 32 : 0); i < r1; i += nstep) {
+  if (threadIdx.x < 32) {   // one warp: an FP64 reciprocal root
+    const double v = hn2 > 0.0 ? rsqrt(hn2) : 0.0;
+    if (threadIdx.x == 0) inv_s = v;
+  }
+  double* vn = a.V + (int64_t)(j + 1) * a.ld;
+  __syncthreads();   // every thread's last w is visible to the CTA
+  const double inv = inv_s;
+  for (int64_t i = r0 + threadIdx.x; i < r1; i += step) {
     const double v = w[i] * inv;
     vn[i] = v;
     if (a.v32 && i < a.m) a.v32[i] = (float)v;
@@ -1470,58 +1685,80 @@ __global__ void __launch_bounds__(NT, WS ? 1 : 2) gm_mgs_kernel(const GmStepArgs
 template <typename TAZ>
 cudaError_t launch_gm_step(double* V, int64_t ld, double* w, int64_t len, int64_t m, const TAZ* az,
                            GmState* st, int maxc, double* Dp, double* sq, double* hsum, double* H, int ldh,
-                           double* cs, double* sn, double* g, float* v32, unsigned* bar, int* err,
+                           double* cs, double* sn, double* g, float* v32, int* err,
                            int num_sms, cudaStream_t s, uint64_t wait_ns, double alpha, int gs,
                            unsigned long long* seq, int expire) {
   static_assert(sizeof(GmStepArgs<TAZ>) < 4096, "kernel parameter block");
-  if (maxc > 128 || gs < 0 || gs > 2 || (gs > 0 && seq == nullptr)) return cudaErrorInvalidValue;
+  if (maxc > 128 || gs < 0 || gs > 2 || seq == nullptr) return cudaErrorInvalidValue;
   const bool mgs = gs > 0;
-  // MGS keeps w in shared memory when one CTA per SM holds its rows (unless gs = 2)
-  const int64_t ws_rows = (len + num_sms - 1) / num_sms;
+  // Classical: up to kGmClusterRows rows one cluster of sixteen CTAs; up to 2^20 a cooperative
+  // launch of at most one CTA per 64 rows and SM; both with w and the basis columns that fit in
+  // shared memory.  From 2^20 rows on (opts.arnoldi = 1) two CTAs per SM with w in global memory
+  // (more loads in flight).  Modified: one per SM with w in shared memory where one CTA's rows
+  // fit (unless gs = 2), else as classical; the last CTA of every form has no rows.
+  const bool lng = len >= ((int64_t)1 << 20);
+  const bool cl = !mgs && len <= kGmClusterRows && !expire;   // the timeout test needs the grid's bounded wait
+  const int64_t cgs_blk = cl ? kGmCluster : std::max<int64_t>(2, std::min<int64_t>(num_sms, (len + 63) / 64 + 1));
+  const int64_t row_ctas = mgs ? std::max(1, num_sms - 1) : cgs_blk - 1;
+  const int64_t ws_rows = (len + row_ctas - 1) / row_ctas;
   const size_t ws_bytes = (size_t)ws_rows * 8;
-  const bool ws = gs == 1 && ws_bytes + kMgsStaticSmem <= 227 * 1024;
-  auto kern = !mgs ? gm_step_kernel<TAZ>
-                   : (ws ? gm_mgs_kernel<TAZ, true, kMgsThreadsWs> : gm_mgs_kernel<TAZ, false, kMgsThreads>);
-  const int threads = !mgs ? kGmThreads : (ws ? kMgsThreadsWs : kMgsThreads);
-  const size_t dyn = ws ? ws_bytes : 0;
+  const size_t room = 227 * 1024 - kMgsStaticSmem;
+  const bool ws = mgs ? (gs == 1 && ws_bytes <= room) : !lng;
+  auto kern = !mgs ? (cl ? gm_step_kernel<TAZ, true, 1> : (ws ? gm_step_kernel<TAZ, true, 0> : gm_step_kernel<TAZ, false, 0>))
+                   : (ws ? gm_mgs_kernel<TAZ, true> : gm_mgs_kernel<TAZ, false>);
+  const int threads = mgs ? kMgsThreads : kGmThreads;
+  // staged columns (classical): all maxc, or as many as fit beside w
+  const size_t col_bytes = (size_t)(ws_rows | 1) * 8;
+  const int slab = (!mgs && ws && ws_bytes < room) ? (int)std::min<int64_t>(maxc, (int64_t)((room - ws_bytes) / col_bytes)) : 0;
+  const size_t dyn = ws ? ws_bytes + col_bytes * (size_t)slab : 0;
   if (ws) {
-    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)dyn);
+    cudaError_t e = allow_dyn_smem(kern, dyn);
+    if (e != cudaSuccess) return e;
+  }
+  if (cl) {
+    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
     if (e != cudaSuccess) return e;
   }
   int occ = 0;
   cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, kern, threads, dyn);
   if (e != cudaSuccess) return e;
   if (occ < 1) return cudaErrorInvalidConfiguration;
-  // co-resident CTAs (cooperative launch): two per SM for long vectors (more loads in
-  // flight), one per SM otherwise (fewer partials to sum); shared w: one per SM
-  const int nblk = ws ? num_sms : num_sms * ((occ >= 2 && len >= ((int64_t)1 << 20)) ? 2 : 1);
-  GmStepArgs<TAZ> a{V, ld, len, m, w, az, st, maxc, 0, Dp, sq, hsum, H, cs, sn, g, v32, bar, err};
+  const int nblk = ws ? (int)row_ctas + 1 : std::max(2, num_sms * (occ >= 2 && lng ? 2 : 1));
+  GmStepArgs<TAZ> a{V, ld, len, m, w, az, st, maxc, 0, Dp, sq, hsum, H, cs, sn, g, v32, err};
   a.ldh = ldh;
-  a.ldd = 2 * num_sms;   // the caller's Dp holds (maxc + 1) x 2 num_sms values
+  a.ldd = 4 * num_sms;   // the caller's Dp holds (maxc + 17) x 4 num_sms values
   a.wait_ns = wait_ns > 0 ? wait_ns : kWaitLimitNs;
   a.alpha = alpha;
   a.seq = seq;
   a.expire = expire;
+  a.slab = slab;
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3((unsigned)nblk);
   cfg.blockDim = dim3(threads);
   cfg.dynamicSmemBytes = dyn;
   cfg.stream = s;
   cudaLaunchAttribute attr[1];
-  attr[0].id = cudaLaunchAttributeCooperative;
-  attr[0].val.cooperative = 1;
+  if (cl) {
+    attr[0].id = cudaLaunchAttributeClusterDimension;
+    attr[0].val.clusterDim.x = kGmCluster;
+    attr[0].val.clusterDim.y = 1;
+    attr[0].val.clusterDim.z = 1;
+  } else {
+    attr[0].id = cudaLaunchAttributeCooperative;
+    attr[0].val.cooperative = 1;
+  }
   cfg.attrs = attr;
   cfg.numAttrs = 1;
   return cudaLaunchKernelEx(&cfg, kern, a);
 }
 template cudaError_t launch_gm_step<float>(double*, int64_t, double*, int64_t, int64_t, const float*, GmState*,
                                            int, double*, double*, double*, double*, int, double*, double*,
-                                           double*, float*, unsigned*, int*, int, cudaStream_t, uint64_t,
-                                           double, int, unsigned long long*, int);
+                                           double*, float*, int*, int, cudaStream_t, uint64_t, double, int,
+                                           unsigned long long*, int);
 template cudaError_t launch_gm_step<double>(double*, int64_t, double*, int64_t, int64_t, const double*,
                                             GmState*, int, double*, double*, double*, double*, int, double*,
-                                            double*, double*, float*, unsigned*, int*, int, cudaStream_t,
-                                            uint64_t, double, int, unsigned long long*, int);
+                                            double*, double*, float*, int*, int, cudaStream_t, uint64_t, double,
+                                            int, unsigned long long*, int);
 
 // y = H[:k,:k]^-1 g[:k]  (k = st->j): one warp, column-oriented back substitution
 __global__ void gm_solve_kernel(const GmState* st, const double* H, int ldh, const double* g, double* y) {
@@ -1883,7 +2120,7 @@ __global__ void __launch_bounds__(kGmThreads)
     }
     __syncthreads();
   }
-  gm_partials(g.V, g.ld, g.w, r0, r1, ncols, g.Dp, (int)nb, red, blk);
+  gm_partials(g.V, g.ld, nullptr, 0, 0, g.w, r0, r1, ncols, g.Dp, (int)nb, red, blk);
 }
 
 // phase B / B' (one CTA per problem): column sums of the partials in block order, then the
@@ -1965,10 +2202,14 @@ __global__ void __launch_bounds__(kGmThreads)
   const int64_t blk = (int64_t)blockIdx.x - start[pr], nb = (int64_t)start[pr + 1] - start[pr];
   const int64_t len = g.m + g.n, chunk = (len + nb - 1) / nb;
   const int64_t r0 = blk * chunk, r1 = min(len, r0 + chunk);
-  for (int c = threadIdx.x; c <= ncols; c += blockDim.x) hs[c] = hsrc[c == ncols ? ncols + 1 : c];
+  for (int c = threadIdx.x; c < ncols; c += blockDim.x) hs[c] = hsrc[c];
+  if (threadIdx.x < 32) {   // one warp: an FP64 root and quotient
+    const double hn2 = hsrc[ncols + 1];
+    const double v = hn2 > 0.0 ? rsqrt(hn2) : 0.0;
+    if (threadIdx.x == 0) hs[ncols] = v;
+  }
   __syncthreads();
-  const double hn2 = hs[ncols];
-  const double inv = hn2 > 0.0 ? 1.0 / sqrt(hn2) : 0.0;
+  const double inv = hs[ncols];
   double* vn = g.V + (int64_t)(j + 1) * g.ld;
   const int64_t step = blockDim.x;
   int64_t i = r0 + threadIdx.x;
@@ -1994,15 +2235,17 @@ __global__ void __launch_bounds__(kGmThreads)
 // phase D (one warp per problem): Hessenberg column h (+ h2), Givens step, j + 1
 __global__ void garn_finish_kernel(const GGm* __restrict__ tab) {
   __shared__ double hcol[130];
+  __shared__ double pre[260];
   const GGm& g = tab[blockIdx.x];
   GmState* st = g.st;
   if (st->done) return;
   const int j = st->j, ncols = j + 1;
   const int re = st->reorth;
+  gm_finish_prefetch(st, g.cs, g.sn, g.g, pre);
   for (int c = threadIdx.x; c < ncols; c += 32) hcol[c] = re ? g.hs1[c] + g.hs2[c] : g.hs1[c];
   __syncwarp();
   const double hn2 = re ? g.hs2[ncols + 1] : g.hs1[ncols + 1];
-  gm_finish_warp(hn2, st, hcol, g.H, g.ldh, g.cs, g.sn, g.g);
+  gm_finish_warp(hn2, j, pre, st, hcol, g.H, g.ldh, g.cs, g.sn, g.g);
 }
 
 cudaError_t launch_grouped_arnoldi(const GGm* tab, const int* start, int64_t ctas, int nprob, cudaStream_t st) {
