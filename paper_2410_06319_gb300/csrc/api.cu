@@ -132,8 +132,7 @@ void stage_qr(Ctx& c, const double* Y, double* R, double* xs, RCopies* rc) {
     StageTimer t(c.h, ST_QR);
     const bool f64 = (c.up == LSQ_F64);
     void* work = ws(c.h, "qrwork", (size_t)c.s * (c.n + 1) * (f64 ? 8 : 4));
-    // norms, diag(R), then either tau and T (blocked QR) or n + 1 column flags (FP64 QR)
-    const size_t tail = std::max<size_t>((32 + 32 * 32) * 8, (size_t)(c.n + 1) * 4);
+    const size_t tail = qr_aux_tail(c.n);
     double* aux = static_cast<double*>(ws(c.h, "qraux", (2 * c.n + 8) * 8 + tail));
     unsigned* bar = static_cast<unsigned*>(ws(c.h, "qrbar", 64));
     double* cvec = static_cast<double*>(ws(c.h, "qrc", c.n * 8));

@@ -370,399 +370,325 @@ __global__ void qr_finalize_kernel(const T* __restrict__ W, int64_t s, int64_t n
   qr_finalize_body<T>(W, s, n, diagR, R, c, blockIdx.x);
 }
 
-// ------------------------------------------------------------ blocked variant
-// Panels of NB columns: one CTA factors the panel W[p:s, p:p+kb] in shared
-// memory (column Householder steps with block reductions), leaving the vectors
-// v_j below the diagonal, tau_j = 1 / (alpha (alpha + |x_1|)) and the compact-WY
-// factor T (Q_panel = I - V T V^T, T upper triangular, Schreiber-Van Loan
-// recurrence); then every trailing column y (including the right-hand side) is
-// updated as y -= V (T^T (V^T y)) by a grid of CTAs.  Same reflectors and the
-// same arithmetic order per column as the unblocked kernel, blocked.
-constexpr int kQrPanelThreads = 1024;
-
-template <typename T>
-__device__ __forceinline__ T block_sum_1024(T v, T* red) {
-  v = warp_sum(v);
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  __syncthreads();
-  if (lane == 0) red[warp] = v;
-  __syncthreads();
-  T t = (threadIdx.x < 32) ? red[threadIdx.x] : T(0);
-  if (warp == 0) t = warp_sum(t);
-  if (threadIdx.x == 0) red[32] = t;
-  __syncthreads();
-  return red[32];
-}
-
-// Block-wide sums of NB per-thread values (entries c < lo are ignored).
-template <typename T, int NB>
-__device__ __forceinline__ void block_vsum(T (&pd)[NB], int lo, T (*red)[NB + 1], T* out) {
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+// ------------------------------------------------------------ register-block variant
+// Column blocks of NB, one CTA per block, the block's columns in registers for the whole
+// factorization (thread t holds rows t, t + NT, ... of every column); one launch.  CTA q waits
+// for the flag of each block P < q in turn, applies its reflectors (compact WY,
+// with V, tau and the Gram entries read from global memory), then factors its own block,
+// publishes V (below the diagonal of W, R above) and those, and raises its flag; so the next block's chain runs while
+// the others still apply.  Column Householder steps take one block reduction each: the dot
+// products x_j^T x_c of the pivot column with every column of the block at once (c = j is the
+// squared norm), from which v = x_j + sgn alpha e_j gives v^T x_c = x_j^T x_c + sgn alpha x_c[j].  The
+// registers rotate by one column a step, so the step is a loop and not NB copies of its
+// code; after NB steps every column is back in its place, and the products with finished
+// columns are the Gram entries g_lj = v_l^T v_j.  With them the block's reflectors apply as
+// w_a = tau_a (v_a^T x - sum_{l < a} g_la w_l), x -= V w (the triangular system of the compact-WY
+// form; forming T itself inside the column steps took half of a step's time).
+//
+// Bound by the chain of the blocks (flag, V from L2, two products, NB column steps).  Panels
+// of 16 columns on one CTA of 1024 threads, unrolled over the columns (each launch fetched
+// some 10,000 instructions once), two reductions a column, and a launch for each trailing
+// update took 1.93 ms at s = 2000, n = 500 in FP32, and a grid barrier per column 1.9 ms at s =
+// 748, n = 187 in FP64; now 0.95 and 1.34 ms.  NB: 8 in FP32; 4 in FP64, where a CTA's arithmetic (two FMAs a
+// clock an SM) weighs as much as the latency.
+template <typename T, int N>
+__device__ __forceinline__ T warp_reduce_scatter(T (&v)[N], int lane) {
+  // after the call lane l holds the warp total of v[l / (32 / N)]
+  static_assert(N == 4 || N == 8 || N == 16 || N == 32, "a power of two up to the warp");
+  int cnt = N;
 #pragma unroll
-  for (int c = 0; c < NB; ++c) {
-    if (c >= lo) {
-      const T v = warp_sum(pd[c]);
-      if (lane == 0) red[warp][c] = v;
-    }
-  }
-  __syncthreads();
-  if (threadIdx.x < NB && (int)threadIdx.x >= lo) {
-    T t = 0;
-    for (int w = 0; w < (int)(blockDim.x >> 5); ++w) t += red[w][threadIdx.x];
-    out[threadIdx.x] = t;
-  }
-  __syncthreads();
-}
-
-template <typename T, int NB>
-__global__ void __launch_bounds__(kQrPanelThreads)
-    qr_panel_kernel(T* __restrict__ W, int64_t s, int64_t p, int kb, double* __restrict__ diagR,
-                    T* __restrict__ tau, T* __restrict__ Tm) {
-  extern __shared__ __align__(16) unsigned char qp_smem[];
-  T* P = reinterpret_cast<T*>(qp_smem);        // [kb][len] panel, column-major
-  __shared__ T red[32][NB + 1];
-  __shared__ T wv[NB];
-  __shared__ T tj_s;
-  const int64_t len = s - p;
-  for (int c = 0; c < kb; ++c)
-    for (int64_t t = threadIdx.x; t < len; t += blockDim.x) P[c * len + t] = W[(p + c) * s + p + t];
-  __syncthreads();
-  for (int j = 0; j < kb; ++j) {
-    T* x = P + j * len;
-    T pd[NB];
+  for (int o = 16; o >= 1; o >>= 1) {
+    if (cnt > 1) {
+      const bool upper = (lane & o) != 0;
+      const int half = cnt / 2;
 #pragma unroll
-    for (int c = 0; c < NB; ++c) pd[c] = 0;
-    for (int64_t t = j + threadIdx.x; t < len; t += blockDim.x) pd[0] += x[t] * x[t];
-    block_vsum<T, NB>(pd, 0, red, wv);
-    if (threadIdx.x == 0) {
-      const T alpha = sqrt(wv[0]);
-      const T x0 = x[j];
-      const T sgn = (x0 >= T(0)) ? T(1) : T(-1);
-      const T tj = (alpha > T(0)) ? T(1) / (alpha * (alpha + fabs(x0))) : T(0);
-      x[j] = x0 + sgn * alpha;               // v_j lives in rows j.. of panel column j
-      diagR[p + j] = (double)(-sgn * alpha);
-      tau[j] = tj;
-      tj_s = tj;
-    }
-    __syncthreads();
-    const T tj = tj_s;
-    // w_c = tau_j v_j^T y_c for all remaining panel columns at once, then y_c -= w_c v_j
-#pragma unroll
-    for (int c = 0; c < NB; ++c) pd[c] = 0;
-    for (int64_t t = j + threadIdx.x; t < len; t += blockDim.x) {
-      const T xv = x[t];
-#pragma unroll
-      for (int c = 0; c < NB; ++c)
-        if (c > j && c < kb) pd[c] += xv * P[c * len + t];
-    }
-    block_vsum<T, NB>(pd, j + 1, red, wv);
-    for (int64_t t = j + threadIdx.x; t < len; t += blockDim.x) {
-      const T xv = x[t];
-#pragma unroll
-      for (int c = 0; c < NB; ++c)
-        if (c > j && c < kb) P[c * len + t] -= (wv[c] * tj) * xv;
-    }
-    __syncthreads();
-  }
-  // T factor: T_jj = tau_j ; T[0:j, j] = -tau_j T[0:j, 0:j] (V[:, 0:j]^T v_j)
-  if ((int)threadIdx.x < kb) Tm[threadIdx.x * NB + threadIdx.x] = tau[threadIdx.x];
-  __syncthreads();
-  for (int j = 1; j < kb; ++j) {
-    const T* vj = P + j * len;
-    T pd[NB];
-#pragma unroll
-    for (int c = 0; c < NB; ++c) pd[c] = 0;
-    for (int64_t t = j + threadIdx.x; t < len; t += blockDim.x) {   // v_j is zero above row j
-      const T vv = vj[t];
-#pragma unroll
-      for (int c = 0; c < NB; ++c)
-        if (c < j) pd[c] += P[c * len + t] * vv;
-    }
-    block_vsum<T, NB>(pd, 0, red, wv);
-    if (threadIdx.x == 0) {
-      const T tjj = tau[j];
-      for (int i = 0; i < j; ++i) {
-        T acc = 0;
-        for (int l = i; l < j; ++l) acc += Tm[l * NB + i] * wv[l];
-        Tm[j * NB + i] = -tjj * acc;
+      for (int t = 0; t < N / 2; ++t) {
+        if (t < half) {
+          const T send = upper ? v[t] : v[t + half];
+          const T keep = upper ? v[t + half] : v[t];
+          v[t] = keep + __shfl_xor_sync(0xffffffffu, send, o);
+        }
       }
+      cnt = half;
+    } else {
+      v[0] += __shfl_xor_sync(0xffffffffu, v[0], o);
     }
-    __syncthreads();
   }
-  if (threadIdx.x < NB) {
-    const int j = threadIdx.x;
-    for (int i = 0; i < NB; ++i)
-      if (i > j || j >= kb) Tm[j * NB + i] = T(0);
-  }
-  // write back: rows 0..j-1 of column j are R entries, rows j.. hold v_j
-  for (int c = 0; c < kb; ++c)
-    for (int64_t t = threadIdx.x; t < len; t += blockDim.x) W[(p + c) * s + p + t] = P[c * len + t];
+  return v[0];
 }
 
-// y -= V T^T V^T y for trailing columns c in [p + kb, n] (column n = Omega b).
-template <typename T, int NB>
-__global__ void __launch_bounds__(256)
-    qr_trail_kernel(T* __restrict__ W, int64_t s, int64_t n, int64_t p, int kb,
-                    const T* __restrict__ Tm) {
-  __shared__ T red[NB][9];
-  __shared__ T wv[NB];
-  const int64_t len = s - p;
-  const T* V = W + p * s + p;                  // column j of V at V + j * s (rows j.. are valid)
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  for (int64_t col = p + kb + blockIdx.x; col <= n; col += gridDim.x) {
-    T* y = W + col * s + p;
-    // w = V^T y (v_j has an implicit zero above row j)
-    for (int j = warp; j < kb; j += 8) {
-      const T* vj = V + (int64_t)j * s;
-      T pd = 0;
-      for (int64_t t = j + lane; t < len; t += 32) pd += vj[t] * y[t];
-      pd = warp_sum(pd);
-      if (lane == 0) wv[j] = pd;
-    }
-    __syncthreads();
-    // w2 = T^T w (T upper triangular): w2_j = sum_{i <= j} T(i, j) w_i
-    if (threadIdx.x < kb) {
-      const int j = threadIdx.x;
-      T acc = 0;
-      for (int i = 0; i <= j; ++i) acc += Tm[j * NB + i] * wv[i];
-      red[j][0] = acc;
-    }
-    __syncthreads();
-    for (int64_t t = threadIdx.x; t < len; t += blockDim.x) {
-      T acc = 0;
-      const int jmax = (t < kb - 1) ? (int)t : kb - 1;
-      for (int j = 0; j <= jmax; ++j) acc += V[(int64_t)j * s + t] * red[j][0];
-      y[t] -= acc;
-    }
-    __syncthreads();
-  }
-}
-
-// ------------------------------------------------------ register-panel variant
-// The same blocked algorithm with the panel held in registers: 1024 threads,
-// thread t owns panel rows t, t + 1024, ... (RPT rows), NB columns each.  A
-// column costs two block reductions: ||x_j|| (with x_j[j] broadcast through
-// shared memory so every thread forms alpha, tau and v_jj itself), then one
-// reduction of v_j^T x_c for all other panel columns at once -- c > j are the
-// update coefficients, c < j are the Gram entries v_c^T v_j from which warp 0
-// extends the compact-WY factor T (T[0:j, j] = -tau_j T[0:j, 0:j] G[0:j, j]).
-// Within a warp the NB partial sums are reduced by recursive halving (NB
-// shuffles instead of 5 NB).
-constexpr int kQrRegThreads = 1024;
-
-// After the call lane l holds the warp total of v[l >> 1] (N = 16).
-template <int N>
-__device__ __forceinline__ float warp_reduce_scatter(float (&v)[N], int lane) {
-  static_assert(N == 16, "16 values over 32 lanes");
-#pragma unroll
-  for (int o = 16, cnt = N; o >= 2; o >>= 1, cnt >>= 1) {
-    const bool upper = (lane & o) != 0;
-    const int half = cnt / 2;
-#pragma unroll
-    for (int t = 0; t < N / 2; ++t) {
-      if (t < half) {
-        const float send = upper ? v[t] : v[t + half];
-        const float keep = upper ? v[t + half] : v[t];
-        v[t] = keep + __shfl_xor_sync(0xffffffffu, send, o);
-      }
-    }
-  }
-  return v[0] + __shfl_xor_sync(0xffffffffu, v[0], 1);
-}
-
-template <int NB, int RPT>
-__global__ void __launch_bounds__(kQrRegThreads, 1)
-    qr_panel_reg_kernel(float* __restrict__ W, int64_t s, int64_t p, int kb, double* __restrict__ diagR,
-                        float* __restrict__ tau, float* __restrict__ Tm) {
-  __shared__ float redA[32];
-  __shared__ float redB[32][NB];
-  __shared__ float Ts[NB * NB];
-  __shared__ float x0s;
+template <typename T, int NB, int NT, int RPT>
+__global__ void __launch_bounds__(NT, 1)
+    qr_block_kernel(T* __restrict__ W, int64_t s, int64_t n, double* __restrict__ diagR, T* __restrict__ Tg,
+                    unsigned* __restrict__ flag, int* err) {
+  constexpr int NW = NT / 32;
+  constexpr int HA = NB * NB > 32 ? 32 / NB : NB;   // reflectors at a time in the products
+  constexpr int NH = NB / HA;
+  constexpr int LB = NT <= 256 ? NB : NB / 2;       // columns of V loaded at a time
+  __shared__ T red[2][NW][NB * NB];
+  // Gs: g_la at l + a * NB (l < a), tau_a at a + a * NB
+  __shared__ T Ws[NB * NB], Gs[NB * NB], prow[2][NB];
+  __shared__ T sc[2], rd[NB];
+  extern __shared__ __align__(16) unsigned char qb_smem[];
+  T* Vs = reinterpret_cast<T*>(qb_smem);   // [NB][RPT * NT]: the block of reflectors being applied
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  const int64_t len = s - p;
-  float x[RPT][NB];
+  const int q = (int)blockIdx.x;
+  const int64_t c0 = (int64_t)q * NB;
+  const int ncol = (int)min((int64_t)NB, n + 1 - c0);
+  T x[RPT][NB];
 #pragma unroll
   for (int i = 0; i < RPT; ++i) {
-    const int64_t r = tid + (int64_t)i * kQrRegThreads;
+    const int64_t r = tid + (int64_t)i * NT;
 #pragma unroll
-    for (int c = 0; c < NB; ++c) x[i][c] = (r < len && c < kb) ? W[(p + c) * s + p + r] : 0.0f;
+    for (int c = 0; c < NB; ++c) x[i][c] = (r < s && c < ncol) ? W[(c0 + c) * s + r] : T(0);
   }
-#pragma unroll
-  for (int j = 0; j < NB; ++j) {
-    if (j < kb) {
-      // ---- alpha = ||x_j[j:]||, tau_j, v_jj
-      float part = 0.0f;
-#pragma unroll
-      for (int i = 0; i < RPT; ++i) {
-        const int64_t r = tid + (int64_t)i * kQrRegThreads;
-        if (r >= j) part += x[i][j] * x[i][j];
-      }
-      part = warp_sum(part);
-      if (lane == 0) redA[warp] = part;
-      if (tid == j) x0s = x[0][j];
-      __syncthreads();
-      const float n2 = warp_sum(redA[lane]);
-      const float x0 = x0s;
-      const float alpha = sqrtf(n2);
-      const float sgn = (x0 >= 0.0f) ? 1.0f : -1.0f;
-      const float tj = (alpha > 0.0f) ? 1.0f / (alpha * (alpha + fabsf(x0))) : 0.0f;
-      if (tid == j) {
-        x[0][j] = x0 + sgn * alpha;          // v_j lives in rows j.. of panel column j
-        diagR[p + j] = (double)(-sgn * alpha);
-        tau[j] = tj;
-      }
-      // ---- d_c = v_j^T x_c for every other column (rows >= j; v_j is zero above)
-      float pw[NB];
-#pragma unroll
-      for (int c = 0; c < NB; ++c) {
-        pw[c] = 0.0f;
-        if (c != j) {
-#pragma unroll
-          for (int i = 0; i < RPT; ++i) {
-            const int64_t r = tid + (int64_t)i * kQrRegThreads;
-            if (r >= j) pw[c] += x[i][j] * x[i][c];
+  // ---- reflectors of the earlier blocks
+  for (int P = 0; P < q; ++P) {
+    int ok = 1;
+    if (tid == 0) {
+      const unsigned* fp = flag + P;
+      auto raised = [&]() {
+        unsigned f;
+        asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(f) : "l"(fp) : "memory");
+        return f != 0u;
+      };
+      if (!raised()) {
+        const uint64_t t0 = globaltimer_ns();
+        while (!raised()) {
+          if (globaltimer_ns() - t0 > kWaitLimitNs) {
+            set_error(err, DEV_TIMEOUT_GRID);
+            ok = 0;
+            break;
           }
         }
       }
-      const float wsum = warp_reduce_scatter<NB>(pw, lane);
-      if ((lane & 1) == 0) redB[warp][lane >> 1] = wsum;
-      __syncthreads();
-      float d = 0.0f;
-      if (lane < NB) {
-#pragma unroll 8
-        for (int w = 0; w < 32; ++w) d += redB[w][lane];
-      }
-      // ---- trailing panel columns: x_c -= tau_j d_c v_j
+    }
+    if (__syncthreads_and(ok) == 0) return;
+    const int64_t p = (int64_t)P * NB;
+    if (tid < NB * NB) Gs[tid] = __ldcg(Tg + (int64_t)P * NB * NB + tid);
+    // a thread stages its own rows of V (from L2; zero above each diagonal entry), all loads in
+    // flight together where the registers allow it
+    const T* V = W + p * s;
 #pragma unroll
-      for (int c = j + 1; c < NB; ++c) {
-        const float coef = tj * __shfl_sync(0xffffffffu, d, c);
+    for (int a0 = 0; a0 < NB; a0 += LB) {
+      T v[LB][RPT];
+#pragma unroll
+      for (int a = 0; a < LB; ++a)
 #pragma unroll
         for (int i = 0; i < RPT; ++i) {
-          const int64_t r = tid + (int64_t)i * kQrRegThreads;
-          if (r >= j) x[i][c] -= coef * x[i][j];
+          const int64_t r = tid + (int64_t)i * NT;
+          v[a][i] = (r >= p + a0 + a && r < s) ? __ldcg(V + (a0 + a) * s + r) : T(0);
         }
-      }
-      // ---- T column j (warp 0): T_jj = tau_j, T[a, j] = -tau_j sum_{l=a}^{j-1} T[a, l] G[l, j]
-      if (warp == 0) {
-        float tcol = 0.0f;
 #pragma unroll
-        for (int l = 0; l < j; ++l) {
-          const float g = __shfl_sync(0xffffffffu, d, l);
-          if (lane <= l) tcol += Ts[lane + l * NB] * g;
+      for (int a = 0; a < LB; ++a)
+#pragma unroll
+        for (int i = 0; i < RPT; ++i) Vs[(a0 + a) * (RPT * NT) + tid + i * NT] = v[a][i];
+    }
+#pragma unroll
+    for (int h = 0; h < NH; ++h) {
+      T acc[HA * NB];
+#pragma unroll
+      for (int e = 0; e < HA * NB; ++e) acc[e] = T(0);
+#pragma unroll
+      for (int i = 0; i < RPT; ++i) {
+        {   // V is zero outside its rows
+          const int r = tid + i * NT;
+          T v[HA];
+#pragma unroll
+          for (int a = 0; a < HA; ++a) v[a] = Vs[(h * HA + a) * (RPT * NT) + r];
+#pragma unroll
+          for (int a = 0; a < HA; ++a)
+#pragma unroll
+            for (int c = 0; c < NB; ++c) acc[a * NB + c] = fma(v[a], x[i][c], acc[a * NB + c]);
         }
-        if (lane < j) Ts[lane + j * NB] = -tj * tcol;
-        if (lane == j) Ts[j + j * NB] = tj;
-        if (lane > j && lane < NB) Ts[lane + j * NB] = 0.0f;
-        __syncwarp();
       }
-    } else if (warp == 0 && lane < NB) {
-      Ts[lane + j * NB] = 0.0f;
+      const T w = warp_reduce_scatter<T, HA * NB>(acc, lane);
+      constexpr int LP = 32 / (HA * NB);   // lanes per value
+      if (lane % LP == 0) red[0][warp][h * HA * NB + lane / LP] = w;
+    }
+    __syncthreads();
+    if (tid < NB * NB) {
+      T w = T(0);
+#pragma unroll
+      for (int k = 0; k < NW; ++k) w += red[0][k][tid];
+      Ws[tid] = w;
+    }
+    __syncthreads();
+    if (tid < NB) {   // column tid of the block: forward substitution
+      T w[NB];
+#pragma unroll
+      for (int a = 0; a < NB; ++a) {
+        T u = Ws[a * NB + tid];
+#pragma unroll
+        for (int l = 0; l < a; ++l) u = fma(-Gs[l + a * NB], w[l], u);
+        w[a] = Gs[a + a * NB] * u;
+        Ws[a * NB + tid] = w[a];
+      }
+    }
+    __syncthreads();
+#pragma unroll
+    for (int h = 0; h < NH; ++h) {
+      T w2[HA * NB];
+#pragma unroll
+      for (int e = 0; e < HA * NB; ++e) w2[e] = Ws[h * HA * NB + e];
+#pragma unroll
+      for (int i = 0; i < RPT; ++i) {
+        {   // V is zero outside its rows
+          const int r = tid + i * NT;
+          T v[HA];
+#pragma unroll
+          for (int a = 0; a < HA; ++a) v[a] = Vs[(h * HA + a) * (RPT * NT) + r];
+#pragma unroll
+          for (int c = 0; c < NB; ++c) {
+            T y = x[i][c];
+#pragma unroll
+            for (int a = 0; a < HA; ++a) y = fma(-v[a], w2[a * NB + c], y);
+            x[i][c] = y;
+          }
+        }
+      }
     }
   }
+  // ---- factor the own block
+  const int kb = (int)max((int64_t)0, min((int64_t)NB, n - c0));
+  if (tid < NB * NB) Gs[tid] = T(0);
   __syncthreads();
-  for (int e = tid; e < NB * NB; e += blockDim.x) Tm[e] = Ts[e];
+#pragma unroll 1
+  for (int j = 0; j < NB; ++j) {
+    // x[.][c] holds column (j + c) % NB of the block
+    if (j < kb) {
+      const int pr = (int)c0 + j;
+      const int par = j & 1;
+      T d[NB];
+#pragma unroll
+      for (int c = 0; c < NB; ++c) d[c] = T(0);
+#pragma unroll
+      for (int i = 0; i < RPT; ++i) {
+        const int r = tid + i * NT;
+        const T xj = r >= pr ? x[i][0] : T(0);
+#pragma unroll
+        for (int c = 0; c < NB; ++c) d[c] = fma(xj, x[i][c], d[c]);
+        if (r == pr) {
+#pragma unroll
+          for (int c = 0; c < NB; ++c) prow[par][c] = x[i][c];
+        }
+      }
+      const T dw = warp_reduce_scatter<T, NB>(d, lane);
+      constexpr int LP = 32 / NB;
+      if (lane % LP == 0) red[par][warp][lane / LP] = dw;
+      __syncthreads();
+      T tot = T(0), sa, tau;   // lane l: value l % NB, summed over a share of the warps, then over the shares
+      const T x0 = prow[par][0];
+      auto totals = [&]() {
+#pragma unroll
+        for (int k = 0; k < (NW + LP - 1) / LP; ++k)
+          if (lane / NB + k * LP < NW) tot += red[par][lane / NB + k * LP][lane % NB];
+#pragma unroll
+        for (int o = NB; o < 32; o <<= 1) tot += __shfl_xor_sync(0xffffffffu, tot, o);
+      };
+      auto scalars = [&](T n2) {
+        const T alpha = sqrt(n2);
+        sa = (x0 >= T(0)) ? alpha : -alpha;
+        tau = (alpha > T(0)) ? T(1) / (alpha * (alpha + fabs(x0))) : T(0);
+      };
+      if constexpr (sizeof(T) == 4) {
+        totals();
+        scalars(__shfl_sync(0xffffffffu, tot, 0));
+      } else {   // FP64 is scarce: the sums, the root and the quotient in one warp
+        if (warp == 0) {
+          totals();
+          scalars(__shfl_sync(0xffffffffu, tot, 0));
+          if (lane < NB) red[par][0][lane] = tot;   // every warp's share has been read by this warp alone
+          if (lane == 0) {
+            sc[0] = sa;
+            sc[1] = tau;
+          }
+        }
+        __syncthreads();
+        tot = red[par][0][lane % NB];
+        sa = sc[0];
+        tau = sc[1];
+      }
+      T v[RPT];   // v_j: zero above the pivot row, where x keeps R
+#pragma unroll
+      for (int i = 0; i < RPT; ++i) {
+        const int r = tid + i * NT;
+        if (r == pr) x[i][0] += sa;
+        v[i] = r >= pr ? x[i][0] : T(0);
+        // the column is final: R above the pivot row, v_j from it down
+        if (r < s) W[(int64_t)pr * s + r] = x[i][0];
+      }
+#pragma unroll
+      for (int c = 1; c < NB; ++c) {
+        const T vx = fma(sa, prow[par][c], __shfl_sync(0xffffffffu, tot, c));
+        if (c < NB - j) {
+          const T coef = tau * vx;
+#pragma unroll
+          for (int i = 0; i < RPT; ++i) x[i][c] = fma(-coef, v[i], x[i][c]);
+        }
+      }
+      if (warp == 0) {   // lane c >= NB - j: v_l^T v_j of the finished column l = c - (NB - j)
+        if (lane < NB && lane >= NB - j) Gs[lane - (NB - j) + j * NB] = fma(sa, prow[par][lane], tot);
+        if (lane == 0) {
+          Gs[j + j * NB] = tau;
+          rd[j] = -sa;
+        }
+      }
+    }
+#pragma unroll
+    for (int i = 0; i < RPT; ++i) {
+      const T first = x[i][0];
+#pragma unroll
+      for (int c = 0; c + 1 < NB; ++c) x[i][c] = x[i][c + 1];
+      x[i][NB - 1] = first;
+    }
+  }
+  // ---- the right-hand side's column, if the block holds it; tau and the Gram entries; the flag
 #pragma unroll
   for (int i = 0; i < RPT; ++i) {
-    const int64_t r = tid + (int64_t)i * kQrRegThreads;
+    const int64_t r = tid + (int64_t)i * NT;
 #pragma unroll
     for (int c = 0; c < NB; ++c)
-      if (r < len && c < kb) W[(p + c) * s + p + r] = x[i][c];
-  }
-}
-
-// y -= V T^T V^T y for the trailing columns (V in registers, one block
-// reduction per column; reduction buffers alternate so one barrier suffices).
-template <int NB, int RPT>
-__global__ void __launch_bounds__(kQrRegThreads, 1)
-    qr_trail_reg_kernel(float* __restrict__ W, int64_t s, int64_t n, int64_t p, int kb,
-                        const float* __restrict__ Tm) {
-  __shared__ float red[2][32][NB];
-  __shared__ float Ts[NB * NB];
-  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  const int64_t len = s - p;
-  for (int e = tid; e < NB * NB; e += blockDim.x) Ts[e] = Tm[e];
-  float V[RPT][NB];
-#pragma unroll
-  for (int i = 0; i < RPT; ++i) {
-    const int64_t r = tid + (int64_t)i * kQrRegThreads;
-#pragma unroll
-    for (int c = 0; c < NB; ++c) V[i][c] = (r < len && c < kb && r >= c) ? W[(p + c) * s + p + r] : 0.0f;
+      if (c >= kb && c < ncol && r < s) W[(c0 + c) * s + r] = x[i][c];
   }
   __syncthreads();
-  int par = 0;
-  for (int64_t col = p + kb + blockIdx.x; col <= n; col += gridDim.x, par ^= 1) {
-    float* y = W + col * s + p;
-    float yv[RPT];
-#pragma unroll
-    for (int i = 0; i < RPT; ++i) {
-      const int64_t r = tid + (int64_t)i * kQrRegThreads;
-      yv[i] = (r < len) ? y[r] : 0.0f;
-    }
-    float pw[NB];
-#pragma unroll
-    for (int c = 0; c < NB; ++c) {
-      pw[c] = 0.0f;
-#pragma unroll
-      for (int i = 0; i < RPT; ++i) pw[c] += V[i][c] * yv[i];
-    }
-    const float wsum = warp_reduce_scatter<NB>(pw, lane);
-    if ((lane & 1) == 0) red[par][warp][lane >> 1] = wsum;
-    __syncthreads();
-    float w = 0.0f;
-    if (lane < NB) {
-#pragma unroll 8
-      for (int q = 0; q < 32; ++q) w += red[par][q][lane];
-    }
-    // w2 = T^T w: w2_c = sum_{a <= c} T[a, c] w_a
-    float w2 = 0.0f;
-#pragma unroll
-    for (int a = 0; a < NB; ++a) {
-      const float wa = __shfl_sync(0xffffffffu, w, a);
-      if (lane < NB && a <= lane) w2 += Ts[a + lane * NB] * wa;
-    }
-#pragma unroll
-    for (int c = 0; c < NB; ++c) {
-      const float w2c = __shfl_sync(0xffffffffu, w2, c);
-#pragma unroll
-      for (int i = 0; i < RPT; ++i) yv[i] -= V[i][c] * w2c;
-    }
-#pragma unroll
-    for (int i = 0; i < RPT; ++i) {
-      const int64_t r = tid + (int64_t)i * kQrRegThreads;
-      if (r < len) y[r] = yv[i];
-    }
-  }
+  if (tid < NB * NB) Tg[(int64_t)q * NB * NB + tid] = Gs[tid];
+  if (tid < kb) diagR[c0 + tid] = (double)rd[tid];
+  __threadfence();
+  __syncthreads();
+  if (tid == 0) atomicExch(flag + q, 1u);
 }
 
-template <int RPT>
-static cudaError_t run_qr_reg(const double* Y, int64_t s, int64_t n, float* W, double* aux, double* R,
-                              double* c, int num_sms, cudaStream_t st) {
-  constexpr int NB = 16;
+// The register-block form: `aux` as launch_qr's, block factors and flags behind diag(R).
+template <typename T, int NB, int NT, int RPT>
+static cudaError_t run_qr_block(const double* Y, int64_t s, int64_t n, T* W, double* aux, double* R, double* c,
+                                int* err, cudaStream_t st) {
   const int64_t total = s * (n + 1);
-  convert_y_kernel<float><<<(unsigned)((total + 255) / 256), 256, 0, st>>>(Y, W, total);
+  const unsigned nblk = (unsigned)((n + 1 + NB - 1) / NB);
+  convert_y_kernel<T><<<(unsigned)((total + 255) / 256), 256, 0, st>>>(Y, W, total);
   cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) return e;
   double* diagR = aux + n;
-  float* tau = reinterpret_cast<float*>(aux + 2 * n + 8);
-  float* Tm = tau + NB;
-  for (int64_t p = 0; p < n; p += NB) {
-    const int kb = (int)std::min<int64_t>(NB, n - p);
-    qr_panel_reg_kernel<NB, RPT><<<1, kQrRegThreads, 0, st>>>(W, s, p, kb, diagR, tau, Tm);
-    const int64_t ncols = n + 1 - (p + kb);
-    if (ncols > 0) {
-      const unsigned grid = (unsigned)std::min<int64_t>(ncols, (int64_t)num_sms);
-      qr_trail_reg_kernel<NB, RPT><<<grid, kQrRegThreads, 0, st>>>(W, s, n, p, kb, Tm);
-    }
-  }
-  e = cudaGetLastError();
+  T* Tg = reinterpret_cast<T*>(aux + 2 * n + 8);
+  unsigned* flag = reinterpret_cast<unsigned*>(Tg + (size_t)nblk * NB * NB);
+  e = cudaMemsetAsync(flag, 0, nblk * sizeof(unsigned), st);
   if (e != cudaSuccess) return e;
-  qr_finalize_kernel<float><<<(unsigned)n, 256, 0, st>>>(W, s, n, diagR, R, c);
+  T* Wp = W;
+  int64_t sp = s, np = n;
+  void* args[] = {&Wp, &sp, &np, &diagR, &Tg, &flag, &err};
+  const size_t smem = (size_t)NB * RPT * NT * sizeof(T);
+  e = allow_dyn_smem(qr_block_kernel<T, NB, NT, RPT>, smem);
+  if (e != cudaSuccess) return e;
+  e = cudaLaunchCooperativeKernel((const void*)qr_block_kernel<T, NB, NT, RPT>, dim3(nblk), dim3(NT), args, smem, st);
+  if (e != cudaSuccess) return e;
+  qr_finalize_kernel<T><<<(unsigned)n, 256, 0, st>>>(W, s, n, diagR, R, c);
   return cudaGetLastError();
 }
 
-template <typename T>
-static bool qr_blocked_fits(int64_t s, int nb) {
-  return (size_t)s * nb * sizeof(T) <= 200 * 1024;
+// Bytes of the region behind diag(R) in aux that a factorization of n columns may use.
+size_t qr_aux_tail(int64_t n) {
+  const size_t f32 = (size_t)((n + 1 + 7) / 8) * (64 * 4 + 4), f64 = (size_t)((n + 1 + 3) / 4) * (16 * 8 + 4);
+  return std::max(std::max(f32, f64), (size_t)(n + 1) * 4);   // or n + 1 column flags (qr64s_kernel)
 }
 
 template <typename T>
@@ -835,46 +761,26 @@ static cudaError_t run_qr64(const double* Y, int64_t s, int64_t n, double* W, do
   return cudaGetLastError();
 }
 
-template <typename T, int NB>
-static cudaError_t run_qr_blocked(const double* Y, int64_t s, int64_t n, T* W, double* aux, double* R,
-                                  double* c, int num_sms, cudaStream_t st) {
-  const int64_t total = s * (n + 1);
-  convert_y_kernel<T><<<(unsigned)((total + 255) / 256), 256, 0, st>>>(Y, W, total);
-  cudaError_t e = cudaGetLastError();
-  if (e != cudaSuccess) return e;
-  double* diagR = aux + n;
-  T* tau = reinterpret_cast<T*>(aux + 2 * n + 8);
-  T* Tm = tau + NB;
-  const size_t smem = (size_t)s * NB * sizeof(T);
-  e = allow_dyn_smem(qr_panel_kernel<T, NB>, smem);
-  if (e != cudaSuccess) return e;
-  for (int64_t p = 0; p < n; p += NB) {
-    const int kb = (int)std::min<int64_t>(NB, n - p);
-    qr_panel_kernel<T, NB><<<1, kQrPanelThreads, (size_t)(s - p) * kb * sizeof(T), st>>>(W, s, p, kb, diagR,
-                                                                                        tau, Tm);
-    const int64_t ncols = n + 1 - (p + kb);
-    if (ncols > 0) {
-      const unsigned grid = (unsigned)std::min<int64_t>(ncols, 4 * (int64_t)num_sms);
-      qr_trail_kernel<T, NB><<<grid, 256, 0, st>>>(W, s, n, p, kb, Tm);
-    }
-  }
-  e = cudaGetLastError();
-  if (e != cudaSuccess) return e;
-  qr_finalize_kernel<T><<<(unsigned)n, 256, 0, st>>>(W, s, n, diagR, R, c);
-  return cudaGetLastError();
-}
-
 cudaError_t launch_qr(bool fp64, const double* Y, int64_t s, int64_t n, void* work, double* aux,
                       unsigned* bar, double* R, double* c, int* err, int num_sms, cudaStream_t st) {
-  if (!fp64 && s <= kQrRegThreads)
-    return run_qr_reg<1>(Y, s, n, static_cast<float*>(work), aux, R, c, num_sms, st);
-  if (!fp64 && s <= 2 * kQrRegThreads)
-    return run_qr_reg<2>(Y, s, n, static_cast<float*>(work), aux, R, c, num_sms, st);
-  if (!fp64 && qr_blocked_fits<float>(s, 24))
-    return run_qr_blocked<float, 24>(Y, s, n, static_cast<float*>(work), aux, R, c, num_sms, st);
-  if (fp64)
-    return run_qr64(Y, s, n, static_cast<double*>(work), aux, bar, R, c, err, num_sms, st);
-  return run_qr<float>(Y, s, n, static_cast<float*>(work), aux, bar, R, c, err, num_sms, st);
+  if (!fp64) {
+    float* W = static_cast<float*>(work);
+    // one CTA per block of eight columns, all co-resident (n <= 1024: at most 129), rows of a
+    // column in at most eight registers of each thread
+    if ((n + 1 + 7) / 8 <= num_sms) {
+      if (s <= 512) return run_qr_block<float, 8, 256, 2>(Y, s, n, W, aux, R, c, err, st);
+      if (s <= 1024) return run_qr_block<float, 8, 256, 4>(Y, s, n, W, aux, R, c, err, st);
+      if (s <= 2048) return run_qr_block<float, 8, 256, 8>(Y, s, n, W, aux, R, c, err, st);
+      if (s <= 4096) return run_qr_block<float, 8, 512, 8>(Y, s, n, W, aux, R, c, err, st);
+    }
+    return run_qr<float>(Y, s, n, W, aux, bar, R, c, err, num_sms, st);
+  }
+  double* W = static_cast<double*>(work);
+  if ((n + 1 + 3) / 4 <= num_sms) {
+    if (s <= 512) return run_qr_block<double, 4, 128, 4>(Y, s, n, W, aux, R, c, err, st);
+    if (s <= 1024) return run_qr_block<double, 4, 128, 8>(Y, s, n, W, aux, R, c, err, st);
+  }
+  return run_qr64(Y, s, n, W, aux, bar, R, c, err, num_sms, st);
 }
 
 
@@ -883,6 +789,20 @@ cudaError_t launch_qr(bool fp64, const double* Y, int64_t s, int64_t n, void* wo
 // memory, whole trailing columns per warp (lanes over rows, one warp sum per dot
 // product); the warp that updates column k+1 also sums its squares below the diagonal
 // for the next step's norm.  W (s x (n + 1), ld = s) stays in global memory.
+template <typename T>
+__device__ __forceinline__ T block_sum_1024(T v, T* red) {
+  v = warp_sum(v);
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  __syncthreads();
+  if (lane == 0) red[warp] = v;
+  __syncthreads();
+  T t = (threadIdx.x < 32) ? red[threadIdx.x] : T(0);
+  if (warp == 0) t = warp_sum(t);
+  if (threadIdx.x == 0) red[32] = t;
+  __syncthreads();
+  return red[32];
+}
+
 template <typename T>
 __global__ void __launch_bounds__(1024) grouped_qr_kernel(const GQr<T>* __restrict__ tab) {
   const GQr<T>& g = tab[blockIdx.x];

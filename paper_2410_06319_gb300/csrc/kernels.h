@@ -147,7 +147,8 @@ cudaError_t launch_sparse_sketch(const SparsePlan& p, const double* A, int64_t l
 // ---------------------------------------------------------------- QR
 // Householder QR of Y (s x (n+1), col-major) in FP32 (fp64 = false) or FP64.
 // Outputs R (FP64, n x n col-major, diag >= 0) and c (FP64, n).  `work` holds
-// s*(n+1) elements of the arithmetic type; `aux` >= (2n + 8) doubles.
+// s*(n+1) elements of the arithmetic type; `aux` >= (2n + 8) doubles and qr_aux_tail(n) bytes.
+size_t qr_aux_tail(int64_t n);
 cudaError_t launch_qr(bool fp64, const double* Y, int64_t s, int64_t n, void* work, double* aux,
                       unsigned* bar, double* R, double* c, int* err, int num_sms, cudaStream_t st);
 
