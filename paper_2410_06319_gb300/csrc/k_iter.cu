@@ -177,6 +177,150 @@ __device__ __forceinline__ void pass_body(PassArgs<T> p, int64_t blk, int64_t nb
   }
 }
 
+// The FP32 pass of the grouped launches (LSQR, FGMRES; rows of at most 64 float4): the body
+// above with each warp's rows streamed through a ring of its own in shared memory, kRingPairs
+// row pairs ahead with asynchronous copies.  A lane copies and reads the same pieces, so the
+// ring needs no barrier.  Two rows a warp in flight, as the register form has, left HBM waiting
+// (381 us an FGMRES pass and 480 us an LSQR pass over 1.8 GB); now 294 and 410 (with 3 or 4 pairs
+// fewer CTAs fit an SM: 2 % and 1 % more for a batch of 32).
+constexpr int kRingPairs = 2;
+template <int MODE>
+__device__ __forceinline__ void pass_ring_body(PassArgs<float> p, int64_t blk, int64_t nblk) {
+  static_assert(MODE == PM_LSQR || MODE == PM_FGM, "FP32 passes");
+  if (p.done && *p.done) return;
+  if (p.jp) {
+    const int64_t j = *p.jp;
+    p.x += j * p.xstr;
+    p.v += j * p.vstr;
+  }
+  constexpr int VPL = 2, VW = 4;
+  extern __shared__ __align__(16) unsigned char pass_smem[];
+  __shared__ double sqred[8];
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int64_t gw = blk * 8 + warp, tw = nblk * 8;
+  const int width = p.nv * VW;
+  float* ring = reinterpret_cast<float*>(pass_smem) + (size_t)warp * 2 * kRingPairs * width;
+  float xv[VPL][VW], acc[VPL][VW];
+#pragma unroll
+  for (int v = 0; v < VPL; ++v) {
+    const int idx = lane + 32 * v;
+    if (idx < p.nv) {
+      load_vec<float, VW>(p.x + (int64_t)idx * VW, xv[v], false);
+    } else {
+      for (int k = 0; k < VW; ++k) xv[v][k] = 0.0f;
+    }
+#pragma unroll
+    for (int k = 0; k < VW; ++k) acc[v][k] = 0.0f;
+  }
+  const float cu = (MODE == PM_LSQR) ? (float)((p.cu_ptr ? *p.cu_ptr : 1.0) * p.cu_mul) : 0.0f;
+  // rows i and i + tw into slots 2 s and 2 s + 1
+  auto fetch = [&](int64_t i, int s) {
+#pragma unroll
+    for (int e = 0; e < 2; ++e) {
+      const int64_t row = i + e * tw;
+      if (row < p.m) {
+#pragma unroll
+        for (int v = 0; v < VPL; ++v) {
+          const int idx = lane + 32 * v;
+          if (idx < p.nv)
+            asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(
+                             smem_u32(ring + (size_t)(2 * s + e) * width + idx * VW)),
+                         "l"(p.A + row * p.lda + (int64_t)idx * VW)
+                         : "memory");
+        }
+      }
+    }
+    asm volatile("cp.async.commit_group;" ::: "memory");
+  };
+#pragma unroll
+  for (int s = 0; s < kRingPairs; ++s) fetch(gw + 2 * s * tw, s);
+  double sqacc = 0.0;   // as in the body above
+  float qkeep = 0.0f;
+  int qn = 0, slot = 0;
+  for (int64_t i = gw; i < p.m; i += 2 * tw) {
+    const int64_t i2 = i + tw;
+    const bool has2 = i2 < p.m;
+    const float s0 = MODE == PM_LSQR ? p.uin[i] : p.v[i];
+    const float s1 = has2 ? (MODE == PM_LSQR ? p.uin[i2] : p.v[i2]) : 0.0f;
+    asm volatile("cp.async.wait_group %0;" ::"n"(kRingPairs - 1) : "memory");
+    float a[VPL][VW], a2[VPL][VW];
+    float d = 0.0f, d2 = 0.0f;
+#pragma unroll
+    for (int v = 0; v < VPL; ++v) {
+      const int idx = lane + 32 * v;
+      if (idx < p.nv) {
+        load_vec<float, VW>(ring + (size_t)(2 * slot) * width + idx * VW, a[v], false);
+      } else {
+        for (int k = 0; k < VW; ++k) a[v][k] = 0.0f;
+      }
+      if (has2 && idx < p.nv) {
+        load_vec<float, VW>(ring + (size_t)(2 * slot + 1) * width + idx * VW, a2[v], false);
+      } else {
+        for (int k = 0; k < VW; ++k) a2[v][k] = 0.0f;
+      }
+#pragma unroll
+      for (int k = 0; k < VW; ++k) {
+        d = fma(a[v][k], xv[v][k], d);
+        d2 = fma(a2[v][k], xv[v][k], d2);
+      }
+    }
+    warp_sum2(d, d2);   // the sums need every piece read: the slot can be filled again
+    fetch(i + 2 * kRingPairs * tw, slot);
+    slot = slot + 1 == kRingPairs ? 0 : slot + 1;
+    float c1, c2;
+    if constexpr (MODE == PM_LSQR) {
+      c1 = d + cu * s0;
+      c2 = has2 ? d2 + cu * s1 : 0.0f;
+      if (lane == 0) p.uout[i] = c1;
+      if (lane == qn) qkeep = c1;
+      if (has2) {
+        if (lane == 0) p.uout[i2] = c2;
+        if (lane == qn + 1) qkeep = c2;
+      }
+      qn += 2;
+      if (qn == 32) {
+        sqacc = fma((double)qkeep, (double)qkeep, sqacc);
+        qkeep = 0.0f;
+        qn = 0;
+      }
+    } else {
+      c1 = s0;
+      c2 = s1;
+      if (lane == 0) p.az[i] = d;
+      if (lane == 0 && has2) p.az[i2] = d2;
+    }
+#pragma unroll
+    for (int v = 0; v < VPL; ++v)
+#pragma unroll
+      for (int k = 0; k < VW; ++k) acc[v][k] = fma(c1, a[v][k], fma(c2, a2[v][k], acc[v][k]));
+  }
+  asm volatile("cp.async.wait_all;" ::: "memory");
+  // CTA reduction of acc (fixed order over warps), each warp's sums in its own ring
+#pragma unroll
+  for (int v = 0; v < VPL; ++v) {
+    const int idx = lane + 32 * v;
+    if (idx < p.nv)
+      for (int k = 0; k < VW; ++k) ring[idx * VW + k] = acc[v][k];
+  }
+  if (MODE == PM_LSQR) {
+    sqacc = warp_sum(fma((double)qkeep, (double)qkeep, sqacc));
+    if (lane == 0) sqred[warp] = sqacc;
+  }
+  __syncthreads();
+  const float* all = reinterpret_cast<const float*>(pass_smem);
+  for (int c = threadIdx.x; c < p.n; c += blockDim.x) {
+    float s = 0.0f;
+#pragma unroll
+    for (int w = 0; w < 8; ++w) s += all[(size_t)w * 2 * kRingPairs * width + c];
+    p.Pblk[blk * p.n + c] = s;
+  }
+  if (MODE == PM_LSQR && threadIdx.x == 0) {
+    double s = 0.0;
+    for (int w = 0; w < 8; ++w) s += sqred[w];
+    p.sq[blk] = s;
+  }
+}
+
 template <typename T, int VW, int VPL, int MODE>
 __global__ void __launch_bounds__(256) pass_kernel(PassArgs<T> p) {
   pass_body<T, VW, VPL, MODE>(p, blockIdx.x, gridDim.x);
@@ -1902,7 +2046,10 @@ __global__ void __launch_bounds__(256)
                         int64_t items) {
   for (int64_t it = blockIdx.x; it < items; it += gridDim.x) {
     const int pr = group_of(start, nprob, it);
-    pass_body<T, VW, VPL, MODE>(tab[pr], it - start[pr], (int64_t)start[pr + 1] - start[pr]);
+    if constexpr (sizeof(T) == 4)
+      pass_ring_body<MODE>(tab[pr], it - start[pr], (int64_t)start[pr + 1] - start[pr]);
+    else
+      pass_body<T, VW, VPL, MODE>(tab[pr], it - start[pr], (int64_t)start[pr + 1] - start[pr]);
     __syncthreads();   // the item's shared-memory reduction is read before the next item writes it
   }
 }
@@ -1920,6 +2067,7 @@ cudaError_t launch_grouped_pass(int mode, int vw, int vpl, const PassArgs<T>* ta
     return cudaGetLastError();
   };
   if constexpr (sizeof(T) == 4) {
+    smem *= 2 * kRingPairs;   // the caller's size is 8 warps x one row
     if (vw != 4 || vpl != 2) return cudaErrorInvalidValue;
     if (mode == PM_LSQR) return go(grouped_pass_kernel<float, 4, 2, PM_LSQR>);
     if (mode == PM_FGM) return go(grouped_pass_kernel<float, 4, 2, PM_FGM>);
