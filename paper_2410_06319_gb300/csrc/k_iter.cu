@@ -71,6 +71,7 @@ __device__ __forceinline__ void pass_body(PassArgs<T> p, int64_t blk, int64_t nb
   __shared__ double sqred[8];
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int64_t gw = blk * 8 + warp, tw = nblk * 8;
+  const int nvl = (p.nv + 31) >> 5;   // vectors a lane uses (the grouped launches have one VPL for all problems)
   T xv[VPL][VW], acc[VPL][VW];
 #pragma unroll
   for (int v = 0; v < VPL; ++v) {
@@ -85,7 +86,11 @@ __device__ __forceinline__ void pass_body(PassArgs<T> p, int64_t blk, int64_t nb
   }
   T cu = T(0);
   if (MODE == PM_LSQR) cu = (T)((p.cu_ptr ? *p.cu_ptr : 1.0) * p.cu_mul);
+  // q^2 is summed in FP64, 32 rows at a time: lane l keeps the q of the rows l, l + 32, ... of the
+  // warp's sequence (an FP64 product per row is one more serial step of 67 cycles)
   double sqacc = 0.0;
+  T qkeep = T(0);
+  int qn = 0;
   for (int64_t i = gw; i < p.m; i += 2 * tw) {
     const int64_t i2 = i + tw;
     const bool has2 = i2 < p.m;
@@ -109,27 +114,30 @@ __device__ __forceinline__ void pass_body(PassArgs<T> p, int64_t blk, int64_t nb
     T d = 0, d2 = 0;
 #pragma unroll
     for (int v = 0; v < VPL; ++v)
+      if (sizeof(T) == 4 || VPL >= 16 || v < nvl)   // FP64 instructions are what an FP64 pass costs
 #pragma unroll
-      for (int k = 0; k < VW; ++k) {
-        d = fma(a[v][k], xv[v][k], d);
-        d2 = fma(a2[v][k], xv[v][k], d2);
-      }
+        for (int k = 0; k < VW; ++k) {
+          d = fma(a[v][k], xv[v][k], d);
+          d2 = fma(a2[v][k], xv[v][k], d2);
+        }
     warp_sum2(d, d2);
     T c1, c2 = T(0);
     if (MODE == PM_LSQR) {
       const T q = d + cu * p.uin[i];
       c1 = q;
-      if (lane == 0) {
-        p.uout[i] = q;
-        sqacc += (double)q * (double)q;
-      }
+      if (lane == 0) p.uout[i] = q;
+      if (lane == qn) qkeep = q;
       if (has2) {
         const T q2 = d2 + cu * p.uin[i2];
         c2 = q2;
-        if (lane == 0) {
-          p.uout[i2] = q2;
-          sqacc += (double)q2 * (double)q2;
-        }
+        if (lane == 0) p.uout[i2] = q2;
+        if (lane == qn + 1) qkeep = q2;
+      }
+      qn += 2;
+      if (qn == 32) {
+        sqacc = fma((double)qkeep, (double)qkeep, sqacc);
+        qkeep = T(0);
+        qn = 0;
       }
     } else if (MODE == PM_FGM) {
       c1 = p.v[i];
@@ -150,8 +158,9 @@ __device__ __forceinline__ void pass_body(PassArgs<T> p, int64_t blk, int64_t nb
     }
 #pragma unroll
     for (int v = 0; v < VPL; ++v)
+      if (sizeof(T) == 4 || VPL >= 16 || v < nvl)
 #pragma unroll
-      for (int k = 0; k < VW; ++k) acc[v][k] = fma(c1, a[v][k], fma(c2, a2[v][k], acc[v][k]));
+        for (int k = 0; k < VW; ++k) acc[v][k] = fma(c1, a[v][k], fma(c2, a2[v][k], acc[v][k]));
   }
   // CTA reduction of acc (fixed order over warps)
   const int width = p.nv * VW;
@@ -162,7 +171,10 @@ __device__ __forceinline__ void pass_body(PassArgs<T> p, int64_t blk, int64_t nb
       for (int k = 0; k < VW; ++k) red[warp * width + idx * VW + k] = acc[v][k];
     }
   }
-  if (MODE == PM_LSQR && lane == 0) sqred[warp] = sqacc;
+  if (MODE == PM_LSQR) {
+    sqacc = warp_sum(fma((double)qkeep, (double)qkeep, sqacc));
+    if (lane == 0) sqred[warp] = sqacc;
+  }
   __syncthreads();
   for (int c = threadIdx.x; c < p.n; c += blockDim.x) {
     T s = 0;
@@ -327,15 +339,22 @@ __global__ void __launch_bounds__(256) pass_kernel(PassArgs<T> p) {
 }
 
 // ------------------------------------------------------------ bulk-streamed passes
-// A producer warp streams stages of 8 consecutive rows of A into a shared-memory
-// ring with cp.async.bulk (completion on an mbarrier); eight consumer warps take
-// one row of each stage.  Each CTA owns a contiguous range of rows.  The per-row
-// scalars of the next stage are loaded one stage ahead.
+// A producer warp streams stages of 16 consecutive rows of A into a shared-memory
+// ring with cp.async.bulk (completion on an mbarrier).  FP32 (bound by HBM): sixteen consumer
+// warps take a row of each stage.  FP64 (bound by its pipe, 20 cycles an instruction of a warp
+// on the SM, 67 between two of one warp, dependent or not): eight warps take two rows, whose
+// sums share a reduction (five additions instead of ten), in one chain of FMAs; with a row a
+// warp and four interleaved chains, n = 187 took 38 us at m = 20011 (FGMRES) and n = 500
+// 274 us at m = 1e5 (residual); now 27 and 240.  Each CTA owns a contiguous range of rows.
+// The per-row scalars of the next stage are loaded one stage ahead.
 //   PM_LSQR: q = A t + cu u ; u_out = q ; P = A^T q ; sq = sum q^2
 //   PM_FGM : az = A z ; P = A^T v            (v_top + az is formed by the Arnoldi step)
 //   PM_RES : f = b - r - A x ; P = A^T (-r)
 constexpr int kBulkRows = 16;
-constexpr int kBulkThreads = (kBulkRows + 1) * 32;
+template <typename T>
+constexpr int kBulkRw = sizeof(T) == 8 ? 2 : 1;                          // rows of a warp
+template <typename T>
+constexpr int kBulkThreads = (kBulkRows / kBulkRw<T> + 1) * 32;
 
 template <typename T>
 struct BulkArgs {
@@ -362,7 +381,7 @@ struct BulkArgs {
 };
 
 template <typename T, int VW, int VPL, int MODE>
-__global__ void __launch_bounds__(kBulkThreads, 1) pass_bulk_kernel(BulkArgs<T> p) {
+__global__ void __launch_bounds__(kBulkThreads<T>, 1) pass_bulk_kernel(BulkArgs<T> p) {
   if (p.done && *p.done) return;
   if (MODE == PM_FGM && p.jp) {
     const int64_t j = *p.jp;
@@ -373,7 +392,8 @@ __global__ void __launch_bounds__(kBulkThreads, 1) pass_bulk_kernel(BulkArgs<T> 
   const uint32_t stage_bytes = (uint32_t)(kBulkRows * p.lda * sizeof(T));
   uint64_t* bars = reinterpret_cast<uint64_t*>(bulk_smem + (size_t)p.stages * stage_bytes);
   const uint32_t full0 = smem_u32(bars), empty0 = smem_u32(bars + p.stages);
-  __shared__ double sqred[kBulkRows];
+  constexpr int RW = kBulkRw<T>, CW = kBulkRows / RW;   // rows of a warp, consumer warps
+  __shared__ double sqred[CW];
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int64_t r0 = (int64_t)blockIdx.x * p.rows_per_cta;
   const int64_t r1 = min(p.m, r0 + p.rows_per_cta);
@@ -381,7 +401,7 @@ __global__ void __launch_bounds__(kBulkThreads, 1) pass_bulk_kernel(BulkArgs<T> 
   if (threadIdx.x == 0) {
     for (int k = 0; k < p.stages; ++k) {
       mbar_init(full0 + 8 * k, 1);
-      mbar_init(empty0 + 8 * k, kBulkRows);
+      mbar_init(empty0 + 8 * k, CW);
     }
     fence_barrier_init();
   }
@@ -392,7 +412,7 @@ __global__ void __launch_bounds__(kBulkThreads, 1) pass_bulk_kernel(BulkArgs<T> 
 #pragma unroll
     for (int k = 0; k < VW; ++k) acc[v][k] = T(0);
   float sqacc = 0.f;
-  if (warp == kBulkRows) {
+  if (warp == CW) {
     // ---------------- producer
     if (lane == 0) {
       const uint64_t pol = l2_policy_evict_first();   // A is read once per pass
@@ -409,7 +429,8 @@ __global__ void __launch_bounds__(kBulkThreads, 1) pass_bulk_kernel(BulkArgs<T> 
       }
     }
   } else {
-    // ---------------- consumers: warp `warp` takes row `warp` of every stage
+    // ---------------- consumers: warp `warp` takes rows RW warp .. RW warp + RW - 1 of every stage
+    const int nvl = (p.nv + 31) >> 5;   // vectors a lane uses
     T xv[VPL][VW];
 #pragma unroll
     for (int v = 0; v < VPL; ++v) {
@@ -425,74 +446,118 @@ __global__ void __launch_bounds__(kBulkThreads, 1) pass_bulk_kernel(BulkArgs<T> 
     // base + l; the next window is loaded while the current one is consumed
     // scalars in the pass precision (no FP64 conversions in the FP32 passes)
     using S = typename std::conditional<MODE == PM_RES, double, T>::type;
-    auto load_window = [&](int base, S& s0, S& s1) {
+    auto load_window = [&](int base, S (&s0)[RW], S (&s1)[RW]) {
       const int it = base + lane;
-      const int64_t row = r0 + (int64_t)it * kBulkRows + warp;
-      s0 = S(0);
-      s1 = S(0);
-      if (it < nst && row < r1) {
-        if constexpr (MODE == PM_LSQR) s0 = p.uin[row];
-        if constexpr (MODE == PM_FGM) s0 = p.v[row];
-        if constexpr (MODE == PM_RES) {
-          s0 = p.r[row];
-          s1 = p.b[row];
+#pragma unroll
+      for (int e = 0; e < RW; ++e) {
+        const int64_t row = r0 + (int64_t)it * kBulkRows + warp * RW + e;
+        s0[e] = S(0);
+        s1[e] = S(0);
+        if (it < nst && row < r1) {
+          if constexpr (MODE == PM_LSQR) s0[e] = p.uin[row];
+          if constexpr (MODE == PM_FGM) s0[e] = p.v[row];
+          if constexpr (MODE == PM_RES) {
+            s0[e] = p.r[row];
+            s1[e] = p.b[row];
+          }
         }
       }
     };
-    S w0, w1, x0n, x1n;
+    S w0[RW], w1[RW], x0n[RW], x1n[RW];
     load_window(0, w0, w1);
     load_window(32, x0n, x1n);
     for (int it = 0; it < nst; ++it) {
       if ((it & 31) == 0 && it > 0) {
-        w0 = x0n;
-        w1 = x1n;
+#pragma unroll
+        for (int e = 0; e < RW; ++e) {
+          w0[e] = x0n[e];
+          w1[e] = x1n[e];
+        }
         load_window(it + 32, x0n, x1n);
       }
-      const S c0 = __shfl_sync(0xffffffffu, w0, it & 31);
-      const S c1s = (MODE == PM_RES) ? __shfl_sync(0xffffffffu, w1, it & 31) : S(0);
+      S c0[RW], c1s[RW];
+#pragma unroll
+      for (int e = 0; e < RW; ++e) {
+        c0[e] = __shfl_sync(0xffffffffu, w0[e], it & 31);
+        c1s[e] = (MODE == PM_RES) ? __shfl_sync(0xffffffffu, w1[e], it & 31) : S(0);
+      }
       const int slot = it % p.stages;
       const uint32_t ph = (uint32_t)(it / p.stages) & 1u;
       if (!mbar_wait(full0 + 8 * slot, ph, p.err, DEV_TIMEOUT_FULL)) break;
-      const int64_t row = r0 + (int64_t)it * kBulkRows + warp;
+      const int64_t row = r0 + (int64_t)it * kBulkRows + warp * RW;
       if (row < r1) {
-        const T* srow = reinterpret_cast<const T*>(bulk_smem + (size_t)slot * stage_bytes) + warp * p.lda;
-        T a[VPL][VW];
-#pragma unroll
-        for (int v = 0; v < VPL; ++v) {
+        const bool has2 = RW == 2 && row + 1 < r1;   // a missing second row counts as zeros
+        const T* srow = reinterpret_cast<const T*>(bulk_smem + (size_t)slot * stage_bytes) + warp * RW * p.lda;
+        T a[RW == 1 ? VPL : 1][VW];   // FP32 keeps the row; FP64 (pipe-bound) reads it again for A^T
+        // vector v of row e of the warp
+        auto row_vec = [&](int e, int v, T (&o)[VW]) {
           const int idx = lane + 32 * v;
-          if (idx < p.nv) {
-            load_vec<T, VW>(srow + idx * VW, a[v], false);
+          if (idx < p.nv && (e == 0 || has2)) {
+            load_vec<T, VW>(srow + e * p.lda + idx * VW, o, false);
           } else {
-            for (int k = 0; k < VW; ++k) a[v][k] = T(0);
+            for (int k = 0; k < VW; ++k) o[k] = T(0);
           }
-        }
-        // four interleaved chains: in LSQR the row's A^T q update waits on this sum
-        T dq[4] = {T(0), T(0), T(0), T(0)};
+        };
+        T d[RW];
+        if constexpr (RW == 1) {
 #pragma unroll
-        for (int v = 0; v < VPL; ++v)
+          for (int v = 0; v < VPL; ++v) row_vec(0, v, a[v]);
+          // four interleaved chains: in LSQR the row's A^T q update waits on this sum
+          T dq[4] = {T(0), T(0), T(0), T(0)};
 #pragma unroll
-          for (int k = 0; k < VW; ++k) dq[(v * VW + k) & 3] = fma(a[v][k], xv[v][k], dq[(v * VW + k) & 3]);
-        T d = (dq[0] + dq[1]) + (dq[2] + dq[3]);
-        d = warp_sum(d);
-        T coef;
-        if (MODE == PM_LSQR) {
-          const T q = d + cu * (T)c0;
-          coef = q;
-          if (lane == 0) {
-            p.uout[row] = q;
-            sqacc = fmaf((float)q, (float)q, sqacc);
-          }
-        } else if (MODE == PM_FGM) {
-          coef = (T)c0;
-          if (lane == 0) p.az[row] = d;
+          for (int v = 0; v < VPL; ++v)
+#pragma unroll
+            for (int k = 0; k < VW; ++k)
+              dq[(v * VW + k) & 3] = fma(a[v][k], xv[v][k], dq[(v * VW + k) & 3]);
+          d[0] = warp_sum((dq[0] + dq[1]) + (dq[2] + dq[3]));
         } else {
-          coef = (T)(-c0);
-          if (lane == 0) p.f[row] = (c1s - c0) - (double)d;
+          d[0] = T(0);
+          d[RW - 1] = T(0);
+#pragma unroll
+          for (int v = 0; v < VPL; ++v)
+            if (v < nvl) {
+              T y0[VW], y1[VW];
+              row_vec(0, v, y0);
+              row_vec(1, v, y1);
+#pragma unroll
+              for (int k = 0; k < VW; ++k) {
+                d[0] = fma(y0[k], xv[v][k], d[0]);
+                d[RW - 1] = fma(y1[k], xv[v][k], d[RW - 1]);
+              }
+            }
+          warp_sum2(d[0], d[RW - 1]);
+        }
+        T coef[RW];
+#pragma unroll
+        for (int e = 0; e < RW; ++e) {
+          const bool in = e == 0 || has2;
+          if (MODE == PM_LSQR) {
+            const T q = d[e] + cu * (T)c0[e];
+            coef[e] = q;
+            if (lane == 0 && in) {
+              p.uout[row + e] = q;
+              sqacc = fmaf((float)q, (float)q, sqacc);
+            }
+          } else if (MODE == PM_FGM) {
+            coef[e] = (T)c0[e];
+            if (lane == 0 && in) p.az[row + e] = d[e];
+          } else {
+            coef[e] = (T)(-c0[e]);
+            if (lane == 0 && in) p.f[row + e] = (c1s[e] - c0[e]) - (double)d[e];
+          }
         }
 #pragma unroll
         for (int v = 0; v < VPL; ++v)
+          if constexpr (RW == 1) {
 #pragma unroll
-          for (int k = 0; k < VW; ++k) acc[v][k] = fma(coef, a[v][k], acc[v][k]);
+            for (int k = 0; k < VW; ++k) acc[v][k] = fma(coef[0], a[v][k], acc[v][k]);
+          } else if (v < nvl) {
+            T y0[VW], y1[VW];
+            row_vec(0, v, y0);
+            row_vec(1, v, y1);
+#pragma unroll
+            for (int k = 0; k < VW; ++k) acc[v][k] = fma(coef[0], y0[k], fma(coef[RW - 1], y1[k], acc[v][k]));
+          }
       }
       __syncwarp();
       if (lane == 0) mbar_arrive(empty0 + 8 * slot);
@@ -501,7 +566,7 @@ __global__ void __launch_bounds__(kBulkThreads, 1) pass_bulk_kernel(BulkArgs<T> 
   __syncthreads();   // every stage consumed: the ring is free for the reduction
   const int width = p.nv * VW;
   T* red = reinterpret_cast<T*>(bulk_smem);
-  if (warp < kBulkRows) {
+  if (warp < CW) {
 #pragma unroll
     for (int v = 0; v < VPL; ++v) {
       const int idx = lane + 32 * v;
@@ -515,12 +580,12 @@ __global__ void __launch_bounds__(kBulkThreads, 1) pass_bulk_kernel(BulkArgs<T> 
   for (int c = threadIdx.x; c < p.n; c += blockDim.x) {
     T s = 0;
 #pragma unroll
-    for (int w = 0; w < kBulkRows; ++w) s += red[w * width + c];
+    for (int w = 0; w < CW; ++w) s += red[w * width + c];
     p.Pblk[(int64_t)blockIdx.x * p.n + c] = s;
   }
   if (MODE == PM_LSQR && threadIdx.x == 0) {
     double s = 0.0;
-    for (int w = 0; w < kBulkRows; ++w) s += sqred[w];
+    for (int w = 0; w < CW; ++w) s += sqred[w];
     p.sq[blockIdx.x] = s;
   }
 }
@@ -544,7 +609,7 @@ static cudaError_t dispatch_bulk(BulkArgs<T> p, int nblk, int num_sms_unused, cu
   auto go = [&](auto kern) -> cudaError_t {
     cudaError_t e = allow_dyn_smem(kern, smem);
     if (e != cudaSuccess) return e;
-    kern<<<nblk, kBulkThreads, smem, st>>>(p);
+    kern<<<nblk, kBulkThreads<T>, smem, st>>>(p);
     return cudaGetLastError();
   };
   if (vpl <= 1) return go(pass_bulk_kernel<T, VW, 1, MODE>);
