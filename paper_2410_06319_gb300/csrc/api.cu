@@ -57,7 +57,8 @@ void stage_sketch(Ctx& c, double* Y, const float* a32) {
     float* partial = static_cast<float*>(ws(c.h, "partial", (size_t)p.splits * ncols * p.s_pad * 4));
     {
       KernTimer kt(c.h, K_SKETCH, c.o.timing);
-      L(launch_sketch_tc(p, tm, c.seed, partial, c.h->d_err, c.st));
+      auto* work = static_cast<unsigned*>(ws(c.h, "sk_work", (1 + 2 * (size_t)kSkHandMax) * 4));
+      L(launch_sketch_tc(p, tm, c.seed, partial, work, c.h->d_err, c.st));
     }
     KernTimer kt(c.h, K_SKETCH_SUM, c.o.timing);
     L(launch_sketch_reduce(partial, false, p.splits, ncols, c.s, p.s_pad, kexp, Y, c.st));

@@ -44,6 +44,8 @@ struct SketchTcArgs {
   uint32_t k0, k1;
   float* partial;
   int* err;
+  int hand, items;   // items done by two CTAs, and all items (sketch_hand_items); 0: one CTA each
+  unsigned* work;    // hand > 0: ticket, then two flags an item, zero before the launch
 };
 
 // A grouped sketch launch: problem p owns CTAs [start[p], start[p + 1]); tab[p] and
@@ -114,8 +116,11 @@ cudaError_t launch_grouped_cast(int fmt, const GCast* tab, const int* colmax_sta
 // Grouped sketch_reduce: ceil(s / 256) x (n + 1) CTAs per problem.
 cudaError_t launch_grouped_sketch_reduce(const GReduce* tab, const int* start, int64_t ctas, int nprob,
                                          cudaStream_t st);
+// work: 1 + 2 kSkHandMax words for items that two CTAs share (sketch_hand_items).
+constexpr int kSkHandMax = 255;
+int sketch_hand_items(int64_t items, int64_t steps, int64_t slots);
 cudaError_t launch_sketch_tc(const SketchPlan& p, const CUtensorMap& tm, uint64_t seed,
-                             float* partial, int* err, cudaStream_t st);
+                             float* partial, unsigned* work, int* err, cudaStream_t st);
 uint32_t sketch_rec_cap(const SketchPlan& p);
 int64_t sketch_rec_lists(const SketchPlan& p);
 // CUDA-core sketch in FP64 (fmt F64) or FP32 (fmt F32) from the FP64 data.
