@@ -162,6 +162,12 @@ __device__ __forceinline__ uint32_t cl_map(uint32_t saddr, uint32_t rank) {
   asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(saddr), "r"(rank));
   return r;
 }
+// a value into another CTA's shared memory (raddr from cl_map)
+template <typename T>
+__device__ __forceinline__ void st_cluster(uint32_t raddr, T v) {
+  if constexpr (sizeof(T) == 4) asm volatile("st.shared::cluster.b32 [%0], %1;" ::"r"(raddr), "r"(*reinterpret_cast<const uint32_t*>(&v)) : "memory");
+  else asm volatile("st.shared::cluster.b64 [%0], %1;" ::"r"(raddr), "l"(*reinterpret_cast<const uint64_t*>(&v)) : "memory");
+}
 // every thread of every CTA of the cluster (release / acquire)
 __device__ __forceinline__ void cl_sync() {
   asm volatile("barrier.cluster.arrive.release.aligned;\n barrier.cluster.wait.acquire.aligned;" ::: "memory");

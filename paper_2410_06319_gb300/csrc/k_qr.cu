@@ -179,175 +179,6 @@ __global__ void __launch_bounds__(kQr64Threads, 1)
   }
 }
 
-// FP64 variant with the columns resident in shared memory (s <= 4096 and at most
-// kQr64sMaxCols columns per CTA), with look-ahead.  CTA b owns columns b, b + nb, ...
-// (cyclic, so every CTA keeps a share of the trailing matrix to the end) and keeps them in
-// shared memory for the whole factorization; each thread holds v_k for its rows in
-// registers.  A CTA touches only its own columns, so steps need no grid barrier: step k
-// waits (bounded) for the flag ready[k] that the owner of column k raises once column k
-// (updated by reflectors 0..k-1) and its norm are in global memory.  The owner of column
-// k+1 updates that column first, publishes it, then updates its other columns; the rest of
-// the trailing update overlaps the next pivot's critical path.  ready[] (n + 1 words) must
-// be zero at launch.  At the end the owner of column n (b) writes it back.
-constexpr int kQr64sMaxCols = 8;
-constexpr int kQr64sRows = 8;          // rows per thread: s <= 512 * 8
-
-__device__ __forceinline__ double block_sum_512(double v, double* nred) {
-  v = warp_sum(v);
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
-  __syncthreads();
-  if (lane == 0) nred[warp] = v;
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    double q = 0.0;
-    for (int w = 0; w < nw; ++w) q += nred[w];
-    nred[16] = q;
-  }
-  __syncthreads();
-  return nred[16];
-}
-
-__global__ void __launch_bounds__(kQr64Threads, 1)
-    qr64s_kernel(double* __restrict__ W, int64_t s, int64_t n, double* __restrict__ norms,
-                 double* __restrict__ diagR, unsigned* __restrict__ ready, int* err) {
-  extern __shared__ __align__(16) unsigned char qr_smem[];
-  double* cols = reinterpret_cast<double*>(qr_smem);   // [owned][s]
-  __shared__ double red[16 * 9];
-  __shared__ double wsum[8];
-  __shared__ double nred[17];
-  __shared__ int ok_s;
-  const int nb = (int)gridDim.x, b = (int)blockIdx.x;
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
-  const int64_t ncols = n + 1;
-  int owned = 0;
-  for (int64_t j = b; j < ncols; j += nb) ++owned;
-  for (int c = 0; c < owned; ++c) {
-    const int64_t j = b + (int64_t)c * nb;
-    for (int64_t t = threadIdx.x; t < s; t += blockDim.x) cols[c * s + t] = W[j * s + t];
-  }
-  __syncthreads();
-  if (b == 0) {   // column 0 is ready as it stands: its norm, then the flag
-    double part = 0.0;
-    for (int64_t t = threadIdx.x; t < s; t += blockDim.x) part = fma(cols[t], cols[t], part);
-    const double nn = block_sum_512(part, nred);
-    if (threadIdx.x == 0) {
-      norms[0] = nn;
-      __threadfence();
-      atomicExch(ready, 1u);
-    }
-  }
-  for (int64_t k = 0; k < n; ++k) {
-    // ---- wait for column k and its norm
-    if (threadIdx.x == 0) {
-      volatile unsigned* vr = ready + k;
-      int ok = 1;
-      if (*vr == 0u) {
-        const uint64_t t0 = globaltimer_ns();
-        while (*vr == 0u) {
-          if (globaltimer_ns() - t0 > kWaitLimitNs) {
-            set_error(err, DEV_TIMEOUT_GRID);
-            ok = 0;
-            break;
-          }
-        }
-      }
-      __threadfence();
-      ok_s = ok;
-    }
-    __syncthreads();
-    if (!ok_s) return;
-    const double* colk = W + k * s;
-    const double alpha = sqrt(__ldcg(norms + k));
-    const double x0 = __ldcg(colk + k);
-    const double sgn = (x0 >= 0.0) ? 1.0 : -1.0;
-    const double tau = (alpha > 0.0) ? 1.0 / (alpha * (alpha + fabs(x0))) : 0.0;
-    if (b == 0 && threadIdx.x == 0) diagR[k] = -sgn * alpha;
-    double v[kQr64sRows];
-#pragma unroll
-    for (int r = 0; r < kQr64sRows; ++r) {
-      const int64_t t = threadIdx.x + (int64_t)r * blockDim.x;
-      v[r] = (t < k || t >= s) ? 0.0 : (t == k ? x0 + sgn * alpha : __ldcg(colk + t));
-    }
-    // owned columns with index > k, from c_first on; the next pivot k+1 first if owned
-    int c_first = 0;
-    if (k + 1 > b) c_first = (int)((k + 1 - b + nb - 1) / nb);
-    const int64_t jn = k + 1;
-    if (jn < n && jn % nb == b) {
-      const int cn = (int)(jn / nb);       // == c_first
-      double d = 0.0;
-#pragma unroll
-      for (int r = 0; r < kQr64sRows; ++r) {
-        const int64_t t = threadIdx.x + (int64_t)r * blockDim.x;
-        if (t < s) d = fma(v[r], cols[cn * s + t], d);
-      }
-      const double wn = block_sum_512(d, nred) * tau;
-      double sq = 0.0;
-#pragma unroll
-      for (int r = 0; r < kQr64sRows; ++r) {
-        const int64_t t = threadIdx.x + (int64_t)r * blockDim.x;
-        if (t < s && t >= k) {
-          const double val = fma(-wn, v[r], cols[cn * s + t]);
-          cols[cn * s + t] = val;
-          if (t >= jn) sq = fma(val, val, sq);
-        }
-      }
-      const double nn = block_sum_512(sq, nred);
-      for (int64_t t = threadIdx.x; t < s; t += blockDim.x) W[jn * s + t] = cols[cn * s + t];
-      __syncthreads();
-      if (threadIdx.x == 0) {
-        norms[jn] = nn;
-        __threadfence();
-        atomicExch(ready + jn, 1u);
-      }
-      c_first = cn + 1;
-    }
-    // ---- the other owned trailing columns, up to eight at a time
-    if (c_first < owned) {
-      double d[8];
-#pragma unroll
-      for (int q = 0; q < 8; ++q) d[q] = 0.0;
-#pragma unroll
-      for (int q = 0; q < 8; ++q) {
-        const int c = c_first + q;
-        if (c < owned) {
-#pragma unroll
-          for (int r = 0; r < kQr64sRows; ++r) {
-            const int64_t t = threadIdx.x + (int64_t)r * blockDim.x;
-            if (t < s) d[q] = fma(v[r], cols[c * s + t], d[q]);
-          }
-        }
-      }
-      const double tot = warp_reduce8(d);
-      if ((lane & 3) == 0) red[warp * 9 + ((lane >> 2) & 7)] = tot;
-      __syncthreads();
-      if (threadIdx.x < 8) {
-        double q = 0.0;
-        for (int w = 0; w < nw; ++w) q += red[w * 9 + threadIdx.x];
-        wsum[threadIdx.x] = q * tau;
-      }
-      __syncthreads();
-#pragma unroll
-      for (int q = 0; q < 8; ++q) {
-        const int c = c_first + q;
-        if (c < owned) {
-          const double wq = wsum[q];
-#pragma unroll
-          for (int r = 0; r < kQr64sRows; ++r) {
-            const int64_t t = threadIdx.x + (int64_t)r * blockDim.x;
-            if (t < s && t >= k) cols[c * s + t] = fma(-wq, v[r], cols[c * s + t]);
-          }
-        }
-      }
-    }
-    __syncthreads();
-  }
-  // columns 0..n-1 are final in W since they were published; only b's column is left
-  if (n % nb == b) {
-    const int c = (int)(n / nb);
-    for (int64_t t = threadIdx.x; t < s; t += blockDim.x) W[n * s + t] = cols[c * s + t];
-  }
-}
-
 // R (FP64, col-major, diag >= 0) and c from the factored work matrix.
 template <typename T>
 __device__ __forceinline__ void qr_finalize_body(const T* __restrict__ W, int64_t s, int64_t n,
@@ -389,8 +220,9 @@ __global__ void qr_finalize_kernel(const T* __restrict__ W, int64_t s, int64_t n
 // of 16 columns on one CTA of 1024 threads, unrolled over the columns (each launch fetched
 // some 10,000 instructions once), two reductions a column, and a launch for each trailing
 // update took 1.93 ms at s = 2000, n = 500 in FP32, and a grid barrier per column 1.9 ms at s =
-// 748, n = 187 in FP64; now 0.95 and 1.34 ms.  NB: 8 in FP32; 4 in FP64, where a CTA's arithmetic (two FMAs a
+// 748, n = 187 in FP64; now 0.95 and 0.96 ms.  NB: 8 in FP32; 4 in FP64, where a CTA's arithmetic (two FMAs a
 // clock an SM) weighs as much as the latency.
+constexpr int min_int(int a, int b) { return a < b ? a : b; }
 template <typename T, int N>
 __device__ __forceinline__ T warp_reduce_scatter(T (&v)[N], int lane) {
   // after the call lane l holds the warp total of v[l / (32 / N)]
@@ -417,28 +249,58 @@ __device__ __forceinline__ T warp_reduce_scatter(T (&v)[N], int lane) {
   return v[0];
 }
 
-template <typename T, int NB, int NT, int RPT>
+//
+// C > 1: a block's rows are spread over a cluster of C CTAs, so that the chain of a block (in FP64
+// one instruction of a warp takes 67 cycles) has C SMs; the partial sums go to every CTA of the
+// cluster, one cluster barrier a reduction.  Blocks are taken by ticket (flag[nblk]), so they
+// need not all be resident: a block waits only for blocks that run already.  FP64 with the
+// columns in shared memory and a flag per column (one SM's FP64 rate bound the pivot column):
+// s = 2000, n = 500 5.9 ms, s = 4000, n = 1000 14.8 ms; now 3.1 and 12.3 (5.8 of them FMAs).
+template <typename T, int NB, int NT, int RPT, int C>
 __global__ void __launch_bounds__(NT, 1)
     qr_block_kernel(T* __restrict__ W, int64_t s, int64_t n, double* __restrict__ diagR, T* __restrict__ Tg,
-                    unsigned* __restrict__ flag, int* err) {
+                    unsigned* __restrict__ flag, int nblk, int* err) {
   constexpr int NW = NT / 32;
-  constexpr int HA = NB * NB > 32 ? 32 / NB : NB;   // reflectors at a time in the products
+  constexpr int HA = min_int(NB, 32 / NB);   // reflectors at a time in the products
   constexpr int NH = NB / HA;
-  constexpr int LB = NT <= 256 ? NB : NB / 2;       // columns of V loaded at a time
+  constexpr int LB = NB;                            // columns of V loaded at a time
   __shared__ T red[2][NW][NB * NB];
   // Gs: g_la at l + a * NB (l < a), tau_a at a + a * NB
   __shared__ T Ws[NB * NB], Gs[NB * NB], prow[2][NB];
   __shared__ T sc[2], rd[NB];
   extern __shared__ __align__(16) unsigned char qb_smem[];
   T* Vs = reinterpret_cast<T*>(qb_smem);   // [NB][RPT * NT]: the block of reflectors being applied
+  // C > 1: the CTAs' shares of the products of a block (by its parity) and of a column (by the
+  // column's), and the pivot row; the ticket
+  __shared__ T cw[C > 1 ? 2 : 1][C][NB * NB], cd[C > 1 ? 2 : 1][C][NB];
+  __shared__ unsigned ticket;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  const int q = (int)blockIdx.x;
+  const int rank = C > 1 ? (int)cl_rank() : 0;
+  int q = (int)blockIdx.x;
+  if constexpr (C > 1) {
+    cl_sync();   // the whole cluster runs
+    if (rank == 0 && tid == 0) {
+      const unsigned k = atomicAdd(flag + nblk, 1u);
+      for (int d = 0; d < C; ++d) st_cluster(cl_map(smem_u32(&ticket), (uint32_t)d), k);
+    }
+    cl_sync();
+    q = (int)ticket;
+  }
+  // Row i of a thread.  The 128-row pieces go round the cluster, so that its CTAs keep equal
+  // shares while the factored rows grow; FP64 leaves out the pieces that hold none of a
+  // reflector's rows.
+  auto row = [&](int i) { return (i * C + rank) * NT + tid; };
+  auto idle = [&](int i, int64_t first) {
+    if constexpr (sizeof(T) == 4) return false;
+    else return (int64_t)(i * C + rank + 1) * NT <= first || (int64_t)(i * C + rank) * NT >= s;
+  };
+  bool live = true;                           // C > 1: no wait has run out
   const int64_t c0 = (int64_t)q * NB;
   const int ncol = (int)min((int64_t)NB, n + 1 - c0);
   T x[RPT][NB];
 #pragma unroll
   for (int i = 0; i < RPT; ++i) {
-    const int64_t r = tid + (int64_t)i * NT;
+    const int64_t r = row(i);
 #pragma unroll
     for (int c = 0; c < NB; ++c) x[i][c] = (r < s && c < ncol) ? W[(c0 + c) * s + r] : T(0);
   }
@@ -450,9 +312,9 @@ __global__ void __launch_bounds__(NT, 1)
       auto raised = [&]() {
         unsigned f;
         asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(f) : "l"(fp) : "memory");
-        return f != 0u;
+        return f >= (unsigned)C;
       };
-      if (!raised()) {
+      if (live && !raised()) {
         const uint64_t t0 = globaltimer_ns();
         while (!raised()) {
           if (globaltimer_ns() - t0 > kWaitLimitNs) {
@@ -463,7 +325,10 @@ __global__ void __launch_bounds__(NT, 1)
         }
       }
     }
-    if (__syncthreads_and(ok) == 0) return;
+    if (__syncthreads_and(ok) == 0) {
+      if constexpr (C == 1) return;
+      else live = false;   // the cluster's barriers need every CTA: go on without waiting
+    }
     const int64_t p = (int64_t)P * NB;
     if (tid < NB * NB) Gs[tid] = __ldcg(Tg + (int64_t)P * NB * NB + tid);
     // a thread stages its own rows of V (from L2; zero above each diagonal entry), all loads in
@@ -476,8 +341,8 @@ __global__ void __launch_bounds__(NT, 1)
       for (int a = 0; a < LB; ++a)
 #pragma unroll
         for (int i = 0; i < RPT; ++i) {
-          const int64_t r = tid + (int64_t)i * NT;
-          v[a][i] = (r >= p + a0 + a && r < s) ? __ldcg(V + (a0 + a) * s + r) : T(0);
+          const int64_t r = row(i);
+          v[a][i] = (!idle(i, p) && r >= p + a0 + a && r < s) ? __ldcg(V + (a0 + a) * s + r) : T(0);
         }
 #pragma unroll
       for (int a = 0; a < LB; ++a)
@@ -491,7 +356,7 @@ __global__ void __launch_bounds__(NT, 1)
       for (int e = 0; e < HA * NB; ++e) acc[e] = T(0);
 #pragma unroll
       for (int i = 0; i < RPT; ++i) {
-        {   // V is zero outside its rows
+        if (!idle(i, p)) {   // V is zero outside its rows
           const int r = tid + i * NT;
           T v[HA];
 #pragma unroll
@@ -507,13 +372,31 @@ __global__ void __launch_bounds__(NT, 1)
       if (lane % LP == 0) red[0][warp][h * HA * NB + lane / LP] = w;
     }
     __syncthreads();
-    if (tid < NB * NB) {
-      T w = T(0);
+    if constexpr (C == 1) {
+      if (tid < NB * NB) {
+        T w = T(0);
 #pragma unroll
-      for (int k = 0; k < NW; ++k) w += red[0][k][tid];
-      Ws[tid] = w;
+        for (int k = 0; k < NW; ++k) w += red[0][k][tid];
+        Ws[tid] = w;
+      }
+      __syncthreads();
+    } else {
+      // warp d sends this CTA's share to the CTAs d, d + NW, ...
+      for (int e = lane; e < NB * NB; e += 32) {
+        T w = T(0);
+#pragma unroll
+        for (int k = 0; k < NW; ++k) w += red[0][k][e];
+        for (int d = warp; d < C; d += NW) st_cluster(cl_map(smem_u32(&cw[P & 1][rank][e]), (uint32_t)d), w);
+      }
+      cl_sync();
+      if (tid < NB * NB) {
+        T w = T(0);
+#pragma unroll
+        for (int d = 0; d < C; ++d) w += cw[P & 1][d][tid];
+        Ws[tid] = w;
+      }
+      __syncthreads();
     }
-    __syncthreads();
     if (tid < NB) {   // column tid of the block: forward substitution
       T w[NB];
 #pragma unroll
@@ -533,7 +416,7 @@ __global__ void __launch_bounds__(NT, 1)
       for (int e = 0; e < HA * NB; ++e) w2[e] = Ws[h * HA * NB + e];
 #pragma unroll
       for (int i = 0; i < RPT; ++i) {
-        {   // V is zero outside its rows
+        if (!idle(i, p)) {   // V is zero outside its rows
           const int r = tid + i * NT;
           T v[HA];
 #pragma unroll
@@ -564,25 +447,45 @@ __global__ void __launch_bounds__(NT, 1)
       for (int c = 0; c < NB; ++c) d[c] = T(0);
 #pragma unroll
       for (int i = 0; i < RPT; ++i) {
-        const int r = tid + i * NT;
+        const int r = row(i);
+        if (idle(i, pr)) continue;
         const T xj = r >= pr ? x[i][0] : T(0);
 #pragma unroll
         for (int c = 0; c < NB; ++c) d[c] = fma(xj, x[i][c], d[c]);
         if (r == pr) {
 #pragma unroll
-          for (int c = 0; c < NB; ++c) prow[par][c] = x[i][c];
+          for (int c = 0; c < NB; ++c) {
+            if constexpr (C == 1) {
+              prow[par][c] = x[i][c];
+            } else {
+              for (int d = 0; d < C; ++d) st_cluster(cl_map(smem_u32(&prow[par][c]), (uint32_t)d), x[i][c]);
+            }
+          }
         }
       }
       const T dw = warp_reduce_scatter<T, NB>(d, lane);
       constexpr int LP = 32 / NB;
       if (lane % LP == 0) red[par][warp][lane / LP] = dw;
       __syncthreads();
+      if constexpr (C > 1) {
+        // a CTA's share by lanes 0 .. NB - 1 of each warp, which sends it to the CTAs warp, warp + NW, ...
+        if (lane < NB) {
+          T w = T(0);
+#pragma unroll
+          for (int k = 0; k < NW; ++k) w += red[par][k][lane];
+          for (int d = warp; d < C; d += NW) st_cluster(cl_map(smem_u32(&cd[par][rank][lane]), (uint32_t)d), w);
+        }
+        cl_sync();
+      }
       T tot = T(0), sa, tau;   // lane l: value l % NB, summed over a share of the warps, then over the shares
       const T x0 = prow[par][0];
       auto totals = [&]() {
 #pragma unroll
-        for (int k = 0; k < (NW + LP - 1) / LP; ++k)
-          if (lane / NB + k * LP < NW) tot += red[par][lane / NB + k * LP][lane % NB];
+        for (int k = 0; k < ((C > 1 ? C : NW) + LP - 1) / LP; ++k)
+          if (lane / NB + k * LP < (C > 1 ? C : NW)) {
+            if constexpr (C > 1) tot += cd[par][lane / NB + k * LP][lane % NB];
+            else tot += red[par][lane / NB + k * LP][lane % NB];
+          }
 #pragma unroll
         for (int o = NB; o < 32; o <<= 1) tot += __shfl_xor_sync(0xffffffffu, tot, o);
       };
@@ -612,7 +515,7 @@ __global__ void __launch_bounds__(NT, 1)
       T v[RPT];   // v_j: zero above the pivot row, where x keeps R
 #pragma unroll
       for (int i = 0; i < RPT; ++i) {
-        const int r = tid + i * NT;
+        const int r = row(i);
         if (r == pr) x[i][0] += sa;
         v[i] = r >= pr ? x[i][0] : T(0);
         // the column is final: R above the pivot row, v_j from it down
@@ -624,7 +527,8 @@ __global__ void __launch_bounds__(NT, 1)
         if (c < NB - j) {
           const T coef = tau * vx;
 #pragma unroll
-          for (int i = 0; i < RPT; ++i) x[i][c] = fma(-coef, v[i], x[i][c]);
+          for (int i = 0; i < RPT; ++i)
+            if (!idle(i, pr)) x[i][c] = fma(-coef, v[i], x[i][c]);
         }
       }
       if (warp == 0) {   // lane c >= NB - j: v_l^T v_j of the finished column l = c - (NB - j)
@@ -646,21 +550,24 @@ __global__ void __launch_bounds__(NT, 1)
   // ---- the right-hand side's column, if the block holds it; tau and the Gram entries; the flag
 #pragma unroll
   for (int i = 0; i < RPT; ++i) {
-    const int64_t r = tid + (int64_t)i * NT;
+    const int64_t r = row(i);
 #pragma unroll
     for (int c = 0; c < NB; ++c)
       if (c >= kb && c < ncol && r < s) W[(c0 + c) * s + r] = x[i][c];
   }
   __syncthreads();
-  if (tid < NB * NB) Tg[(int64_t)q * NB * NB + tid] = Gs[tid];
-  if (tid < kb) diagR[c0 + tid] = (double)rd[tid];
+  if (rank == 0) {
+    if (tid < NB * NB) Tg[(int64_t)q * NB * NB + tid] = Gs[tid];
+    if (tid < kb) diagR[c0 + tid] = (double)rd[tid];
+  }
   __threadfence();
   __syncthreads();
-  if (tid == 0) atomicExch(flag + q, 1u);
+  if (tid == 0) atomicAdd(flag + q, 1u);
+  if constexpr (C > 1) cl_sync();   // no CTA leaves while another may still send to it
 }
 
 // The register-block form: `aux` as launch_qr's, block factors and flags behind diag(R).
-template <typename T, int NB, int NT, int RPT>
+template <typename T, int NB, int NT, int RPT, int C = 1>
 static cudaError_t run_qr_block(const double* Y, int64_t s, int64_t n, T* W, double* aux, double* R, double* c,
                                 int* err, cudaStream_t st) {
   const int64_t total = s * (n + 1);
@@ -671,15 +578,36 @@ static cudaError_t run_qr_block(const double* Y, int64_t s, int64_t n, T* W, dou
   double* diagR = aux + n;
   T* Tg = reinterpret_cast<T*>(aux + 2 * n + 8);
   unsigned* flag = reinterpret_cast<unsigned*>(Tg + (size_t)nblk * NB * NB);
-  e = cudaMemsetAsync(flag, 0, nblk * sizeof(unsigned), st);
+  e = cudaMemsetAsync(flag, 0, (nblk + 1) * sizeof(unsigned), st);   // and the ticket
   if (e != cudaSuccess) return e;
   T* Wp = W;
   int64_t sp = s, np = n;
-  void* args[] = {&Wp, &sp, &np, &diagR, &Tg, &flag, &err};
-  const size_t smem = (size_t)NB * RPT * NT * sizeof(T);
-  e = allow_dyn_smem(qr_block_kernel<T, NB, NT, RPT>, smem);
+  int nb = (int)nblk;
+  size_t smem = (size_t)NB * RPT * NT * sizeof(T);
+  // at most three CTAs an SM: with more, the FP64 instructions of the block that all others wait
+  // for queue behind theirs (s = 4000, n = 1000: 13.2 ms with four, 12.3 with three, 17 with two)
+  if (C > 1) smem = std::max(smem, (size_t)74 * 1024);
+  auto kern = qr_block_kernel<T, NB, NT, RPT, C>;
+  e = allow_dyn_smem(kern, smem);
   if (e != cudaSuccess) return e;
-  e = cudaLaunchCooperativeKernel((const void*)qr_block_kernel<T, NB, NT, RPT>, dim3(nblk), dim3(NT), args, smem, st);
+  if constexpr (C == 1) {
+    void* args[] = {&Wp, &sp, &np, &diagR, &Tg, &flag, &nb, &err};
+    e = cudaLaunchCooperativeKernel((const void*)kern, dim3(nblk), dim3(NT), args, smem, st);
+  } else {
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(nblk * C);
+    cfg.blockDim = dim3(NT);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = st;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeClusterDimension;
+    attr[0].val.clusterDim.x = C;
+    attr[0].val.clusterDim.y = 1;
+    attr[0].val.clusterDim.z = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    e = cudaLaunchKernelEx(&cfg, kern, Wp, sp, np, diagR, Tg, flag, nb, err);
+  }
   if (e != cudaSuccess) return e;
   qr_finalize_kernel<T><<<(unsigned)n, 256, 0, st>>>(W, s, n, diagR, R, c);
   return cudaGetLastError();
@@ -687,8 +615,8 @@ static cudaError_t run_qr_block(const double* Y, int64_t s, int64_t n, T* W, dou
 
 // Bytes of the region behind diag(R) in aux that a factorization of n columns may use.
 size_t qr_aux_tail(int64_t n) {
-  const size_t f32 = (size_t)((n + 1 + 7) / 8) * (64 * 4 + 4), f64 = (size_t)((n + 1 + 3) / 4) * (16 * 8 + 4);
-  return std::max(std::max(f32, f64), (size_t)(n + 1) * 4);   // or n + 1 column flags (qr64s_kernel)
+  const size_t f32 = (size_t)((n + 1 + 7) / 8) * (64 * 4 + 4) + 4, f64 = (size_t)((n + 1 + 3) / 4) * (16 * 8 + 4) + 4;
+  return std::max(f32, f64);
 }
 
 template <typename T>
@@ -732,30 +660,19 @@ static cudaError_t run_qr64(const double* Y, int64_t s, int64_t n, double* W, do
   e = cudaMemsetAsync(bar, 0, 2 * sizeof(unsigned), st);
   if (e != cudaSuccess) return e;
   const int grid = num_sms;                      // one CTA per SM (co-resident: occ >= 1)
-  const int64_t per_cta = (n + 1 + grid - 1) / grid;
-  const bool resident = s <= (int64_t)kQr64Threads * kQr64sRows && per_cta <= kQr64sMaxCols &&
-                        (size_t)per_cta * s * 8 <= 227 * 1024 - 2048;
-  auto kern = resident ? qr64s_kernel : qr64_kernel;
-  const size_t smem = resident ? (size_t)per_cta * s * 8 : (size_t)s * 8;
-  e = allow_dyn_smem(kern, smem);
+  const size_t smem = (size_t)s * 8;
+  e = allow_dyn_smem(qr64_kernel, smem);
   if (e != cudaSuccess) return e;
   int occ = 0;
-  e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, kern, kQr64Threads, smem);
+  e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, qr64_kernel, kQr64Threads, smem);
   if (e != cudaSuccess) return e;
   if (occ < 1) return cudaErrorInvalidConfiguration;
   double* norms = aux;
   double* diagR = aux + n;
-  // the resident kernel's per-column flags follow diag(R) in aux (n + 1 words, zeroed here)
-  unsigned* ready = reinterpret_cast<unsigned*>(aux + 2 * n + 8);
-  if (resident) {
-    e = cudaMemsetAsync(ready, 0, (size_t)(n + 1) * sizeof(unsigned), st);
-    if (e != cudaSuccess) return e;
-  }
-  unsigned* sync = resident ? ready : bar;
   double* Wp = W;
   int64_t sp = s, np = n;
-  void* args[] = {&Wp, &sp, &np, &norms, &diagR, &sync, &err};
-  e = cudaLaunchCooperativeKernel((const void*)kern, dim3((unsigned)grid), dim3(kQr64Threads), args, smem, st);
+  void* args[] = {&Wp, &sp, &np, &norms, &diagR, &bar, &err};
+  e = cudaLaunchCooperativeKernel((const void*)qr64_kernel, dim3((unsigned)grid), dim3(kQr64Threads), args, smem, st);
   if (e != cudaSuccess) return e;
   qr_finalize_kernel<double><<<(unsigned)n, 256, 0, st>>>(W, s, n, diagR, R, c);
   return cudaGetLastError();
@@ -771,15 +688,20 @@ cudaError_t launch_qr(bool fp64, const double* Y, int64_t s, int64_t n, void* wo
       if (s <= 512) return run_qr_block<float, 8, 256, 2>(Y, s, n, W, aux, R, c, err, st);
       if (s <= 1024) return run_qr_block<float, 8, 256, 4>(Y, s, n, W, aux, R, c, err, st);
       if (s <= 2048) return run_qr_block<float, 8, 256, 8>(Y, s, n, W, aux, R, c, err, st);
-      if (s <= 4096) return run_qr_block<float, 8, 512, 8>(Y, s, n, W, aux, R, c, err, st);
     }
+    // past that a cluster of eight (s = 4000, n = 1000: 2.94 ms with 512 threads of eight rows on one
+    // CTA, 2.06 so; at s <= 2048 the cluster's barriers cost more than they give: 0.94 and 0.96)
+    if (s > 2048 && s <= 4096) return run_qr_block<float, 8, 256, 2, 8>(Y, s, n, W, aux, R, c, err, st);
     return run_qr<float>(Y, s, n, W, aux, bar, R, c, err, num_sms, st);
   }
   double* W = static_cast<double*>(work);
-  if ((n + 1 + 3) / 4 <= num_sms) {
-    if (s <= 512) return run_qr_block<double, 4, 128, 4>(Y, s, n, W, aux, R, c, err, st);
-    if (s <= 1024) return run_qr_block<double, 4, 128, 8>(Y, s, n, W, aux, R, c, err, st);
-  }
+  // FP64: rows of a block over clusters of four or eight CTAs, fewer rows a thread than a
+  // wider CTA would have (s = 1000, n = 250: 1.81 ms on one CTA of 128 threads, 1.24 so)
+  if (s <= 256) return run_qr_block<double, 4, 64, 1, 4>(Y, s, n, W, aux, R, c, err, st);
+  if (s <= 512) return run_qr_block<double, 4, 128, 1, 4>(Y, s, n, W, aux, R, c, err, st);
+  if (s <= 1024) return run_qr_block<double, 4, 64, 2, 8>(Y, s, n, W, aux, R, c, err, st);
+  if (s <= 2048) return run_qr_block<double, 4, 64, 4, 8>(Y, s, n, W, aux, R, c, err, st);
+  if (s <= 4096) return run_qr_block<double, 4, 128, 4, 8>(Y, s, n, W, aux, R, c, err, st);
   return run_qr64(Y, s, n, W, aux, bar, R, c, err, num_sms, st);
 }
 
