@@ -479,7 +479,8 @@ lsq_status lsq_batch_grouped(lsq_handle* h, int32_t nprob, const lsq_problem* pr
     check_dev_error(h);
     // ------------------------------------------------------------ QR (a4), R copies, x_s
     std::vector<size_t> szW(np), szN(np), szNN(np), szR32(np), szR64(np), szD32(np), szD64(np);
-    std::vector<int64_t> ncol(np), nblk32(np);
+    std::vector<int64_t> ncol(np), nblk32(np), nqr(np);
+    int64_t maxs = 0;
     const bool qr64 = u_p == LSQ_F64;
     for (int p = 0; p < np; ++p) {
       const int64_t n = b.n[p], ld32 = tri_ld(n, 4), ld64 = tri_ld(n, 8);
@@ -492,6 +493,8 @@ lsq_status lsq_batch_grouped(lsq_handle* h, int32_t nprob, const lsq_problem* pr
       szD64[p] = (size_t)cdiv(n, 32) * 1024 * 8;
       ncol[p] = n;
       nblk32[p] = cdiv(n, 32);
+      nqr[p] = cdiv(n + 1, qr64 ? kQrCols<double> : kQrCols<float>);
+      maxs = std::max(maxs, b.s[p]);
     }
     Arena aW = make_arena(h, "b_qrw", szW), aDg = make_arena(h, "b_diag", szN), aR = make_arena(h, "b_R", szNN),
           aCv = make_arena(h, "b_c", szN), aR32 = make_arena(h, "b_R32", szR32), aL32 = make_arena(h, "b_L32", szR32),
@@ -500,7 +503,9 @@ lsq_status lsq_batch_grouped(lsq_handle* h, int32_t nprob, const lsq_problem* pr
           aDU64 = make_arena(h, "b_DU64", szD64), aDL64 = make_arena(h, "b_DL64", szD64),
           aX0 = make_arena(h, "b_x0", szN);
     double* kapd = static_cast<double*>(ws(h, "b_kap", (size_t)np * 8));
-    Groups gcol = make_groups(h, "b_gqrcol", ncol), gblk = make_groups(h, "b_gqrblk", nblk32);
+    Groups gcol = make_groups(h, "b_gqrcol", ncol), gblk = make_groups(h, "b_gqrblk", nblk32),
+           gqr = make_groups(h, "b_gqrq", nqr);
+    void* qwork = ws(h, "b_qrt", (size_t)gqr.total * ((qr64 ? 16 * 8 : 64 * 4) + 4) + 4);
     std::vector<Tri<float>> tri32(np);
     std::vector<Tri<double>> tri64(np);
     {
@@ -519,13 +524,15 @@ lsq_status lsq_batch_grouped(lsq_handle* h, int32_t nprob, const lsq_problem* pr
         for (int p = 0; p < np; ++p)
           tq[p] = GQr<double>{aY.at<double>(p), aW.at<double>(p), b.s[p], b.n[p], aDg.at<double>(p), aR.at<double>(p),
                               aCv.at<double>(p)};
-        LB(launch_grouped_qr<double>(upload(h, "b_tq", tq), gcol.dev, gcol.total, np, 256, b.st));
+        LB(launch_grouped_qr<double>(upload(h, "b_tq", tq), gqr.dev, gqr.total, gcol.dev, gcol.total, np, maxs, qwork,
+                                     h->d_err, b.st));
       } else {
         std::vector<GQr<float>> tq(np);
         for (int p = 0; p < np; ++p)
           tq[p] = GQr<float>{aY.at<double>(p), aW.at<float>(p), b.s[p], b.n[p], aDg.at<double>(p), aR.at<double>(p),
                              aCv.at<double>(p)};
-        LB(launch_grouped_qr<float>(upload(h, "b_tq", tq), gcol.dev, gcol.total, np, 256, b.st));
+        LB(launch_grouped_qr<float>(upload(h, "b_tq", tq), gqr.dev, gqr.total, gcol.dev, gcol.total, np, maxs, qwork,
+                                    h->d_err, b.st));
       }
       LB(launch_grouped_prepare_r(upload(h, "b_tprep", tprep), gcol.dev, gcol.total, gblk.dev, gblk.total, np,
                                   b.st));

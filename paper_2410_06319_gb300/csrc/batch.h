@@ -155,7 +155,7 @@ struct GPrepR {
 cudaError_t launch_grouped_prepare_r(const GPrepR* tab, const int* col_start, int64_t col_ctas,
                                      const int* blk_start, int64_t blk_ctas, int nprob, cudaStream_t st);
 
-// ---- k_qr.cu: Householder QR of each problem's sketch, one CTA per problem (s <= 1024)
+// ---- k_qr.cu: Householder QR of each problem's sketch, one launch (s <= 1024)
 template <typename T>
 struct GQr {
   const double* Y;   // s x (n + 1), column-major
@@ -165,8 +165,11 @@ struct GQr {
   double* R;         // n x n, column-major, diag >= 0
   double* c;         // n: (Q^T Omega b)[:n]
 };
+// Columns of a block of the QR; `work` holds (NB * NB * sizeof(T) + 4) bytes a block and 4 more.
 template <typename T>
-cudaError_t launch_grouped_qr(const GQr<T>* tab, const int* col_start, int64_t col_ctas, int nprob, int64_t max_n,
-                              cudaStream_t st);
+constexpr int kQrCols = sizeof(T) == 4 ? 8 : 4;
+template <typename T>
+cudaError_t launch_grouped_qr(const GQr<T>* tab, const int* blk_start, int64_t blocks, const int* col_start,
+                              int64_t col_ctas, int nprob, int64_t max_s, void* work, int* err, cudaStream_t st);
 
 }  // namespace lsq

@@ -256,10 +256,29 @@ __device__ __forceinline__ T warp_reduce_scatter(T (&v)[N], int lane) {
 // need not all be resident: a block waits only for blocks that run already.  FP64 with the
 // columns in shared memory and a flag per column (one SM's FP64 rate bound the pivot column):
 // s = 2000, n = 500 5.9 ms, s = 4000, n = 1000 14.8 ms; now 3.1 and 12.3 (5.8 of them FMAs).
+// The CTA's (or cluster's) next item.
+template <int C>
+__device__ __forceinline__ int qr_ticket(unsigned* counter) {
+  __shared__ unsigned ticket;
+  if constexpr (C > 1) {
+    cl_sync();   // the whole cluster runs
+    if (cl_rank() == 0 && threadIdx.x == 0) {
+      const unsigned k = atomicAdd(counter, 1u);
+      for (int d = 0; d < C; ++d) st_cluster(cl_map(smem_u32(&ticket), (uint32_t)d), k);
+    }
+    cl_sync();
+  } else {
+    if (threadIdx.x == 0) ticket = atomicAdd(counter, 1u);
+    __syncthreads();
+  }
+  return (int)ticket;
+}
+
+// Block q of the factorization of Y; W receives V and R, Tg and flag hold the blocks' factors and flags.
 template <typename T, int NB, int NT, int RPT, int C>
-__global__ void __launch_bounds__(NT, 1)
-    qr_block_kernel(T* __restrict__ W, int64_t s, int64_t n, double* __restrict__ diagR, T* __restrict__ Tg,
-                    unsigned* __restrict__ flag, int nblk, int* err) {
+__device__ __forceinline__ void qr_block_body(const double* __restrict__ Y, T* __restrict__ W, int64_t s, int64_t n,
+                                              double* __restrict__ diagR, T* __restrict__ Tg,
+                                              unsigned* __restrict__ flag, int q, int* err) {
   constexpr int NW = NT / 32;
   constexpr int HA = min_int(NB, 32 / NB);   // reflectors at a time in the products
   constexpr int NH = NB / HA;
@@ -271,21 +290,10 @@ __global__ void __launch_bounds__(NT, 1)
   extern __shared__ __align__(16) unsigned char qb_smem[];
   T* Vs = reinterpret_cast<T*>(qb_smem);   // [NB][RPT * NT]: the block of reflectors being applied
   // C > 1: the CTAs' shares of the products of a block (by its parity) and of a column (by the
-  // column's), and the pivot row; the ticket
+  // column's), and the pivot row
   __shared__ T cw[C > 1 ? 2 : 1][C][NB * NB], cd[C > 1 ? 2 : 1][C][NB];
-  __shared__ unsigned ticket;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int rank = C > 1 ? (int)cl_rank() : 0;
-  int q = (int)blockIdx.x;
-  if constexpr (C > 1) {
-    cl_sync();   // the whole cluster runs
-    if (rank == 0 && tid == 0) {
-      const unsigned k = atomicAdd(flag + nblk, 1u);
-      for (int d = 0; d < C; ++d) st_cluster(cl_map(smem_u32(&ticket), (uint32_t)d), k);
-    }
-    cl_sync();
-    q = (int)ticket;
-  }
   // Row i of a thread.  The 128-row pieces go round the cluster, so that its CTAs keep equal
   // shares while the factored rows grow; FP64 leaves out the pieces that hold none of a
   // reflector's rows.
@@ -302,7 +310,7 @@ __global__ void __launch_bounds__(NT, 1)
   for (int i = 0; i < RPT; ++i) {
     const int64_t r = row(i);
 #pragma unroll
-    for (int c = 0; c < NB; ++c) x[i][c] = (r < s && c < ncol) ? W[(c0 + c) * s + r] : T(0);
+    for (int c = 0; c < NB; ++c) x[i][c] = (r < s && c < ncol) ? (T)Y[(c0 + c) * s + r] : T(0);
   }
   // ---- reflectors of the earlier blocks
   for (int P = 0; P < q; ++P) {
@@ -566,19 +574,23 @@ __global__ void __launch_bounds__(NT, 1)
   if constexpr (C > 1) cl_sync();   // no CTA leaves while another may still send to it
 }
 
+template <typename T, int NB, int NT, int RPT, int C>
+__global__ void __launch_bounds__(NT, 1)
+    qr_block_kernel(const double* __restrict__ Y, T* __restrict__ W, int64_t s, int64_t n, double* __restrict__ diagR,
+                    T* __restrict__ Tg, unsigned* __restrict__ flag, int nblk, int* err) {
+  const int q = C > 1 ? qr_ticket<C>(flag + nblk) : (int)blockIdx.x;
+  qr_block_body<T, NB, NT, RPT, C>(Y, W, s, n, diagR, Tg, flag, q, err);
+}
+
 // The register-block form: `aux` as launch_qr's, block factors and flags behind diag(R).
 template <typename T, int NB, int NT, int RPT, int C = 1>
 static cudaError_t run_qr_block(const double* Y, int64_t s, int64_t n, T* W, double* aux, double* R, double* c,
                                 int* err, cudaStream_t st) {
-  const int64_t total = s * (n + 1);
   const unsigned nblk = (unsigned)((n + 1 + NB - 1) / NB);
-  convert_y_kernel<T><<<(unsigned)((total + 255) / 256), 256, 0, st>>>(Y, W, total);
-  cudaError_t e = cudaGetLastError();
-  if (e != cudaSuccess) return e;
   double* diagR = aux + n;
   T* Tg = reinterpret_cast<T*>(aux + 2 * n + 8);
   unsigned* flag = reinterpret_cast<unsigned*>(Tg + (size_t)nblk * NB * NB);
-  e = cudaMemsetAsync(flag, 0, (nblk + 1) * sizeof(unsigned), st);   // and the ticket
+  cudaError_t e = cudaMemsetAsync(flag, 0, (nblk + 1) * sizeof(unsigned), st);   // and the ticket
   if (e != cudaSuccess) return e;
   T* Wp = W;
   int64_t sp = s, np = n;
@@ -591,7 +603,7 @@ static cudaError_t run_qr_block(const double* Y, int64_t s, int64_t n, T* W, dou
   e = allow_dyn_smem(kern, smem);
   if (e != cudaSuccess) return e;
   if constexpr (C == 1) {
-    void* args[] = {&Wp, &sp, &np, &diagR, &Tg, &flag, &nb, &err};
+    void* args[] = {&Y, &Wp, &sp, &np, &diagR, &Tg, &flag, &nb, &err};
     e = cudaLaunchCooperativeKernel((const void*)kern, dim3(nblk), dim3(NT), args, smem, st);
   } else {
     cudaLaunchConfig_t cfg = {};
@@ -606,7 +618,7 @@ static cudaError_t run_qr_block(const double* Y, int64_t s, int64_t n, T* W, dou
     attr[0].val.clusterDim.z = 1;
     cfg.attrs = attr;
     cfg.numAttrs = 1;
-    e = cudaLaunchKernelEx(&cfg, kern, Wp, sp, np, diagR, Tg, flag, nb, err);
+    e = cudaLaunchKernelEx(&cfg, kern, Y, Wp, sp, np, diagR, Tg, flag, nb, err);
   }
   if (e != cudaSuccess) return e;
   qr_finalize_kernel<T><<<(unsigned)n, 256, 0, st>>>(W, s, n, diagR, R, c);
@@ -707,67 +719,45 @@ cudaError_t launch_qr(bool fp64, const double* Y, int64_t s, int64_t n, void* wo
 
 
 // ============================================================ grouped (batched) QR
-// One 1024-thread CTA per problem (s <= 1024): the reflectors of qr_kernel, v in shared
-// memory, whole trailing columns per warp (lanes over rows, one warp sum per dot
-// product); the warp that updates column k+1 also sums its squares below the diagonal
-// for the next step's norm.  W (s x (n + 1), ld = s) stays in global memory.
-template <typename T>
-__device__ __forceinline__ T block_sum_1024(T v, T* red) {
-  v = warp_sum(v);
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  __syncthreads();
-  if (lane == 0) red[warp] = v;
-  __syncthreads();
-  T t = (threadIdx.x < 32) ? red[threadIdx.x] : T(0);
-  if (warp == 0) t = warp_sum(t);
-  if (threadIdx.x == 0) red[32] = t;
-  __syncthreads();
-  return red[32];
+// The register-block form for all problems in one launch (s <= 1024): the blocks of problem p
+// are items start[p] .. start[p + 1] - 1, taken by ticket, so an item waits only for items that run
+// already.  One CTA of 1024 threads per problem, with W in global memory, took as long as its
+// largest problem's chain (n = 256, s = 1024: 4.2 ms; GQRNOW now for a batch of 32).
+template <typename T, int NB, int NT, int RPT, int C>
+__global__ void __launch_bounds__(NT, 1)
+    grouped_qr_kernel(const GQr<T>* __restrict__ tab, const int* __restrict__ start, int nprob, T* __restrict__ Tg,
+                      unsigned* __restrict__ flag, int* err) {
+  const int t = qr_ticket<C>(flag + start[nprob]);
+  const int p = group_of(start, nprob, t);
+  const GQr<T> g = tab[p];
+  qr_block_body<T, NB, NT, RPT, C>(g.Y, g.W, g.s, g.n, g.diagR, Tg + (int64_t)start[p] * NB * NB, flag + start[p],
+                                   t - start[p], err);
 }
 
-template <typename T>
-__global__ void __launch_bounds__(1024) grouped_qr_kernel(const GQr<T>* __restrict__ tab) {
-  const GQr<T>& g = tab[blockIdx.x];
-  const int64_t s = g.s, n = g.n;
-  T* W = g.W;
-  __shared__ T vs[1024];
-  __shared__ T red[33];
-  __shared__ T nrm_next;
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
-  for (int64_t e = threadIdx.x; e < s * (n + 1); e += blockDim.x) W[e] = (T)g.Y[e];
-  __syncthreads();
-  T part = 0;
-  for (int64_t t = threadIdx.x; t < s; t += blockDim.x) part += W[t] * W[t];
-  T nn = block_sum_1024(part, red);
-  for (int64_t k = 0; k < n; ++k) {
-    const T* colk = W + k * s;
-    const T alpha = sqrt(nn);
-    const T x0 = colk[k];
-    const T sgn = (x0 >= T(0)) ? T(1) : T(-1);
-    const T scale = (alpha > T(0)) ? T(1) / (alpha * (alpha + fabs(x0))) : T(0);
-    if (threadIdx.x == 0) g.diagR[k] = (double)(-sgn * alpha);
-    const int64_t len = s - k;
-    for (int64_t t = threadIdx.x; t < len; t += blockDim.x) vs[t] = (t == 0) ? x0 + sgn * alpha : colk[k + t];
-    __syncthreads();
-    for (int64_t j = k + 1 + warp; j <= n; j += nw) {
-      T* colj = W + j * s + k;
-      T d = 0;
-      for (int64_t t = lane; t < len; t += 32) d += vs[t] * colj[t];
-      const T wj = warp_sum(d) * scale;
-      T sq = 0;
-      for (int64_t t = lane; t < len; t += 32) {
-        const T val = colj[t] - wj * vs[t];
-        colj[t] = val;
-        if (t >= 1) sq += val * val;
-      }
-      if (j == k + 1) {
-        sq = warp_sum(sq);
-        if (lane == 0) nrm_next = sq;
-      }
-    }
-    __syncthreads();
-    nn = nrm_next;
-  }
+template <typename T, int NB, int NT, int RPT, int C>
+static cudaError_t run_grouped_qr(const GQr<T>* tab, const int* start, int64_t blocks, int nprob, void* work, int* err,
+                                  cudaStream_t st) {
+  T* Tg = static_cast<T*>(work);
+  unsigned* flag = reinterpret_cast<unsigned*>(Tg + (size_t)blocks * NB * NB);
+  cudaError_t e = cudaMemsetAsync(flag, 0, (blocks + 1) * sizeof(unsigned), st);   // and the ticket
+  if (e != cudaSuccess) return e;
+  const size_t smem = (size_t)NB * RPT * NT * sizeof(T);
+  auto kern = grouped_qr_kernel<T, NB, NT, RPT, C>;
+  e = allow_dyn_smem(kern, smem);
+  if (e != cudaSuccess) return e;
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3((unsigned)(blocks * C));
+  cfg.blockDim = dim3(NT);
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = st;
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeClusterDimension;
+  attr[0].val.clusterDim.x = C;
+  attr[0].val.clusterDim.y = 1;
+  attr[0].val.clusterDim.z = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = C > 1 ? 1 : 0;
+  return cudaLaunchKernelEx(&cfg, kern, tab, start, nprob, Tg, flag, err);
 }
 
 template <typename T>
@@ -778,17 +768,24 @@ __global__ void grouped_qr_finalize_kernel(const GQr<T>* __restrict__ tab, const
 }
 
 template <typename T>
-cudaError_t launch_grouped_qr(const GQr<T>* tab, const int* col_start, int64_t col_ctas, int nprob, int64_t max_n,
-                              cudaStream_t st) {
+cudaError_t launch_grouped_qr(const GQr<T>* tab, const int* blk_start, int64_t blocks, const int* col_start,
+                              int64_t col_ctas, int nprob, int64_t max_s, void* work, int* err, cudaStream_t st) {
   if (nprob <= 0) return cudaSuccess;
-  (void)max_n;
-  grouped_qr_kernel<T><<<(unsigned)nprob, 1024, 0, st>>>(tab);
-  cudaError_t e = cudaGetLastError();
+  if (max_s > 1024) return cudaErrorInvalidValue;
+  cudaError_t e;
+  if constexpr (sizeof(T) == 4)
+    e = max_s <= 512 ? run_grouped_qr<T, 8, 256, 2, 1>(tab, blk_start, blocks, nprob, work, err, st)
+                     : run_grouped_qr<T, 8, 256, 4, 1>(tab, blk_start, blocks, nprob, work, err, st);
+  else
+    e = max_s <= 512 ? run_grouped_qr<T, 4, 128, 1, 4>(tab, blk_start, blocks, nprob, work, err, st)
+                     : run_grouped_qr<T, 4, 64, 2, 8>(tab, blk_start, blocks, nprob, work, err, st);
   if (e != cudaSuccess) return e;
   grouped_qr_finalize_kernel<T><<<(unsigned)col_ctas, 256, 0, st>>>(tab, col_start, nprob);
   return cudaGetLastError();
 }
-template cudaError_t launch_grouped_qr<float>(const GQr<float>*, const int*, int64_t, int, int64_t, cudaStream_t);
-template cudaError_t launch_grouped_qr<double>(const GQr<double>*, const int*, int64_t, int, int64_t, cudaStream_t);
+template cudaError_t launch_grouped_qr<float>(const GQr<float>*, const int*, int64_t, const int*, int64_t, int, int64_t, void*,
+                                              int*, cudaStream_t);
+template cudaError_t launch_grouped_qr<double>(const GQr<double>*, const int*, int64_t, const int*, int64_t, int, int64_t,
+                                               void*, int*, cudaStream_t);
 
 }  // namespace lsq
