@@ -189,42 +189,44 @@ __device__ __forceinline__ void pass_body(PassArgs<T> p, int64_t blk, int64_t nb
   }
 }
 
-// The FP32 pass of the grouped launches (LSQR, FGMRES; rows of at most 64 float4): the body
+// The pass of the grouped launches (rows of at most 64 float4 or 256 doubles): the body
 // above with each warp's rows streamed through a ring of its own in shared memory, kRingPairs
 // row pairs ahead with asynchronous copies.  A lane copies and reads the same pieces, so the
 // ring needs no barrier.  Two rows a warp in flight, as the register form has, left HBM waiting
-// (381 us an FGMRES pass and 480 us an LSQR pass over 1.8 GB); now 294 and 410 (with 3 or 4 pairs
-// fewer CTAs fit an SM: 2 % and 1 % more for a batch of 32).
+// (381 us an FGMRES pass and 480 us an LSQR pass over 1.8 GB); now 288 and 384 (with 3 or 4 pairs
+// fewer CTAs fit an SM: 2 % and 1 % more for a batch of 32).  FP64 residual, 3.6 GB: 3.98 ms, 2.9 now
+// (1.4 of them FMAs).
 constexpr int kRingPairs = 2;
-template <int MODE>
-__device__ __forceinline__ void pass_ring_body(PassArgs<float> p, int64_t blk, int64_t nblk) {
-  static_assert(MODE == PM_LSQR || MODE == PM_FGM, "FP32 passes");
+template <typename T, int VW, int VPL, int MODE>
+__device__ __forceinline__ void pass_ring_body(PassArgs<T> p, int64_t blk, int64_t nblk) {
+  constexpr int CB = VW * (int)sizeof(T);   // bytes of a copy
+  static_assert(CB == 16 || CB == 8, "asynchronous copies");
   if (p.done && *p.done) return;
   if (p.jp) {
     const int64_t j = *p.jp;
     p.x += j * p.xstr;
     p.v += j * p.vstr;
   }
-  constexpr int VPL = 2, VW = 4;
   extern __shared__ __align__(16) unsigned char pass_smem[];
   __shared__ double sqred[8];
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int64_t gw = blk * 8 + warp, tw = nblk * 8;
   const int width = p.nv * VW;
-  float* ring = reinterpret_cast<float*>(pass_smem) + (size_t)warp * 2 * kRingPairs * width;
-  float xv[VPL][VW], acc[VPL][VW];
+  T* ring = reinterpret_cast<T*>(pass_smem) + (size_t)warp * 2 * kRingPairs * width;
+  const int nvl = (p.nv + 31) >> 5;   // vectors a lane uses
+  T xv[VPL][VW], acc[VPL][VW];
 #pragma unroll
   for (int v = 0; v < VPL; ++v) {
     const int idx = lane + 32 * v;
     if (idx < p.nv) {
-      load_vec<float, VW>(p.x + (int64_t)idx * VW, xv[v], false);
+      load_vec<T, VW>(p.x + (int64_t)idx * VW, xv[v], false);
     } else {
-      for (int k = 0; k < VW; ++k) xv[v][k] = 0.0f;
+      for (int k = 0; k < VW; ++k) xv[v][k] = T(0);
     }
 #pragma unroll
-    for (int k = 0; k < VW; ++k) acc[v][k] = 0.0f;
+    for (int k = 0; k < VW; ++k) acc[v][k] = T(0);
   }
-  const float cu = (MODE == PM_LSQR) ? (float)((p.cu_ptr ? *p.cu_ptr : 1.0) * p.cu_mul) : 0.0f;
+  const T cu = (MODE == PM_LSQR) ? (T)((p.cu_ptr ? *p.cu_ptr : 1.0) * p.cu_mul) : T(0);
   // rows i and i + tw into slots 2 s and 2 s + 1
   auto fetch = [&](int64_t i, int s) {
 #pragma unroll
@@ -234,11 +236,12 @@ __device__ __forceinline__ void pass_ring_body(PassArgs<float> p, int64_t blk, i
 #pragma unroll
         for (int v = 0; v < VPL; ++v) {
           const int idx = lane + 32 * v;
-          if (idx < p.nv)
-            asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(
-                             smem_u32(ring + (size_t)(2 * s + e) * width + idx * VW)),
-                         "l"(p.A + row * p.lda + (int64_t)idx * VW)
-                         : "memory");
+          if (idx < p.nv) {
+            const uint32_t dst = smem_u32(ring + (size_t)(2 * s + e) * width + idx * VW);
+            const T* src = p.A + row * p.lda + (int64_t)idx * VW;
+            if constexpr (CB == 16) asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(dst), "l"(src) : "memory");
+            else asm volatile("cp.async.ca.shared.global [%0], [%1], 8;" ::"r"(dst), "l"(src) : "memory");
+          }
         }
       }
     }
@@ -247,42 +250,54 @@ __device__ __forceinline__ void pass_ring_body(PassArgs<float> p, int64_t blk, i
 #pragma unroll
   for (int s = 0; s < kRingPairs; ++s) fetch(gw + 2 * s * tw, s);
   double sqacc = 0.0;   // as in the body above
-  float qkeep = 0.0f;
+  T qkeep = T(0);
   int qn = 0, slot = 0;
   for (int64_t i = gw; i < p.m; i += 2 * tw) {
     const int64_t i2 = i + tw;
     const bool has2 = i2 < p.m;
-    const float s0 = MODE == PM_LSQR ? p.uin[i] : p.v[i];
-    const float s1 = has2 ? (MODE == PM_LSQR ? p.uin[i2] : p.v[i2]) : 0.0f;
-    asm volatile("cp.async.wait_group %0;" ::"n"(kRingPairs - 1) : "memory");
-    float a[VPL][VW], a2[VPL][VW];
-    float d = 0.0f, d2 = 0.0f;
-#pragma unroll
-    for (int v = 0; v < VPL; ++v) {
-      const int idx = lane + 32 * v;
-      if (idx < p.nv) {
-        load_vec<float, VW>(ring + (size_t)(2 * slot) * width + idx * VW, a[v], false);
-      } else {
-        for (int k = 0; k < VW; ++k) a[v][k] = 0.0f;
+    T s0, s1 = T(0), b0 = T(0), b1 = T(0);
+    if constexpr (MODE == PM_RES) {
+      s0 = (T)p.r[i];
+      b0 = (T)p.b[i];
+      if (has2) {
+        s1 = (T)p.r[i2];
+        b1 = (T)p.b[i2];
       }
-      if (has2 && idx < p.nv) {
-        load_vec<float, VW>(ring + (size_t)(2 * slot + 1) * width + idx * VW, a2[v], false);
-      } else {
-        for (int k = 0; k < VW; ++k) a2[v][k] = 0.0f;
-      }
-#pragma unroll
-      for (int k = 0; k < VW; ++k) {
-        d = fma(a[v][k], xv[v][k], d);
-        d2 = fma(a2[v][k], xv[v][k], d2);
-      }
+    } else {
+      const T* sv = MODE == PM_LSQR ? p.uin : p.v;
+      s0 = sv[i];
+      if (has2) s1 = sv[i2];
     }
-    warp_sum2(d, d2);   // the sums need every piece read: the slot can be filled again
-    fetch(i + 2 * kRingPairs * tw, slot);
-    slot = slot + 1 == kRingPairs ? 0 : slot + 1;
-    float c1, c2;
+    asm volatile("cp.async.wait_group %0;" ::"n"(kRingPairs - 1) : "memory");
+    const T* ra = ring + (size_t)(2 * slot) * width;
+    const T* rb = ra + width;
+    // a row's pieces: zero past its end (and for a second row that is none)
+    auto pieces = [&](int v, T (&a)[VW], T (&a2)[VW]) {
+      const int idx = lane + 32 * v;
+#pragma unroll
+      for (int k = 0; k < VW; ++k) a[k] = a2[k] = T(0);
+      if (idx < p.nv) {
+        load_vec<T, VW>(ra + idx * VW, a, false);
+        if (has2) load_vec<T, VW>(rb + idx * VW, a2, false);
+      }
+    };
+    T d = T(0), d2 = T(0);
+#pragma unroll
+    for (int v = 0; v < VPL; ++v)
+      if (sizeof(T) == 4 || v < nvl) {
+        T a[VW], a2[VW];
+        pieces(v, a, a2);
+#pragma unroll
+        for (int k = 0; k < VW; ++k) {
+          d = fma(a[k], xv[v][k], d);
+          d2 = fma(a2[k], xv[v][k], d2);
+        }
+      }
+    warp_sum2(d, d2);
+    T c1, c2;
     if constexpr (MODE == PM_LSQR) {
       c1 = d + cu * s0;
-      c2 = has2 ? d2 + cu * s1 : 0.0f;
+      c2 = has2 ? d2 + cu * s1 : T(0);
       if (lane == 0) p.uout[i] = c1;
       if (lane == qn) qkeep = c1;
       if (has2) {
@@ -292,19 +307,32 @@ __device__ __forceinline__ void pass_ring_body(PassArgs<float> p, int64_t blk, i
       qn += 2;
       if (qn == 32) {
         sqacc = fma((double)qkeep, (double)qkeep, sqacc);
-        qkeep = 0.0f;
+        qkeep = T(0);
         qn = 0;
       }
-    } else {
+    } else if constexpr (MODE == PM_FGM) {
       c1 = s0;
       c2 = s1;
       if (lane == 0) p.az[i] = d;
       if (lane == 0 && has2) p.az[i2] = d2;
+    } else {
+      c1 = -s0;
+      c2 = -s1;
+      if (lane == 0) p.f[i] = (b0 - s0) - d;
+      if (lane == 0 && has2) p.f[i2] = (b1 - s1) - d2;
     }
+    // the pieces again from the ring: held in registers over the sum they would cost a CTA an SM
+    asm volatile("" ::: "memory");
 #pragma unroll
     for (int v = 0; v < VPL; ++v)
+      if (sizeof(T) == 4 || v < nvl) {
+        T a[VW], a2[VW];
+        pieces(v, a, a2);
 #pragma unroll
-      for (int k = 0; k < VW; ++k) acc[v][k] = fma(c1, a[v][k], fma(c2, a2[v][k], acc[v][k]));
+        for (int k = 0; k < VW; ++k) acc[v][k] = fma(c1, a[k], fma(c2, a2[k], acc[v][k]));
+      }
+    fetch(i + 2 * kRingPairs * tw, slot);
+    slot = slot + 1 == kRingPairs ? 0 : slot + 1;
   }
   asm volatile("cp.async.wait_all;" ::: "memory");
   // CTA reduction of acc (fixed order over warps), each warp's sums in its own ring
@@ -319,9 +347,9 @@ __device__ __forceinline__ void pass_ring_body(PassArgs<float> p, int64_t blk, i
     if (lane == 0) sqred[warp] = sqacc;
   }
   __syncthreads();
-  const float* all = reinterpret_cast<const float*>(pass_smem);
+  const T* all = reinterpret_cast<const T*>(pass_smem);
   for (int c = threadIdx.x; c < p.n; c += blockDim.x) {
-    float s = 0.0f;
+    T s = T(0);
 #pragma unroll
     for (int w = 0; w < 8; ++w) s += all[(size_t)w * 2 * kRingPairs * width + c];
     p.Pblk[blk * p.n + c] = s;
@@ -2111,10 +2139,7 @@ __global__ void __launch_bounds__(256)
                         int64_t items) {
   for (int64_t it = blockIdx.x; it < items; it += gridDim.x) {
     const int pr = group_of(start, nprob, it);
-    if constexpr (sizeof(T) == 4)
-      pass_ring_body<MODE>(tab[pr], it - start[pr], (int64_t)start[pr + 1] - start[pr]);
-    else
-      pass_body<T, VW, VPL, MODE>(tab[pr], it - start[pr], (int64_t)start[pr + 1] - start[pr]);
+    pass_ring_body<T, VW, VPL, MODE>(tab[pr], it - start[pr], (int64_t)start[pr + 1] - start[pr]);
     __syncthreads();   // the item's shared-memory reduction is read before the next item writes it
   }
 }
@@ -2131,8 +2156,8 @@ cudaError_t launch_grouped_pass(int mode, int vw, int vpl, const PassArgs<T>* ta
     kern<<<(unsigned)g, 256, smem, st>>>(tab, start, nprob, ctas);
     return cudaGetLastError();
   };
+  smem *= 2 * kRingPairs;   // the caller's size is 8 warps x one row
   if constexpr (sizeof(T) == 4) {
-    smem *= 2 * kRingPairs;   // the caller's size is 8 warps x one row
     if (vw != 4 || vpl != 2) return cudaErrorInvalidValue;
     if (mode == PM_LSQR) return go(grouped_pass_kernel<float, 4, 2, PM_LSQR>);
     if (mode == PM_FGM) return go(grouped_pass_kernel<float, 4, 2, PM_FGM>);
