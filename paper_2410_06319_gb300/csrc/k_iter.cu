@@ -71,7 +71,7 @@ __device__ __forceinline__ void pass_body(PassArgs<T> p, int64_t blk, int64_t nb
   __shared__ double sqred[8];
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int64_t gw = blk * 8 + warp, tw = nblk * 8;
-  const int nvl = (p.nv + 31) >> 5;   // vectors a lane uses (the grouped launches have one VPL for all problems)
+  const int nvl = (p.nv + 31) >> 5;   // vectors a lane uses (VPL is a power of two)
   T xv[VPL][VW], acc[VPL][VW];
 #pragma unroll
   for (int v = 0; v < VPL; ++v) {

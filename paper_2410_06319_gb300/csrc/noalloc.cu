@@ -5,7 +5,7 @@
 //
 // Scratch layout (one copy per device, 256-byte aligned):
 //   [0, kWorkBytes)                 working copy of Y (s x (n+1), FP32 or FP64)
-//   [kWorkBytes, +kAuxBytes)        norms, diag(R), the compact-WY T factors and flags
+//   [kWorkBytes, +kAuxBytes)        norms, diag(R), the blocks' factors and flags
 //   [kWorkBytes + kAuxBytes, +256)  grid-barrier counter and generation word
 //                                   (two unsigned), then the error word (int)
 // Must start at zero on every call: the two barrier words and the error word.
