@@ -1997,22 +1997,48 @@ template cudaError_t launch_gm_step<double>(double*, int64_t, double*, int64_t, 
                                             double*, double*, float*, int*, int, cudaStream_t, uint64_t, double,
                                             int, unsigned long long*, int);
 
-// y = H[:k,:k]^-1 g[:k]  (k = st->j): one warp, column-oriented back substitution
-__global__ void gm_solve_kernel(const GmState* st, const double* H, int ldh, const double* g, double* y) {
-  extern __shared__ double hs[];   // k x k, column-major
-  __shared__ double rhs[130];
-  const int k = st->j, lane = threadIdx.x;
-  for (int c = 0; c < k; ++c)
-    for (int i = lane; i <= c; i += 32) hs[c * k + i] = H[(int64_t)c * ldh + i];
-  for (int i = lane; i < k; i += 32) rhs[i] = g[i];
-  __syncwarp();
-  for (int i = k - 1; i >= 0; --i) {
-    const double yi = rhs[i] / hs[i * k + i];
-    __syncwarp();
-    for (int l = lane; l < i; l += 32) rhs[l] -= hs[i * k + l] * yi;
-    if (lane == 0) y[i] = yi;
-    __syncwarp();
+// y = H[:k,:k]^-1 g[:k] (k <= 128): column-oriented back substitution by one warp, the right-hand
+// side in registers.  H comes in by 128 threads and the diagonal's reciprocals are formed side
+// by side, since an FP64 quotient is a chain of some 500 cycles: yi = a / d is a product and one
+// residual correction (a / d itself where 1 / d is not finite or zero).  With the quotients in
+// the chain and one warp's loads k = 40 took 57 us, 25 now.
+constexpr int kGmSolveThreads = 128;
+__device__ __forceinline__ void gm_solve_body(int k, const double* __restrict__ H, int ldh,
+                                              const double* __restrict__ g, double* __restrict__ y, double* hs) {
+  __shared__ double rinv[kGmSolveThreads];
+  const int tid = threadIdx.x;
+#pragma unroll 4
+  for (int e = tid; e < k * k; e += kGmSolveThreads) {
+    const int c = e / k, i = e % k;
+    hs[e] = i <= c ? H[(int64_t)c * ldh + i] : 0.0;
   }
+  if (tid < k) rinv[tid] = 1.0 / H[(int64_t)tid * ldh + tid];
+  __syncthreads();
+  if (tid >= 32) return;
+  constexpr int NQ = kGmSolveThreads / 32;
+  double x[NQ];
+#pragma unroll
+  for (int q = 0; q < NQ; ++q) x[q] = tid + 32 * q < k ? g[tid + 32 * q] : 0.0;
+#pragma unroll
+  for (int q = NQ - 1; q >= 0; --q) {
+    for (int ii = min(31, k - 1 - 32 * q); ii >= 0; --ii) {
+      const int i = 32 * q + ii;
+      const double* col = hs + (size_t)i * k;
+      const double a = __shfl_sync(0xffffffffu, x[q], ii), d = col[i], ri = rinv[i];
+      double yi = a * ri;
+      yi = fma(fma(-yi, d, a), ri, yi);
+      if (!(fabs(ri) > 0.0 && fabs(ri) <= 1.7976931348623157e308)) yi = a / d;
+#pragma unroll
+      for (int p = 0; p <= q; ++p)
+        if (tid + 32 * p < i) x[p] = fma(-col[tid + 32 * p], yi, x[p]);
+      if (tid == 0) y[i] = yi;
+    }
+  }
+}
+__global__ void __launch_bounds__(kGmSolveThreads)
+    gm_solve_kernel(const GmState* st, const double* H, int ldh, const double* g, double* y) {
+  extern __shared__ double hs[];   // k x k, column-major
+  gm_solve_body(st->j, H, ldh, g, y, hs);
 }
 
 // d[i] += sum_c B[c][i] y[c] for i < len (B column-major, ld); partial sums of
@@ -2066,7 +2092,7 @@ cudaError_t launch_gm_solve(const GmState* st, const double* H, int ldh, const d
     cudaError_t e = allow_dyn_smem(gm_solve_kernel, smem);
     if (e != cudaSuccess) return e;
   }
-  gm_solve_kernel<<<1, 32, smem, s>>>(st, H, ldh, g, y);
+  gm_solve_kernel<<<1, kGmSolveThreads, smem, s>>>(st, H, ldh, g, y);
   return cudaGetLastError();
 }
 template <typename TB>
@@ -2499,25 +2525,13 @@ cudaError_t launch_grouped_arnoldi(const GGm* tab, const int* start, int64_t cta
   return cudaGetLastError();
 }
 
-// update: y = H^-1 g (one warp per problem), then r += alpha V_top y, x += Z y over the
+// update: y = H^-1 g (one CTA per problem), then r += alpha V_top y, x += Z y over the
 // problem's CTAs with the partial sums of ||alpha V_top y||^2, ||r||^2, ||Z y||^2, ||x||^2
-__global__ void grouped_gm_solve_kernel(const GGm* __restrict__ tab) {
+__global__ void __launch_bounds__(kGmSolveThreads) grouped_gm_solve_kernel(const GGm* __restrict__ tab) {
   extern __shared__ double hsm[];   // k x k, column-major
-  __shared__ double rhs[130];
   const GGm& g = tab[blockIdx.x];
   if (*g.skip) return;
-  const int k = g.st->j, lane = threadIdx.x;
-  for (int c = 0; c < k; ++c)
-    for (int i = lane; i <= c; i += 32) hsm[c * k + i] = g.H[(int64_t)c * g.ldh + i];
-  for (int i = lane; i < k; i += 32) rhs[i] = g.g[i];
-  __syncwarp();
-  for (int i = k - 1; i >= 0; --i) {
-    const double yi = rhs[i] / hsm[i * k + i];
-    __syncwarp();
-    for (int l = lane; l < i; l += 32) rhs[l] -= hsm[i * k + l] * yi;
-    if (lane == 0) g.y[i] = yi;
-    __syncwarp();
-  }
+  gm_solve_body(g.st->j, g.H, g.ldh, g.g, g.y, hsm);
 }
 
 __global__ void grouped_gm_apply_kernel(const GGm* __restrict__ tab, const int* __restrict__ start, int nprob) {
@@ -2576,7 +2590,7 @@ cudaError_t launch_grouped_gm_update(const GGm* tab, const int* start, int64_t c
   const size_t smem = (size_t)kMaxGmresBatch * kMaxGmresBatch * 8;
   cudaError_t e = allow_dyn_smem(grouped_gm_solve_kernel, smem);
   if (e != cudaSuccess) return e;
-  grouped_gm_solve_kernel<<<(unsigned)nprob, 32, smem, st>>>(tab);
+  grouped_gm_solve_kernel<<<(unsigned)nprob, kGmSolveThreads, smem, st>>>(tab);
   grouped_gm_apply_kernel<<<(unsigned)ctas, 256, 0, st>>>(tab, start, nprob);
   grouped_gm_norms_kernel<<<(unsigned)nprob, 256, 0, st>>>(tab, start);
   return cudaGetLastError();

@@ -51,3 +51,21 @@ def test_fp64_products(lsq, handle, length, n, u_r):
                                 {"arnoldi": form}, x, r)
         ex, _ = exact.forward_errors(x.cpu().numpy(), r.cpu().numpy(), xstar, rstar)
         assert ex <= 1e2 * n * 2.0 ** -53 * 10, (form, ex)
+
+
+@pytest.mark.parametrize("cap", [1, 31, 32, 33, 64, 65, 97, 127])
+def test_back_substitution_lengths(lsq, handle, cap):
+    """A tolerance that is never reached makes every correction take `cap` columns: the triangular
+    system of the update ends at every place of a register and of a warp."""
+    m, n = 700, 150
+    P = randsvd_problem(m, n, 1e2, rho=1e-2, seed=cap)
+    xstar, rstar = exact.reference_solution(P.A, P.b)
+    x, r = zeros(n), zeros(m)
+    st, info = lsq.lsq_lsir(handle, dev(P.A), dev(P.b), m, n, 600, "bf16x3", "f32", "f32", "f64", 1e-6, 7,
+                            {"gmres_maxit": cap, "gmres_tol": 1e-30, "ir_maxit": 6}, x, r)
+    assert info.gmres_its[0] == cap
+    ex, er = exact.forward_errors(x.cpu().numpy(), r.cpu().numpy(), xstar, rstar)
+    if cap > 30:
+        assert ex <= 4 * U32 and er <= 4 * U32, (ex, er)
+    else:   # one column a correction: each must not increase the error of LSQR's start
+        assert np.isfinite(ex) and ex <= 1e-3
