@@ -773,12 +773,14 @@ cudaError_t launch_grouped_qr(const GQr<T>* tab, const int* blk_start, int64_t b
   if (nprob <= 0) return cudaSuccess;
   if (max_s > 1024) return cudaErrorInvalidValue;
   cudaError_t e;
+  // the two forms of a type differ in the rows a thread holds alone: to a problem with s <= 512 the
+  // longer form adds rows of zeros, so its bits do not depend on the batch's largest s
   if constexpr (sizeof(T) == 4)
     e = max_s <= 512 ? run_grouped_qr<T, 8, 256, 2, 1>(tab, blk_start, blocks, nprob, work, err, st)
                      : run_grouped_qr<T, 8, 256, 4, 1>(tab, blk_start, blocks, nprob, work, err, st);
   else
     e = max_s <= 512 ? run_grouped_qr<T, 4, 128, 1, 4>(tab, blk_start, blocks, nprob, work, err, st)
-                     : run_grouped_qr<T, 4, 64, 2, 8>(tab, blk_start, blocks, nprob, work, err, st);
+                     : run_grouped_qr<T, 4, 128, 2, 4>(tab, blk_start, blocks, nprob, work, err, st);
   if (e != cudaSuccess) return e;
   grouped_qr_finalize_kernel<T><<<(unsigned)col_ctas, 256, 0, st>>>(tab, col_start, nprob);
   return cudaGetLastError();
