@@ -189,7 +189,7 @@ LsqrState stage_lsqr(Ctx& c, const W* Aw, int64_t ldw, const Tri<W>& tri, const 
   c.h->launches += 1;
   // u = b - A x0, A^T u  (t = -x0 so that q = A t + 1 * b)
   L((launch_axpby<double, double, W>(x0, -1.0, nullptr, 0.0, t, n, c.st)));
-  L(launch_pass_lsqr_any<W>(Aw, ldw, m, n, t, bw, nullptr, 1.0, u, P, sq, c.nblk, nullptr, c.st));
+  L(launch_pass_lsqr_any<W>(Aw, ldw, m, n, t, bw, nullptr, 1.0, u, P, sq, c.nblk, nullptr, c.st, &dst->normb));
   L(launch_lsqr_colsum<W>(P, c.nblk, n, sq, dst, true, sv, c.st));
   L(launch_lsqr_step<W>(tri, sv, v, w, z, t, vt, spart, dst, true, c.st));
   c.h->launches += 1;

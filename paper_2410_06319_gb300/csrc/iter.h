@@ -55,11 +55,13 @@ struct GmState {
 };
 
 // LSQR pass over A (FP32 copy or FP64): q_i = (A t)_i + cu * u_i (cu read from *cu_ptr
-// times cu_mul); u_out = q; Pblk[blk][c] = sum_rows q_i A_ic; sq[blk] = sum q_i^2.
+// times cu_mul); u_out = q; Pblk[blk][c] = sum_rows q_i A_ic; sq[blk] = sum q_i^2.  sq_ref (device,
+// may be null): a norm that the size of q goes with, where q is not normalised.
 template <typename TP>
 cudaError_t launch_pass_lsqr_any(const TP* A, int64_t lda, int64_t m, int64_t n, const TP* t,
                                  const TP* u_in, const double* cu_ptr, double cu_mul, TP* u_out,
-                                 TP* Pblk, double* sq, int nblk, const int* done, cudaStream_t st);
+                                 TP* Pblk, double* sq, int nblk, const int* done, cudaStream_t st,
+                                 const double* sq_ref = nullptr);
 template <typename T>
 cudaError_t launch_lsqr_colsum(const T* P, int nblk, int64_t n, const double* sq, LsqrState* st,
                                bool init, T* out, cudaStream_t s);

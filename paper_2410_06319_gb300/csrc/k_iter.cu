@@ -397,6 +397,7 @@ struct BulkArgs {
   T* uout;
   const double* cu_ptr;
   double cu_mul;
+  const double* sq_ref;        // SCALED: a norm that the size of q goes with
   const T* v;                  // FGM coefficient vector
   T* az;
   const double* r;             // RES
@@ -408,7 +409,13 @@ struct BulkArgs {
   int* err;
 };
 
-template <typename T, int VW, int VPL, int MODE>
+// 2^-e for ref in [2^e, 2^(e + 1)), |e| <= 126; 1 for 0 and non-finite ref
+__device__ __forceinline__ float pow2_near_inverse(double ref) {
+  const int e = (int)((__double_as_longlong(ref) >> 52) & 0x7FF);
+  return e == 0 || e == 0x7FF ? 1.0f : __uint_as_float((uint32_t)(127 - min(126, max(-126, e - 1023))) << 23);
+}
+
+template <typename T, int VW, int VPL, int MODE, bool SCALED = false>
 __global__ void __launch_bounds__(kBulkThreads<T>, 1) pass_bulk_kernel(BulkArgs<T> p) {
   if (p.done && *p.done) return;
   if (MODE == PM_FGM && p.jp) {
@@ -439,7 +446,13 @@ __global__ void __launch_bounds__(kBulkThreads<T>, 1) pass_bulk_kernel(BulkArgs<
   for (int v = 0; v < VPL; ++v)
 #pragma unroll
     for (int k = 0; k < VW; ++k) acc[v][k] = T(0);
-  float sqacc = 0.f;
+  // Sum of q^2.  FP64: as in pass_body, 32 rows at a time.  FP32: in single (FP64 sums cost this form
+  // 10 to 40 %: n = 600, m = 1e6 400 us, 565); SCALED, for the start's residual, which has the scale
+  // of b: of q times a power of two, since squares of |q| above 1.8e19 or below 1e-23 leave the range.
+  // (An instantiation of its own: the product cost the iterations' passes up to 4 %.)
+  constexpr bool WIDE = sizeof(T) == 8;
+  T sqacc = T(0), qkeep = T(0);
+  const float qs = SCALED ? pow2_near_inverse(*p.sq_ref) : 1.0f;
   if (warp == CW) {
     // ---------------- producer
     if (lane == 0) {
@@ -564,8 +577,12 @@ __global__ void __launch_bounds__(kBulkThreads<T>, 1) pass_bulk_kernel(BulkArgs<
             coef[e] = q;
             if (lane == 0 && in) {
               p.uout[row + e] = q;
-              sqacc = fmaf((float)q, (float)q, sqacc);
+              if constexpr (!WIDE) {
+                const float qe = SCALED ? q * qs : q;
+                sqacc = fmaf(qe, qe, sqacc);
+              }
             }
+            if (WIDE && lane == ((it * RW) & 31) + e && in) qkeep = q;
           } else if (MODE == PM_FGM) {
             coef[e] = (T)c0[e];
             if (lane == 0 && in) p.az[row + e] = d[e];
@@ -573,6 +590,10 @@ __global__ void __launch_bounds__(kBulkThreads<T>, 1) pass_bulk_kernel(BulkArgs<
             coef[e] = (T)(-c0[e]);
             if (lane == 0 && in) p.f[row + e] = (c1s[e] - c0[e]) - (double)d[e];
           }
+        }
+        if (MODE == PM_LSQR && WIDE && ((it + 1) * RW & 31) == 0) {
+          sqacc = fma(qkeep, qkeep, sqacc);
+          qkeep = T(0);
         }
 #pragma unroll
         for (int v = 0; v < VPL; ++v)
@@ -602,7 +623,10 @@ __global__ void __launch_bounds__(kBulkThreads<T>, 1) pass_bulk_kernel(BulkArgs<
         for (int k = 0; k < VW; ++k) red[warp * width + idx * VW + k] = acc[v][k];
       }
     }
-    if (MODE == PM_LSQR && lane == 0) sqred[warp] = (double)sqacc;
+    if (MODE == PM_LSQR) {
+      if constexpr (WIDE) sqacc = warp_sum(fma(qkeep, qkeep, sqacc));
+      if (lane == 0) sqred[warp] = (double)sqacc;
+    }
   }
   __syncthreads();
   for (int c = threadIdx.x; c < p.n; c += blockDim.x) {
@@ -614,13 +638,17 @@ __global__ void __launch_bounds__(kBulkThreads<T>, 1) pass_bulk_kernel(BulkArgs<
   if (MODE == PM_LSQR && threadIdx.x == 0) {
     double s = 0.0;
     for (int w = 0; w < CW; ++w) s += sqred[w];
+    if constexpr (SCALED) {
+      const double iqs = (double)__uint_as_float((254u << 23) - __float_as_uint(qs));   // 1 / qs
+      s = s * iqs * iqs;
+    }
     p.sq[blockIdx.x] = s;
   }
 }
 
 int bulk_blocks(int num_sms) { return num_sms; }
 
-template <typename T, int VW, int MODE>
+template <typename T, int VW, int MODE, bool SCALED = false>
 static cudaError_t dispatch_bulk(BulkArgs<T> p, int nblk, int num_sms_unused, cudaStream_t st) {
   const int vpl = (p.nv + 31) / 32;
   const size_t stage_bytes = (size_t)kBulkRows * p.lda * sizeof(T);
@@ -640,12 +668,12 @@ static cudaError_t dispatch_bulk(BulkArgs<T> p, int nblk, int num_sms_unused, cu
     kern<<<nblk, kBulkThreads<T>, smem, st>>>(p);
     return cudaGetLastError();
   };
-  if (vpl <= 1) return go(pass_bulk_kernel<T, VW, 1, MODE>);
-  if (vpl <= 2) return go(pass_bulk_kernel<T, VW, 2, MODE>);
-  if (vpl <= 4) return go(pass_bulk_kernel<T, VW, 4, MODE>);
-  if (vpl <= 8) return go(pass_bulk_kernel<T, VW, 8, MODE>);
+  if (vpl <= 1) return go(pass_bulk_kernel<T, VW, 1, MODE, SCALED>);
+  if (vpl <= 2) return go(pass_bulk_kernel<T, VW, 2, MODE, SCALED>);
+  if (vpl <= 4) return go(pass_bulk_kernel<T, VW, 4, MODE, SCALED>);
+  if (vpl <= 8) return go(pass_bulk_kernel<T, VW, 8, MODE, SCALED>);
   if constexpr (VW <= 2) {
-    if (vpl <= 16) return go(pass_bulk_kernel<T, VW, 16, MODE>);
+    if (vpl <= 16) return go(pass_bulk_kernel<T, VW, 16, MODE, SCALED>);
   }
   return cudaErrorInvalidValue;
 }
@@ -697,7 +725,8 @@ static bool bulk_fits(int64_t lda, int64_t nv) {
 template <typename T>
 cudaError_t launch_pass_lsqr_t(const T* A, int64_t lda, int64_t m, int64_t n, const T* t,
                                const T* u_in, const double* cu_ptr, double cu_mul, T* u_out, T* Pblk,
-                               double* sq, int nblk, const int* done, cudaStream_t st) {
+                               double* sq, int nblk, const int* done, cudaStream_t st,
+                               const double* sq_ref) {
   int vw = 4;
   bool bulk = aligned16(A);
   if constexpr (sizeof(T) == 4) {
@@ -711,9 +740,10 @@ cudaError_t launch_pass_lsqr_t(const T* A, int64_t lda, int64_t m, int64_t n, co
     BulkArgs<T> b{};
     b.A = A; b.lda = lda; b.m = m; b.n = (int)n;
     b.x = t; b.uin = u_in; b.uout = u_out; b.cu_ptr = cu_ptr; b.cu_mul = cu_mul;
-    b.Pblk = Pblk; b.sq = sq; b.done = done;
+    b.Pblk = Pblk; b.sq = sq; b.done = done; b.sq_ref = sq_ref;
     if constexpr (sizeof(T) == 4) {
       b.nv = (int)((lda + 3) / 4);
+      if (sq_ref) return dispatch_bulk<float, 4, PM_LSQR, true>(b, nblk, 0, st);
       return dispatch_bulk<float, 4, PM_LSQR>(b, nblk, 0, st);
     } else {
       if (vw == 2) {
@@ -867,15 +897,17 @@ template cudaError_t launch_colsum<float, double>(const float*, int, int64_t, co
 template <typename TP>
 cudaError_t launch_pass_lsqr_any(const TP* A, int64_t lda, int64_t m, int64_t n, const TP* t,
                                  const TP* u_in, const double* cu_ptr, double cu_mul, TP* u_out,
-                                 TP* Pblk, double* sq, int nblk, const int* done, cudaStream_t st) {
-  return launch_pass_lsqr_t<TP>(A, lda, m, n, t, u_in, cu_ptr, cu_mul, u_out, Pblk, sq, nblk, done, st);
+                                 TP* Pblk, double* sq, int nblk, const int* done, cudaStream_t st,
+                                 const double* sq_ref) {
+  return launch_pass_lsqr_t<TP>(A, lda, m, n, t, u_in, cu_ptr, cu_mul, u_out, Pblk, sq, nblk, done, st, sq_ref);
 }
 template cudaError_t launch_pass_lsqr_any<float>(const float*, int64_t, int64_t, int64_t, const float*,
                                                  const float*, const double*, double, float*, float*,
-                                                 double*, int, const int*, cudaStream_t);
+                                                 double*, int, const int*, cudaStream_t, const double*);
 template cudaError_t launch_pass_lsqr_any<double>(const double*, int64_t, int64_t, int64_t, const double*,
                                                   const double*, const double*, double, double*,
-                                                  double*, double*, int, const int*, cudaStream_t);
+                                                  double*, double*, int, const int*, cudaStream_t,
+                                                  const double*);
 
 // ------------------------------------------------------------ fused LSQR step
 // beta = ||q|| from the per-CTA sums of squares (every CTA recomputes it);
