@@ -128,11 +128,13 @@ typedef struct lsq_opts {
                              m range (each split is summed in FP32, the splits in FP64);
                              0 -> the library's choice */
   int32_t wait_limit_us;  /* limit of each grid-sync wait of the FGMRES Arnoldi step in
-                             microseconds; 0 -> 2 s */
-  int32_t expire_sync;    /* 1: the Arnoldi step's grid-sync arrival count starts past its
-                             completion value, so the first wait runs out after wait_limit_us
-                             and the call returns LSQ_E_TIMEOUT (tests the timeout path; the
-                             handle stays usable) */
+                             microseconds; 0 -> 2 s.  (Vectors of up to 2048 rows run on one
+                             thread-block cluster where the device can place one; that form has
+                             no such wait.) */
+  int32_t expire_sync;    /* 1: the Arnoldi step's grid sync waits for one arrival more than the
+                             grid makes, so the first wait runs out after wait_limit_us and the
+                             call returns LSQ_E_TIMEOUT (tests the timeout path; the handle stays
+                             usable) */
   int32_t sketch_kind;    /* 0: Gaussian embedding (Sec. 2, generated in the GEMM, precision u_s);
                              1: sparse sign embedding (Sec. 2): Omega = zeta^-1/2 (omega_1 ..
                              omega_m), omega_j with sparse_zeta entries +-1 in distinct rows

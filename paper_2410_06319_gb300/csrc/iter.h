@@ -92,6 +92,13 @@ cudaError_t launch_gm_scale0(double* V0, int64_t len, const GmState* st, float* 
 // (maxc + 1); maxc <= 128.  Each sync waits at most wait_ns (0: the library's limit; expire: one
 // arrival more than the grid makes); a wait that runs out records DEV_TIMEOUT_GRID in *err
 // and sets st->done, so the rest of the batch is skipped.
+constexpr int kGmCluster = 16;             // CTAs of the cluster: the largest size
+constexpr int64_t kGmClusterRows = 2048;   // longest vectors it takes
+// Whether the step runs on one cluster, of which `clusters` fit the device: classical Gram-Schmidt of
+// short vectors.  The timeout test (expire) needs the grid's bounded wait.
+inline bool gm_one_cluster(int64_t len, int gs, int expire, int clusters) {
+  return gs == 0 && len <= kGmClusterRows && !expire && clusters > 0;
+}
 template <typename TAZ>
 cudaError_t launch_gm_step(double* V, int64_t ld, double* w, int64_t len, int64_t m, const TAZ* az,
                            GmState* st, int maxc, double* Dp, double* sq, double* hsum, double* H, int ldh,

@@ -1644,8 +1644,6 @@ __device__ __forceinline__ void gm_row_update2(const double* __restrict__ V, int
 
 // SUMS = 1: the partials of the cluster's CTAs, part[c] in each one's shared memory, added in
 // rank order by every CTA.
-constexpr int kGmCluster = 16;   // the largest size
-constexpr int64_t kGmClusterRows = 2048;
 __device__ __forceinline__ void gm_cluster_sums(double* part, int cols, double* hs) {
   cl_sync();   // every CTA's partials are written
   for (int c = threadIdx.x; c < cols; c += blockDim.x) {
@@ -1951,6 +1949,35 @@ __global__ void __launch_bounds__(kMgsThreads, WS ? 1 : 2) gm_mgs_kernel(const G
   }
 }
 
+// Shared memory for w and the staged columns.
+constexpr size_t kGmRoom = 227 * 1024 - kMgsStaticSmem;
+
+// Clusters of kGmCluster CTAs that fit the device with all of kGmRoom (a non-portable size: none where
+// sixteen SMs of one group are not to be had, as in a slice of the GPU).
+template <typename TAZ>
+static int gm_clusters() {
+  auto kern = gm_step_kernel<TAZ, true, 1>;
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3(kGmCluster);
+  cfg.blockDim = dim3(kGmThreads);
+  cfg.dynamicSmemBytes = kGmRoom;
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeClusterDimension;
+  attr[0].val.clusterDim.x = kGmCluster;
+  attr[0].val.clusterDim.y = 1;
+  attr[0].val.clusterDim.z = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = 1;
+  int clusters = 0;
+  if (allow_dyn_smem(kern, kGmRoom) != cudaSuccess ||
+      cudaFuncSetAttribute(kern, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) != cudaSuccess ||
+      cudaOccupancyMaxActiveClusters(&clusters, kern, &cfg) != cudaSuccess) {
+    cudaGetLastError();   // no such clusters: the grid form serves
+    return 0;
+  }
+  return clusters;
+}
+
 template <typename TAZ>
 cudaError_t launch_gm_step(double* V, int64_t ld, double* w, int64_t len, int64_t m, const TAZ* az,
                            GmState* st, int maxc, double* Dp, double* sq, double* hsum, double* H, int ldh,
@@ -1960,32 +1987,27 @@ cudaError_t launch_gm_step(double* V, int64_t ld, double* w, int64_t len, int64_
   static_assert(sizeof(GmStepArgs<TAZ>) < 4096, "kernel parameter block");
   if (maxc > 128 || gs < 0 || gs > 2 || seq == nullptr) return cudaErrorInvalidValue;
   const bool mgs = gs > 0;
-  // Classical: up to kGmClusterRows rows one cluster of sixteen CTAs; up to 2^20 a cooperative
-  // launch of at most one CTA per 64 rows and SM; both with w and the basis columns that fit in
+  // Classical: up to kGmClusterRows rows one cluster of sixteen CTAs (gm_one_cluster); up to 2^20 a
+  // cooperative launch of at most one CTA per 64 rows and SM; both with w and the basis columns that fit in
   // shared memory.  From 2^20 rows on (opts.arnoldi = 1) two CTAs per SM with w in global memory
   // (more loads in flight).  Modified: one per SM with w in shared memory where one CTA's rows
   // fit (unless gs = 2), else as classical; the last CTA of every form has no rows.
   const bool lng = len >= ((int64_t)1 << 20);
-  const bool cl = !mgs && len <= kGmClusterRows && !expire;   // the timeout test needs the grid's bounded wait
+  const bool cl = gm_one_cluster(len, gs, expire, 1) && gm_one_cluster(len, gs, expire, gm_clusters<TAZ>());
   const int64_t cgs_blk = cl ? kGmCluster : std::max<int64_t>(2, std::min<int64_t>(num_sms, (len + 63) / 64 + 1));
   const int64_t row_ctas = mgs ? std::max(1, num_sms - 1) : cgs_blk - 1;
   const int64_t ws_rows = (len + row_ctas - 1) / row_ctas;
   const size_t ws_bytes = (size_t)ws_rows * 8;
-  const size_t room = 227 * 1024 - kMgsStaticSmem;
-  const bool ws = mgs ? (gs == 1 && ws_bytes <= room) : !lng;
+  const bool ws = mgs ? (gs == 1 && ws_bytes <= kGmRoom) : !lng;
   auto kern = !mgs ? (cl ? gm_step_kernel<TAZ, true, 1> : (ws ? gm_step_kernel<TAZ, true, 0> : gm_step_kernel<TAZ, false, 0>))
                    : (ws ? gm_mgs_kernel<TAZ, true> : gm_mgs_kernel<TAZ, false>);
   const int threads = mgs ? kMgsThreads : kGmThreads;
   // staged columns (classical): all maxc, or as many as fit beside w
   const size_t col_bytes = (size_t)(ws_rows | 1) * 8;
-  const int slab = (!mgs && ws && ws_bytes < room) ? (int)std::min<int64_t>(maxc, (int64_t)((room - ws_bytes) / col_bytes)) : 0;
+  const int slab = (!mgs && ws && ws_bytes < kGmRoom) ? (int)std::min<int64_t>(maxc, (int64_t)((kGmRoom - ws_bytes) / col_bytes)) : 0;
   const size_t dyn = ws ? ws_bytes + col_bytes * (size_t)slab : 0;
   if (ws) {
     cudaError_t e = allow_dyn_smem(kern, dyn);
-    if (e != cudaSuccess) return e;
-  }
-  if (cl) {
-    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
     if (e != cudaSuccess) return e;
   }
   int occ = 0;
