@@ -27,7 +27,7 @@ STATUS = {0: "LSQ_OK", 1: "LSQ_NOT_CONVERGED", -1: "LSQ_E_INVAL", -2: "LSQ_E_RAN
 
 #: kernels timed with opts.timing (order of lsq_info.kern_ms)
 KERNELS = ["sketch_gemm", "lsqr_pass", "fgmres_pass", "residual_pass", "arnoldi_step", "fgmres_trsv",
-           "sketch_fix", "spare7"]
+           "sketch_sum", "spare7"]
 
 
 class Opts(ctypes.Structure):
