@@ -147,14 +147,26 @@ void stage_qr(Ctx& c, const double* Y, double* R, double* xs, RCopies* rc) {
   }
 }
 
-struct LsqrOut {
-  LsqrState st;
+// Columns from which an FP32 solve of a single iteration is quicker with two substitutions a step than
+// with R^-1, which takes n^3 / 6 FP64 FMAs to form: R given, m = 4096, us with R^-1 / substituting: n = 600
+// 471 / 473, 704 539 / 526, 1000 857 / 710; two iterations: n = 1000 869 / 897.  (FP64, whose
+// substitutions take twice as long: n = 1000 908 / 1744 with one iteration, so always R^-1.)
+constexpr int64_t kLsqrSubstCols = 640;
+
+// The vectors of an LSQR solve in working precision W.
+template <typename W>
+struct LsqrWork {
+  const W* Aw;
+  int64_t ldw;
+  W *u, *t, *sv, *vt, *v, *w, *z, *P;
+  double *sq, *spart;
+  LsqrState* dst;
+  int maxit;
 };
 
-// Alg. 2 (LSQR start): preconditioned LSQR in working precision W from x0 -> x.
+// u = b - A x0, beta = ||u||, A^T u / beta.
 template <typename W>
-LsqrState stage_lsqr(Ctx& c, const W* Aw, int64_t ldw, const Tri<W>& tri, const double* x0,
-                     double* x) {
+LsqrWork<W> lsqr_begin(Ctx& c, const W* Aw, int64_t ldw, const double* x0) {
   StageTimer tmr(c.h, ST_LSQR);
   const int64_t n = c.n, m = c.m;
   const int64_t nvec = round_up(n, 4) + 4;
@@ -191,8 +203,23 @@ LsqrState stage_lsqr(Ctx& c, const W* Aw, int64_t ldw, const Tri<W>& tri, const 
   L((launch_axpby<double, double, W>(x0, -1.0, nullptr, 0.0, t, n, c.st)));
   L(launch_pass_lsqr_any<W>(Aw, ldw, m, n, t, bw, nullptr, 1.0, u, P, sq, c.nblk, nullptr, c.st, &dst->normb));
   L(launch_lsqr_colsum<W>(P, c.nblk, n, sq, dst, true, sv, c.st));
+  return LsqrWork<W>{Aw, ldw, u, t, sv, vt, v, w, z, P, sq, spart, dst, maxit};
+}
+
+// Alg. 2 (LSQR start): preconditioned LSQR in working precision W from x0 -> x, after lsqr_begin,
+// by products with tri.X or, without it, substitutions.
+template <typename W>
+LsqrState stage_lsqr(Ctx& c, const LsqrWork<W>& g, const Tri<W>& tri, const double* x0, double* x) {
+  StageTimer tmr(c.h, ST_LSQR);
+  const int64_t n = c.n, m = c.m, ldw = g.ldw;
+  const W* Aw = g.Aw;
+  W *u = g.u, *t = g.t, *sv = g.sv, *vt = g.vt, *v = g.v, *w = g.w, *z = g.z, *P = g.P;
+  double *sq = g.sq, *spart = g.spart;
+  LsqrState* dst = g.dst;
+  const int maxit = g.maxit;
+  const int step_launches = tri.X ? 2 : 1;
   L(launch_lsqr_step<W>(tri, sv, v, w, z, t, vt, spart, dst, true, c.st));
-  c.h->launches += 1;
+  c.h->launches += step_launches - 1;
   auto body = [&]() {
     for (int k = 0; k < kBatch; ++k) {
       const int* dn = &dst->done;
@@ -202,7 +229,7 @@ LsqrState stage_lsqr(Ctx& c, const W* Aw, int64_t ldw, const Tri<W>& tri, const 
       }
       L(launch_lsqr_colsum<W>(P, c.nblk, n, sq, dst, false, sv, c.st));
       L(launch_lsqr_step<W>(tri, sv, v, w, z, t, vt, spart, dst, false, c.st));
-      c.h->launches += 1;
+      c.h->launches += step_launches - 1;
     }
   };
   // CUDA events cannot be timed inside graphs: with opts.timing the batch is launched directly
@@ -212,7 +239,8 @@ LsqrState stage_lsqr(Ctx& c, const W* Aw, int64_t ldw, const Tri<W>& tri, const 
                                           graph_key(sizeof(W) == 4 ? "lsqr32" : "lsqr64",
                                                     {PV(Aw), ldw, m, n, PV(t), PV(u), PV(P), PV(sq),
                                                      PV(sv), PV(v), PV(w), PV(z), PV(vt), PV(spart), PV(dst),
-                                                     PV(tri.X), PV(tri.XT), c.nblk}),
+                                                     PV(tri.X), PV(tri.XT), PV(tri.R), PV(tri.L), PV(tri.DU),
+                                                     PV(tri.DL), c.nblk}),
                                           body);
   int done = 0, its = 0;
   LsqrState out{};
@@ -228,7 +256,8 @@ LsqrState stage_lsqr(Ctx& c, const W* Aw, int64_t ldw, const Tri<W>& tri, const 
     if (its > maxit + kBatch) break;  // defensive: the device flag ends the loop
   }
   // x = x0 + R^-1 z
-  L((launch_trimv<W, W, W>(false, tri, z, t, nullptr, c.st)));
+  if (tri.X) L((launch_trimv<W, W, W>(false, tri, z, t, nullptr, c.st)));
+  else L((launch_trsv<W, W, W>(true, tri, z, 1.0, t, nullptr, c.st)));
   L((launch_axpby<W, double, double>(t, 1.0, x0, 1.0, x, n, c.st)));
   return out;
 }
@@ -496,6 +525,38 @@ bool stage_refine(Ctx& c, const TOP* Aop, int64_t ldop, RCopies& rc, double* x, 
   return converged;
 }
 
+// The checks of A, b and R, and LSQR.  alone: no refinement with products in W follows, which would
+// need R^-1 in any case.
+template <typename W>
+LsqrState run_lsqr(Ctx& c, const W* Aw, int64_t ldw, RCopies& rc, bool alone, const double* x0, double* x,
+                   lsq_info* info) {
+  // A solve of a single iteration, by the cap or since ||b - A x0|| is within the tolerance already.
+  // Only where that could matter is the residual taken before R^-1 (whose kernel covers the host's
+  // launches of it) and read, with R's condition estimate.
+  const bool ask = sizeof(W) == 4 && alone && c.n >= kLsqrSubstCols;
+  bool one = ask && c.o.lsqr_maxit == 1;
+  LsqrWork<W> g{};
+  if (ask) {
+    g = lsqr_begin<W>(c, Aw, ldw, x0);
+    CK(cudaMemcpyAsync(c.h->h_pinned + 64, g.dst, sizeof(LsqrState), cudaMemcpyDeviceToHost, c.st));
+  }
+  CK(cudaMemcpyAsync(c.h->h_pinned + 32, rc.kappa, 8, cudaMemcpyDeviceToHost, c.st));
+  check_dev_error(c.h);   // waits; a NaN or an infinity in A or b (column-max pass)
+  double kap;
+  std::memcpy(&kap, c.h->h_pinned + 32, 8);
+  info->kappa_R_est = kap;
+  if (!(kap < INFINITY)) throw StatusFail{LSQ_E_RANK};
+  if (c.us != LSQ_AUTO && kap * unit_roundoff(c.us) >= 1.0) info->flags |= LSQ_WARN_COND;
+  if (ask) {
+    LsqrState s0;
+    std::memcpy(&s0, c.h->h_pinned + 64, sizeof(s0));
+    one = one || s0.beta <= s0.tol * s0.normb;
+  }
+  const Tri<W> tri = one ? rc.get<W>() : stage_inverse<W>(c, rc);
+  if (!ask) g = lsqr_begin<W>(c, Aw, ldw, x0);
+  return stage_lsqr<W>(c, g, tri, x0, x);
+}
+
 // Common front part of lsq_lsqr / lsq_lsir: sketch + QR (or R_in), LSQR.
 struct Front {
   RCopies rc;
@@ -504,7 +565,8 @@ struct Front {
   LsqrState ls;
 };
 
-Front run_front(Ctx& c, double* x, lsq_info* info) {
+// alone: see run_lsqr
+Front run_front(Ctx& c, double* x, lsq_info* info, bool alone) {
   Front fr{};
   fr.a32 = stage_cast(c);
   double* R;
@@ -547,15 +609,8 @@ Front run_front(Ctx& c, double* x, lsq_info* info) {
     if (c.o.x0_in) CK(cudaMemcpyAsync(fr.x0, c.o.x0_in, c.n * 8, cudaMemcpyDeviceToDevice, c.st));
   }
   info->us_used = (int32_t)c.us;
-  const double kap = read_scalar(c, fr.rc.kappa);
-  check_dev_error(c.h);   // a NaN or an infinity in A or b (column-max pass)
-  info->kappa_R_est = kap;
-  if (!(kap < INFINITY)) throw StatusFail{LSQ_E_RANK};
-  if (c.us != LSQ_AUTO && kap * unit_roundoff(c.us) >= 1.0) info->flags |= LSQ_WARN_COND;
-  if (c.uw == LSQ_F32)
-    fr.ls = stage_lsqr<float>(c, fr.a32, c.lda32, stage_inverse<float>(c, fr.rc), fr.x0, x);
-  else
-    fr.ls = stage_lsqr<double>(c, c.A, c.lda, stage_inverse<double>(c, fr.rc), fr.x0, x);
+  if (c.uw == LSQ_F32) fr.ls = run_lsqr<float>(c, fr.a32, c.lda32, fr.rc, alone, fr.x0, x, info);
+  else fr.ls = run_lsqr<double>(c, c.A, c.lda, fr.rc, alone, fr.x0, x, info);
   info->lsqr_its = fr.ls.its;
   info->lsqr_flag = fr.ls.flag;
   info->lsqr_normr = fr.ls.normr;
@@ -717,7 +772,7 @@ lsq_status lsq_lsqr(lsq_handle* h, const double* A, const double* b, int64_t m, 
   std::memset(inf, 0, sizeof(*inf));
   return run_guarded(h, inf, [&]() {
     StageTimer tt(c.h, ST_TOTAL);
-    Front fr = run_front(c, x, inf);
+    Front fr = run_front(c, x, inf, true);
     return fr.ls.flag != 0 ? LSQ_OK : LSQ_NOT_CONVERGED;
   });
 }
@@ -735,7 +790,7 @@ lsq_status lsq_lsir(lsq_handle* h, const double* A, const double* b, int64_t m, 
   return run_guarded(h, inf, [&]() {
     StageTimer tt(c.h, ST_TOTAL);
     double* x0 = static_cast<double*>(ws(c.h, "ir_x0", (c.n + 4) * 8));
-    Front fr = run_front(c, x0, inf);
+    Front fr = run_front(c, x0, inf, c.o.ops_escalated != 0 || c.o.ir_maxit == 1);
     double* rr = r ? r : static_cast<double*>(ws(c.h, "ir_r", c.m * 8));
     double* r0 = static_cast<double*>(ws(c.h, "ir_r0", c.m * 8));
     // r0 = b - A x0 in the working precision (Alg. 2 (initial residual))

@@ -65,9 +65,11 @@ cudaError_t launch_pass_lsqr_any(const TP* A, int64_t lda, int64_t m, int64_t n,
 template <typename T>
 cudaError_t launch_lsqr_colsum(const T* P, int nblk, int64_t n, const double* sq, LsqrState* st,
                                bool init, T* out, cudaStream_t s);
+// With f.X (launch_trinv): two launches, vv and part (n / 8 values) their scratch.  Without it (FP32):
+// one launch of one CTA that substitutes.
 template <typename T>
 cudaError_t launch_lsqr_step(const Tri<T>& f, const T* s, T* v, T* w, T* z, T* t, T* vv, double* part,
-                             LsqrState* st, bool init, cudaStream_t strm);   // part: n / 8 values
+                             LsqrState* st, bool init, cudaStream_t strm);
 
 template <typename TX, typename TY, typename TO>
 cudaError_t launch_axpby(const TX* x, double a, const TY* y, double b, TO* out, int64_t len,

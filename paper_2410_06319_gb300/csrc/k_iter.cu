@@ -1132,6 +1132,13 @@ __global__ void __launch_bounds__(kTrimvWarps * 32)
   }
 }
 
+// The step on one CTA with two substitutions, for a solve of a single iteration.
+__global__ void __launch_bounds__(kTrsvThreads)
+    lsqr_step_kernel(const Tri<float> f, const float* __restrict__ s, float* __restrict__ v, float* __restrict__ w,
+                     float* __restrict__ z, float* __restrict__ t, LsqrState* st, bool init) {
+  lsqr_step_body<float>(f, s, v, w, z, t, st, init);
+}
+
 template <typename T>
 cudaError_t launch_lsqr_colsum(const T* P, int nblk, int64_t n, const double* sq, LsqrState* st,
                                bool init, T* out, cudaStream_t s) {
@@ -1142,7 +1149,18 @@ cudaError_t launch_lsqr_colsum(const T* P, int nblk, int64_t n, const double* sq
 template <typename T>
 cudaError_t launch_lsqr_step(const Tri<T>& f, const T* s, T* v, T* w, T* z, T* t, T* vv, double* part,
                              LsqrState* st, bool init, cudaStream_t strm) {
-  if (f.n > 1024 || !f.X || !f.XT) return cudaErrorInvalidValue;
+  if (f.n > 1024) return cudaErrorInvalidValue;
+  if (!f.X || !f.XT) {
+    if constexpr (sizeof(T) == 4) {
+      const size_t smem = TrsvSmem<T>::bytes;
+      cudaError_t e = allow_dyn_smem(lsqr_step_kernel, smem);
+      if (e != cudaSuccess) return e;
+      lsqr_step_kernel<<<1, kTrsvThreads, smem, strm>>>(f, s, v, w, z, t, st, init);
+      return cudaGetLastError();
+    } else {
+      return cudaErrorInvalidValue;
+    }
+  }
   const unsigned grid = (unsigned)((f.n + kTrimvWarps - 1) / kTrimvWarps);
   lsqr_step1_kernel<T><<<grid, kTrimvWarps * 32, 0, strm>>>(f.XT, f.ld, (int)f.n, s, v, vv, part, st, init);
   lsqr_step2_kernel<T><<<grid, kTrimvWarps * 32, 0, strm>>>(f.X, f.ld, (int)f.n, vv, part, v, w, z, t, st, init);
