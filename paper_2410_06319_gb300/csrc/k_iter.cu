@@ -58,6 +58,10 @@ __device__ __forceinline__ void load_vec(const T* p, T (&o)[VW], bool streaming)
   for (int k = 0; k < VW; ++k) o[k] = e[k];
 }
 
+// The register form, for rows the bulk ring does not take (odd or unaligned FP64 strides, FP64
+// beyond 800 columns).  Every lane works on all VPL vectors, padding included: tests that leave out
+// the vectors past the row (as the other forms have for FP64) cost it 2 to 10 % at every width
+// (residual, m = 60,000 with an odd stride: n = 187 112 us without, 124 with; n = 256 116, 125).
 template <typename T, int VW, int VPL, int MODE>
 __device__ __forceinline__ void pass_body(PassArgs<T> p, int64_t blk, int64_t nblk) {
   if (p.done && *p.done) return;
@@ -71,7 +75,6 @@ __device__ __forceinline__ void pass_body(PassArgs<T> p, int64_t blk, int64_t nb
   __shared__ double sqred[8];
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int64_t gw = blk * 8 + warp, tw = nblk * 8;
-  const int nvl = (p.nv + 31) >> 5;   // vectors a lane uses (VPL is a power of two)
   T xv[VPL][VW], acc[VPL][VW];
 #pragma unroll
   for (int v = 0; v < VPL; ++v) {
@@ -86,11 +89,7 @@ __device__ __forceinline__ void pass_body(PassArgs<T> p, int64_t blk, int64_t nb
   }
   T cu = T(0);
   if (MODE == PM_LSQR) cu = (T)((p.cu_ptr ? *p.cu_ptr : 1.0) * p.cu_mul);
-  // q^2 is summed in FP64, 32 rows at a time: lane l keeps the q of the rows l, l + 32, ... of the
-  // warp's sequence (an FP64 product per row is one more serial step of 67 cycles)
-  double sqacc = 0.0;
-  T qkeep = T(0);
-  int qn = 0;
+  double sqacc = 0.0;   // lane 0: q^2 in FP64
   for (int64_t i = gw; i < p.m; i += 2 * tw) {
     const int64_t i2 = i + tw;
     const bool has2 = i2 < p.m;
@@ -114,30 +113,27 @@ __device__ __forceinline__ void pass_body(PassArgs<T> p, int64_t blk, int64_t nb
     T d = 0, d2 = 0;
 #pragma unroll
     for (int v = 0; v < VPL; ++v)
-      if (sizeof(T) == 4 || VPL >= 16 || v < nvl)   // FP64 instructions are what an FP64 pass costs
 #pragma unroll
-        for (int k = 0; k < VW; ++k) {
-          d = fma(a[v][k], xv[v][k], d);
-          d2 = fma(a2[v][k], xv[v][k], d2);
-        }
+      for (int k = 0; k < VW; ++k) {
+        d = fma(a[v][k], xv[v][k], d);
+        d2 = fma(a2[v][k], xv[v][k], d2);
+      }
     warp_sum2(d, d2);
     T c1, c2 = T(0);
     if (MODE == PM_LSQR) {
       const T q = d + cu * p.uin[i];
       c1 = q;
-      if (lane == 0) p.uout[i] = q;
-      if (lane == qn) qkeep = q;
+      if (lane == 0) {
+        p.uout[i] = q;
+        sqacc = fma((double)q, (double)q, sqacc);
+      }
       if (has2) {
         const T q2 = d2 + cu * p.uin[i2];
         c2 = q2;
-        if (lane == 0) p.uout[i2] = q2;
-        if (lane == qn + 1) qkeep = q2;
-      }
-      qn += 2;
-      if (qn == 32) {
-        sqacc = fma((double)qkeep, (double)qkeep, sqacc);
-        qkeep = T(0);
-        qn = 0;
+        if (lane == 0) {
+          p.uout[i2] = q2;
+          sqacc = fma((double)q2, (double)q2, sqacc);
+        }
       }
     } else if (MODE == PM_FGM) {
       c1 = p.v[i];
@@ -158,9 +154,8 @@ __device__ __forceinline__ void pass_body(PassArgs<T> p, int64_t blk, int64_t nb
     }
 #pragma unroll
     for (int v = 0; v < VPL; ++v)
-      if (sizeof(T) == 4 || VPL >= 16 || v < nvl)
 #pragma unroll
-        for (int k = 0; k < VW; ++k) acc[v][k] = fma(c1, a[v][k], fma(c2, a2[v][k], acc[v][k]));
+      for (int k = 0; k < VW; ++k) acc[v][k] = fma(c1, a[v][k], fma(c2, a2[v][k], acc[v][k]));
   }
   // CTA reduction of acc (fixed order over warps)
   const int width = p.nv * VW;
@@ -171,10 +166,7 @@ __device__ __forceinline__ void pass_body(PassArgs<T> p, int64_t blk, int64_t nb
       for (int k = 0; k < VW; ++k) red[warp * width + idx * VW + k] = acc[v][k];
     }
   }
-  if (MODE == PM_LSQR) {
-    sqacc = warp_sum(fma((double)qkeep, (double)qkeep, sqacc));
-    if (lane == 0) sqred[warp] = sqacc;
-  }
+  if (MODE == PM_LSQR && lane == 0) sqred[warp] = sqacc;
   __syncthreads();
   for (int c = threadIdx.x; c < p.n; c += blockDim.x) {
     T s = 0;
@@ -249,7 +241,9 @@ __device__ __forceinline__ void pass_ring_body(PassArgs<T> p, int64_t blk, int64
   };
 #pragma unroll
   for (int s = 0; s < kRingPairs; ++s) fetch(gw + 2 * s * tw, s);
-  double sqacc = 0.0;   // as in the body above
+  // q^2 is summed in FP64, 32 rows at a time: lane l keeps the q of the rows l, l + 32, ... of the
+  // warp's sequence (an FP64 product per row is one more serial step of 67 cycles)
+  double sqacc = 0.0;
   T qkeep = T(0);
   int qn = 0, slot = 0;
   for (int64_t i = gw; i < p.m; i += 2 * tw) {
@@ -446,7 +440,7 @@ __global__ void __launch_bounds__(kBulkThreads<T>, 1) pass_bulk_kernel(BulkArgs<
   for (int v = 0; v < VPL; ++v)
 #pragma unroll
     for (int k = 0; k < VW; ++k) acc[v][k] = T(0);
-  // Sum of q^2.  FP64: as in pass_body, 32 rows at a time.  FP32: in single (FP64 sums cost this form
+  // Sum of q^2.  FP64: 32 rows at a time, as in pass_ring_body.  FP32: in single (FP64 sums cost this form
   // 10 to 40 %: n = 600, m = 1e6 400 us, 565); SCALED, for the start's residual, which has the scale
   // of b: of q times a power of two, since squares of |q| above 1.8e19 or below 1e-23 leave the range.
   // (An instantiation of its own: the product cost the iterations' passes up to 4 %.)
