@@ -125,7 +125,8 @@ typedef struct lsq_opts {
                              skips sketch and QR inside lsq_lsqr/lsq_lsir */
   const double* x0_in;    /* optional device LSQR start (n); used with R_in */
   int64_t sketch_kchunk;  /* tensor-core sketch: at most this many rows of A per split of the
-                             m range (each split is summed in FP32, the splits in FP64);
+                             m range (each split is summed in FP32, the splits in FP64), in
+                             whole K steps of 64 rows (E4M3: 128) and at least one;
                              0 -> the library's choice */
   int32_t wait_limit_us;  /* limit of each grid-sync wait of the FGMRES Arnoldi step in
                              microseconds; 0 -> 2 s.  (Vectors of up to 2048 rows run on one
@@ -350,11 +351,12 @@ lsq_status lsq_lsir_host(lsq_handle* h, const double* A, const double* b, int64_
  * the Gaussian sketch; no Y_in, R_in, ops_escalated or timing): every stage runs
  * as one grouped launch over all problems -- the cast, one tensor-core sketch
  * grid over every problem's (tile, column group, split) items with per-problem
- * tensor maps and Philox keys, one QR CTA per problem, and one pass launch per
- * LSQR or FGMRES iteration covering every problem's rows, with per-problem done
- * flags -- and the iteration batches replay as CUDA graphs.  A problem's result
- * does not depend on the rest of the batch; it matches lsq_lsir's on the same
- * problem to rounding (the passes and the QR block the work differently).
+ * tensor maps and Philox keys, one QR launch over every problem's column blocks,
+ * and one pass launch per LSQR or FGMRES iteration covering every problem's rows,
+ * with per-problem done flags -- and the iteration batches replay as CUDA graphs.
+ * A problem's result does not depend on the rest of the batch; it matches
+ * lsq_lsir's on the same problem to rounding (the passes and the QR block the work
+ * differently).
  * Per-problem mode (opts->batch_mode = 1, or a batch outside that range): the
  * problems run concurrently on up to four internal streams (one worker thread
  * and one workspace per stream, created on first use and owned by the handle),

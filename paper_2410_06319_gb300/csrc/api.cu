@@ -349,7 +349,7 @@ GmOut stage_fgmres(Ctx& c, const TOP* Aop, int64_t ldop, const Tri<TOP>& tri, co
         }
         {
           KernTimer kt(c.h, K_ARNOLDI, c.o.timing);
-          L(launch_gm_step<double>(V, ld, wv, ld, m, nullptr, gst, maxc, Dp, sqp, hh, H, ldh, cs, sn, g, nullptr,
+          L(launch_gm_step<double>(V, ld, wv, ld, m, nullptr, gst, maxc, Dp, hh, H, ldh, cs, sn, g, nullptr,
                                    c.h->d_err, c.h->num_sms, c.st, wait_ns, c.alpha, mgs, gseq,
                                    c.o.expire_sync));
         }
@@ -379,7 +379,7 @@ GmOut stage_fgmres(Ctx& c, const TOP* Aop, int64_t ldop, const Tri<TOP>& tri, co
       // lost more than half of ||w||^2 ("twice is enough"); Givens step; new column
       {
         KernTimer kt(c.h, K_ARNOLDI, c.o.timing);
-        L(launch_gm_step<TOP>(V, ld, wv, ld, m, az, gst, maxc, Dp, sqp, hh, H, ldh, cs, sn, g, v32,
+        L(launch_gm_step<TOP>(V, ld, wv, ld, m, az, gst, maxc, Dp, hh, H, ldh, cs, sn, g, v32,
                               c.h->d_err, c.h->num_sms, c.st, wait_ns, c.alpha, mgs, gseq, c.o.expire_sync));
       }
     }

@@ -20,8 +20,11 @@ using namespace lsq;
 
 constexpr size_t kAlign = 256;
 constexpr int64_t kPassRowsPerCta = 1024;   // rows of A per CTA of a grouped pass
-constexpr int64_t kArnRowsPerCta = 4096;    // rows of the (m + n) vectors per Arnoldi CTA: 32 problems of
-                                            // 1e5 rows fill 3 waves of two CTAs per SM to 94 % (8192: 70 %)
+// Rows of the (m + n) vectors per Arnoldi CTA; fixed, since a problem's sums must not depend on the rest of the
+// batch.  32 problems of 1e5 rows fill 3 waves of two CTAs per SM to 94 % (8192 rows: 70 %).  Batches of two to
+// five such problems leave most SMs idle and would want less (2048 rows, ms: batches of 32 / 5 / 2 101.2 / 24.4
+// / 15.7 against 100.1 / 25.0 / 19.2): the large batch, whose time is the longer, decided.
+constexpr int64_t kArnRowsPerCta = 4096;
 
 size_t align_up(size_t v) { return (v + kAlign - 1) / kAlign * kAlign; }
 

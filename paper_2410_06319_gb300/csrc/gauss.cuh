@@ -245,7 +245,7 @@ __device__ __forceinline__ bool gauss_pair_est(uint32_t a, uint32_t b, uint32_t&
 // ------------------------------------------------------------ double-float evaluation
 // The undecided pairs: the definition's value in double-float (an unevaluated sum of two
 // FP32 numbers) on the FP32 pipe, about 250 instructions a pair against ~95 FP64 operations
-// (GB300 issues a warp's FP64 operation over 64 cycles).  Relative error of an entry: each
+// (64 cycles of a quarter of the SM each).  Relative error of an entry: each
 // product, quotient and sum below 2^-43; the FP32 tails of the series enter scaled by at
 // most 2.6e-5 (ln), 4e-7 (sin) and 3.7e-6 (cos) times 2^-23: below 2^-38 in all.  An entry
 // further than kDfRel = 2^-36 from a rounding boundary of u_s is decided; the rest (about

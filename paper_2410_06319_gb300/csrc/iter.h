@@ -103,7 +103,7 @@ inline bool gm_one_cluster(int64_t len, int gs, int expire, int clusters) {
 }
 template <typename TAZ>
 cudaError_t launch_gm_step(double* V, int64_t ld, double* w, int64_t len, int64_t m, const TAZ* az,
-                           GmState* st, int maxc, double* Dp, double* sq, double* hsum, double* H, int ldh,
+                           GmState* st, int maxc, double* Dp, double* hsum, double* H, int ldh,
                            double* cs, double* sn, double* g, float* v32, int* err,
                            int num_sms, cudaStream_t s, uint64_t wait_ns = 0, double alpha = 1.0,
                            int gs = 0, unsigned long long* seq = nullptr, int expire = 0);

@@ -363,9 +363,8 @@ __global__ void __launch_bounds__(256) pass_kernel(PassArgs<T> p) {
 // ------------------------------------------------------------ bulk-streamed passes
 // A producer warp streams stages of 16 consecutive rows of A into a shared-memory
 // ring with cp.async.bulk (completion on an mbarrier).  FP32 (bound by HBM): sixteen consumer
-// warps take a row of each stage.  FP64 (bound by its pipe, 20 cycles an instruction of a warp
-// on the SM, 67 between two of one warp, dependent or not): eight warps take two rows, whose
-// sums share a reduction (five additions instead of ten), in one chain of FMAs; with a row a
+// warps take a row of each stage.  FP64 (bound by its pipe; the
+// rates: common.cuh): eight warps take two rows, whose sums share a reduction (five additions instead of ten), in one chain of FMAs; with a row a
 // warp and four interleaved chains, n = 187 took 38 us at m = 20011 (FGMRES) and n = 500
 // 274 us at m = 1e5 (residual); now 27 and 240.  Each CTA owns a contiguous range of rows.
 // The per-row scalars of the next stage are loaded one stage ahead.
@@ -1046,6 +1045,9 @@ __device__ __forceinline__ void lsqr_step_body(const Tri<T>& f, const T* __restr
 //      vectors v, w, z.  (A CTA that starts after CTA 0 has set done skips its rows of t: no
 //      pass reads them then.)
 // On one CTA with two triangular solves the step took 20 us at n = 50 and 46 us at n = 500.
+// Accuracy: k_trsv.cu (trinv_kernel).  FP64 solves (tol 1e-14), median error of eight problems of m = 2000, n = 50
+// / m = 6000, n = 180 against extended precision, substituting: kappa 1e3 1.6e-15 / 2.2e-15, 1e6 9.4e-11 / 6.7e-11, 1e9
+// 1.5e-8 / 3.3e-9; now (with q^2 summed in FP64 too): 1.8e-15 / 2.0e-15, 3.0e-11 / 4.0e-11, 3.0e-9 / 1.9e-9.
 template <typename T>
 __global__ void __launch_bounds__(kTrimvWarps * 32)
     lsqr_step1_kernel(const T* __restrict__ XT, int64_t ld, int n, const T* __restrict__ s, const T* __restrict__ v,
@@ -1367,7 +1369,6 @@ struct GmStepArgs {
   GmState* st;
   int maxc, ldh;
   double* Dp;     // [maxc + 1][ldd] partials, one column per block (row ncols: the squared norm)
-  double* sq;     // unused (kept for the launch signature)
   double* hsum;   // [maxc + 1] column sums
   double* H;
   double* cs;
@@ -1443,8 +1444,7 @@ __device__ __forceinline__ double gm_task(const double* __restrict__ V, int64_t 
 
 // Partials of V^T w and ||w||^2 over the CTA's rows [r0, r1) into Dp[c * ldd + blk], c <= ncols.
 // nfit: the first nfit columns (a multiple of eight, or all) are also in shared memory, row i
-// of column c at Vs[c * vld + i] (vld odd).  Two forms, by the FP64 instructions they take (20
-// cycles of the SM's pipe each):
+// of column c at Vs[c * vld + i] (vld odd).  Two forms, by the FP64 instructions they take:
 //  * lanes over rows, a warp per (group of eight sums, slice of rows), a nine-addition
 //    reduction per task;
 //  * lanes over the sums (all columns in shared memory, at most 32 sums): a row per
@@ -1819,10 +1819,11 @@ __global__ void __launch_bounds__(kGmThreads, WS ? 1 : 2) gm_step_kernel(const G
 // the eight products of block k with w (sweep K: ||w||^2); each sweep ends in one grid sum.
 // 2(j+1) FP64 FMAs per row, the least any Gram-Schmidt form needs for j+1 projections
 // (classical Gram-Schmidt with its second pass takes 4(j+1)); GB300's FP64 rate, not HBM,
-// bounds the step at m in the millions.  The columns of a block are orthonormal to working
-// accuracy, so projecting on eight at once loses no more than one after the other does,
-// with an eighth of the grid sums (about 4 us each: column by column, m = 1e6, j = 20 took 222
-// us a step, 152 us now, 67 us of them FMAs).
+// bounds the step at m in the millions.  Projecting on eight columns at once can leave
+// the basis less orthogonal than one after the other does (||V^T V - I|| 0.9 to 2.3 times as large,
+// emulated on the preconditioned augmented system, kappa 10 to 1e7); FGMRES takes the same iterations
+// to the same residual.  It needs an eighth of the grid sums (about 4 us each: column by column,
+// m = 1e6, j = 20 took 222 us a step, 152 us now, 67 us of them FMAs).
 // Each row stays with one thread from sweep to sweep, so w needs no barrier between
 // sweeps.  WS: the CTA's rows of w live in shared memory for the whole step (one CTA per
 // SM; rows of [r; x] up to 152 x ~27,000), so a sweep reads only block k from HBM and block k-1
@@ -1992,7 +1993,7 @@ static int gm_clusters() {
 
 template <typename TAZ>
 cudaError_t launch_gm_step(double* V, int64_t ld, double* w, int64_t len, int64_t m, const TAZ* az,
-                           GmState* st, int maxc, double* Dp, double* sq, double* hsum, double* H, int ldh,
+                           GmState* st, int maxc, double* Dp, double* hsum, double* H, int ldh,
                            double* cs, double* sn, double* g, float* v32, int* err,
                            int num_sms, cudaStream_t s, uint64_t wait_ns, double alpha, int gs,
                            unsigned long long* seq, int expire) {
@@ -2027,7 +2028,7 @@ cudaError_t launch_gm_step(double* V, int64_t ld, double* w, int64_t len, int64_
   if (e != cudaSuccess) return e;
   if (occ < 1) return cudaErrorInvalidConfiguration;
   const int nblk = ws ? (int)row_ctas + 1 : std::max(2, num_sms * (occ >= 2 && lng ? 2 : 1));
-  GmStepArgs<TAZ> a{V, ld, len, m, w, az, st, maxc, 0, Dp, sq, hsum, H, cs, sn, g, v32, err};
+  GmStepArgs<TAZ> a{V, ld, len, m, w, az, st, maxc, 0, Dp, hsum, H, cs, sn, g, v32, err};
   a.ldh = ldh;
   a.ldd = 4 * num_sms;   // the caller's Dp holds (maxc + 17) x 4 num_sms values
   a.wait_ns = wait_ns > 0 ? wait_ns : kWaitLimitNs;
@@ -2055,11 +2056,11 @@ cudaError_t launch_gm_step(double* V, int64_t ld, double* w, int64_t len, int64_
   return cudaLaunchKernelEx(&cfg, kern, a);
 }
 template cudaError_t launch_gm_step<float>(double*, int64_t, double*, int64_t, int64_t, const float*, GmState*,
-                                           int, double*, double*, double*, double*, int, double*, double*,
+                                           int, double*, double*, double*, int, double*, double*,
                                            double*, float*, int*, int, cudaStream_t, uint64_t, double, int,
                                            unsigned long long*, int);
 template cudaError_t launch_gm_step<double>(double*, int64_t, double*, int64_t, int64_t, const double*,
-                                            GmState*, int, double*, double*, double*, double*, int, double*,
+                                            GmState*, int, double*, double*, double*, int, double*,
                                             double*, double*, float*, int*, int, cudaStream_t, uint64_t, double,
                                             int, unsigned long long*, int);
 

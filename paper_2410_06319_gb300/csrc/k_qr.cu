@@ -5,10 +5,11 @@
 //
 // Reflector k (Golub & Van Loan): x = W[k:, k], alpha = ||x||, v = x + sign(x_1)
 // alpha e_1, H = I - v v^T / (alpha (alpha + |x_1|)); R_kk = -sign(x_1) alpha.
-// One cooperative launch runs all n steps; per step every block loads v into
-// shared memory, each block updates whole trailing columns (block-wide
-// reductions), the block owning column k+1 also leaves its squared norm for
-// the next step, and a bounded grid barrier separates the steps.
+//
+// s <= 4096 (and the batch, s <= 1024): column blocks in registers, one launch (qr_block_kernel).
+// Longer columns: qr_kernel (FP32) and qr64_kernel (FP64), one cooperative launch of n steps; per step
+// every CTA loads v into shared memory and updates whole trailing columns, the one owning column k+1
+// also leaves its squared norm for the next step, and a bounded grid barrier separates the steps.
 #include <algorithm>
 #include <cooperative_groups.h>
 
@@ -251,7 +252,7 @@ __device__ __forceinline__ T warp_reduce_scatter(T (&v)[N], int lane) {
 
 //
 // C > 1: a block's rows are spread over a cluster of C CTAs, so that the chain of a block (in FP64
-// one instruction of a warp takes 67 cycles) has C SMs; the partial sums go to every CTA of the
+// a warp issues an instruction in 67 cycles) has C SMs; the partial sums go to every CTA of the
 // cluster, one cluster barrier a reduction.  Blocks are taken by ticket (flag[nblk]), so they
 // need not all be resident: a block waits only for blocks that run already.  FP64 with the
 // columns in shared memory and a flag per column (one SM's FP64 rate bound the pivot column):
@@ -294,7 +295,7 @@ __device__ __forceinline__ void qr_block_body(const double* __restrict__ Y, T* _
   __shared__ T cw[C > 1 ? 2 : 1][C][NB * NB], cd[C > 1 ? 2 : 1][C][NB];
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int rank = C > 1 ? (int)cl_rank() : 0;
-  // Row i of a thread.  The 128-row pieces go round the cluster, so that its CTAs keep equal
+  // Row i of a thread.  The pieces of NT rows go round the cluster, so that its CTAs keep equal
   // shares while the factored rows grow; FP64 leaves out the pieces that hold none of a
   // reflector's rows.
   auto row = [&](int i) { return (i * C + rank) * NT + tid; };
@@ -597,7 +598,9 @@ static cudaError_t run_qr_block(const double* Y, int64_t s, int64_t n, T* W, dou
   int nb = (int)nblk;
   size_t smem = (size_t)NB * RPT * NT * sizeof(T);
   // at most three CTAs an SM: with more, the FP64 instructions of the block that all others wait
-  // for queue behind theirs (s = 4000, n = 1000: 13.2 ms with four, 12.3 with three, 17 with two)
+  // for queue behind theirs (s = 4000, n = 1000: 13.2 ms with four, 12.3 with three, 17 with two;
+  // without the limit / with it, ms: s = 2000, n = 500 3.48 / 3.15, 1000 x 250 1.30 / 1.26, 500 x 125 and
+  // FP32 the same)
   if (C > 1) smem = std::max(smem, (size_t)74 * 1024);
   auto kern = qr_block_kernel<T, NB, NT, RPT, C>;
   e = allow_dyn_smem(kern, smem);

@@ -8,8 +8,9 @@
 //    columns of [A | b] in TMEM (FP32), a split of the m range.  Warp 0 feeds
 //    Bt tiles by TMA, warp 1 issues tcgen05.mma (kind::f16 or kind::f8f6f4),
 //    sixteen generator warps synthesise the sketch tile fl_s(G) in registers
-//    and store it swizzled into shared memory; four warps drain TMEM into an
-//    FP32 partial per split.  G is never stored in global memory.
+//    and store it swizzled into shared memory, fixer warps settle the entries
+//    that their estimate leaves open, and the generators drain TMEM into an FP32
+//    partial per split.  G is never stored in global memory.
 //  * CUDA-core sketch for u_s = F64 / F32 (no tensor-core format).
 //  * reduce: FP64 sum of the split partials, times s^-1/2 and 2^-k_j.
 #include <cudaTypedefs.h>
@@ -390,7 +391,7 @@ constexpr size_t kSkSmem = 232448;           // the SM's shared memory: one CTA 
 // waiting for the refill's latency.  Rings, 128-byte rows and fixer groups together: BF16, m =
 // 1e5, n = 500, s = 2000 459 -> 355 us (instruction issue of the generators), F16, m = 2e5, n =
 // 1000, s = 3000 2.50 -> 1.65 ms, BF16X3, m = 2e5, n = 1000, s = 4000 4.99 -> 3.5 ms (tensor
-// pipe 42 -> 60 %).
+// pipe 42 -> 59 %).
 constexpr int sk_a_ring(int nt) { return nt == 1 ? 4 : 3; }
 constexpr int kSkBRing = 16;
 constexpr size_t kSkCtrl = 5120;             // barriers and queue counters (512 bytes), queues
@@ -414,16 +415,16 @@ __device__ __forceinline__ uint32_t swz_chunk(int row, int kc) {
 // Y partial = fl_s(G)[128 rows] x (sum over NT planes of Bt)[bn columns] over one split of m.
 //
 // A stage passes through three groups of warps: the generators write the tile from FP32
-// estimates and queue the pairs that the estimate leaves undecided (gauss.cuh: about 1 %
-// for BF16, 3 % for F16); the fixers evaluate those in double-float and patch the tile while
-// the generators are on the next stage; the MMA warp multiplies it.  So the GEMM always
-// multiplies fl_s(G) itself.
+// estimates and queue the pairs that the estimate leaves undecided (gauss.cuh); the fixers
+// evaluate those in double-float and patch the tile while the generators are on the next stage;
+// the MMA warp multiplies it.  So the GEMM always multiplies fl_s(G) itself.
 //
 // What bounds it: the generators' instruction issue where n is below about 500 a format
-// term, the tensor pipe and the refill of Bt beyond.  (With the earlier FP32 estimate, 176
-// instructions a pair against 72 now, BF16, m = 1e5, n = 500, s = 2000 took 706 us.)  Before, the GEMM multiplied the estimates, kept lists of the undecided
-// pairs and a second kernel evaluated them in FP64 and corrected the partials: 17 ms beside
-// the GEMM's 17 ms for F16 at m = 1e6, n = 1000, s = 3000, a host round trip to see whether
+// term; beyond, a stage's way through generators, fixers and MMA with the refill of Bt (F16, n =
+// 1000: issue 56 %, tensor pipe 30 % busy; BF16X3 37 % and 59 %).  (With the earlier FP32 estimate,
+// 176 instructions a pair against 72 now, BF16, m = 1e5, n = 500, s = 2000 took 706 us.)  Before,
+// the GEMM multiplied the estimates, kept lists of the undecided pairs and a second kernel
+// evaluated them in FP64 and corrected the partials: 17 ms beside the GEMM's 17 ms for F16 at m = 1e6, n = 1000, s = 3000, a host round trip to see whether
 // a list had overflowed, and in E4M3, whose subnormal range no estimate decided, always a
 // second GEMM with every such pair in FP64 (131 ms at m = 6e5, n = 601, s = 1803).
 //
